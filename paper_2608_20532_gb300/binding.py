@@ -300,9 +300,8 @@ class Store:
                                             m.ctypes.data if m is not None else None, ctypes.byref(h),
                                             ok.ctypes.data, _stream(stream)), "f2_merge_bases")
         d = np.zeros(int(num_groups), np.int32)
-        for c in range(len(g)):
-            if g[c] >= 0:
-                d[g[c]] = self.n_bits[c] + (0 if self.raw else 1)
+        member = g >= 0
+        d[g[member]] = self.n_bits[member] + (0 if self.raw else 1)
         return Store(d, raw=True, device=self.device, _handle=h), ok[:int(num_groups)]
 
     def learn_timing(self, stream=None) -> np.ndarray:

@@ -370,7 +370,8 @@ struct f2_store {
     bool widths_ready;
     std::vector<int32_t> n_bits;
     std::vector<int64_t> slot_off, xw_off, pw_off;
-    // device memory
+    // device memory: the arrays up to full_first are parts of one allocation
+    void* slab;
     f2::CtxDesc* desc;
     int32_t* rank;
     uint8_t* contra;
