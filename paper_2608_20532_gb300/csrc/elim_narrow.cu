@@ -1,0 +1,41 @@
+// Elimination of the contexts of SMALL_WD + 1 .. NARROW_WD words (96 < d <= 288).
+#include "elim.cuh"
+
+namespace f2 {
+namespace {
+
+// CTA-owned contexts first (longest first), then warp-owned ones, 16 warps per
+// SM at 128 registers.  Launched with CTAs of eight warps or, in long calls, of
+// four: a CTA-owned context's insertions run one warp at a time, so smaller
+// groups waste less; in a short call the longest CTA-owned contexts bound the
+// call and keep eight warps each.
+__global__ void __launch_bounds__(LEARN_WARPS * 32, 2) elim_narrow_kernel(StoreDev s, LearnArgs a)
+{
+    extern __shared__ __align__(16) uint32_t smem[];
+    elim_queues<CLS_CTA, CLS_WARP, CLS_RESUME>(s, a, smem, a.warp_region_words, [&](int c, auto cta, uint32_t* region, int words) {
+        switch (s.desc[c].wd) {
+        case 4: elim_one<4, decltype(cta)::value>(s, a, c, region, words); break;
+        case 5: elim_one<5, decltype(cta)::value>(s, a, c, region, words); break;
+        case 6: elim_one<6, decltype(cta)::value>(s, a, c, region, words); break;
+        case 7: elim_one<7, decltype(cta)::value>(s, a, c, region, words); break;
+        case 8: elim_one<8, decltype(cta)::value>(s, a, c, region, words); break;
+        case 9: elim_one<9, decltype(cta)::value>(s, a, c, region, words); break;
+        default: break;
+        }
+    });
+}
+
+}  // namespace
+
+cudaError_t elim_launch_narrow(const StoreDev& sd, LearnArgs la, int max_words, int warps, int num_sms, cudaStream_t cs)
+{
+    return launch_queues(elim_narrow_kernel, sd, la, max_words, la.warp_region_words, warps, 16 / warps, num_sms, cs);
+}
+
+cudaError_t elim_load_narrow()
+{
+    cudaFuncAttributes fa;
+    return cudaFuncGetAttributes(&fa, elim_narrow_kernel);
+}
+
+}  // namespace f2

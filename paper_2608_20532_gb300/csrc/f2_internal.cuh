@@ -30,8 +30,8 @@ constexpr int NARROW_WD = 9;         // widest row (32-bit words) handled by the
 constexpr int LEARN_WARPS = 8;       // warps per CTA of the narrow learn kernel
 constexpr int WIDE_WARPS = 8;        // warps per CTA of the wide learn kernel
 constexpr int PLAN_BUCKETS = 48;     // log2(work) buckets for longest-first ordering
-constexpr int DEFAULT_WARP_REGION_BYTES = 12288;  // shared memory of one warp-owned context
-constexpr int DEFAULT_SMALL_REGION_BYTES = 4096;  // the same in the small-width kernel (d <= 96)
+constexpr int DEFAULT_WARP_REGION_BYTES = 13824;  // shared memory of one warp-owned context
+constexpr int DEFAULT_SMALL_REGION_BYTES = 9472;  // the same in the small-width kernel (d <= 96)
 constexpr int64_t DEFAULT_ENCODE_DIRECT_MAX = 65536;  // encode passes this small skip the grouping
 constexpr int64_t DEFAULT_LONG_CALL_ROWS = int64_t(1) << 25;  // learn calls this long: 4-warp CTAs (4..9 words)
 constexpr int64_t DEFAULT_HANDOFF_REPS = 0;  // representatives left for a saturated context to hand off (0: never)
@@ -72,8 +72,10 @@ enum Class {
     CLS_DDW_QUAD = 10,
     CLS_DDW_WARP = 11,
     CLS_WIDE_M = 12,   // elimination of rows of 10..17 words (a narrower instance of the wide kernel)
-    CLS_RESUME = 13,   // handed-off contexts sent back by the check (their queue head only)
-    NUM_CLASSES = 14
+    CLS_RESUME = 13,   // handed-off contexts sent back by the check (their queue heads only),
+    CLS_RESUME_S = 14, // taken up by the 4..9-word, small-width and 10..17-word kernels
+    CLS_RESUME_W = 15,
+    NUM_CLASSES = 16
 };
 static_assert(NUM_CLASSES <= CNT_BEGIN - CNT_HEAD, "counter blocks hold one entry per class");
 constexpr int SMALL_WD = 3;

@@ -35,12 +35,11 @@
 // to large ones; contexts wider than 288 bits (d up to 1025) are eliminated
 // by a separate wide kernel.  Single-block plan kernels validate the CSR
 // batch and order the work longest-first.
-#include <limits.h>
 #include <string.h>
 
 #include <mutex>
 
-#include "f2_internal.cuh"
+#include "elim.cuh"
 
 using namespace f2;
 
@@ -78,36 +77,6 @@ struct CheckArgs {
     int32_t* resume_from;
 };
 
-struct LearnArgs {
-    const int64_t* row_off;
-    const int64_t* x_off;
-    const uint32_t* x;
-    const uint4* y;
-    const int32_t* rep_list;   // representatives (row indices, per-context at row_off[c]); NULL = every row
-    const int32_t* rep_dup;    // duplicates of each representative (NULL = none)
-    const int32_t* rep_count;  // representatives per context (NULL = all rows)
-    const int32_t* queue;
-    int* counters;
-    int warp_region_words;
-    // contexts that reach full rank with rows left (not deduplicated): listed
-    // here, the rest of their rows checked by verify_full_kernel
-    int* late_count;
-    int32_t* late_list;
-    int32_t* late_start;
-    unsigned long long* timing;  // per-context timestamps (F2_OPT_TIMING), NULL = off
-    int tables;                  // reduce against a lookup table of the snapshot where it pays
-    int small_region_words;      // shared memory of a warp-owned context of the small-width kernel
-    int cta_region_words;        // shared memory of a CTA-owned context (the launch's dynamic size)
-    // a CTA-owned context whose rank has not grown for HANDOFF_QUIET rounds,
-    // with at least handoff_min representatives left, stops and is listed
-    // here: check_snap_kernel checks the rest against its basis in parallel
-    int handoff_min;             // 0 = never
-    int* snap_count;
-    int32_t* snap_list;
-    int32_t* snap_start;         // its first representative left
-    const int32_t* resume_from;  // resume_kernel: the first representative of each listed context
-};
-
 struct DedupArgs {
     const int64_t* row_off;
     const int64_t* x_off;
@@ -123,35 +92,7 @@ struct DedupArgs {
     int32_t* shard_done;         // [C]: shards of a split context finished (the last one compacts)
 };
 
-// Per-context timestamps of a learn call (diagnostics, F2_OPT_TIMING):
-// TIME_WORDS words per context -- %globaltimer at the start and end of its
-// duplicate pass and of its elimination, then the SM ids that ran them.
-constexpr int TIME_WORDS = 6;
-__device__ __forceinline__ unsigned smid()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void time_mark(unsigned long long* timing, int c, int slot)
-{
-    if (timing) {
-        timing[(size_t)TIME_WORDS * c + slot] = global_ns();
-        timing[(size_t)TIME_WORDS * c + 4 + (slot >> 1)] = smid();
-    }
-}
-
-// Shared-memory control area of an elimination group (32-bit words).
-constexpr int CTL_P = 0;       // pivot mask, 48 words
-constexpr int CTL_NPR = 48;    // pivots added during the current round, 48 words
-constexpr int CTL_CAND = 96;   // per-warp candidate ballots, 32 words
-constexpr int CTL_RANK = 160;  // rank
-constexpr int CTL_CNT = 162;   // contradiction count (uint64, 8-byte aligned)
-constexpr int CTL_FIRST = 164; // first contradiction index (int64)
-constexpr int CTL_WORDS = 176; // size of the control area (16-byte multiple)
-
 constexpr int FULL_THREADS = 1024;  // verify_full_kernel: one table shared by 32 warps
-constexpr int FULL_CHUNK = 2048;   // rows of a full-rank context claimed at a time
 
 // Pass 1: 16 warps per CTA, two CTAs per SM (64 registers a thread: the pass
 // is bound by dependent per-row chains, so warps hide latency better than
@@ -197,28 +138,7 @@ constexpr int DD_PROMOTE_MIN_ROWS = 1024;
 constexpr int DD_SHARD_MIN_ROWS = 2048;
 static_assert(DD_WARPS * DD_WARP_REGION * 4 <= DD_SMEM, "warp regions exceed the dedup shared memory");
 
-__host__ __device__ __forceinline__ int elim_words(int d, int wd) { return CTL_WORDS + d * row_stride(wd); }
-
-// Dispatch on a width 1..9 (feature words) to a template instantiation.
-#define F2_SMALL_SWITCH(wd, CALL)    \
-    switch (wd) {                    \
-    case 1: CALL(1); break;          \
-    case 2: CALL(2); break;          \
-    case 3: CALL(3); break;          \
-    default: break;                  \
-    }
-
-#define F2_BIG_SWITCH(wd, CALL)      \
-    switch (wd) {                    \
-    case 4: CALL(4); break;          \
-    case 5: CALL(5); break;          \
-    case 6: CALL(6); break;          \
-    case 7: CALL(7); break;          \
-    case 8: CALL(8); break;          \
-    case 9: CALL(9); break;          \
-    default: break;                  \
-    }
-
+// Dispatch on a feature-row width to a template instantiation.
 #define F2_XWIDE_SWITCH(wd, CALL)    \
     switch (wd) {                    \
     case 10: CALL(10); break;        \
@@ -246,61 +166,6 @@ __host__ __device__ __forceinline__ int elim_words(int d, int wd) { return CTL_W
     }
 
 
-__device__ __forceinline__ bool nonzero4(const uint4& v) { return (v.x | v.y | v.z | v.w) != 0u; }
-
-__device__ __forceinline__ void xor4(uint4& a, const uint4& b)
-{
-    a.x ^= b.x;
-    a.y ^= b.y;
-    a.z ^= b.z;
-    a.w ^= b.w;
-}
-
-// Bit v set iff feature word v (< wd) still has a non-pivot column.  Words
-// made only of pivot columns are never XOR-ed: the residual is zero there.
-template <int WD>
-__device__ __forceinline__ uint64_t mixed_words(const uint32_t (&P)[WD], int d, int wd)
-{
-    uint64_t m = 0;
-#pragma unroll
-    for (int v = 0; v < WD; ++v) {
-        if (v < wd) {
-            const uint32_t valid = (v < wd - 1 || (d & 31) == 0) ? 0xffffffffu : ((1u << (d & 31)) - 1u);
-            if (P[v] != valid) m |= 1ull << v;
-        }
-    }
-    return m;
-}
-
-// Feature words exactly as supplied (bits >= n cleared), and the word.
-template <int WD>
-__device__ __forceinline__ void load_raw(const uint32_t* __restrict__ xrow, const uint4* __restrict__ yrow,
-                                         bool valid, int n, int xw, uint32_t (&xin)[WD], uint4& y)
-{
-#pragma unroll
-    for (int v = 0; v < WD; ++v) {
-        uint32_t t = 0;
-        if (valid && v < xw) t = __ldg(xrow + v);
-        if (v == xw - 1 && (n & 31)) t &= (1u << (n & 31)) - 1u;
-        xin[v] = t;
-    }
-    y = valid ? __ldg(yrow) : make_uint4(0, 0, 0, 0);
-}
-
-// q = [1 || x] (index 0 = constant) or x itself for raw feature rows.
-template <int WD>
-__device__ __forceinline__ void make_q(const uint32_t (&xin)[WD], bool valid, uint32_t raw, uint32_t (&q)[WD])
-{
-    if (raw) {
-#pragma unroll
-        for (int v = 0; v < WD; ++v) q[v] = xin[v];
-    } else {
-        q[0] = (xin[0] << 1) | (valid ? 1u : 0u);
-#pragma unroll
-        for (int v = 1; v < WD; ++v) q[v] = (xin[v] << 1) | (xin[v - 1] >> 31);
-    }
-}
-
 // 32-bit hash of an observation (feature words and word): FNV-1a over the
 // words, then a murmur-style finalizer.
 template <int WD>
@@ -319,13 +184,6 @@ __device__ __forceinline__ uint32_t hash_row(const uint32_t (&xin)[WD], const ui
     h *= 0xC2B2AE35u;
     h ^= h >> 16;
     return h;
-}
-
-template <bool CTA>
-__device__ __forceinline__ void group_sync()
-{
-    if (CTA) __syncthreads();
-    else __syncwarp();
 }
 
 // ------------------------------------------------------------------ pass 1
@@ -738,642 +596,6 @@ __global__ void __launch_bounds__(DD_THREADS, DD_CTAS_PER_SM) dedup_kernel(Store
     }
 }
 
-// Step (1) against the snapshot S.  On return the residual is zero at every
-// pivot column of words that are not "mixed"; the caller masks with ~P.
-template <int WD>
-__device__ __forceinline__ void reduce_snapshot(uint32_t (&xr)[WD], uint4& yr, const uint32_t* __restrict__ S,
-                                                const uint32_t (&P)[WD], uint64_t mixed)
-{
-    constexpr int RS = row_stride(WD);
-    // A stored row never changes another pivot bit of the lane's row, so the
-    // bit that selects row b is the row's own bit b however the rows are
-    // ordered: two pivots are taken per step, their loads issued together.
-#pragma unroll
-    for (int w = 0; w < WD; ++w) {
-        uint32_t uw = __reduce_or_sync(FULL, xr[w] & P[w]);
-        const bool xwork = (mixed & ((2ull << w) - 1ull)) != 0;
-        const uint32_t sel = xr[w];
-        while (uw) {
-            const int b0 = __ffs(uw) - 1;
-            uw &= uw - 1;
-            const bool two = uw != 0u;
-            const int b1 = two ? __ffs(uw) - 1 : b0;
-            uw &= uw - 1;
-            const uint32_t* row0 = S + (32 * w + b0) * RS;
-            const uint32_t* row1 = S + (32 * w + b1) * RS;
-            const uint32_t m0 = 0u - ((sel >> b0) & 1u);
-            const uint32_t m1 = two ? 0u - ((sel >> b1) & 1u) : 0u;
-            const uint4 z0 = *reinterpret_cast<const uint4*>(row0);
-            const uint4 z1 = *reinterpret_cast<const uint4*>(row1);
-            yr.x ^= (z0.x & m0) ^ (z1.x & m1);
-            yr.y ^= (z0.y & m0) ^ (z1.y & m1);
-            yr.z ^= (z0.z & m0) ^ (z1.z & m1);
-            yr.w ^= (z0.w & m0) ^ (z1.w & m1);
-            if (xwork) {
-#pragma unroll
-                for (int v4 = 0; v4 <= w / 4; ++v4) {
-                    const uint4 xa = *reinterpret_cast<const uint4*>(row0 + 4 + 4 * v4);
-                    const uint4 xb = *reinterpret_cast<const uint4*>(row1 + 4 + 4 * v4);
-                    const uint32_t ea[4] = {xa.x, xa.y, xa.z, xa.w};
-                    const uint32_t eb[4] = {xb.x, xb.y, xb.z, xb.w};
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int v = 4 * v4 + j;
-                        if (v <= w && v < WD)
-                            if ((mixed >> v) & 1ull) xr[v] ^= (ea[j] & m0) ^ (eb[j] & m1);
-                    }
-                }
-            }
-        }
-    }
-}
-
-// Reduce a candidate (already zero at the snapshot's pivots) against rows
-// inserted earlier in the same round (CTA mode).  Per lane.
-template <int WD>
-__device__ __forceinline__ void reduce_new(uint32_t (&xr)[WD], uint4& yr, const uint32_t* __restrict__ S,
-                                           const uint32_t* __restrict__ NPR)
-{
-    constexpr int RS = row_stride(WD);
-#pragma unroll
-    for (int w = 0; w < WD; ++w) {
-        uint32_t m = xr[w] & NPR[w];
-        while (m) {
-            const int b = __ffs(m) - 1;
-            m &= m - 1;
-            const uint32_t* row = S + (32 * w + b) * RS;
-            xor4(yr, *reinterpret_cast<const uint4*>(row));
-#pragma unroll
-            for (int v = 0; v <= w; ++v) xr[v] ^= row[4 + v];
-        }
-    }
-}
-
-// Steps (4)-(5) for the candidate lanes of one warp, in lane (= stream)
-// order.  Returns the number of rows inserted; NP receives their pivots.
-// P (the pivots before this call) is not modified.
-template <int WD>
-__device__ int insert_block(uint32_t (&xr)[WD], uint4& yr, uint32_t cand, uint32_t* __restrict__ S,
-                            const uint32_t (&P)[WD], int d, int lane, long long idx, long long& first,
-                            unsigned long long& cnt, uint32_t (&NP)[WD], bool& contra_lane, uint32_t weight)
-{
-    constexpr int RS = row_stride(WD);
-    int pk = -1;
-    uint32_t newp = 0;
-    while (cand) {
-        const int i = __ffs(cand) - 1;
-        cand &= cand - 1;
-        int mine = -1;
-#pragma unroll
-        for (int v = 0; v < WD; ++v)
-            if (xr[v]) mine = 32 * v + 31 - __clz(xr[v]);
-        const int k = __shfl_sync(FULL, mine, i);
-        if (k < 0) {  // reduced to zero by rows inserted earlier in this block
-            if (lane == i && nonzero4(yr)) {
-                cnt += weight;
-                first = min(first, idx);
-                contra_lane = true;
-            }
-            continue;
-        }
-        const int kw = k >> 5;
-        const uint32_t kb = 1u << (k & 31);
-        uint32_t sel = 0;
-#pragma unroll
-        for (int v = 0; v < WD; ++v)
-            if (v == kw) sel = xr[v];
-        const bool hit = (lane != i) && (sel & kb);
-#pragma unroll
-        for (int v = 0; v < WD; ++v) {
-            const uint32_t t = __shfl_sync(FULL, xr[v], i);
-            if (hit) xr[v] ^= t;
-        }
-        uint4 bz;
-        bz.x = __shfl_sync(FULL, yr.x, i);
-        bz.y = __shfl_sync(FULL, yr.y, i);
-        bz.z = __shfl_sync(FULL, yr.z, i);
-        bz.w = __shfl_sync(FULL, yr.w, i);
-        if (hit) xor4(yr, bz);
-        if (lane == i) pk = k;
-        newp |= 1u << i;
-    }
-#pragma unroll
-    for (int v = 0; v < WD; ++v) NP[v] = 0;
-    if (!newp) return 0;
-    if (pk >= 0) {
-        uint32_t* row = S + pk * RS;
-        *reinterpret_cast<uint4*>(row) = yr;
-#pragma unroll
-        for (int v = 0; v < RS - 4; ++v) row[4 + v] = (v < WD) ? xr[v] : 0u;
-    }
-#pragma unroll
-    for (int v = 0; v < WD; ++v)
-        NP[v] = __reduce_or_sync(FULL, (pk >= 0 && (pk >> 5) == v) ? (1u << (pk & 31)) : 0u);
-    __syncwarp();
-    // step (5): clear the new pivot columns from every previously stored row
-    for (int j = lane; j < d; j += 32) {
-        uint32_t pj = 0;
-#pragma unroll
-        for (int v = 0; v < WD; ++v)
-            if (v == (j >> 5)) pj = P[v];
-        if (!((pj >> (j & 31)) & 1u)) continue;
-        uint32_t* rj = S + j * RS;
-        uint32_t xj[WD];
-        uint32_t hits = 0;
-#pragma unroll
-        for (int v = 0; v < WD; ++v) {
-            xj[v] = rj[4 + v];
-            hits |= xj[v] & NP[v];
-        }
-        if (!hits) continue;
-        uint4 zj = *reinterpret_cast<const uint4*>(rj);
-#pragma unroll
-        for (int v = 0; v < WD; ++v) {
-            uint32_t m = xj[v] & NP[v];
-            while (m) {
-                const int b = __ffs(m) - 1;
-                m &= m - 1;
-                const uint32_t* rk = S + (32 * v + b) * RS;
-                xor4(zj, *reinterpret_cast<const uint4*>(rk));
-#pragma unroll
-                for (int u = 0; u <= v; ++u) xj[u] ^= rk[4 + u];
-            }
-        }
-        *reinterpret_cast<uint4*>(rj) = zj;
-#pragma unroll
-        for (int v = 0; v < WD; ++v) rj[4 + v] = xj[v];
-    }
-    __syncwarp();
-    return __popc(newp);
-}
-
-// The stored basis moves between global and shared memory by its pivot rows
-// only: an empty slot is zero in the store and never read in shared memory
-// (every read of S selects a pivot), and a slot that became a pivot stays one.
-template <int WD>
-__device__ void basis_to_smem(const StoreDev& s, const CtxDesc& cd, uint32_t* S, const uint32_t* Ps, int t, int nt)
-{
-    constexpr int RS = row_stride(WD);
-    for (int k = t; k < cd.d; k += nt) {
-        if (!((Ps[k >> 5] >> (k & 31)) & 1u)) continue;
-        uint32_t* row = S + k * RS;
-        *reinterpret_cast<uint4*>(row) = s.bz[cd.slot_off + k];
-        const uint32_t* src = s.bx + cd.xw_off + (int64_t)k * cd.wd;
-        for (int v = 0; v < RS - 4; ++v) row[4 + v] = (v < cd.wd) ? src[v] : 0u;
-    }
-}
-
-template <int WD>
-__device__ void basis_from_smem(const StoreDev& s, const CtxDesc& cd, const uint32_t* S, const uint32_t* Ps, int t,
-                                int nt)
-{
-    constexpr int RS = row_stride(WD);
-    for (int k = t; k < cd.d; k += nt) {
-        if (!((Ps[k >> 5] >> (k & 31)) & 1u)) continue;
-        const uint32_t* row = S + k * RS;
-        s.bz[cd.slot_off + k] = *reinterpret_cast<const uint4*>(row);
-        uint32_t* dst = s.bx + cd.xw_off + (int64_t)k * cd.wd;
-        for (int v = 0; v < cd.wd; ++v) dst[v] = row[4 + v];
-    }
-}
-
-__device__ __forceinline__ void warp_stats(long long& first, unsigned long long& cnt)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        first = min(first, __shfl_xor_sync(FULL, first, o));
-        cnt += __shfl_xor_sync(FULL, cnt, o);
-    }
-}
-
-__device__ __forceinline__ void commit_stats(const StoreDev& s, int c, long long first, unsigned long long cnt)
-{
-    if (cnt) {
-        s.n_contra[c] += cnt;
-        s.contra[c] = 1;
-        if (s.first_contra[c] < 0) s.first_contra[c] = first;
-    }
-}
-
-// ------------------------------------------------------------------ pass 2
-
-// Set compressed residual bit tt (< 32 * TABLE_MAX_RW).
-__device__ __forceinline__ void set_rbit(uint32_t (&er)[TABLE_MAX_RW], int tt)
-{
-#pragma unroll
-    for (int u = 0; u < TABLE_MAX_RW; ++u)
-        if ((tt >> 5) == u) er[u] |= 1u << (tt & 31);
-}
-
-constexpr int FL_WORDS = 64;  // free-coordinate list of a table: 128 uint16 entries
-
-// The lookup table (layout in f2_internal.cuh) of the basis held in shared
-// memory: pivot rows S (row stride row_stride(WD)), pivot mask P, rank; FL
-// receives the non-pivot coordinates in increasing order (the meaning of the
-// compressed residual bits).  All nt threads of the group take part.
-template <int WD, bool CTA>
-__device__ void build_table_smem(const uint32_t* __restrict__ S, const uint32_t (&P)[WD], int d, int wd, int rank,
-                                 uint32_t* __restrict__ TB, uint16_t* __restrict__ FL, int t, int nt)
-{
-    constexpr int RS = row_stride(WD);
-    const int np = (d + 3) >> 2, rw = (d - rank + 31) >> 5;
-    uint32_t f[WD];  // non-pivot coordinates of each word
-    int pre[WD];     // non-pivot coordinates in the words before
-    {
-        int acc = 0;
-#pragma unroll
-        for (int w = 0; w < WD; ++w) {
-            const uint32_t valid = (w < wd) ? ((w == wd - 1 && (d & 31)) ? ((1u << (d & 31)) - 1u) : 0xffffffffu) : 0u;
-            f[w] = ~P[w] & valid;
-            pre[w] = acc;
-            acc += __popc(f[w]);
-        }
-    }
-    uint2* const Zl = reinterpret_cast<uint2*>(TB);
-    uint2* const Zh = Zl + 16 * np;
-    uint32_t* const R = TB + 64 * np;
-    for (int j = t; j < 4 * np; j += nt) {
-        uint4 z = make_uint4(0, 0, 0, 0);
-        uint32_t er[TABLE_MAX_RW] = {0, 0, 0, 0};
-        if (j < d) {
-            const int w = j >> 5, b = j & 31;
-            uint32_t fw = 0;
-            int pw = 0;
-#pragma unroll
-            for (int u = 0; u < WD; ++u)
-                if (u == w) {
-                    fw = f[u];
-                    pw = pre[u];
-                }
-            if ((fw >> b) & 1u) {  // a non-pivot coordinate: its unit vector
-                const int tt = pw + __popc(fw & ((1u << b) - 1u));
-                set_rbit(er, tt);
-                FL[tt] = (uint16_t)j;
-            } else {  // a pivot: z_j and r_j on the non-pivot coordinates
-                const uint32_t* row = S + j * RS;
-                z = *reinterpret_cast<const uint4*>(row);
-#pragma unroll
-                for (int u = 0; u < WD; ++u) {
-                    if (u <= w) {
-                        uint32_t bits = row[4 + u] & f[u];
-                        while (bits) {
-                            const int bb = __ffs(bits) - 1;
-                            bits &= bits - 1u;
-                            set_rbit(er, pre[u] + __popc(f[u] & ((1u << bb) - 1u)));
-                        }
-                    }
-                }
-            }
-        }
-        const int e = 16 * (j >> 2) + (1 << (j & 3));
-        Zl[e] = make_uint2(z.x, z.y);
-        Zh[e] = make_uint2(z.z, z.w);
-#pragma unroll
-        for (int u = 0; u < TABLE_MAX_RW; ++u)
-            if (u < rw) R[u * 16 * np + e] = er[u];
-        if ((j & 3) == 0) {
-            const int e0 = 16 * (j >> 2);
-            Zl[e0] = make_uint2(0, 0);
-            Zh[e0] = make_uint2(0, 0);
-#pragma unroll
-            for (int u = 0; u < TABLE_MAX_RW; ++u)
-                if (u < rw) R[u * 16 * np + e0] = 0u;
-        }
-    }
-    group_sync<CTA>();
-    // entries of two or more coordinates: XOR of their single entries
-    for (int k = t; k < 16 * np; k += nt) {
-        const int v = k & 15;
-        if (__popc(v) < 2) continue;
-        const int eb = k & ~15;
-        uint2 lo = make_uint2(0, 0), hi = make_uint2(0, 0);
-        uint32_t rr[TABLE_MAX_RW] = {0, 0, 0, 0};
-#pragma unroll
-        for (int bb = 0; bb < 4; ++bb) {
-            if ((v >> bb) & 1) {
-                const int es = eb + (1 << bb);
-                const uint2 l = Zl[es], h = Zh[es];
-                lo.x ^= l.x;
-                lo.y ^= l.y;
-                hi.x ^= h.x;
-                hi.y ^= h.y;
-#pragma unroll
-                for (int u = 0; u < TABLE_MAX_RW; ++u)
-                    if (u < rw) rr[u] ^= R[u * 16 * np + es];
-            }
-        }
-        Zl[k] = lo;
-        Zh[k] = hi;
-#pragma unroll
-        for (int u = 0; u < TABLE_MAX_RW; ++u)
-            if (u < rw) R[u * 16 * np + k] = rr[u];
-    }
-    group_sync<CTA>();
-}
-
-// The full residual (feature words, zero at the pivots) from its compressed
-// form: bit tt is the non-pivot coordinate FL[tt].
-template <int WD>
-__device__ __forceinline__ void decompress_residual(const uint32_t (&cr)[TABLE_MAX_RW], int rw,
-                                                    const uint16_t* __restrict__ FL, uint32_t (&xr)[WD])
-{
-#pragma unroll
-    for (int v = 0; v < WD; ++v) xr[v] = 0u;
-#pragma unroll
-    for (int u = 0; u < TABLE_MAX_RW; ++u) {
-        uint32_t bits = (u < rw) ? cr[u] : 0u;
-        while (bits) {
-            const int bb = __ffs(bits) - 1;
-            bits &= bits - 1u;
-            const int coord = FL[32 * u + bb];
-#pragma unroll
-            for (int v = 0; v < WD; ++v)
-                if ((coord >> 5) == v) xr[v] |= 1u << (coord & 31);
-        }
-    }
-}
-
-// Snapshot reduction by table: acc of the word parts into yr, the residual
-// (zero at the pivots) into xr; returns whether it is nonzero.
-template <int WD>
-__device__ __forceinline__ bool reduce_by_table(uint32_t (&xr)[WD], uint4& yr, const uint32_t* __restrict__ TB,
-                                                const uint16_t* __restrict__ FL, int np, int rw)
-{
-    uint32_t q[WD];
-#pragma unroll
-    for (int v = 0; v < WD; ++v) q[v] = xr[v];
-    uint4 acc;
-    uint32_t cr[TABLE_MAX_RW] = {0, 0, 0, 0};
-    switch (rw) {
-    case 0: {
-        uint32_t r0[1];
-        table_reduce<0, WD>(TB, np, q, acc, r0);
-        break;
-    }
-    case 1: {
-        uint32_t r1[1];
-        table_reduce<1, WD>(TB, np, q, acc, r1);
-        cr[0] = r1[0];
-        break;
-    }
-    case 2: {
-        uint32_t r2[2];
-        table_reduce<2, WD>(TB, np, q, acc, r2);
-        cr[0] = r2[0];
-        cr[1] = r2[1];
-        break;
-    }
-    case 3: {
-        uint32_t r3[3];
-        table_reduce<3, WD>(TB, np, q, acc, r3);
-        cr[0] = r3[0];
-        cr[1] = r3[1];
-        cr[2] = r3[2];
-        break;
-    }
-    default: {
-        uint32_t r4[4];
-        table_reduce<4, WD>(TB, np, q, acc, r4);
-        cr[0] = r4[0];
-        cr[1] = r4[1];
-        cr[2] = r4[2];
-        cr[3] = r4[3];
-        break;
-    }
-    }
-    yr.x ^= acc.x;
-    yr.y ^= acc.y;
-    yr.z ^= acc.z;
-    yr.w ^= acc.w;
-    const bool nz = (cr[0] | cr[1] | cr[2] | cr[3]) != 0u;
-    if (nz) decompress_residual<WD>(cr, rw, FL, xr);
-    else {
-#pragma unroll
-        for (int v = 0; v < WD; ++v) xr[v] = 0u;
-    }
-    return nz;
-}
-
-// Hand-off of saturated contexts (see LearnArgs): the quiet rounds before
-// it, the widest basis the check can hold (shared memory words, a slot per
-// coordinate) and its chunks of representatives; the row widths of the two
-// instances of the wide kernel (the 10..17-word one takes part).
-constexpr int HANDOFF_QUIET = 2;
-constexpr int CHECK_BASIS_WORDS = 14336;  // 56 KB
-constexpr int CHECK_CHUNK = 512;
-constexpr int HANDOFF_CALL_FACTOR = 16;  // calls of fewer rows than this many hand-off minimums hand off none
-constexpr int WIDE_WD = 33;    // widest row (d <= 1056)
-constexpr int WIDE_M_WD = 17;  // rows of 10..17 words (d <= 544): half the registers, two CTAs per SM
-
-// One group (a warp, or the whole CTA) streams the representatives of
-// context c through its basis.
-template <int WD, bool CTA>
-__device__ void elim_ctx(const StoreDev& s, const LearnArgs& a, int c, uint32_t* region, int region_words)
-{
-    const int G = CTA ? (int)(blockDim.x >> 5) : 1;
-    const int lane = threadIdx.x & 31;
-    const int warp = CTA ? (int)(threadIdx.x >> 5) : 0;
-    const int t = 32 * warp + lane;
-    const int nt = 32 * G;
-    const CtxDesc cd = s.desc[c];
-    uint32_t* ctl = region;
-    uint32_t* Ps = ctl + CTL_P;
-    uint32_t* NPR = ctl + CTL_NPR;
-    uint32_t* wc = ctl + CTL_CAND;
-    int* rank_s = reinterpret_cast<int*>(ctl + CTL_RANK);
-    unsigned long long* cnt_s = reinterpret_cast<unsigned long long*>(ctl + CTL_CNT);
-    long long* first_s = reinterpret_cast<long long*>(ctl + CTL_FIRST);
-    uint32_t* S = region + CTL_WORDS;
-    const int rank0 = s.rank[c];
-    if (t < 48) {
-        Ps[t] = (t < cd.wd && rank0 != 0) ? s.pivot[cd.pw_off + t] : 0u;
-        NPR[t] = 0u;
-    }
-    if (t == 0) {
-        *rank_s = rank0;
-        *cnt_s = 0ull;
-        *first_s = LLONG_MAX;
-    }
-    group_sync<CTA>();
-    if (rank0 != 0) {
-        basis_to_smem<WD>(s, cd, S, Ps, t, nt);
-        group_sync<CTA>();
-    }
-    uint32_t P[WD];
-#pragma unroll
-    for (int v = 0; v < WD; ++v) P[v] = Ps[v];
-    uint64_t mixed = mixed_words<WD>(P, cd.d, cd.wd);
-    // lookup table of the snapshot (rebuilt after a round that inserted):
-    // after the basis rows, the free-coordinate list at the region's end
-    constexpr int RS = row_stride(WD);
-    uint32_t* const TB = S + cd.d * RS;
-    uint16_t* const FL = reinterpret_cast<uint16_t*>(region + region_words - FL_WORDS);
-    const int tab_cap = region_words - FL_WORDS - CTL_WORDS - cd.d * RS;
-    const int np = (cd.d + 3) >> 2;
-    bool dirty = true;
-    const long long seen = s.rows_seen[c];
-    const int64_t r0 = a.row_off[c];
-    const int64_t T = a.row_off[c + 1] - r0;
-    const int rc = a.rep_count ? a.rep_count[c] : -((int)T + 2);
-    const bool deduped = rc >= 0;
-    const int R = deduped ? rc : -(rc + 2);
-    const int32_t* reps = deduped ? a.rep_list + r0 : nullptr;
-    const int32_t* dups = deduped ? a.rep_dup + r0 : nullptr;
-    const uint32_t* xc = a.x + a.x_off[c];
-    const uint4* yc = a.y + r0;
-    long long first = LLONG_MAX;
-    unsigned long long cnt = 0;
-    // prefetched round
-    const int k0 = a.resume_from ? a.resume_from[c] : 0;  // the first representative of this launch
-    int nk = k0 + t;
-    bool nvalid = nk < R;
-    int ni = nvalid ? (reps ? __ldg(reps + nk) : nk) : 0;
-    uint32_t nw = (nvalid && dups) ? (uint32_t)__ldg(dups + nk) : 0u;
-    uint32_t xn[WD];
-    uint4 yn;
-    load_raw<WD>(xc + (int64_t)ni * cd.xw, yc + ni, nvalid, cd.n, cd.xw, xn, yn);
-    int stop_at = -1;
-    int snap_at = -1;  // handed off from this representative on
-    int quiet = 0;     // rounds in a row that inserted nothing
-    int parity = 0;
-    for (int base = k0; base < R; base += nt, parity ^= 1) {
-        const bool valid = nvalid;
-        const int i = ni;
-        const uint32_t weight = 1u + nw;
-        uint32_t xr[WD];
-        make_q<WD>(xn, valid, s.raw, xr);
-        uint4 yr = yn;
-        nk += nt;
-        nvalid = nk < R;
-        ni = nvalid ? (reps ? __ldg(reps + nk) : nk) : 0;
-        nw = (nvalid && dups) ? (uint32_t)__ldg(dups + nk) : 0u;
-        load_raw<WD>(xc + (int64_t)ni * cd.xw, yc + ni, nvalid, cd.n, cd.xw, xn, yn);
-        // step (1) against the snapshot: by lookup table where the table fits
-        // and costs fewer instructions than walking the pivots (about d/4
-        // lookups a row against about rank/2 two-pivot steps), else by walk
-        int tmode = 0;  // 1 + residual words of the table, 0 = walk
-        // (CTA-owned contexts only: their many rounds after the basis stops
-        // growing repay the rebuilds; a warp-owned context has few rounds,
-        // most of them inserting, and keeps the small shared-memory region
-        // that lets more warps run)
-        if constexpr (CTA && WD <= TABLE_MAX_WD) {
-            if (a.tables) {
-                const int rk = *rank_s;
-                const int rw = (cd.d - rk + 31) >> 5;
-                if (rw <= TABLE_MAX_RW && table_words(cd.d, rk) <= tab_cap && 4 * rk >= 5 * np) {
-                    tmode = 1 + rw;
-                    if (dirty) {
-                        build_table_smem<WD, CTA>(S, P, cd.d, cd.wd, rk, TB, FL, t, nt);
-                        dirty = false;
-                    }
-                }
-            }
-        }
-        uint32_t nz = 0;
-        if (tmode) {
-            nz = reduce_by_table<WD>(xr, yr, TB, FL, np, tmode - 1) ? 1u : 0u;
-        } else {
-            reduce_snapshot<WD>(xr, yr, S, P, mixed);
-#pragma unroll
-            for (int v = 0; v < WD; ++v) {
-                xr[v] &= ~P[v];
-                nz |= xr[v];
-            }
-        }
-        bool contra_lane = false;
-        if (valid && !nz && nonzero4(yr)) {
-            cnt += weight;
-            first = min(first, seen + (long long)i);
-            contra_lane = true;
-        }
-        const uint32_t cand = __ballot_sync(FULL, valid && nz != 0u);
-        uint32_t wmask;
-        if (CTA) {
-            // two alternating ballot buffers: a round without candidates
-            // ends without a barrier, so the next round's ballots must not
-            // overwrite this round's before every warp has read them
-            uint32_t* const wcp = wc + 16 * parity;
-            if (lane == 0) wcp[warp] = cand;
-            __syncthreads();
-            wmask = 0;
-            for (int ww = 0; ww < G; ++ww)
-                if (wcp[ww]) wmask |= 1u << ww;
-        } else {
-            wmask = cand ? 1u : 0u;
-        }
-        if (wmask) {
-            const int first_warp = __ffs(wmask) - 1;
-            for (uint32_t wm = wmask; wm; wm &= wm - 1) {
-                const int ww = __ffs(wm) - 1;
-                if (warp == ww) {
-                    if (CTA && ww != first_warp) reduce_new<WD>(xr, yr, S, NPR);
-                    uint32_t NP[WD];
-                    const int added = insert_block<WD>(xr, yr, cand, S, P, cd.d, lane, seen + (long long)i, first, cnt,
-                                                       NP, contra_lane, weight);
-                    if (lane == 0 && added) {
-#pragma unroll
-                        for (int v = 0; v < WD; ++v) {
-                            Ps[v] = P[v] | NP[v];
-                            NPR[v] |= NP[v];
-                        }
-                        *rank_s += added;
-                    }
-                }
-                group_sync<CTA>();
-#pragma unroll
-                for (int v = 0; v < WD; ++v) P[v] = Ps[v];
-            }
-            mixed = mixed_words<WD>(P, cd.d, cd.wd);
-            dirty = true;
-            if (CTA) {
-                if (t < 48) NPR[t] = 0u;
-            }
-            // (wide contexts) full rank with at least a chunk of rows left:
-            // every later row is a check only (the rows are their own
-            // representatives here)
-            if constexpr (WD > NARROW_WD) {
-                if (!deduped && a.late_list && R - (base + nt) >= FULL_CHUNK && *rank_s == cd.d) {
-                    stop_at = base + nt;
-                    break;
-                }
-            }
-        }
-        if constexpr (CTA && (WD <= NARROW_WD || WD == WIDE_M_WD)) {
-            // every rank >= 1 saturated context with many representatives
-            // left: hand the rest off to the parallel check (block-uniform)
-            quiet = wmask ? 0 : quiet + 1;
-            if (a.handoff_min > 0 && !a.resume_from && quiet >= HANDOFF_QUIET && R - (base + nt) >= a.handoff_min &&
-                *rank_s < cd.d && cd.d * row_stride(WD) <= CHECK_BASIS_WORDS) {
-                snap_at = base + nt;
-                break;
-            }
-        }
-        (void)contra_lane;
-    }
-    warp_stats(first, cnt);
-    if (lane == 0 && cnt) {
-        atomicAdd(cnt_s, cnt);
-        atomicMin(first_s, first);
-    }
-    group_sync<CTA>();
-    if (t < cd.wd) s.pivot[cd.pw_off + t] = Ps[t];
-    basis_from_smem<WD>(s, cd, S, Ps, t, nt);
-    if (t == 0) {
-        s.rank[c] = *rank_s;
-        commit_stats(s, c, *first_s, *cnt_s);
-        if (snap_at >= 0) {  // rows_seen is advanced by check_snap_kernel (or resume_kernel)
-            a.snap_start[c] = snap_at;
-            a.snap_list[atomicAdd(a.snap_count, 1)] = c;
-        } else if (stop_at < 0) {
-            s.rows_seen[c] = seen + T;
-        } else {  // rows_seen is advanced by verify_full_kernel
-            a.late_start[c] = stop_at;
-            a.late_list[atomicAdd(a.late_count, 1)] = c;
-        }
-    }
-    group_sync<CTA>();
-}
-
 __device__ __forceinline__ int64_t check_slot(const CheckArgs& a, int c)
 {
     return a.row_off[c] / CHECK_CHUNK + c;  // the context's first chunk record (chunks never overlap)
@@ -1394,16 +616,16 @@ __device__ void check_chunk(const StoreDev& s, const CheckArgs& a, int c, int kb
         const int k = base + (int)threadIdx.x;
         const bool valid = k < ke;
         const int i = valid ? (reps ? __ldg(reps + k) : k) : 0;
-        uint32_t xin[WD], q[WD];
-        uint4 yr;
-        load_raw<WD>(xc + (int64_t)i * cd.xw, yc + i, valid, cd.n, cd.xw, xin, yr);
-        make_q<WD>(xin, valid, s.raw, q);
-        reduce_snapshot<WD>(q, yr, S, P, mixed);
+        uint32_t xin[WD], q[1][WD];
+        uint4 yr[1];
+        load_raw<WD>(xc + (int64_t)i * cd.xw, yc + i, valid, cd.n, cd.xw, xin, yr[0]);
+        make_q<WD>(xin, valid, s.raw, q[0]);
+        reduce_rows<WD, 1>(q, yr, S, P, mixed);
         uint32_t resid = 0;
 #pragma unroll
-        for (int w = 0; w < WD; ++w) resid |= q[w] & ~P[w];
+        for (int w = 0; w < WD; ++w) resid |= q[0][w] & ~P[w];
         // 2: outside the span, 1: a contradiction, 0: redundant
-        if (valid) flags[k - kb] = resid ? 2 : (nonzero4(yr) ? 1 : 0);
+        if (valid) flags[k - kb] = resid ? 2 : (nonzero4(yr[0]) ? 1 : 0);
     }
 }
 
@@ -1547,94 +769,6 @@ __global__ void __launch_bounds__(256) check_snap_kernel(StoreDev s, CheckArgs a
             }
         }
         __syncthreads();
-    }
-}
-
-// Narrow elimination: CTA-owned contexts first (longest first), then
-// warp-owned ones.  SMALL: the contexts of at most SMALL_WD words, with
-// fixed 4 KB warp regions and a register budget for three CTAs per SM (80
-// registers, no spills; four CTAs at 64 registers spill and ran 6% slower
-// on the 78k-context, 81M-row learn); else
-// the contexts of SMALL_WD + 1 .. NARROW_WD words.
-static_assert(DEFAULT_SMALL_REGION_BYTES / 4 >= 32 * SMALL_WD * row_stride(SMALL_WD) + CTL_WORDS + FL_WORDS,
-              "a warp region holds the basis of any small-width context");
-
-//
-// NW: warps of a CTA.  The 4..9-word kernel has an instance of four-warp CTAs
-// (four per SM, the same warps per SM) for long calls: a CTA-owned context's
-// insertions run one warp at a time while the group's other warps wait, so
-// smaller groups waste less; in a short call the longest CTA-owned contexts
-// bound the call and keep eight warps each.
-template <bool SMALL, int NW = LEARN_WARPS>
-__global__ void __launch_bounds__(NW * 32, SMALL ? 3 : 16 / NW) elim_narrow_kernel(StoreDev s, LearnArgs a)
-{
-    constexpr int C_CTA = SMALL ? CLS_CTA_S : CLS_CTA;
-    constexpr int C_WARP = SMALL ? CLS_WARP_S : CLS_WARP;
-    extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ int s_item;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_cta = a.counters[CNT_COUNT + C_CTA];
-    const int b_cta = a.counters[CNT_BEGIN + C_CTA];
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_item = atomicAdd(a.counters + CNT_HEAD + C_CTA, 1);
-        __syncthreads();
-        const int item = s_item;
-        if (item >= n_cta) break;
-        const int c = a.queue[b_cta + item];
-        const int wd = s.desc[c].wd;
-        if (threadIdx.x == 0) time_mark(a.timing, c, 2);
-#define F2_CALL_CTA(W) elim_ctx<W, true>(s, a, c, smem, a.cta_region_words)
-        if (SMALL) {
-            F2_SMALL_SWITCH(wd, F2_CALL_CTA)
-        } else {
-            F2_BIG_SWITCH(wd, F2_CALL_CTA)
-        }
-#undef F2_CALL_CTA
-        if (threadIdx.x == 0) time_mark(a.timing, c, 3);
-    }
-    const int n_w = a.counters[CNT_COUNT + C_WARP];
-    const int b_w = a.counters[CNT_BEGIN + C_WARP];
-    const int region_words = SMALL ? a.small_region_words : a.warp_region_words;
-    uint32_t* region = smem + warp * region_words;
-    for (;;) {
-        int item = 0;
-        if (lane == 0) item = atomicAdd(a.counters + CNT_HEAD + C_WARP, 1);
-        item = __shfl_sync(FULL, item, 0);
-        if (item >= n_w) break;
-        const int c = a.queue[b_w + item];
-        const int wd = s.desc[c].wd;
-        if (lane == 0) time_mark(a.timing, c, 2);
-#define F2_CALL_WARP(W) elim_ctx<W, false>(s, a, c, region, region_words)
-        if (SMALL) {
-            F2_SMALL_SWITCH(wd, F2_CALL_WARP)
-        } else {
-            F2_BIG_SWITCH(wd, F2_CALL_WARP)
-        }
-#undef F2_CALL_WARP
-        if (lane == 0) time_mark(a.timing, c, 3);
-    }
-}
-
-
-// Wide elimination: every context by a whole CTA, rows of up to WDT words.
-template <int WDT, int CLS>
-__global__ void __launch_bounds__(WIDE_WARPS * 32, WDT <= WIDE_M_WD ? 2 : 1) elim_wide_kernel(StoreDev s, LearnArgs a)
-{
-    extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ int s_item;
-    const int n = a.counters[CNT_COUNT + CLS];
-    const int b = a.counters[CNT_BEGIN + CLS];
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_item = atomicAdd(a.counters + CNT_HEAD + CLS, 1);
-        __syncthreads();
-        const int item = s_item;
-        if (item >= n) break;
-        const int c = a.queue[b + item];
-        if (threadIdx.x == 0) time_mark(a.timing, c, 2);
-        elim_ctx<WDT, true>(s, a, c, smem, a.cta_region_words);
-        if (threadIdx.x == 0) time_mark(a.timing, c, 3);
     }
 }
 
@@ -2146,48 +1280,7 @@ __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, F
     }
 }
 
-// The contexts the check sent back: eliminated in stream order from their
-// first representative outside the snapshot (no further hand-off), one CTA
-// each.  Every width that can hand off has an instance here.
-__global__ void __launch_bounds__(LEARN_WARPS * 32, 1) resume_kernel(StoreDev s, LearnArgs a, const int* resume_count,
-                                                                     const int32_t* resume_list)
-{
-    extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ int s_item;
-    const int n = *resume_count;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_item = atomicAdd(a.counters + CNT_HEAD + CLS_RESUME, 1);
-        __syncthreads();
-        const int item = s_item;
-        if (item >= n) break;
-        const int c = resume_list[item];
-        const int wd = s.desc[c].wd;
-#define F2_CALL_RESUME(W) elim_ctx<W, true>(s, a, c, smem, a.cta_region_words)
-        switch (wd) {
-        case 1: F2_CALL_RESUME(1); break;
-        case 2: F2_CALL_RESUME(2); break;
-        case 3: F2_CALL_RESUME(3); break;
-        case 4: F2_CALL_RESUME(4); break;
-        case 5: F2_CALL_RESUME(5); break;
-        case 6: F2_CALL_RESUME(6); break;
-        case 7: F2_CALL_RESUME(7); break;
-        case 8: F2_CALL_RESUME(8); break;
-        case 9: F2_CALL_RESUME(9); break;
-        default: F2_CALL_RESUME(WIDE_M_WD); break;
-        }
-#undef F2_CALL_RESUME
-    }
-}
-
 // Which elimination kernels a store needs, and their widest bases.
-
-size_t narrow_smem(int max_narrow_words, int warp_region_words, int nw)
-{
-    const size_t cta = 4 * (size_t)max_narrow_words;
-    const size_t warps = 4 * (size_t)nw * (size_t)warp_region_words;
-    return cta > warps ? cta : warps;
-}
 
 // Calls of at least this many rows run the 4..9-word elimination in CTAs of
 // four warps (see elim_narrow_kernel; F2_OPT_LONG_CALL_ROWS).
@@ -2265,65 +1358,27 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
     pa.counters = la.counters;
     int rc = launch_plan(sd, pa, num_sms, cs);
     if (rc != F2_OK) return rc;
-    cudaError_t e;
-    auto narrow = [&](auto kernel, size_t smem, cudaStream_t ks, int nw) -> int {
-        cudaError_t er = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (er != cudaSuccess) return f2_cuda_status(er);
-        int per_sm = 0;
-        er = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, nw * 32, smem);
-        if (er != cudaSuccess) return f2_cuda_status(er);
-        if (per_sm < 1) per_sm = 1;
-        LearnArgs lk = lx;
-        lk.cta_region_words = (int)(smem / 4);
-        kernel<<<num_sms * per_sm, nw * 32, smem, ks>>>(sd, lk);
-        return f2_cuda_status(cudaGetLastError());
-    };
-    // the three width classes hold disjoint contexts: with a second stream
-    // their kernels overlap (each fills the others' tails)
+    // the width classes hold disjoint contexts: with a second stream their
+    // kernels overlap (each fills the others' tails)
     Fork solo{cs, nullptr, nullptr, nullptr};
     Fork& f = fk ? *fk : solo;
     int left = (int)wv.has_narrow + (int)wv.has_wide + (int)wv.has_wide_m + (int)wv.has_small;
-    auto wide = [&](auto kernel, int max_d, int wdt) -> int {
-        const size_t smem = 4 * (size_t)elim_words(max_d, wdt);
-        cudaError_t er = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (er != cudaSuccess) return f2_cuda_status(er);
-        int per_sm = 0;
-        er = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, WIDE_WARPS * 32, smem);
-        if (er != cudaSuccess) return f2_cuda_status(er);
-        if (per_sm < 1) per_sm = 1;
-        const cudaStream_t ks = f.next(left--);
-        if (f.e != cudaSuccess) return f2_cuda_status(f.e);
-        LearnArgs lk = lx;
-        lk.cta_region_words = (int)(smem / 4);
-        kernel<<<num_sms * per_sm, WIDE_WARPS * 32, smem, ks>>>(sd, lk);
-        return f2_cuda_status(cudaGetLastError());
+    auto eliminate = [&](const LearnArgs& lk) -> cudaError_t {
+        cudaError_t er = cudaSuccess;
+        auto stream = [&]() { return lk.resume_from ? cs : f.next(left--); };
+        const bool resume = lk.resume_from != nullptr;
+        if (er == cudaSuccess && wv.has_wide && !resume)  // wider contexts hand nothing off
+            er = elim_launch_wide(sd, lk, wv.max_wide_d, false, num_sms, stream());
+        if (er == cudaSuccess && wv.has_wide_m)
+            er = elim_launch_wide(sd, lk, wv.max_wide_m_d, true, num_sms, stream());
+        if (er == cudaSuccess && wv.has_narrow)
+            er = elim_launch_narrow(sd, lk, wv.max_narrow_words, total_rows >= long_rows && !resume ? 4 : LEARN_WARPS,
+                                    num_sms, stream());
+        if (er == cudaSuccess && wv.has_small) er = elim_launch_small(sd, lk, wv.max_small_words, num_sms, stream());
+        return er == cudaSuccess ? f.e : er;
     };
-    if (wv.has_wide) {
-        rc = wide(elim_wide_kernel<WIDE_WD, CLS_WIDE>, wv.max_wide_d, WIDE_WD);
-        if (rc != F2_OK) return rc;
-    }
-    if (wv.has_wide_m) {
-        rc = wide(elim_wide_kernel<WIDE_M_WD, CLS_WIDE_M>, wv.max_wide_m_d, WIDE_M_WD);
-        if (rc != F2_OK) return rc;
-    }
-    const size_t small_words = (size_t)LEARN_WARPS * (size_t)la.small_region_words;
-    const size_t small_smem = 4 * (small_words > (size_t)wv.max_small_words ? small_words : (size_t)wv.max_small_words);
-    if (wv.has_narrow) {
-        const cudaStream_t ks = f.next(left--);
-        if (f.e != cudaSuccess) return f2_cuda_status(f.e);
-        if (total_rows >= long_rows)
-            rc = narrow(elim_narrow_kernel<false, 4>, narrow_smem(wv.max_narrow_words, la.warp_region_words, 4), ks, 4);
-        else
-            rc = narrow(elim_narrow_kernel<false>, narrow_smem(wv.max_narrow_words, la.warp_region_words, LEARN_WARPS),
-                        ks, LEARN_WARPS);
-        if (rc != F2_OK) return rc;
-    }
-    if (wv.has_small) {
-        const cudaStream_t ks = f.next(left--);
-        if (f.e != cudaSuccess) return f2_cuda_status(f.e);
-        rc = narrow(elim_narrow_kernel<true>, small_smem, ks, LEARN_WARPS);
-        if (rc != F2_OK) return rc;
-    }
+    cudaError_t e = eliminate(lx);
+    if (e != cudaSuccess) return f2_cuda_status(e);
     e = f.join();
     if (e != cudaSuccess) return f2_cuda_status(e);
     if (check && la.handoff_min > 0) {
@@ -2336,18 +1391,12 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
         check_snap_kernel<<<num_sms * 2, 256, csmem, cs>>>(sd, *check);
         e = cudaGetLastError();
         if (e != cudaSuccess) return f2_cuda_status(e);
-        int words = wv.max_small_words > wv.max_narrow_words ? wv.max_small_words : wv.max_narrow_words;
-        if (wv.has_wide_m && elim_words(wv.max_wide_m_d, WIDE_M_WD) > words)
-            words = elim_words(wv.max_wide_m_d, WIDE_M_WD);
-        const size_t rsmem = 4 * (size_t)words;
-        e = cudaFuncSetAttribute(resume_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem);
-        if (e != cudaSuccess) return f2_cuda_status(e);
         LearnArgs lr = lx;
         lr.handoff_min = 0;
         lr.resume_from = check->resume_from;
-        lr.cta_region_words = words;
-        resume_kernel<<<num_sms, LEARN_WARPS * 32, rsmem, cs>>>(sd, lr, check->resume_count, check->resume_list);
-        e = cudaGetLastError();
+        lr.resume_list = check->resume_list;
+        lr.resume_count = check->resume_count;
+        e = eliminate(lr);
         if (e != cudaSuccess) return f2_cuda_status(e);
     }
     {  // full-rank contexts: at the start of the call (the plan decides on the
@@ -2552,6 +1601,8 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
     la.snap_list = st->hand + 2;
     la.snap_start = st->hand + 2 + C;
     la.resume_from = nullptr;
+    la.resume_list = nullptr;
+    la.resume_count = nullptr;
     if (!st->widths_ready) {  // fixed by the widths: computed once per store
         st->widths = width_summary(st->n_bits.data(), st->num_ctx, (st->flags & F2_FLAG_RAW_FEATURES) != 0);
         st->widths_ready = true;
@@ -2735,11 +1786,9 @@ cudaError_t noalloc_load_kernels()
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, plan_scan_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, plan_scatter_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, plan_small_kernel);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, elim_narrow_kernel<true>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, elim_narrow_kernel<false>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, elim_narrow_kernel<false, 4>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, elim_wide_kernel<WIDE_WD, CLS_WIDE>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, elim_wide_kernel<WIDE_M_WD, CLS_WIDE_M>);
+    if (e == cudaSuccess) e = elim_load_small();
+    if (e == cudaSuccess) e = elim_load_narrow();
+    if (e == cudaSuccess) e = elim_load_wide();
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, verify_full_kernel);
     return e;
 }
@@ -2846,6 +1895,8 @@ extern "C" int f2_learn_batched_noalloc(int32_t num_ctx, const int32_t* n_bits_h
     la.snap_list = nullptr;
     la.snap_start = nullptr;
     la.resume_from = nullptr;
+    la.resume_list = nullptr;
+    la.resume_count = nullptr;
     la.warp_region_words = NOALLOC_WARP_REGION_WORDS;
     const Widths wv = width_summary(n_bits_host, num_ctx, raw);
     return launch_elimination(sd, la, row_off_dev, x_off_dev, total_rows, total_x_words, nullptr, NOALLOC_HEAVY_ROWS,
