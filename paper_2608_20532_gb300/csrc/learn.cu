@@ -136,6 +136,14 @@ constexpr int DD_QUAD_SHARE = 4;
 // its barriers, the shards' compaction) outweigh what the split saves.
 constexpr int DD_PROMOTE_MIN_ROWS = 1024;
 constexpr int DD_SHARD_MIN_ROWS = 2048;
+// Contexts of at most this many rows in a call skip the duplicate pass: a
+// warp opens a basis with 128 rows at once, repeats or not, and a CTA takes
+// 256 rows a round, so their repeats cost less than finding them.  A call
+// without longer contexts leaves the duplicate pass and the second plan with
+// nothing to do: eight batches of 32 rows for each of 4,096 contexts went from
+// 625 to 444 us.
+constexpr int DEDUP_MIN_WARP = 128;
+constexpr int DEDUP_MIN_CTA = 1024;
 static_assert(DD_WARPS * DD_WARP_REGION * 4 <= DD_SMEM, "warp regions exceed the dedup shared memory");
 
 // Dispatch on a feature-row width to a template instantiation.
@@ -513,6 +521,7 @@ __global__ void __launch_bounds__(DD_THREADS, DD_CTAS_PER_SM) dedup_kernel(Store
     __shared__ int s_item[DD_WARPS];
     __shared__ int wcnt[DD_WARPS * DD_K];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (a.counters[CNT_DEDUPED] == 0) return;
     {
         const int n = a.counters[CNT_COUNT + C_CTA];
         const int b = a.counters[CNT_BEGIN + C_CTA];
@@ -778,12 +787,14 @@ __global__ void __launch_bounds__(256) check_snap_kernel(StoreDev s, CheckArgs a
 // width); within a class, buckets run from the most work to the least and,
 // inside a bucket, widths in increasing order (so few template variants run
 // at once).
-//   mode 0 (dedup plan): every valid non-empty context with at most DD_XW
-//     feature words goes to the warp, quad or CTA dedup queue by its row
-//     count; rep_count[c] becomes 0 (filled by the dedup pass), -1 (invalid,
+//   mode 0 (dedup plan): every valid non-empty context of more than dedup_min
+//     rows and at most DD_XW_WIDE feature words goes to the warp, quad or CTA
+//     dedup queue by its row count, the others straight to an elimination
+//     queue; rep_count[c] becomes 0 (filled by the dedup pass), -1 (invalid,
 //     skipped) or -(T+2) (every row is its own representative);
 //   mode 1 (elimination plan): contexts with rows to eliminate go to the
-//     warp, CTA or wide elimination queue.
+//     warp, CTA or wide elimination queue.  After a mode-0 plan that sent no
+//     context to the duplicate pass it has nothing to do and returns.
 constexpr int PLAN_SUB = PLAN_BUCKETS * NARROW_WD;  // (bucket, width) keys per class
 constexpr int PLAN_KEYS = NUM_CLASSES * PLAN_SUB;
 static_assert(PLAN_KEYS <= PLAN_HIST_WORDS, "the plan histogram holds every key");
@@ -798,6 +809,8 @@ struct PlanArgs {
     int warp_region_words;
     int64_t heavy_rows;
     int64_t warp_work;
+    int dedup_min; // mode 0: contexts of at most this many rows are not deduplicated
+    int after;     // mode 1: a mode-0 plan ran before
     int scale;     // mode 1: scale heavy_rows / warp_work to the totals of the duplicate pass
     int num_sms;
     long long shard_work;  // mode 0: rows x (xw + 4) of one shard share; 0 = no splitting
@@ -839,6 +852,7 @@ __device__ __forceinline__ int plan_key_of(const StoreDev& s, const PlanArgs& p,
     nsh_out = 0;
     const CtxDesc cd = s.desc[c];
     int64_t R;
+    bool direct = p.mode == 1;  // to an elimination queue
     if (p.mode == 1 && p.rep_count) {
         R = p.rep_count[c];
         if (R <= -2) R = -(R + 2);
@@ -851,11 +865,11 @@ __device__ __forceinline__ int plan_key_of(const StoreDev& s, const PlanArgs& p,
         if (!ok) record_status(s.status, F2_ERR_ROWS);
         R = ok ? rows : -1;
         if (p.mode == 0 && p.rep_count) {
-            // wide rows are not deduplicated; rows of a full-rank context
-            // are checked one by one (verify_full_kernel)
-            if (R > 0 && (cd.xw > DD_XW_WIDE || s.rank[c] == cd.d)) {
+            // wide rows and short contexts are not deduplicated; rows of a
+            // full-rank context are checked one by one (verify_full_kernel)
+            if (R > 0 && (cd.xw > DD_XW_WIDE || R <= p.dedup_min || s.rank[c] == cd.d)) {
                 p.rep_count[c] = (int32_t)(-(R + 2));
-                R = 0;
+                direct = true;
             } else {
                 p.rep_count[c] = (R > 0) ? 0 : (int32_t)R;
             }
@@ -865,7 +879,7 @@ __device__ __forceinline__ int plan_key_of(const StoreDev& s, const PlanArgs& p,
     if (R > 0) {
         int cls;
         unsigned long long work;
-        if (p.mode == 0) {
+        if (!direct) {
             cls = (R <= DD_WARP_MAX_ROWS) ? CLS_DD_WARP : (R <= DD_QUAD_MAX_ROWS ? CLS_DD_QUAD : CLS_DD_CTA);
             if (cd.xw > DD_XW) cls += CLS_DDW_CTA - CLS_DD_CTA;  // the 10..16-word instance
             work = (unsigned long long)R * (unsigned long long)(cd.xw + 4);
@@ -879,7 +893,7 @@ __device__ __forceinline__ int plan_key_of(const StoreDev& s, const PlanArgs& p,
             work = (unsigned long long)R * (unsigned long long)(cd.wd + 4) * (unsigned long long)cd.d;
         }
         int nsh = 1;
-        if (p.mode == 0 && p.shard_work > 0) {
+        if (!direct && p.shard_work > 0) {
             if (F2_DD_QUAD_PROMOTE && (cls == CLS_DD_QUAD || cls == CLS_DDW_QUAD) && R >= DD_PROMOTE_MIN_ROWS &&
                 (long long)work * DD_QUAD_SHARE > p.shard_work)
                 cls += CLS_DD_CTA - CLS_DD_QUAD;
@@ -896,7 +910,7 @@ __device__ __forceinline__ int plan_key_of(const StoreDev& s, const PlanArgs& p,
         }
         int bucket = 63 - __clzll(work);
         if (bucket >= PLAN_BUCKETS) bucket = PLAN_BUCKETS - 1;
-        const int width = (p.mode == 0 ? cd.xw : cd.wd);
+        const int width = direct ? cd.wd : cd.xw;
         const int sub = (PLAN_BUCKETS - 1 - bucket) * NARROW_WD + (width > NARROW_WD ? NARROW_WD : width) - 1;
         key = cls * PLAN_SUB + sub;
         key |= (nsh - 1) << 16;
@@ -905,8 +919,12 @@ __device__ __forceinline__ int plan_key_of(const StoreDev& s, const PlanArgs& p,
     return key;
 }
 
+// The second plan of a call whose first one left nothing to the duplicate pass.
+__device__ __forceinline__ bool plan_done(const PlanArgs& p) { return p.after && p.counters[CNT_DEDUPED] == 0; }
+
 __global__ void __launch_bounds__(256) plan_key_kernel(StoreDev s, PlanArgs p)
 {
+    if (plan_done(p)) return;
     __shared__ int hist[PLAN_KEYS];
     for (int i = threadIdx.x; i < PLAN_KEYS; i += blockDim.x) hist[i] = 0;
     __syncthreads();
@@ -925,7 +943,7 @@ __global__ void __launch_bounds__(256) plan_key_kernel(StoreDev s, PlanArgs p)
 // Exclusive scan of the key counts `hist` (global or shared) in key order by
 // one block of 1024 threads; hist becomes the cursors and the class blocks of
 // `counters` (first item, count, head) are set.
-__device__ void plan_scan_block(int* hist, int* counters)
+__device__ void plan_scan_block(int* hist, int* counters, int mode)
 {
     constexpr int PER = (PLAN_KEYS + 1023) / 1024;
     __shared__ int wsum[32];
@@ -975,9 +993,16 @@ __device__ void plan_scan_block(int* hist, int* counters)
         counters[CNT_HEAD + t] = 0;
         counters[CNT_COUNT + t] = e - b;
     }
+    if (mode == 0 && t == 0)  // items of the duplicate pass (its classes are consecutive keys)
+        counters[CNT_DEDUPED] = (hist[(CLS_DD_WARP + 1) * PLAN_SUB] - hist[CLS_DD_CTA * PLAN_SUB]) +
+                                (hist[(CLS_DDW_WARP + 1) * PLAN_SUB] - hist[CLS_DDW_CTA * PLAN_SUB]);
 }
 
-__global__ void __launch_bounds__(1024) plan_scan_kernel(PlanArgs p) { plan_scan_block(p.hist, p.counters); }
+__global__ void __launch_bounds__(1024) plan_scan_kernel(PlanArgs p)
+{
+    if (plan_done(p)) return;
+    plan_scan_block(p.hist, p.counters, p.mode);
+}
 
 // Queue item(s) of context c with key kv at the cursor of its key.
 __device__ __forceinline__ void plan_place(const PlanArgs& p, int* cursor, int c, int kv)
@@ -994,6 +1019,7 @@ __device__ __forceinline__ void plan_place(const PlanArgs& p, int* cursor, int c
 
 __global__ void __launch_bounds__(256) plan_scatter_kernel(StoreDev s, PlanArgs p)
 {
+    if (plan_done(p)) return;
     // the lanes of a warp with the same key take their slots with one atomic
     const int lane = threadIdx.x & 31;
     for (int b = blockIdx.x * blockDim.x; b < s.num_ctx; b += gridDim.x * blockDim.x) {
@@ -1021,22 +1047,26 @@ constexpr int PLAN_SMALL_MAX = 8192;
 __global__ void __launch_bounds__(1024) plan_small_kernel(StoreDev s, PlanArgs p)
 {
     __shared__ int hist[PLAN_KEYS];
+    if (plan_done(p)) return;
     for (int i = threadIdx.x; i < PLAN_KEYS; i += blockDim.x) hist[i] = 0;
     __syncthreads();
     const PlanLimits L = plan_limits(p);
-    for (int c = threadIdx.x; c < s.num_ctx; c += blockDim.x) {
-        int nsh;
-        const int kv = plan_key_of(s, p, L, c, nsh);
-        if (kv >= 0) atomicAdd(&hist[kv & 0xFFFF], nsh);
-        p.keybuf[c] = kv;  // read back below by this same thread
+    constexpr int PER = PLAN_SMALL_MAX / 1024;
+    int kv[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int c = j * 1024 + (int)threadIdx.x;
+        kv[j] = -1;
+        int nsh = 0;
+        if (c < s.num_ctx) kv[j] = plan_key_of(s, p, L, c, nsh);
+        if (kv[j] >= 0) atomicAdd(&hist[kv[j] & 0xFFFF], nsh);
     }
     __syncthreads();
-    plan_scan_block(hist, p.counters);
+    plan_scan_block(hist, p.counters, p.mode);
     __syncthreads();
-    for (int c = threadIdx.x; c < s.num_ctx; c += blockDim.x) {
-        const int kv = p.keybuf[c];
-        if (kv >= 0) plan_place(p, hist, c, kv);
-    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j)
+        if (kv[j] >= 0) plan_place(p, hist, j * 1024 + (int)threadIdx.x, kv[j]);
 }
 
 int launch_plan(const StoreDev& sd, const PlanArgs& pa, int num_sms, cudaStream_t cs)
@@ -1346,6 +1376,8 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
     pa.warp_region_words = la.warp_region_words;
     pa.heavy_rows = heavy_rows;
     pa.warp_work = warp_work;
+    pa.dedup_min = 0;
+    pa.after = rep_count != nullptr;
     pa.scale = scale;
     pa.num_sms = num_sms;
     pa.shard_work = 0;
@@ -1521,6 +1553,22 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
         if (rc != F2_OK) return rc;
     }
     Fork fk{cs, st->aux, st->ev_fork, st->ev_join};
+    // Rows from which a context gets a whole CTA: unless set explicitly, it
+    // scales with the batch -- in a short call a warp-owned context of a few
+    // thousand rows, dependent round after round, would outlast everything
+    // else, while in a long one warps keep the SMs fuller
+    // else, and in a store of at most ALL_CTA_PER_SM contexts per SM, every
+    // context gets one: none waits for a CTA, and a CTA takes eight warps'
+    // rows per dependent round
+    int64_t heavy = st->heavy_rows;
+    const bool all_cta = !st->heavy_rows_set && st->num_ctx <= (int64_t)ALL_CTA_PER_SM * st->num_sms;
+    if (all_cta) {
+        heavy = 1;
+    } else if (!st->heavy_rows_set && !dedup) {
+        heavy = total_rows / HEAVY_ROWS_BATCH_DIV;
+        if (heavy < HEAVY_ROWS_MIN) heavy = HEAVY_ROWS_MIN;
+        if (heavy > st->heavy_rows) heavy = st->heavy_rows;
+    }
     if (dedup) {
         PlanArgs pa;
         pa.row_off = row_off;
@@ -1529,9 +1577,11 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
         pa.total_xw = total_x_words;
         pa.rep_count = st->rep_count;
         pa.mode = 0;
-        pa.warp_region_words = 0;
-        pa.heavy_rows = 0;
-        pa.warp_work = 0;
+        pa.warp_region_words = (int)(st->warp_basis_bytes / 4);
+        pa.heavy_rows = heavy;
+        pa.warp_work = st->warp_work;
+        pa.dedup_min = st->handoff_min > 0 ? 0 : (all_cta ? DEDUP_MIN_CTA : DEDUP_MIN_WARP);
+        pa.after = 0;
         pa.scale = 0;
         pa.num_sms = st->num_sms;
         // a shard share: the call's rows x (feature words + 4) over four per SM
@@ -1608,22 +1658,6 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
         st->widths_ready = true;
     }
     const Widths& wv = st->widths;
-    // Rows from which a context gets a whole CTA: unless set explicitly, it
-    // scales with the batch -- in a short call a warp-owned context of a few
-    // thousand rows, dependent round after round, would outlast everything
-    // else, while in a long one warps keep the SMs fuller
-    // else, and in a store of at most ALL_CTA_PER_SM contexts per SM, every
-    // context gets one: none waits for a CTA, and a CTA takes eight warps'
-    // rows per dependent round
-    int64_t heavy = st->heavy_rows;
-    const bool all_cta = !st->heavy_rows_set && st->num_ctx <= (int64_t)ALL_CTA_PER_SM * st->num_sms;
-    if (all_cta) {
-        heavy = 1;
-    } else if (!st->heavy_rows_set && !dedup) {
-        heavy = total_rows / HEAVY_ROWS_BATCH_DIV;
-        if (heavy < HEAVY_ROWS_MIN) heavy = HEAVY_ROWS_MIN;
-        if (heavy > st->heavy_rows) heavy = st->heavy_rows;
-    }
     const int scale = dedup && !all_cta && !st->heavy_rows_set && !st->warp_work_set;
     CheckArgs ca;
     ca.row_off = row_off;
@@ -1644,7 +1678,7 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
     return launch_elimination(sd, la, row_off, x_off, total_rows, total_x_words, dedup ? st->rep_count : nullptr,
                               heavy, st->warp_work, st->queue, st->keybuf, st->plan_hist + PLAN_HIST_WORDS,
                               st->num_sms, wv, st->full_ctr, st->full_cnt, st->full_first, cs, &fk, scale, true,
-                              st->long_call_rows, &ca);
+                              all_cta ? INT64_MAX : st->long_call_rows, &ca);
 }
 
 extern "C" int f2_learn_timing(const f2_store* st, uint64_t* out_host, f2_stream_t stream)
