@@ -45,6 +45,9 @@ struct LearnArgs {
     const int32_t* resume_from;
     const int32_t* resume_list;
     const int* resume_count;
+    // rows of each context of more than 17 words that elim_open_kernel has
+    // taken already
+    int32_t* open_from;
 };
 
 // The elimination kernels' launches, one function per translation unit (each
@@ -53,6 +56,7 @@ struct LearnArgs {
 cudaError_t elim_launch_small(const StoreDev& sd, LearnArgs la, int max_words, int num_sms, cudaStream_t cs);
 cudaError_t elim_launch_narrow(const StoreDev& sd, LearnArgs la, int max_words, int warps, int num_sms,
                                cudaStream_t cs);
+// (for rows of more than 17 words: elim_open_kernel, then the streaming kernel)
 cudaError_t elim_launch_wide(const StoreDev& sd, LearnArgs la, int max_d, bool medium, int num_sms, cudaStream_t cs);
 cudaError_t elim_load_small();
 cudaError_t elim_load_narrow();
@@ -66,6 +70,7 @@ constexpr int CTL_FIRST = 82;  // first contradiction index (int64)
 constexpr int CTL_WORDS = 84;  // size of the control area (16-byte multiple)
 
 constexpr int FULL_CHUNK = 2048;   // rows of a full-rank context claimed at a time
+constexpr int FULL_LATE_MIN = 64;  // rows left for a context that reaches full rank mid-call to be checked that way
 
 __host__ __device__ __forceinline__ int elim_words(int d, int wd) { return CTL_WORDS + d * row_stride(wd); }
 
@@ -1059,6 +1064,7 @@ __device__ void elim_cta(const StoreDev& s, const LearnArgs& a, int c, uint32_t*
     for (int v = 0; v < WD; ++v) st.P[v] = (rank0 && v < cd.wd) ? s.pivot[cd.pw_off + v] : 0u;
     st.rank = rank0;
     st.base = a.resume_from ? a.resume_from[c] : 0;  // the first representative of this launch
+    if constexpr (WD > WIDE_M_WD) st.base = a.open_from[c];
     st.quiet = st.parity = 0;
     st.first = LLONG_MAX;
     st.cnt = 0;
@@ -1066,7 +1072,11 @@ __device__ void elim_cta(const StoreDev& s, const LearnArgs& a, int c, uint32_t*
         *cnt_s = 0ull;
         *first_s = LLONG_MAX;
     }
-    if (rank0) basis_to_smem<WD>(s, cd, S, st.P, lane, warp, G);
+    int stop_at = -1;
+    if constexpr (WD > NARROW_WD) {  // full rank: the rows left are checks only (below)
+        if (!deduped && a.late_list && rank0 == cd.d && rs.R - st.base >= FULL_LATE_MIN) stop_at = st.base;
+    }
+    if (rank0 && stop_at < 0 && st.base < rs.R) basis_to_smem<WD>(s, cd, S, st.P, lane, warp, G);
     __syncthreads();
     uint64_t mixed = mixed_words<WD>(st.P, cd.d, cd.wd);
     uint32_t* const TB = S + cd.d * RS;
@@ -1075,9 +1085,8 @@ __device__ void elim_cta(const StoreDev& s, const LearnArgs& a, int c, uint32_t*
     const int np = (cd.d + 3) >> 2;
     Row<WD> nx;
     fetch_row<WD>(rs, st.base + t, nx);
-    int stop_at = -1;
     int snap_at = -1;  // handed off from this representative on
-    while (st.base < rs.R) {
+    while (st.base < rs.R && stop_at < 0) {
         if constexpr (WD <= TABLE_MAX_WD) {
             // by lookup table where it fits and costs fewer instructions than
             // the walk (about d/4 lookups a row against rank/2 two-pivot steps)
@@ -1152,10 +1161,10 @@ __device__ void elim_cta(const StoreDev& s, const LearnArgs& a, int c, uint32_t*
             wmask = publish_candidates(cand, wc, st.parity, warp, lane, G);
             if (!wmask) mixed = mixed_words<WD>(st.P, cd.d, cd.wd);
         }
-        // (wide contexts) full rank with at least a chunk of rows left: every
-        // later row is a check only (the rows are their own representatives)
+        // (wide contexts) full rank with rows left: every later row is a check
+        // only (the rows are their own representatives)
         if constexpr (WD > NARROW_WD) {
-            if (!deduped && a.late_list && st.quiet == 0 && rs.R - st.base >= FULL_CHUNK && st.rank == cd.d) {
+            if (!deduped && a.late_list && st.quiet == 0 && rs.R - st.base >= FULL_LATE_MIN && st.rank == cd.d) {
                 stop_at = st.base;
                 break;
             }

@@ -11,6 +11,221 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, WDT <= WIDE_M_WD ? 2 : 1) eli
     elim_cta_queue<CLS, RESUME>(s, a, [&](int c) { elim_cta<WDT>(s, a, c, smem, a.cta_region_words); });
 }
 
+// ---------------------------------------------------------------------------
+// The first OPEN_THREADS rows of an empty basis of up to WIDE_WD words, a row
+// a thread, in registers.  The rows go in stream order: the row's warp puts it
+// into shared memory and finds its highest set bit, and after one barrier
+// every thread whose row has that bit XORs it from there (broadcast loads,
+// only the words up to the pivot's).  The rows stay reduced among themselves,
+// so what remains is the reduced basis.  A pivot costs about 40 instructions a
+// warp and a barrier; streaming 256 rows at a time against a basis in shared
+// memory, the 1,025 pivots of a dense 1,024-bit context took 3,000 cycles
+// each, most of it in reading older rows a lane each.  Two batches of 65,536
+// rows for 64 such contexts went from 3,012 to 2,256 us.  Dense rows are a few pivots short of full
+// rank after d rows: up to OPEN_EXTRA further rows are reduced one at a time
+// by all threads (a XOR reduction of the rows their bits select).
+// ---------------------------------------------------------------------------
+constexpr int OPEN_THREADS = 1024;
+constexpr int OPEN_EXTRA = 32;
+constexpr int OPEN_Z = 9;  // uint4 index of the word in a shared row; the features before it
+
+struct OpenSmem {
+    uint4 row[2][OPEN_Z + 1];
+    uint32_t q[WIDE_WD + 3];  // a further row's own bits
+    uint32_t mask[WIDE_WD + 3];
+    int head[2];
+    int holder;
+    unsigned long long cnt;
+    long long first;
+};
+
+template <int W>
+__device__ __forceinline__ void open_xor(uint32_t (&x)[WIDE_WD], uint4& y, const uint4* __restrict__ row, uint32_t m,
+                                         bool own)
+{
+    if ((x[W] & m) != 0u && !own) {
+        xor4(y, row[OPEN_Z]);
+#pragma unroll
+        for (int c = 0; 4 * c <= W; ++c) {
+            const uint4 t = row[c];
+            const uint32_t e[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (4 * c + j <= W) x[4 * c + j] ^= e[j];
+        }
+    }
+}
+
+// XOR the row with pivot k into this thread's row if that has bit k set.
+__device__ __forceinline__ void open_step(int k, uint32_t (&x)[WIDE_WD], uint4& y, const uint4* __restrict__ row,
+                                          bool own)
+{
+    const uint32_t m = 1u << (k & 31);
+#define F2_OPEN(W) case W: open_xor<W>(x, y, row, m, own); break;
+    switch (k >> 5) {
+        F2_OPEN(0) F2_OPEN(1) F2_OPEN(2) F2_OPEN(3) F2_OPEN(4) F2_OPEN(5) F2_OPEN(6) F2_OPEN(7) F2_OPEN(8)
+        F2_OPEN(9) F2_OPEN(10) F2_OPEN(11) F2_OPEN(12) F2_OPEN(13) F2_OPEN(14) F2_OPEN(15) F2_OPEN(16)
+        F2_OPEN(17) F2_OPEN(18) F2_OPEN(19) F2_OPEN(20) F2_OPEN(21) F2_OPEN(22) F2_OPEN(23) F2_OPEN(24)
+        F2_OPEN(25) F2_OPEN(26) F2_OPEN(27) F2_OPEN(28) F2_OPEN(29) F2_OPEN(30) F2_OPEN(31) F2_OPEN(32)
+    default: break;
+    }
+#undef F2_OPEN
+}
+
+// Highest set bit of a row in shared memory, by a warp; -1 if it is zero.
+__device__ __forceinline__ int open_top(const uint4* row, int lane)
+{
+    static_assert(WIDE_WD == 33, "one word past the lanes");
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(row);
+    const uint32_t v = w[lane], last = w[32];
+    const uint32_t b = __ballot_sync(FULL, v != 0u);
+    const int tw = b ? 31 - __clz(b) : 0;
+    const uint32_t t = __shfl_sync(FULL, v, tw);
+    if (last) return 1024 + 31 - __clz(last);
+    return b ? 32 * tw + 31 - __clz(t) : -1;
+}
+
+__global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, LearnArgs a)
+{
+    __shared__ OpenSmem sm;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int n_items = a.counters[CNT_COUNT + CLS_WIDE];
+    const int32_t* const list = a.queue + a.counters[CNT_BEGIN + CLS_WIDE];
+    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+        const int c = list[item];
+        if (s.rank[c] != 0) {
+            if (t == 0) a.open_from[c] = 0;
+            continue;
+        }
+        const CtxDesc cd = s.desc[c];
+        bool deduped;
+        const RowStream rs = row_stream(s, a, cd, c, deduped);
+        const int n = rs.R < OPEN_THREADS ? rs.R : OPEN_THREADS;
+        Row<WIDE_WD> r;
+        fetch_row<WIDE_WD>(rs, t, r);
+        uint32_t x[WIDE_WD];
+        make_q<WIDE_WD>(r.x, r.valid, rs.raw, x);
+        uint4 y = r.y;
+        int pk = -1, rank = 0;
+        __syncthreads();  // the last context's shared memory is done with
+        if (t < WIDE_WD) sm.mask[t] = 0u;
+        if (t == 0) {
+            sm.cnt = 0ull;
+            sm.first = LLONG_MAX;
+        }
+        for (int i = 0; i < n && rank < cd.d; ++i) {
+            if (warp == (i >> 5)) {
+                uint4* const row = sm.row[i & 1];
+                if (t == i) {
+#pragma unroll
+                    for (int v4 = 0; v4 < OPEN_Z; ++v4) {
+                        uint32_t e[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) e[j] = 4 * v4 + j < WIDE_WD ? x[4 * v4 + j < WIDE_WD ? 4 * v4 + j : 0] : 0u;
+                        row[v4] = make_uint4(e[0], e[1], e[2], e[3]);
+                    }
+                    row[OPEN_Z] = y;
+                }
+                __syncwarp();
+                const int k = open_top(row, lane);
+                if (t == i) {
+                    sm.head[i & 1] = k;
+                    pk = k;
+                }
+            }
+            __syncthreads();
+            const int k = sm.head[i & 1];
+            if (k < 0) continue;
+            ++rank;
+            open_step(k, x, y, sm.row[i & 1], t == i);
+        }
+        // rows without a pivot lie in the span of the rows before them
+        if (t < n && pk < 0 && nonzero4(y)) {
+            atomicAdd(&sm.cnt, (unsigned long long)r.weight);
+            atomicMin(&sm.first, rs.seen + (long long)r.i);
+        }
+        int base = n;
+        for (int extra = 0; rank < cd.d && base < rs.R && extra < OPEN_EXTRA; ++extra, ++base) {
+            __syncthreads();
+            uint32_t* const acc = reinterpret_cast<uint32_t*>(sm.row[0]);
+            const int i = rs.reps ? __ldg(rs.reps + base) : base;
+            if (warp == 0) {
+                const uint32_t* xr = rs.xc + (int64_t)i * rs.xw;
+                for (int w = lane; w < WIDE_WD + 3; w += 32) {
+                    auto word = [&](int v) {
+                        if (v < 0 || v >= rs.xw) return 0u;
+                        uint32_t u = __ldg(xr + v);
+                        if (v == rs.xw - 1 && (rs.n & 31)) u &= (1u << (rs.n & 31)) - 1u;
+                        return u;
+                    };
+                    uint32_t q = 0;
+                    if (w < WIDE_WD) q = rs.raw ? word(w) : (word(w) << 1) | (w ? word(w - 1) >> 31 : 1u);
+                    acc[w] = q;
+                    sm.q[w] = q;
+                }
+                if (lane == 0) {
+                    sm.row[0][OPEN_Z] = __ldg(rs.yc + i);
+                    sm.holder = OPEN_THREADS;
+                }
+            }
+            __syncthreads();
+            const bool sel = pk >= 0 && ((sm.q[pk >= 0 ? pk >> 5 : 0] >> (pk & 31)) & 1u);
+            if (__any_sync(FULL, sel)) {
+#pragma unroll
+                for (int v = 0; v < WIDE_WD; ++v) {
+                    const uint32_t g = __reduce_xor_sync(FULL, sel ? x[v] : 0u);
+                    if (lane == 0 && g) atomicXor(acc + v, g);
+                }
+                const uint32_t z[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const uint32_t g = __reduce_xor_sync(FULL, sel ? z[v] : 0u);
+                    if (lane == 0 && g) atomicXor(acc + 4 * OPEN_Z + v, g);
+                }
+            }
+            if (pk < 0) atomicMin(&sm.holder, t);
+            __syncthreads();
+            const int k = open_top(sm.row[0], lane);
+            const uint4 z = sm.row[0][OPEN_Z];
+            if (k < 0) {
+                if (t == 0 && nonzero4(z)) {
+                    sm.cnt += 1u + (rs.dups ? (uint32_t)__ldg(rs.dups + base) : 0u);
+                    if (rs.seen + (long long)i < sm.first) sm.first = rs.seen + (long long)i;
+                }
+                continue;
+            }
+            ++rank;
+            open_step(k, x, y, sm.row[0], false);
+            if (t == sm.holder) {
+#pragma unroll
+                for (int v = 0; v < WIDE_WD; ++v) x[v] = acc[v];
+                y = z;
+                pk = k;
+            } else if (sm.holder == OPEN_THREADS && t == 0) {
+                // every thread holds a pivot: this is the last one (d <= 1,025)
+                s.bz[cd.slot_off + k] = z;
+                for (int v = 0; v < cd.wd; ++v) s.bx[cd.xw_off + (int64_t)k * cd.wd + v] = acc[v];
+                atomicOr(sm.mask + (k >> 5), 1u << (k & 31));
+            }
+        }
+        if (pk >= 0) {
+            s.bz[cd.slot_off + pk] = y;
+            uint32_t* dst = s.bx + cd.xw_off + (int64_t)pk * cd.wd;
+#pragma unroll
+            for (int v = 0; v < WIDE_WD; ++v)
+                if (v < cd.wd) dst[v] = x[v];
+            atomicOr(sm.mask + (pk >> 5), 1u << (pk & 31));
+        }
+        __syncthreads();
+        if (t < cd.wd) s.pivot[cd.pw_off + t] = sm.mask[t];
+        if (t == 0) {
+            s.rank[c] = rank;
+            a.open_from[c] = base;
+            commit_stats(s, c, sm.first, sm.cnt);
+        }
+    }
+}
+
 template <typename K>
 cudaError_t launch(K kernel, const StoreDev& sd, LearnArgs la, int max_d, int wdt, int per_sm, int num_sms,
                    cudaStream_t cs)
@@ -29,13 +244,17 @@ cudaError_t elim_launch_wide(const StoreDev& sd, LearnArgs la, int max_d, bool m
 {
     if (medium)
         return launch(elim_wide_kernel<WIDE_M_WD, CLS_WIDE_M, CLS_RESUME_W>, sd, la, max_d, WIDE_M_WD, 2, num_sms, cs);
+    elim_open_kernel<<<num_sms, OPEN_THREADS, 0, cs>>>(sd, la);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     return launch(elim_wide_kernel<WIDE_WD, CLS_WIDE, CLS_RESUME_W>, sd, la, max_d, WIDE_WD, 1, num_sms, cs);
 }
 
 cudaError_t elim_load_wide()
 {
     cudaFuncAttributes fa;
-    const cudaError_t e = cudaFuncGetAttributes(&fa, elim_wide_kernel<WIDE_M_WD, CLS_WIDE_M, CLS_RESUME_W>);
+    cudaError_t e = cudaFuncGetAttributes(&fa, elim_wide_kernel<WIDE_M_WD, CLS_WIDE_M, CLS_RESUME_W>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, elim_open_kernel);
     return e != cudaSuccess ? e : cudaFuncGetAttributes(&fa, elim_wide_kernel<WIDE_WD, CLS_WIDE, CLS_RESUME_W>);
 }
 

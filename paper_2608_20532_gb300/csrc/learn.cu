@@ -1353,12 +1353,14 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
 {
     // prezeroed: the caller has cleared full_ctr's first 2C words and late
     // count, full_cnt, full_first (to -1) and hist
-    // full_ctr: chunks claimed [C], chunks done [C], late start [C], late list [C], late count
+    // full_ctr: chunks claimed [C], chunks done [C], late start [C], late list [C], late count,
+    // rows taken by elim_open_kernel [C]
     const int C = sd.num_ctx;
     LearnArgs lx = la;
     lx.late_start = full_ctr + 2 * C;
     lx.late_list = full_ctr + 3 * C;
     lx.late_count = full_ctr + 4 * C;
+    lx.open_from = full_ctr + 4 * C + 1;
     if (!prezeroed) {
         cudaError_t e0 = cudaMemsetAsync(full_ctr, 0, sizeof(int) * 2 * (size_t)C, cs);
         if (e0 == cudaSuccess) e0 = cudaMemsetAsync(lx.late_count, 0, sizeof(int), cs);
@@ -1708,7 +1710,7 @@ struct NoallocScratch {
     int32_t keybuf[F2_NOALLOC_MAX_CTX];
     int counters[CNT_WORDS];
     int plan_hist[PLAN_KEYS];
-    int full_ctr[4 * F2_NOALLOC_MAX_CTX + 1];
+    int full_ctr[5 * F2_NOALLOC_MAX_CTX + 1];
     unsigned long long full_cnt[F2_NOALLOC_MAX_CTX];
     unsigned long long full_first[F2_NOALLOC_MAX_CTX];
 };

@@ -227,7 +227,7 @@ extern "C" int f2_create(f2_store** out, int32_t num_ctx, const int32_t* n_bits_
         {(void**)&s->shard_done, sizeof(int32_t) * C},
         {(void**)&s->hand, sizeof(int) * (2 + 6 * C)},
         {(void**)&s->plan_hist, sizeof(int) * 2 * PLAN_HIST_WORDS},  // the two plans of a learn call
-        {(void**)&s->full_ctr, sizeof(int) * (4 * C + 1)},
+        {(void**)&s->full_ctr, sizeof(int) * (5 * C + 1)},
         {(void**)&s->full_cnt, sizeof(unsigned long long) * C},
         {(void**)&s->full_first, sizeof(unsigned long long) * C},
     };
