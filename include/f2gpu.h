@@ -329,10 +329,10 @@ enum f2_option {
                                     the rest of its call off to a parallel check when at least this many
                                     of its representatives are left (a representative outside the basis
                                     sends the rest back to elimination from there); only in calls of at
-                                    least 16x this many rows; default 0 = never. It pays only where a
-                                    few long contexts bound the call: 8192 took a 10,000-context
-                                    wide-feature learn from 1.61 to 1.56 ms, but the 77,926- and
-                                    4,096-context learns 1-7% longer */
+                                    least 16x this many rows; 0 = never. Unless this is set, calls of at
+                                    least 2^20 rows on a store with contexts of 10..17 words hand off
+                                    the contexts that hold an eighth of an SM's share of the call's
+                                    work or more (at least 2048 representatives) */
 };
 int f2_set_option(f2_store* store, int option, int64_t value);
 

@@ -34,7 +34,7 @@ constexpr int DEFAULT_WARP_REGION_BYTES = 13824;  // shared memory of one warp-o
 constexpr int DEFAULT_SMALL_REGION_BYTES = 9472;  // the same in the small-width kernel (d <= 96)
 constexpr int64_t DEFAULT_ENCODE_DIRECT_MAX = 65536;  // encode passes this small skip the grouping
 constexpr int64_t DEFAULT_LONG_CALL_ROWS = 0;  // learn calls this long: 4-warp CTAs (4..9 words)
-constexpr int64_t DEFAULT_HANDOFF_REPS = 0;  // representatives left for a saturated context to hand off (0: never)
+constexpr int64_t DEFAULT_HANDOFF_REPS = -1;  // representatives left for a saturated context to hand off (0: never, -1: by the call's work)
 constexpr int DEFAULT_HEAVY_ROWS = 4096;          // rows from which a context gets a whole CTA (at most)
 constexpr int HEAVY_ROWS_MIN = 1024;              // ... and at least, when it scales with the batch:
 constexpr int HEAVY_ROWS_BATCH_DIV = 20000;       // batch rows / this (no duplicate pass), or
@@ -361,7 +361,7 @@ struct f2_store {
     int dd_shards;              // most CTAs one context's duplicate pass is split over
     int64_t enc_direct_max;     // encode passes of at most this many queries skip the grouping
     int64_t long_call_rows;     // learn calls of at least this many rows: 4-warp CTAs for 4..9-word contexts
-    int64_t handoff_min;        // representatives left for a saturated context to hand off (0: never)
+    int64_t handoff_min;        // representatives left for a saturated context to hand off (0: never, -1: by the call's work)
     int* hand;                  // hand-off lists: counts [2], snap list/start [2C], resume list/from [2C], chunk counters [2C]
     uint4* check_rec;           // the check's chunk records (2 x uint4 each), grown per call
     int64_t check_rec_cap;

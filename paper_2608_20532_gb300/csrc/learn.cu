@@ -1310,6 +1310,17 @@ __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, F
     }
 }
 
+// The default hand-off (see f2_learn_batched): calls of at least this many
+// rows, contexts with at least this many representatives left that are at
+// least HANDOFF_SHARE / 16 of an SM's share of the call's representatives x d.
+// On 10,000 contexts of parsed values (13.6M rows) the learn call took 1,515 us
+// without, 1,415 / 1,286 / 1,347 / 1,400 / 1,398 / 1,583 at 1 / 2 / 3 / 4 / 6 / 8.
+// Calls without rows of 10..17 words gain nothing: 4,096 contexts took 268 us
+// without and 293 or more with it, 77,926 contexts 2,379 and 2,467 or more.
+constexpr int64_t HANDOFF_AUTO_ROWS = int64_t(1) << 20;
+constexpr int HANDOFF_AUTO_REPS = 2048;
+constexpr int HANDOFF_SHARE = 2;
+
 // Which elimination kernels a store needs, and their widest bases.
 
 // Calls of at least this many rows run the 4..9-word elimination in CTAs of
@@ -1514,9 +1525,23 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
         if (e != cudaSuccess) return F2_ERR_OOM;
         st->rep_capacity = total_rows;
     }
+    if (!st->widths_ready) {  // fixed by the widths: computed once per store
+        st->widths = width_summary(st->n_bits.data(), st->num_ctx, (st->flags & F2_FLAG_RAW_FEATURES) != 0);
+        st->widths_ready = true;
+    }
+    const Widths& wv = st->widths;
+    // Hand-off of saturated contexts, in calls long enough to have some.  By
+    // default only in calls with contexts of 10..17 words, whose rows cost
+    // most, and there for the few contexts that hold HANDOFF_SHARE / 16 of an
+    // SM's share of the call's work or more.
+    const bool auto_hand = st->handoff_min < 0 && dedup && wv.has_wide_m && total_rows >= HANDOFF_AUTO_ROWS;
+    const int hand_min = auto_hand ? HANDOFF_AUTO_REPS
+                         : (st->handoff_min > 0 && total_rows >= HANDOFF_CALL_FACTOR * st->handoff_min)
+                             ? (int)st->handoff_min
+                             : 0;
     // every scratch counter of the call, zeroed by one launch
     const size_t C = (size_t)st->num_ctx;
-    if (st->handoff_min > 0) {  // the check's chunk records, grown stream-ordered
+    if (hand_min > 0) {  // the check's chunk records, grown stream-ordered
         const int64_t slots = total_rows / CHECK_CHUNK + (int64_t)C + 1;
         if (slots > st->check_rec_cap) {
             if (st->check_rec) cudaFreeAsync(st->check_rec, cs);
@@ -1533,7 +1558,7 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
         if (!st->timing && f2_dev_alloc(st, (void**)&st->timing, bytes, cs, true) != cudaSuccess) return F2_ERR_OOM;
         zl.add(st->timing, bytes);
     }
-    {  // hand-off: the two list counts and the chunk counters
+    if (hand_min > 0) {  // hand-off: the two list counts and the chunk counters
         zl.add(st->hand, sizeof(int) * 2);
         zl.add(st->hand + 2 + 4 * C, sizeof(int) * 2 * C);
     }
@@ -1646,20 +1671,15 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
     la.tables = st->elim_tables;
     la.small_region_words = (int)(st->small_basis_bytes / 4);
     la.cta_region_words = 0;  // set per launch
-    // hand-off of saturated contexts, in calls long enough to have some
-    la.handoff_min = (st->handoff_min > 0 && total_rows >= HANDOFF_CALL_FACTOR * st->handoff_min)
-                         ? (int)st->handoff_min : 0;
+    la.handoff_min = hand_min;
+    la.handoff_share = auto_hand ? HANDOFF_SHARE : 0;
+    la.num_sms = st->num_sms;
     la.snap_count = st->hand;
     la.snap_list = st->hand + 2;
     la.snap_start = st->hand + 2 + C;
     la.resume_from = nullptr;
     la.resume_list = nullptr;
     la.resume_count = nullptr;
-    if (!st->widths_ready) {  // fixed by the widths: computed once per store
-        st->widths = width_summary(st->n_bits.data(), st->num_ctx, (st->flags & F2_FLAG_RAW_FEATURES) != 0);
-        st->widths_ready = true;
-    }
-    const Widths& wv = st->widths;
     const int scale = dedup && !all_cta && !st->heavy_rows_set && !st->warp_work_set;
     CheckArgs ca;
     ca.row_off = row_off;
@@ -1927,6 +1947,8 @@ extern "C" int f2_learn_batched_noalloc(int32_t num_ctx, const int32_t* n_bits_h
     la.small_region_words = DEFAULT_SMALL_REGION_BYTES / 4;
     la.cta_region_words = 0;
     la.handoff_min = 0;
+    la.handoff_share = 0;
+    la.num_sms = nd->num_sms;
     la.snap_count = nullptr;
     la.snap_list = nullptr;
     la.snap_start = nullptr;
