@@ -110,6 +110,9 @@ constexpr int DD_WARP_REGION = 3 * DD_WARP_E;   // words
 constexpr int DD_QUAD_E = 4 * DD_WARP_E;
 constexpr int DD_CTA_E = 8192;
 constexpr int DD_SMEM = 4 * 3 * DD_CTA_E;       // bytes (also 16 warp regions)
+constexpr int DD_SEG_ROWS = 16384;              // rows a CTA takes at a time (10..16-word rows)
+constexpr int DD_QUAD_REPS = 1024;              // most distinct rows numbered by a quad, by a CTA (as above)
+constexpr int DD_CTA_REPS = 4096;
 constexpr int DD_K = 2;                         // rows per thread per round (feature rows of 1-2 words)
 constexpr int DD_XW = NARROW_WD;                // widest feature row (words) of dedup_kernel<false>
 constexpr int DD_XW_WIDE = 16;                  // widest of dedup_kernel<true> (one row in flight)
@@ -260,6 +263,73 @@ __device__ __forceinline__ void dd_sync()
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)(threadIdx.x >> 5) / G), "r"(32 * G) : "memory");
 }
 
+// The queue item of the context a dedup CTA is on (context, shard, shard
+// count); a CTA-owned pass reads it here, before and again after its rows, so
+// that no register holds it through them.
+__shared__ uint32_t dd_cta_item;
+
+// Closes a context's (or a shard's) pass: publishes its count and, in the last
+// shard of a split context to finish, moves the shards' lists together.
+// Returns whether the context is done.
+template <int G>
+__device__ bool dd_finish(const DedupArgs& a, int c, int nrep, int t)
+{
+    constexpr int NT = 32 * G;
+    int shard = 0, nsh = 1;
+    if constexpr (G == DD_WARPS) {
+        const uint32_t qi = *reinterpret_cast<const volatile uint32_t*>(&dd_cta_item);
+        shard = (int)((qi >> 24) & 7u);
+        nsh = (int)(qi >> 28) + 1;
+    }
+    if (nsh == 1) {
+        if (t == 0) a.rep_count[c] = nrep;
+        dd_sync<G>();
+        return true;
+    }
+    // a split context: publish this shard's count; the last shard to finish
+    // moves the lists of shards 1.. down behind shard 0's (never upward: a
+    // shard's list starts at or after its destination), chunk by chunk
+    // through registers, renumbering their rows from the context's first
+    __shared__ int s_last;
+    __threadfence();  // this thread's list entries, before the count that publishes them
+    dd_sync<G>();
+    if (t == 0) {
+        a.shard_reps[(size_t)DD_MAX_SHARDS * c + shard] = nrep;
+        __threadfence();
+        s_last = (atomicAdd(a.shard_done + c, 1) == nsh - 1);
+    }
+    dd_sync<G>();
+    if (!s_last) return false;
+    __threadfence();
+    const int64_t cbase = a.row_off[c];
+    const int Tall = (int)(a.row_off[c + 1] - cbase);
+    int dst = 0;
+    for (int k = 0; k < nsh; ++k) {
+        const int src = (int)(((long long)Tall * k) / nsh);
+        const int cnt = __ldcg(a.shard_reps + (size_t)DD_MAX_SHARDS * c + k);
+        if (k > 0) {
+            for (int b0 = 0; b0 < cnt; b0 += NT) {
+                const int j = b0 + t;
+                int32_t rl = 0, rd = 0;
+                if (j < cnt) {
+                    rl = __ldcg(a.rep_list + cbase + src + j) + src;
+                    rd = __ldcg(a.rep_dup + cbase + src + j);
+                }
+                dd_sync<G>();
+                if (j < cnt) {
+                    a.rep_list[cbase + dst + j] = rl;
+                    a.rep_dup[cbase + dst + j] = rd;
+                }
+                dd_sync<G>();
+            }
+        }
+        dst += cnt;
+    }
+    if (t == 0) a.rep_count[c] = dst;
+    dd_sync<G>();
+    return true;
+}
+
 // One group of G warps finds the representatives of context c and writes
 // them, in stream order, to rep_list[row_off[c] + k] with their duplicate
 // counts in rep_dup; rep_count[c] = number of representatives.  Each thread
@@ -276,11 +346,6 @@ __device__ __forceinline__ void dd_sync()
 // together, in stream order, and sets rep_count[c].  Returns whether the
 // context is done (false in the shards that did not finish last).
 //
-// The queue item of the context a dedup CTA is on (context, shard, shard
-// count); a CTA-owned pass reads it here, before and again after its rows, so
-// that no register holds it through them.
-__shared__ uint32_t dd_cta_item;
-
 template <int G, int XW>
 __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t* region, int E, int* wcnt)
 {
@@ -448,58 +513,7 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
                   (unsigned long long)nrep * (unsigned long long)cd.d);
         atomicAdd(reinterpret_cast<unsigned long long*>(a.counters + CNT_REPS), (unsigned long long)nrep);
     }
-    if constexpr (G == DD_WARPS) {
-        const uint32_t qi = *reinterpret_cast<const volatile uint32_t*>(&dd_cta_item);
-        shard = (int)((qi >> 24) & 7u);
-        nsh = (int)(qi >> 28) + 1;
-    }
-    if (nsh == 1) {
-        if (t == 0) a.rep_count[c] = nrep;
-        dd_sync<G>();
-        return true;
-    }
-    // a split context: publish this shard's count; the last shard to finish
-    // moves the lists of shards 1.. down behind shard 0's (never upward: a
-    // shard's list starts at or after its destination), chunk by chunk
-    // through registers, renumbering their rows from the context's first
-    __shared__ int s_last;
-    __threadfence();  // this thread's list entries, before the count that publishes them
-    dd_sync<G>();
-    if (t == 0) {
-        a.shard_reps[(size_t)DD_MAX_SHARDS * c + shard] = nrep;
-        __threadfence();
-        s_last = (atomicAdd(a.shard_done + c, 1) == nsh - 1);
-    }
-    dd_sync<G>();
-    if (!s_last) return false;
-    __threadfence();
-    const int64_t cbase = a.row_off[c];
-    const int Tall = (int)(a.row_off[c + 1] - cbase);
-    int dst = 0;
-    for (int k = 0; k < nsh; ++k) {
-        const int src = (int)(((long long)Tall * k) / nsh);
-        const int cnt = __ldcg(a.shard_reps + (size_t)DD_MAX_SHARDS * c + k);
-        if (k > 0) {
-            for (int b0 = 0; b0 < cnt; b0 += NT) {
-                const int j = b0 + t;
-                int32_t rl = 0, rd = 0;
-                if (j < cnt) {
-                    rl = __ldcg(a.rep_list + cbase + src + j) + src;
-                    rd = __ldcg(a.rep_dup + cbase + src + j);
-                }
-                dd_sync<G>();
-                if (j < cnt) {
-                    a.rep_list[cbase + dst + j] = rl;
-                    a.rep_dup[cbase + dst + j] = rd;
-                }
-                dd_sync<G>();
-            }
-        }
-        dst += cnt;
-    }
-    if (t == 0) a.rep_count[c] = dst;
-    dd_sync<G>();
-    return true;
+    return dd_finish<G>(a, c, nrep, t);
 }
 
 __device__ __forceinline__ int pow2_at_least(int v)
@@ -507,6 +521,330 @@ __device__ __forceinline__ int pow2_at_least(int v)
     int e = 64;
     while (e < v) e <<= 1;
     return e;
+}
+
+// ---------------------------------------------------------------------------
+// Pass 1 for feature rows of 10..16 words.  Confirming a repeat from global
+// memory costs such a row 14 to 20 scattered loads, so copies of the distinct
+// rows are kept in shared memory, and a warp never waits for the others between
+// rows.  10,000 contexts of parsed values went from 1,471 to 1,403 us; with
+// rows of up to nine words the form above is as fast or faster (77,926
+// contexts 2,609 us and 2,598 with this one, 4,096 contexts 282 and 287):
+// there the extra instructions cost what the loads save.
+// ---------------------------------------------------------------------------
+// A group's shared memory while it looks for the distinct rows among at most
+// DD_SEG_ROWS consecutive rows of a context.  The distinct rows found so far
+// are numbered; number r has its smallest row index idx[r], its repeats
+// dup[r], and for r < cap a copy of the row itself (ys, xs), so that a repeat
+// is confirmed from shared memory: 32 random rows in global memory cost the
+// L1 a tag lookup each, which bound the pass.  A slot of the hash table holds
+// (16 bits of the hash, r + 1), a bucket four slots that one load fetches: with
+// single slots nearly every round had some lane on its third or fourth probe.
+// Rows that find no room (nrep numbers, the probe limit, a distinct row with
+// their fingerprint in the bucket) are marked in `ovf` and stand for
+// themselves, which is exact.
+// (Word offsets into the CTA's dynamic shared memory.)
+struct DdSmem {
+    int tab, idx, dup;
+    int bm;   // rows that are the first of their content
+    int ovf;  // rows that found no room
+    int pre;  // first rows in the bitmap words before
+    int cnt;  // numbers given out; rows without room (0 or 1)
+    int ys, xs;
+    uint32_t emask;
+    int nrep, cap, words;
+};
+__device__ __forceinline__ uint32_t* dd_smem()
+{
+    extern __shared__ __align__(16) uint32_t smem[];
+    return smem;
+}
+__device__ __forceinline__ uint4 dd_load4(int word)  // volatile: other warps fill it
+{
+    uint4 v;
+    asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "r"(smem_addr(dd_smem() + word))
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4* dd_smem4(int word) { return reinterpret_cast<uint4*>(dd_smem() + word); }
+
+template <int XW>
+__device__ __forceinline__ DdSmem dd_layout(int region, int region_words, int T, int most)
+{
+    DdSmem m;
+    m.words = (T + 31) >> 5;
+    // three quarters of the rows: beyond that most rows have no repeat to find
+    const int want = (((3 * T) >> 2) + 31) & ~31;
+    m.nrep = want < most ? (want < 32 ? 32 : want) : most;
+    const int E = pow2_at_least(m.nrep + m.nrep / 3);
+    m.emask = (uint32_t)(E / 4 - 1);  // buckets of four slots
+    m.tab = region;
+    m.idx = m.tab + E;
+    m.dup = m.idx + m.nrep;
+    m.bm = m.dup + m.nrep;
+    m.ovf = m.bm + m.words;
+    m.pre = m.ovf + m.words;
+    m.cnt = m.pre + m.words;
+    const int used = (E + 2 * m.nrep + 3 * m.words + 2 + 3) & ~3;
+    const int cap = (region_words - used) / (4 + XW);
+    m.cap = cap < m.nrep ? cap : m.nrep;
+    m.ys = region + used;
+    m.xs = region + used + 4 * m.cap;
+    return m;
+}
+
+// Feature words of a row: the widest loads that every row of the context
+// allows (`al`: log2 of the words its rows are aligned to).
+template <int XW>
+__device__ __forceinline__ void load_words(const uint32_t* __restrict__ p, int al, uint32_t (&x)[XW])
+{
+    if (XW % 4 == 0 && al >= 2) {
+#pragma unroll
+        for (int v = 0; v + 3 < XW; v += 4) {
+            const uint4 t = __ldg(reinterpret_cast<const uint4*>(p + v));
+            x[v] = t.x;
+            x[v + 1] = t.y;
+            x[v + 2] = t.z;
+            x[v + 3] = t.w;
+        }
+    } else if (XW % 2 == 0 && al >= 1) {
+#pragma unroll
+        for (int v = 0; v + 1 < XW; v += 2) {
+            const uint2 t = __ldg(reinterpret_cast<const uint2*>(p + v));
+            x[v] = t.x;
+            x[v + 1] = t.y;
+        }
+    } else {
+#pragma unroll
+        for (int v = 0; v < XW; ++v) x[v] = __ldg(p + v);
+    }
+}
+
+// Hash of an observation: a sum of the words times odd constants, mixed.  It
+// only proposes candidates; every match is confirmed by comparing the rows.
+template <int XW>
+__device__ __forceinline__ uint32_t dd_hash(const uint32_t (&x)[XW], const uint4& y)
+{
+    uint32_t h = y.x * 0x9E3779B1u + y.y * 0x85EBCA77u + y.z * 0xC2B2AE3Du + y.w * 0x27D4EB2Fu;
+    uint32_t k = 0x165667B1u;
+#pragma unroll
+    for (int v = 0; v < XW; ++v) {
+        h += x[v] * k;
+        k = k * 0x01000193u + 0x3C6EF372u;  // constants at compile time
+        k |= 1u;
+    }
+    h ^= h >> 16;
+    h *= 0x7FEB352Du;
+    h ^= h >> 15;
+    return h;
+}
+
+// Row (x, y) equals the row numbered r, whose smallest index so far is i0.
+template <int XW>
+__device__ __forceinline__ bool dd_same(const DdSmem& m, int r, const uint32_t (&x)[XW], const uint4& y,
+                                        const uint32_t* __restrict__ xc, const uint4* __restrict__ yc, uint32_t lm)
+{
+    uint4 o;
+    uint32_t diff = 0;
+    if (r < m.cap) {
+        o = *dd_smem4(m.ys + 4 * r);
+#pragma unroll
+        for (int v = 0; v < XW; ++v) diff |= dd_smem()[m.xs + r * XW + v] ^ x[v];
+    } else {
+        const int64_t j = (int64_t)*reinterpret_cast<const volatile uint32_t*>(dd_smem() + m.idx + r);
+        o = __ldg(yc + j);
+#pragma unroll
+        for (int v = 0; v < XW; ++v) {
+            const uint32_t w = __ldg(xc + j * XW + v);
+            diff |= (v == XW - 1 ? w & lm : w) ^ x[v];
+        }
+    }
+    return (diff | (o.x ^ y.x) | (o.y ^ y.y) | (o.z ^ y.z) | (o.w ^ y.w)) == 0u;
+}
+
+// The distinct rows among T <= DD_SEG_ROWS rows, by a group of G warps: their
+// indices (plus `off`), in stream order, and repeats go to rep / dups; returns
+// their number.  Each thread takes K rows a round and no round waits for
+// another, so the warps hide each other's latencies; the first rows are put in
+// order at the end, through a bitmap.
+template <int G, int XW>
+__device__ int dedup_rows(const uint32_t* __restrict__ xc, const uint4* __restrict__ yc, int T, int off, uint32_t lm,
+                          int al, const DdSmem& m, int32_t* __restrict__ rep, int32_t* __restrict__ dups, int* wcnt)
+{
+    constexpr int NT = 32 * G;
+    const int lane = threadIdx.x & 31;
+    const int gw = (G == 1) ? 0 : (int)((threadIdx.x >> 5) % G);  // warp within the group
+    const int t = 32 * gw + lane;
+    for (int e = m.tab + t; e < m.idx; e += NT) dd_smem()[e] = 0u;
+    for (int e = t; e < 2 * m.words; e += NT) dd_smem()[m.bm + (e)] = 0u;  // bm and ovf
+    if (t < 2) dd_smem()[m.cnt + (t)] = 0u;
+    dd_sync<G>();
+    for (int base = 0; base < T; base += NT) {
+        const int i = base + t;
+        const int ic = i < T ? i : T - 1;  // (a row read twice, not counted)
+        const uint4 y = __ldg(yc + ic);
+        uint32_t x[XW];
+        load_words<XW>(xc + (int64_t)ic * XW, al, x);
+        x[XW - 1] &= lm;
+        const uint32_t h = dd_hash<XW>(x, y);
+        const uint32_t fp = (h & 0xFFFF0000u) | 0x80000000u;  // never an empty slot's
+        int bucket = m.tab + 4 * (int)(h & m.emask);
+        int mine = -1;                // a number allocated for this row
+        int same = -1;                // the number of the row it repeats
+        bool pending = i < T, alone = false;
+        for (int p = 0; p < DEDUP_PROBES; ++p) {
+            uint4 e = make_uint4(~0u, ~0u, ~0u, ~0u);
+            if (pending) e = dd_load4(bucket);
+            // the bucket's slot with this fingerprint, its first free slot
+            uint32_t v = 0;
+            if ((e.w ^ fp) < 0x10000u) v = e.w;
+            if ((e.z ^ fp) < 0x10000u) v = e.z;
+            if ((e.y ^ fp) < 0x10000u) v = e.y;
+            if ((e.x ^ fp) < 0x10000u) v = e.x;
+            const int free = e.x == 0u ? 0 : (e.y == 0u ? 1 : (e.z == 0u ? 2 : (e.w == 0u ? 3 : 4)));
+            const bool claim = pending && v == 0u && free < 4;
+            // numbers for the rows that found a free slot, one atomic a warp
+            const uint32_t want = __ballot_sync(FULL, claim && mine == -1);
+            if (want) {
+                uint32_t r0 = 0;
+                if (lane == __ffs(want) - 1) r0 = atomicAdd(dd_smem() + m.cnt, (uint32_t)__popc(want));
+                r0 = __shfl_sync(FULL, r0, __ffs(want) - 1);
+                if ((want >> lane) & 1u) {
+                    mine = (int)r0 + __popc(want & ((1u << lane) - 1u));
+                    if (mine >= m.nrep) {  // no room
+                        mine = -2;
+                        pending = false;
+                        alone = true;
+                    } else {
+                        // the row before the slot that publishes it
+                        if (mine < m.cap) {
+                            *dd_smem4(m.ys + 4 * mine) = y;
+#pragma unroll
+                            for (int u = 0; u < XW; ++u) dd_smem()[m.xs + mine * XW + u] = x[u];
+                        }
+                        dd_smem()[m.idx + mine] = (uint32_t)i;
+                        dd_smem()[m.dup + mine] = 0u;
+                    }
+                }
+                __threadfence_block();
+            }
+            if (claim && mine >= 0) {
+                // (a slot that another row took first: look at the bucket again)
+                if (atomicCAS(dd_smem() + bucket + free, 0u, fp | (uint32_t)(mine + 1)) == 0u) pending = false;
+            } else if (pending && v != 0u) {
+                const int r = (int)(v & 0xFFFFu) - 1;
+                pending = false;
+                if (dd_same<XW>(m, r, x, y, xc, yc, lm)) same = r;
+                else alone = true;  // another row with this fingerprint
+            } else if (pending) {  // a full bucket: the next one
+                bucket += 4;
+                if (bucket == m.idx) bucket = m.tab;
+            }
+            if (!__any_sync(FULL, pending)) break;
+        }
+        if (same >= 0) {
+            if ((uint32_t)i < *reinterpret_cast<const volatile uint32_t*>(dd_smem() + m.idx + same)) atomicMin(dd_smem() + m.idx + same, (uint32_t)i);
+            atomicAdd(dd_smem() + m.dup + same, 1u);
+            if (mine >= 0) dd_smem()[m.idx + (mine)] = ~0u;  // a number given out in vain
+        } else if (pending || alone) {
+            if (mine >= 0) dd_smem()[m.idx + (mine)] = ~0u;
+            atomicOr(dd_smem() + m.ovf + (i >> 5), 1u << (i & 31));
+            dd_smem()[m.cnt + (1)] = 1u;
+        }
+    }
+    dd_sync<G>();
+    const int n = (int)(dd_smem()[m.cnt + (0)] < (uint32_t)m.nrep ? dd_smem()[m.cnt + (0)] : (uint32_t)m.nrep);
+    const bool over = dd_smem()[m.cnt + (1)] != 0u;
+    for (int k = t; k < n; k += NT) {
+        const uint32_t i = dd_smem()[m.idx + (k)];
+        if (i != ~0u) atomicOr(dd_smem() + m.bm + (i >> 5), 1u << (i & 31));
+    }
+    dd_sync<G>();
+    // first rows before each bitmap word (at most one word a thread)
+    uint32_t w = 0;
+    if (t < m.words) {
+        w = dd_smem()[m.bm + (t)] | dd_smem()[m.ovf + (t)];
+        dd_smem()[m.bm + (t)] = w;
+    }
+    int inc = __popc(w);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(FULL, inc, o);
+        if (lane >= o) inc += u;
+    }
+    int before = 0, total = __shfl_sync(FULL, inc, 31);
+    if (G > 1) {
+        if (lane == 31) wcnt[gw] = inc;
+        dd_sync<G>();
+        total = 0;
+#pragma unroll
+        for (int ww = 0; ww < G; ++ww) {
+            const int c = wcnt[ww];
+            if (ww < gw) before += c;
+            total += c;
+        }
+    }
+    if (t < m.words) dd_smem()[m.pre + (t)] = (uint32_t)(before + inc - __popc(w));
+    dd_sync<G>();
+    for (int k = t; k < n; k += NT) {
+        const uint32_t i = dd_smem()[m.idx + (k)];
+        if (i == ~0u) continue;
+        const int pos = (int)dd_smem()[m.pre + (i >> 5)] + __popc(dd_smem()[m.bm + (i >> 5)] & ((1u << (i & 31)) - 1u));
+        rep[pos] = (int)i + off;
+        dups[pos] = (int)dd_smem()[m.dup + (k)];
+    }
+    if (over) {
+        for (int i = t; i < T; i += NT) {
+            if (!((dd_smem()[m.ovf + (i >> 5)] >> (i & 31)) & 1u)) continue;
+            const int pos = (int)dd_smem()[m.pre + (i >> 5)] + __popc(dd_smem()[m.bm + (i >> 5)] & ((1u << (i & 31)) - 1u));
+            rep[pos] = i + off;
+            dups[pos] = 0;
+        }
+    }
+    dd_sync<G>();
+    return total;
+}
+
+// As dedup_ctx; a range longer than DD_SEG_ROWS is taken in pieces, whose
+// repeats of earlier pieces stay, as with shards.
+template <int G, int XW>
+__device__ bool dedup_wide_ctx(const StoreDev& s, const DedupArgs& a, int c, int region, int* wcnt)
+{
+    int shard = 0, nsh = 1;
+    if constexpr (G == DD_WARPS) {
+        const uint32_t qi = dd_cta_item;
+        shard = (int)((qi >> 24) & 7u);
+        nsh = (int)(qi >> 28) + 1;
+    }
+    constexpr int NT = 32 * G;
+    constexpr int SEG = (G == 1) ? DD_WARP_MAX_ROWS : (G == 4 ? DD_QUAD_MAX_ROWS : DD_SEG_ROWS);
+    constexpr int MOST = (G == 1) ? DD_WARP_MAX_ROWS : (G == 4 ? DD_QUAD_REPS : DD_CTA_REPS);
+    static_assert(SEG <= 32 * NT, "a bitmap word a thread");
+    const int t = (G == 1) ? (int)(threadIdx.x & 31) : (int)(threadIdx.x % NT);
+    const int Tc = (int)(a.row_off[c + 1] - a.row_off[c]);
+    const int lo = (int)(((long long)Tc * shard) / nsh);
+    const int64_t r0 = a.row_off[c] + lo;  // this shard's rows, and its part of rep_list / rep_dup
+    const int T = (int)(((long long)Tc * (shard + 1)) / nsh) - lo;
+    const uint32_t* xc = a.x + a.x_off[c] + (int64_t)lo * XW;
+    const uint32_t lm = last_mask(s.desc[c].n);
+    const int al = ((uintptr_t)xc & 15) == 0 ? 2 : (((uintptr_t)xc & 7) == 0 ? 1 : 0);
+    int nrep = 0;
+    for (int s0 = 0; s0 < T; s0 += SEG) {
+        const int n = T - s0 < SEG ? T - s0 : SEG;
+        const DdSmem m = dd_layout<XW>(region, G * DD_WARP_REGION, n, MOST);
+        // (a piece starts at a multiple of SEG rows, so its rows keep the alignment)
+        nrep += dedup_rows<G, XW>(xc + (int64_t)s0 * XW, a.y + r0 + s0, n, s0, lm, al, m, a.rep_list + r0 + nrep,
+                                  a.rep_dup + r0 + nrep, wcnt);
+    }
+    if (t == 0) {
+        // the call's work, for the elimination plan's thresholds
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.counters + CNT_WORK),
+                  (unsigned long long)nrep * (unsigned long long)s.desc[c].d);
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.counters + CNT_REPS), (unsigned long long)nrep);
+    }
+    return dd_finish<G>(a, c, nrep, t);
 }
 
 // Pass 1 kernel: CTA-owned contexts first, then quads, then warps.
@@ -545,12 +883,14 @@ __global__ void __launch_bounds__(DD_THREADS, DD_CTAS_PER_SM) dedup_kernel(Store
             if (threadIdx.x == 0 && ((qi >> 24) & 7u) == 0) time_mark(a.timing, c, 0);
             bool done = true;
 #define F2_DD_CTA(W) done = dedup_ctx<DD_WARPS, W>(s, a, c, smem, E, wcnt)
+#define F2_DDW_CTA(W) done = dedup_wide_ctx<DD_WARPS, W>(s, a, c, 0, wcnt)
             if constexpr (WX) {
-                F2_XWIDE_SWITCH(s.desc[c].xw, F2_DD_CTA)
+                F2_XWIDE_SWITCH(s.desc[c].xw, F2_DDW_CTA)
             } else {
                 F2_NARROW_SWITCH(s.desc[c].xw, F2_DD_CTA)
             }
 #undef F2_DD_CTA
+#undef F2_DDW_CTA
             if (threadIdx.x == 0 && done) time_mark(a.timing, c, 1);
         }
     }
@@ -571,12 +911,14 @@ __global__ void __launch_bounds__(DD_THREADS, DD_CTAS_PER_SM) dedup_kernel(Store
             if (E > DD_QUAD_E) E = DD_QUAD_E;
             if ((warp & 3) == 0 && lane == 0) time_mark(a.timing, c, 0);
 #define F2_DD_QUAD(W) dedup_ctx<4, W>(s, a, c, region, E, wcnt + q * 4 * DD_K)
+#define F2_DDW_QUAD(W) dedup_wide_ctx<4, W>(s, a, c, q * 4 * DD_WARP_REGION, wcnt + q * 4 * DD_K)
             if constexpr (WX) {
-                F2_XWIDE_SWITCH(s.desc[c].xw, F2_DD_QUAD)
+                F2_XWIDE_SWITCH(s.desc[c].xw, F2_DDW_QUAD)
             } else {
                 F2_NARROW_SWITCH(s.desc[c].xw, F2_DD_QUAD)
             }
 #undef F2_DD_QUAD
+#undef F2_DDW_QUAD
             if ((warp & 3) == 0 && lane == 0) time_mark(a.timing, c, 1);
         }
     }
@@ -594,12 +936,14 @@ __global__ void __launch_bounds__(DD_THREADS, DD_CTAS_PER_SM) dedup_kernel(Store
             const int E = pow2_at_least(2 * T);
             if (lane == 0) time_mark(a.timing, c, 0);
 #define F2_DD_WARP(W) dedup_ctx<1, W>(s, a, c, region, E, nullptr)
+#define F2_DDW_WARP(W) dedup_wide_ctx<1, W>(s, a, c, warp * DD_WARP_REGION, nullptr)
             if constexpr (WX) {
-                F2_XWIDE_SWITCH(s.desc[c].xw, F2_DD_WARP)
+                F2_XWIDE_SWITCH(s.desc[c].xw, F2_DDW_WARP)
             } else {
                 F2_NARROW_SWITCH(s.desc[c].xw, F2_DD_WARP)
             }
 #undef F2_DD_WARP
+#undef F2_DDW_WARP
             if (lane == 0) time_mark(a.timing, c, 1);
         }
     }
