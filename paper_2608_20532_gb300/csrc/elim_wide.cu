@@ -13,12 +13,14 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, WDT <= WIDE_M_WD ? 2 : 1) eli
 
 // ---------------------------------------------------------------------------
 // The first OPEN_THREADS rows of an empty basis of up to WIDE_WD words, a row
-// a thread, in registers.  The rows go in stream order: the row's warp puts it
-// into shared memory and finds its highest set bit, and after one barrier
-// every thread whose row has that bit XORs it from there (broadcast loads,
-// only the words up to the pivot's).  The rows stay reduced among themselves,
-// so what remains is the reduced basis.  A pivot costs about 40 instructions a
-// warp and a barrier; streaming 256 rows at a time against a basis in shared
+// a thread, in registers.  The rows go in stream order, OPEN_GROUP at a time:
+// their warp puts one after another into shared memory, finds its highest set
+// bit and applies it to its own rows at once; after one barrier every thread
+// of the other warps whose row has such a bit XORs the row from there
+// (broadcast loads, only the words up to the pivot's).  The rows stay reduced
+// among themselves, so what remains is the reduced basis.  (One row a barrier
+// took 1,475 cycles a pivot, four take 1,310, of which the XORs alone 610: 38
+// integer instructions a warp at half rate.)  Streaming 256 rows at a time against a basis in shared
 // memory, the 1,025 pivots of a dense 1,024-bit context took 3,000 cycles
 // each, most of it in reading older rows a lane each.  Two batches of 65,536
 // rows for 64 such contexts went from 3,012 to 2,256 us.  Dense rows are a few pivots short of full
@@ -26,14 +28,15 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, WDT <= WIDE_M_WD ? 2 : 1) eli
 // by all threads (a XOR reduction of the rows their bits select).
 // ---------------------------------------------------------------------------
 constexpr int OPEN_THREADS = 1024;
+constexpr int OPEN_GROUP = 4;
 constexpr int OPEN_EXTRA = 32;
 constexpr int OPEN_Z = 9;  // uint4 index of the word in a shared row; the features before it
 
 struct OpenSmem {
-    uint4 row[2][OPEN_Z + 1];
+    uint4 row[2][OPEN_GROUP][OPEN_Z + 1];
     uint32_t q[WIDE_WD + 3];  // a further row's own bits
     uint32_t mask[WIDE_WD + 3];
-    int head[2];
+    int head[2][OPEN_GROUP];
     int holder;
     unsigned long long cnt;
     long long first;
@@ -113,31 +116,41 @@ __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, 
             sm.cnt = 0ull;
             sm.first = LLONG_MAX;
         }
-        for (int i = 0; i < n && rank < cd.d; ++i) {
-            if (warp == (i >> 5)) {
-                uint4* const row = sm.row[i & 1];
-                if (t == i) {
+        for (int i0 = 0, buf = 0; i0 < n && rank < cd.d; i0 += OPEN_GROUP, buf ^= 1) {
+            const bool owner = warp == (i0 >> 5);
+            if (owner) {
+#pragma unroll 1
+                for (int j = 0; j < OPEN_GROUP; ++j) {
+                    uint4* const row = sm.row[buf][j];
+                    const bool own = t == i0 + j;
+                    if (own) {
 #pragma unroll
-                    for (int v4 = 0; v4 < OPEN_Z; ++v4) {
-                        uint32_t e[4];
+                        for (int v4 = 0; v4 < OPEN_Z; ++v4) {
+                            uint32_t e[4];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) e[j] = 4 * v4 + j < WIDE_WD ? x[4 * v4 + j < WIDE_WD ? 4 * v4 + j : 0] : 0u;
-                        row[v4] = make_uint4(e[0], e[1], e[2], e[3]);
+                            for (int u = 0; u < 4; ++u)
+                                e[u] = 4 * v4 + u < WIDE_WD ? x[4 * v4 + u < WIDE_WD ? 4 * v4 + u : 0] : 0u;
+                            row[v4] = make_uint4(e[0], e[1], e[2], e[3]);
+                        }
+                        row[OPEN_Z] = y;
                     }
-                    row[OPEN_Z] = y;
-                }
-                __syncwarp();
-                const int k = open_top(row, lane);
-                if (t == i) {
-                    sm.head[i & 1] = k;
-                    pk = k;
+                    __syncwarp();
+                    const int k = open_top(row, lane);
+                    if (own) {
+                        sm.head[buf][j] = k;
+                        pk = k;
+                    }
+                    if (k >= 0) open_step(k, x, y, row, own);
                 }
             }
             __syncthreads();
-            const int k = sm.head[i & 1];
-            if (k < 0) continue;
-            ++rank;
-            open_step(k, x, y, sm.row[i & 1], t == i);
+#pragma unroll 1
+            for (int j = 0; j < OPEN_GROUP; ++j) {
+                const int k = sm.head[buf][j];
+                if (k < 0) continue;
+                ++rank;
+                if (!owner) open_step(k, x, y, sm.row[buf][j], false);
+            }
         }
         // rows without a pivot lie in the span of the rows before them
         if (t < n && pk < 0 && nonzero4(y)) {
@@ -147,7 +160,8 @@ __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, 
         int base = n;
         for (int extra = 0; rank < cd.d && base < rs.R && extra < OPEN_EXTRA; ++extra, ++base) {
             __syncthreads();
-            uint32_t* const acc = reinterpret_cast<uint32_t*>(sm.row[0]);
+            uint4* const arow = sm.row[0][0];
+            uint32_t* const acc = reinterpret_cast<uint32_t*>(arow);
             const int i = rs.reps ? __ldg(rs.reps + base) : base;
             if (warp == 0) {
                 const uint32_t* xr = rs.xc + (int64_t)i * rs.xw;
@@ -164,7 +178,7 @@ __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, 
                     sm.q[w] = q;
                 }
                 if (lane == 0) {
-                    sm.row[0][OPEN_Z] = __ldg(rs.yc + i);
+                    arow[OPEN_Z] = __ldg(rs.yc + i);
                     sm.holder = OPEN_THREADS;
                 }
             }
@@ -185,8 +199,8 @@ __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, 
             }
             if (pk < 0) atomicMin(&sm.holder, t);
             __syncthreads();
-            const int k = open_top(sm.row[0], lane);
-            const uint4 z = sm.row[0][OPEN_Z];
+            const int k = open_top(arow, lane);
+            const uint4 z = arow[OPEN_Z];
             if (k < 0) {
                 if (t == 0 && nonzero4(z)) {
                     sm.cnt += 1u + (rs.dups ? (uint32_t)__ldg(rs.dups + base) : 0u);
@@ -195,7 +209,7 @@ __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, 
                 continue;
             }
             ++rank;
-            open_step(k, x, y, sm.row[0], false);
+            open_step(k, x, y, arow, false);
             if (t == sm.holder) {
 #pragma unroll
                 for (int v = 0; v < WIDE_WD; ++v) x[v] = acc[v];
