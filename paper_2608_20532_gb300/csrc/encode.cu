@@ -127,8 +127,10 @@ __device__ __forceinline__ bool encode_one(const StoreDev& s, const CtxDesc& cd,
 //                      CTA to finish);
 //   enc_scatter_kernel writes (context, query) to its grouped position.
 // ---------------------------------------------------------------------------
-constexpr int ENC_TILE = 2048;
+constexpr int ENC_TILE = 2048;       // most queries a CTA counts
 constexpr int ENC_TILE_THREADS = 256;
+constexpr int ENC_TILE_MIN = 512;    // and fewest, where that fills the SMs (512 .. 2048, a power of two)
+constexpr int ENC_HIST = 8192;       // stores of fewer contexts count into a plain histogram
 constexpr int ENC_TILE_PER = ENC_TILE / ENC_TILE_THREADS;
 constexpr int ENC_HT_BITS = 12;
 constexpr int ENC_HT = 1 << ENC_HT_BITS;
@@ -188,82 +190,113 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T* ws, T& total)
     return r;
 }
 
+// A CTA counts `tile` queries of one chunk per context.  With fewer than
+// ENC_HIST contexts the counters are indexed by the context itself: one shared
+// atomic a query.  Else they form a hash table, claimed by compare-and-swap,
+// and a warp's queries of one context are counted together.  (The shared
+// atomics bound this kernel: with the hash table a 1M-query pass over 4,096
+// contexts spent 38 us here.  With this and the segments of whole waves below
+// the pass and its epilogue went from 144 to 115 us.)
+template <bool HIST>
 __global__ void __launch_bounds__(ENC_TILE_THREADS) enc_count_kernel(int32_t Q, const int32_t* __restrict__ ctx_id,
-                                                                     int32_t num_ctx, int shift, int32_t B,
+                                                                     int32_t num_ctx, int shift, int32_t B, int tile,
                                                                      int32_t* __restrict__ cnt,
                                                                      int32_t* __restrict__ off)
 {
-    __shared__ int32_t key[ENC_HT];
-    __shared__ int32_t hcnt[ENC_HT];
+    __shared__ int32_t slots[HIST ? ENC_HIST : 2 * ENC_HT];
+    int32_t* const key = slots;                         // (hash table)
+    int32_t* const hcnt = HIST ? slots : slots + ENC_HT;
     const int t = threadIdx.x, lane = t & 31;
-    const int64_t base = (int64_t)blockIdx.x * ENC_TILE;
+    const int per = tile / ENC_TILE_THREADS;
+    const int64_t base = (int64_t)blockIdx.x * tile;
     int32_t* const bins = cnt + (int64_t)(base >> shift) * B;  // the tile's chunk
     int32_t bk[ENC_TILE_PER];
 #pragma unroll
     for (int j = 0; j < ENC_TILE_PER; ++j) {  // all loads first
         const int64_t i = base + (int64_t)j * ENC_TILE_THREADS + t;
-        bk[j] = (i < Q) ? bucket_of(__ldg(ctx_id + i), num_ctx) : EMPTY_KEY;
+        bk[j] = (j < per && i < Q) ? bucket_of(__ldg(ctx_id + i), num_ctx) : EMPTY_KEY;
     }
-    for (int h = t; h < ENC_HT; h += ENC_TILE_THREADS) {
-        key[h] = EMPTY_KEY;
-        hcnt[h] = 0;
-    }
-    __syncthreads();
-    const uint32_t below = (1u << lane) - 1u;
-    uint32_t peers[ENC_TILE_PER];
     uint32_t slot[ENC_TILE_PER];
-    int32_t prev[ENC_TILE_PER];
-    bool lead[ENC_TILE_PER];
+    int rank[ENC_TILE_PER];
+    if constexpr (HIST) {
+        for (int h = t; h < B; h += ENC_TILE_THREADS) hcnt[h] = 0;
+        __syncthreads();
 #pragma unroll
-    for (int j = 0; j < ENC_TILE_PER; ++j) {
-        peers[j] = __match_any_sync(FULL, bk[j]);
-        lead[j] = lane == __ffs(peers[j]) - 1 && bk[j] != EMPTY_KEY;
-        slot[j] = ((uint32_t)bk[j] * 2654435761u) >> (32 - ENC_HT_BITS);
-    }
-    // The first probe of every group is issued before any is resolved: at
-    // most half of the table is used, so most groups are placed by it.
+        for (int j = 0; j < ENC_TILE_PER; ++j) {
+            slot[j] = bk[j] < 0 ? 0u : (uint32_t)bk[j];
+            rank[j] = bk[j] < 0 ? 0 : atomicAdd(&hcnt[slot[j]], 1);
+        }
+    } else {
+        for (int h = t; h < ENC_HT; h += ENC_TILE_THREADS) {
+            key[h] = EMPTY_KEY;
+            hcnt[h] = 0;
+        }
+        __syncthreads();
+        const uint32_t below = (1u << lane) - 1u;
+        uint32_t peers[ENC_TILE_PER];
+        int32_t prev[ENC_TILE_PER];
+        bool lead[ENC_TILE_PER];
 #pragma unroll
-    for (int j = 0; j < ENC_TILE_PER; ++j) prev[j] = lead[j] ? atomicCAS(&key[slot[j]], EMPTY_KEY, bk[j]) : EMPTY_KEY;
+        for (int j = 0; j < ENC_TILE_PER; ++j) {
+            peers[j] = __match_any_sync(FULL, bk[j]);
+            lead[j] = lane == __ffs(peers[j]) - 1 && bk[j] != EMPTY_KEY;
+            slot[j] = ((uint32_t)bk[j] * 2654435761u) >> (32 - ENC_HT_BITS);
+        }
+        // The first probe of every group is issued before any is resolved: at
+        // most half of the table is used, so most groups are placed by it.
 #pragma unroll
-    for (int j = 0; j < ENC_TILE_PER; ++j) {
-        if (lead[j]) {
-            // at most ENC_TILE distinct keys in ENC_HT slots: a free or
-            // matching slot is always found within ENC_HT probes
-            for (int probe = 1; probe < ENC_HT && prev[j] != EMPTY_KEY && prev[j] != bk[j]; ++probe) {
-                slot[j] = (slot[j] + 1) & (ENC_HT - 1);
-                prev[j] = atomicCAS(&key[slot[j]], EMPTY_KEY, bk[j]);
+        for (int j = 0; j < ENC_TILE_PER; ++j)
+            prev[j] = lead[j] ? atomicCAS(&key[slot[j]], EMPTY_KEY, bk[j]) : EMPTY_KEY;
+#pragma unroll
+        for (int j = 0; j < ENC_TILE_PER; ++j) {
+            if (lead[j]) {
+                // at most ENC_TILE distinct keys in ENC_HT slots: a free or
+                // matching slot is always found within ENC_HT probes
+                for (int probe = 1; probe < ENC_HT && prev[j] != EMPTY_KEY && prev[j] != bk[j]; ++probe) {
+                    slot[j] = (slot[j] + 1) & (ENC_HT - 1);
+                    prev[j] = atomicCAS(&key[slot[j]], EMPTY_KEY, bk[j]);
+                }
             }
         }
-    }
-    int r0[ENC_TILE_PER];
+        int r0[ENC_TILE_PER];
 #pragma unroll
-    for (int j = 0; j < ENC_TILE_PER; ++j) r0[j] = lead[j] ? atomicAdd(&hcnt[slot[j]], __popc(peers[j])) : 0;
-    int rank[ENC_TILE_PER];
+        for (int j = 0; j < ENC_TILE_PER; ++j) r0[j] = lead[j] ? atomicAdd(&hcnt[slot[j]], __popc(peers[j])) : 0;
 #pragma unroll
-    for (int j = 0; j < ENC_TILE_PER; ++j) {
-        const int leader = __ffs(peers[j]) - 1;
-        slot[j] = __shfl_sync(FULL, slot[j], leader);
-        rank[j] = __shfl_sync(FULL, r0[j], leader) + __popc(peers[j] & below);
+        for (int j = 0; j < ENC_TILE_PER; ++j) {
+            const int leader = __ffs(peers[j]) - 1;
+            slot[j] = __shfl_sync(FULL, slot[j], leader);
+            rank[j] = __shfl_sync(FULL, r0[j], leader) + __popc(peers[j] & below);
+        }
     }
     __syncthreads();
     // one global atomic per distinct context of the tile; all of a thread's
-    // atomics are issued before any result is used
-    constexpr int HPER = ENC_HT / ENC_TILE_THREADS;
-    int got[HPER];
+    // atomics of a step are issued before any result is used (each counter is
+    // its own thread's from here to the barrier)
+    constexpr int HPER = 16;
+    const int n_slots = HIST ? B : ENC_HT;
+    for (int h0 = 0; h0 < n_slots; h0 += HPER * ENC_TILE_THREADS) {
+        int got[HPER];
 #pragma unroll
-    for (int u = 0; u < HPER; ++u) {
-        const int h = u * ENC_TILE_THREADS + t;
-        const int32_t k = key[h];
-        got[u] = (k != EMPTY_KEY) ? atomicAdd(bins + k, hcnt[h]) : 0;
+        for (int u = 0; u < HPER; ++u) {
+            const int h = h0 + u * ENC_TILE_THREADS + t;
+            got[u] = 0;
+            if (h < n_slots) {
+                const int32_t v = hcnt[h];
+                const int32_t k = HIST ? h : key[h];
+                if (v) got[u] = atomicAdd(bins + k, v);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < HPER; ++u) {
+            const int h = h0 + u * ENC_TILE_THREADS + t;
+            if (h < n_slots) hcnt[h] = got[u];
+        }
     }
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < HPER; ++u) hcnt[u * ENC_TILE_THREADS + t] = got[u];
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < ENC_TILE_PER; ++j) {
         const int64_t i = base + (int64_t)j * ENC_TILE_THREADS + t;
-        if (i < Q) off[i] = hcnt[slot[j]] + rank[j];
+        if (j < per && i < Q) off[i] = hcnt[slot[j]] + rank[j];
     }
 }
 
@@ -582,7 +615,7 @@ __global__ void __launch_bounds__(SCAT_THREADS) enc_scatter_kernel(int32_t Q, co
 // ---------------------------------------------------------------------------
 // Pass 2: encode the grouped queries.
 //
-// enc_runs_kernel: a CTA takes RUN_SEG consecutive positions of the grouped
+// enc_runs_kernel: a CTA takes up to RUN_SEG consecutive positions of the grouped
 // order, i.e. a few runs of queries of one context each.  A run of at least
 // RUN_TABLE_MIN queries of a table context is encoded with its table: the
 // CTA copies the tables of its runs from the pool into shared memory with
@@ -595,7 +628,10 @@ __global__ void __launch_bounds__(SCAT_THREADS) enc_scatter_kernel(int32_t Q, co
 // query against them in a warp-uniform walk over the pivots.
 // ---------------------------------------------------------------------------
 constexpr int RUN_THREADS = 512;  // two CTAs per SM: 32 warps
-constexpr int RUN_SEG = 2048;
+constexpr int RUN_SEG = 2048;     // most positions of a segment; a pass takes segments of a length that
+                                  // fills whole waves of CTAs (RUN_SEG_MIN at least)
+constexpr int RUN_SEG_MIN = 512;
+constexpr int RUN_WAVES_MAX = 8;
 constexpr int RUN_PER = RUN_SEG / RUN_THREADS;
 constexpr int MAX_TRUNS = 128;                // table runs of a segment (the rest become items)
 constexpr int RUN_TABLE_MIN = 4;              // shorter runs of a table context become items
@@ -753,7 +789,7 @@ __device__ __forceinline__ void query_group(const StoreDev& s, const RunSmem& sm
     }
 }
 
-__global__ void __launch_bounds__(RUN_THREADS, 2) enc_runs_kernel(StoreDev s, int32_t n_total,
+__global__ void __launch_bounds__(RUN_THREADS, 2) enc_runs_kernel(StoreDev s, int32_t n_total, int seg,
                                                                   const unsigned long long* __restrict__ sorted,
                                                                   const uint32_t* __restrict__ x, int stride,
                                                                   uint4* __restrict__ y,
@@ -769,8 +805,8 @@ __global__ void __launch_bounds__(RUN_THREADS, 2) enc_runs_kernel(StoreDev s, in
     int32_t* const run_ctx = reinterpret_cast<int32_t*>(sm.xs);  // until the feature words are staged
     const int t = threadIdx.x;
     const bool xvec = ((uintptr_t)x % 16) == 0 && (stride % 4) == 0;
-    const int64_t seg0 = (int64_t)blockIdx.x * RUN_SEG;
-    const int n = (int)((n_total - seg0) < RUN_SEG ? (n_total - seg0) : RUN_SEG);
+    const int64_t seg0 = (int64_t)blockIdx.x * seg;
+    const int n = (int)((n_total - seg0) < seg ? (n_total - seg0) : seg);
     if (t == 0) {
         mbar_init(&sm.bar[0], 1);
         mbar_init(&sm.bar[1], 1);
@@ -1320,9 +1356,15 @@ extern "C" int f2_encode_batched(const f2_store* st, int64_t Q, const int32_t* c
             e = f2_fill(zl, cs);
             if (e != cudaSuccess) return f2_cuda_status(e);
         }
-        enc_count_kernel<<<(n + ENC_TILE - 1) / ENC_TILE, ENC_TILE_THREADS, 0, cs>>>(n, ctx_id + q0, st->num_ctx,
-                                                                                   shift, (int32_t)B, cnt,
-                                                                                   st->enc_off);
+        // tiles small enough for two CTAs an SM (they divide a chunk: 2^11 queries or more)
+        int tile = ENC_TILE;
+        while (tile > ENC_TILE_MIN && n < (int64_t)tile * 2 * st->num_sms) tile >>= 1;
+        if (B <= ENC_HIST)
+            enc_count_kernel<true><<<(n + tile - 1) / tile, ENC_TILE_THREADS, 0, cs>>>(
+                n, ctx_id + q0, st->num_ctx, shift, (int32_t)B, tile, cnt, st->enc_off);
+        else
+            enc_count_kernel<false><<<(n + tile - 1) / tile, ENC_TILE_THREADS, 0, cs>>>(
+                n, ctx_id + q0, st->num_ctx, shift, (int32_t)B, tile, cnt, st->enc_off);
         enc_table_kernel<<<tbl_blocks, TBL_THREADS, 0, cs>>>(
             sd, nch, (int32_t)B, cnt, sta, st->enc_hot, st->enc_tab_off, tables ? (long long)st->enc_pool_words : 0,
             pool_used, hot_list, n_hot, tables ? st->enc_table_min : INT_MAX, (long long)st->enc_chunk_min,
@@ -1346,8 +1388,18 @@ extern "C" int f2_encode_batched(const f2_store* st, int64_t Q, const int32_t* c
             e = cudaStreamWaitEvent(cs, st->ev_join, 0);
             if (e != cudaSuccess) return f2_cuda_status(e);
         }
-        enc_runs_kernel<<<(n + RUN_SEG - 1) / RUN_SEG, RUN_THREADS, sizeof(RunSmem), cs>>>(
-            sd, n, st->enc_sorted, xq, x_stride_words, yq, in_span + q0, st->enc_hot, st->enc_tab_off,
+        // Segments that fill whole waves of two CTAs an SM: with RUN_SEG queries
+        // each a pass of 1M left 40% of its second wave idle, one of 100,000
+        // two SMs in three.  A pass of many waves keeps the longest (shorter
+        // ones copy more tables: 818 against 810 us on 10M queries).
+        const int64_t slots = 2 * (int64_t)st->num_sms;
+        const int64_t waves = (n + slots * RUN_SEG - 1) / (slots * RUN_SEG);
+        int64_t seg = waves >= RUN_WAVES_MAX ? RUN_SEG : (n + slots * waves - 1) / (slots * waves);
+        seg = (seg + 31) & ~int64_t(31);
+        if (seg < RUN_SEG_MIN) seg = RUN_SEG_MIN;
+        if (seg > RUN_SEG) seg = RUN_SEG;
+        enc_runs_kernel<<<(int)((n + seg - 1) / seg), RUN_THREADS, sizeof(RunSmem), cs>>>(
+            sd, n, (int)seg, st->enc_sorted, xq, x_stride_words, yq, in_span + q0, st->enc_hot, st->enc_tab_off,
             st->enc_pool, items, n_items);
         enc_short_kernel<<<st->num_sms * short_per_sm, SHORT_THREADS, sizeof(ShortSmem), cs>>>(
             sd, st->enc_sorted, xq, x_stride_words, yq, in_span + q0, items, n_items);
