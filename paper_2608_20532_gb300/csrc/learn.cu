@@ -177,39 +177,7 @@ static_assert(DD_WARPS * DD_WARP_REGION * 4 <= DD_SMEM, "warp regions exceed the
     }
 
 
-// 32-bit hash of an observation (feature words and word): FNV-1a over the
-// words, then a murmur-style finalizer.
-template <int WD>
-__device__ __forceinline__ uint32_t hash_row(const uint32_t (&xin)[WD], const uint4& y)
-{
-    uint32_t h = 0x811C9DC5u;
-#pragma unroll
-    for (int v = 0; v < WD; ++v) h = (h ^ xin[v]) * 0x01000193u;
-    h = (h ^ y.x) * 0x01000193u;
-    h = (h ^ y.y) * 0x01000193u;
-    h = (h ^ y.z) * 0x01000193u;
-    h = (h ^ y.w) * 0x01000193u;
-    h ^= h >> 16;
-    h *= 0x85EBCA6Bu;
-    h ^= h >> 13;
-    h *= 0xC2B2AE35u;
-    h ^= h >> 16;
-    return h;
-}
-
 // ------------------------------------------------------------------ pass 1
-
-__device__ __forceinline__ uint32_t fnv_step(uint32_t h, uint32_t w) { return (h ^ w) * 0x01000193u; }
-
-__device__ __forceinline__ uint32_t fmix32(uint32_t h)
-{
-    h ^= h >> 16;
-    h *= 0x85EBCA6Bu;
-    h ^= h >> 13;
-    h *= 0xC2B2AE35u;
-    h ^= h >> 16;
-    return h;
-}
 
 __device__ __forceinline__ uint32_t last_mask(int n) { return (n & 31) ? ((1u << (n & 31)) - 1u) : 0xffffffffu; }
 
@@ -251,6 +219,52 @@ __device__ __noinline__ int dd_find_insert(uint2* tab, int E, uint32_t h, int64_
         }
     }
     return -1;
+}
+
+// Feature words of a row: the widest loads that every row of the context
+// allows (`al`: log2 of the words its rows are aligned to).
+template <int XW>
+__device__ __forceinline__ void load_words(const uint32_t* __restrict__ p, int al, uint32_t (&x)[XW])
+{
+    if (XW % 4 == 0 && al >= 2) {
+#pragma unroll
+        for (int v = 0; v + 3 < XW; v += 4) {
+            const uint4 t = __ldg(reinterpret_cast<const uint4*>(p + v));
+            x[v] = t.x;
+            x[v + 1] = t.y;
+            x[v + 2] = t.z;
+            x[v + 3] = t.w;
+        }
+    } else if (XW % 2 == 0 && al >= 1) {
+#pragma unroll
+        for (int v = 0; v + 1 < XW; v += 2) {
+            const uint2 t = __ldg(reinterpret_cast<const uint2*>(p + v));
+            x[v] = t.x;
+            x[v + 1] = t.y;
+        }
+    } else {
+#pragma unroll
+        for (int v = 0; v < XW; ++v) x[v] = __ldg(p + v);
+    }
+}
+
+// Hash of an observation: a sum of the words times odd constants, mixed.  It
+// only proposes candidates; every match is confirmed by comparing the rows.
+template <int XW>
+__device__ __forceinline__ uint32_t dd_hash(const uint32_t (&x)[XW], const uint4& y)
+{
+    uint32_t h = y.x * 0x9E3779B1u + y.y * 0x85EBCA77u + y.z * 0xC2B2AE3Du + y.w * 0x27D4EB2Fu;
+    uint32_t k = 0x165667B1u;
+#pragma unroll
+    for (int v = 0; v < XW; ++v) {
+        h += x[v] * k;
+        k = k * 0x01000193u + 0x3C6EF372u;  // constants at compile time
+        k |= 1u;
+    }
+    h ^= h >> 16;
+    h *= 0x7FEB352Du;
+    h ^= h >> 15;
+    return h;
 }
 
 // Group synchronisation for pass 1: a warp, a quad of 4 warps (named
@@ -370,6 +384,7 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
     const uint32_t* xc = a.x + a.x_off[c] + (int64_t)lo * XW;
     const uint4* yc = a.y + r0;
     const uint32_t lm = last_mask(n);
+    const int al = ((uintptr_t)xc & 15) == 0 ? 2 : (((uintptr_t)xc & 7) == 0 ? 1 : 0);
     const uint32_t emask = (uint32_t)(E - 1);
     for (int e = t; e < E; e += NT) {
         tab[e] = make_uint2(0u, 0u);
@@ -389,19 +404,14 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
         for (int j = 0; j < K; ++j) {
             const int i = base + j * NT + t;
             const bool ok = i < T;
-            yv[j] = ok ? __ldg(yc + i) : make_uint4(0, 0, 0, 0);
-#pragma unroll
-            for (int v = 0; v < XW; ++v) {
-                const uint32_t w = ok ? __ldg(xc + (int64_t)i * XW + v) : 0u;
-                xv[j][v] = (v == XW - 1) ? (w & lm) : w;
-            }
+            const int ic = ok ? i : T - 1;  // (a row read twice, not counted)
+            yv[j] = __ldg(yc + ic);
+            load_words<XW>(xc + (int64_t)ic * XW, al, xv[j]);
+            xv[j][XW - 1] &= lm;
         }
 #pragma unroll
         for (int j = 0; j < K; ++j) {
-            uint32_t hh = 0x811C9DC5u;
-#pragma unroll
-            for (int v = 0; v < XW; ++v) hh = fnv_step(hh, xv[j][v]);
-            h[j] = fmix32(fnv_step(fnv_step(fnv_step(fnv_step(hh, yv[j].x), yv[j].y), yv[j].z), yv[j].w));
+            h[j] = dd_hash<XW>(xv[j], yv[j]);
         }
         // probe by fingerprint only (shared memory): the first slot holding
         // this fingerprint, or an empty slot that the row then claims
@@ -447,9 +457,13 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
         for (int j = 0; j < K; ++j) {
             need[j] = mine[j] == -2;
             const int64_t o = need[j] ? (int64_t)ent[j].y : 0;
-            yo[j] = need[j] ? __ldg(yc + o) : make_uint4(0, 0, 0, 0);
+            yo[j] = make_uint4(0, 0, 0, 0);
 #pragma unroll
-            for (int v = 0; v < XW; ++v) xo[j][v] = need[j] ? __ldg(xc + o * XW + v) : 0u;
+            for (int v = 0; v < XW; ++v) xo[j][v] = 0u;
+            if (need[j]) {
+                yo[j] = __ldg(yc + o);
+                load_words<XW>(xc + o * XW, al, xo[j]);
+            }
         }
 #pragma unroll
         for (int j = 0; j < K; ++j) {
@@ -486,12 +500,9 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
         for (int j = 0; j < K; ++j) {
             int before = 0, total = __popc(bal[j]);
             if (G > 1) {
-                total = 0;
-                for (int ww = 0; ww < G; ++ww) {
-                    const int v = wcnt[ww * K + j];
-                    if (ww < gw) before += v;
-                    total += v;
-                }
+                const int v = lane < G ? wcnt[lane * K + j] : 0;
+                total = __reduce_add_sync(FULL, v);
+                before = __reduce_add_sync(FULL, lane < gw ? v : 0);
             }
             if ((bal[j] >> lane) & 1u) {
                 const int pos = nrep + before + __popc(bal[j] & ((1u << lane) - 1u));
@@ -500,7 +511,7 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
             }
             nrep += total;
         }
-        if (G > 1) dd_sync<G>();
+        // (the next round's first barrier comes before it writes wcnt again)
     }
     dd_sync<G>();
     for (int k = t; k < nrep; k += NT) {
@@ -593,52 +604,6 @@ __device__ __forceinline__ DdSmem dd_layout(int region, int region_words, int T,
     m.ys = region + used;
     m.xs = region + used + 4 * m.cap;
     return m;
-}
-
-// Feature words of a row: the widest loads that every row of the context
-// allows (`al`: log2 of the words its rows are aligned to).
-template <int XW>
-__device__ __forceinline__ void load_words(const uint32_t* __restrict__ p, int al, uint32_t (&x)[XW])
-{
-    if (XW % 4 == 0 && al >= 2) {
-#pragma unroll
-        for (int v = 0; v + 3 < XW; v += 4) {
-            const uint4 t = __ldg(reinterpret_cast<const uint4*>(p + v));
-            x[v] = t.x;
-            x[v + 1] = t.y;
-            x[v + 2] = t.z;
-            x[v + 3] = t.w;
-        }
-    } else if (XW % 2 == 0 && al >= 1) {
-#pragma unroll
-        for (int v = 0; v + 1 < XW; v += 2) {
-            const uint2 t = __ldg(reinterpret_cast<const uint2*>(p + v));
-            x[v] = t.x;
-            x[v + 1] = t.y;
-        }
-    } else {
-#pragma unroll
-        for (int v = 0; v < XW; ++v) x[v] = __ldg(p + v);
-    }
-}
-
-// Hash of an observation: a sum of the words times odd constants, mixed.  It
-// only proposes candidates; every match is confirmed by comparing the rows.
-template <int XW>
-__device__ __forceinline__ uint32_t dd_hash(const uint32_t (&x)[XW], const uint4& y)
-{
-    uint32_t h = y.x * 0x9E3779B1u + y.y * 0x85EBCA77u + y.z * 0xC2B2AE3Du + y.w * 0x27D4EB2Fu;
-    uint32_t k = 0x165667B1u;
-#pragma unroll
-    for (int v = 0; v < XW; ++v) {
-        h += x[v] * k;
-        k = k * 0x01000193u + 0x3C6EF372u;  // constants at compile time
-        k |= 1u;
-    }
-    h ^= h >> 16;
-    h *= 0x7FEB352Du;
-    h ^= h >> 15;
-    return h;
 }
 
 // Row (x, y) equals the row numbered r, whose smallest index so far is i0.
