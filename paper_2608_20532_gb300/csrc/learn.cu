@@ -39,7 +39,7 @@
 
 #include <mutex>
 
-#include "elim.cuh"
+#include "full.cuh"
 
 using namespace f2;
 
@@ -1423,22 +1423,6 @@ constexpr int FULL_NP_MAX = 8 * ((MAX_D + 31) / 32);      // 264 groups
 constexpr int FULL_ZH_BYTES = FULL_NP_MAX * 16 * 8;        // 33,792: low plane, then the high plane
 constexpr int FULL_TABLE_WORDS = 2 * FULL_ZH_BYTES / 4 + 256;  // both planes + alignment slack
 
-struct FullArgs {
-    const int64_t* row_off;
-    const int64_t* x_off;
-    const uint32_t* x;
-    const uint4* y;
-    const int32_t* queue;
-    const int* counters;
-    int* ctr;                         // [2C]: chunks claimed, chunks done
-    const int* late_count;            // contexts listed by the elimination kernels
-    const int32_t* late_list;
-    const int32_t* late_start;        // their first row left
-    unsigned long long* cnt;          // [C] contradicting rows of the call
-    unsigned long long* first;        // [C] first contradicting row of the call (all ones: none)
-    int table_words;                  // FULL_TABLE_WORDS
-};
-
 __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, FullArgs a)
 {
     extern __shared__ uint4 full_smem[];
@@ -1461,8 +1445,10 @@ __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, F
             while (q < nq) {
                 const int c = ctx_of(q);
                 const int64_t T = a.row_off[c + 1] - a.row_off[c] - start_of(q, c);
-                k = atomicAdd(a.ctr + c, 1);
-                if ((int64_t)k * FULL_CHUNK < T) break;
+                if (!(a.tensor && full_by_tensor(s.desc[c].n, T))) {
+                    k = atomicAdd(a.ctr + c, 1);
+                    if ((int64_t)k * FULL_CHUNK < T) break;
+                }
                 ++q;
             }
             s_q = q;
@@ -1595,26 +1581,7 @@ __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, F
             atomicMin(&s_first, first);
         }
         __syncthreads();
-        if (t == 0) {
-            if (s_cnt) {
-                atomicAdd(a.cnt + c, s_cnt);
-                atomicMin(a.first + c, s_first);
-            }
-            __threadfence();
-            const int nch = (int)((T - i_first + FULL_CHUNK - 1) / FULL_CHUNK);
-            if (atomicAdd(a.ctr + s.num_ctx + c, 1) == nch - 1) {  // the context's last chunk
-                __threadfence();
-                const unsigned long long tot = atomicAdd(a.cnt + c, 0ull);
-                const unsigned long long fi = atomicMin(a.first + c, ~0ull);
-                const long long seen = s.rows_seen[c];
-                if (tot) {
-                    s.n_contra[c] += tot;
-                    s.contra[c] = 1;
-                    if (s.first_contra[c] < 0) s.first_contra[c] = seen + (long long)fi;
-                }
-                s.rows_seen[c] = seen + T;
-            }
-        }
+        if (t == 0) full_commit(s, a, c, i_first, T, s_cnt, s_first);
         __syncthreads();
     }
 }
@@ -1769,6 +1736,11 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
         fa.cnt = full_cnt;
         fa.first = full_first;
         fa.table_words = FULL_TABLE_WORDS;
+        fa.tensor = wv.max_n >= TC_MIN_N && total_rows >= TC_MIN_ROWS;
+        if (fa.tensor) {
+            e = verify_launch_tc(sd, fa, num_sms, cs);
+            if (e != cudaSuccess) return f2_cuda_status(e);
+        }
         const size_t smem = 4 * ((size_t)fa.table_words + (size_t)FULL_STAGE * (size_t)(wv.max_xw | 1));
         e = cudaFuncSetAttribute(verify_full_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return f2_cuda_status(e);
@@ -1791,6 +1763,7 @@ Widths width_summary(const int32_t* n_bits, int32_t num_ctx, bool raw)
         const int wd = (d + 31) / 32;
         const int words = elim_words(d, wd);
         if (d > w.max_d) w.max_d = d;
+        if (n_bits[c] > w.max_n) w.max_n = n_bits[c];
         if ((n_bits[c] + 31) / 32 > w.max_xw) w.max_xw = (n_bits[c] + 31) / 32;
         if (wd <= SMALL_WD) {
             w.has_small = true;
@@ -2154,6 +2127,7 @@ cudaError_t noalloc_load_kernels()
     if (e == cudaSuccess) e = elim_load_small();
     if (e == cudaSuccess) e = elim_load_narrow();
     if (e == cudaSuccess) e = elim_load_wide();
+    if (e == cudaSuccess) e = verify_load_tc();
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, verify_full_kernel);
     return e;
 }
