@@ -114,7 +114,7 @@ constexpr int DD_SEG_ROWS = 16384;              // rows a CTA takes at a time (1
 constexpr int DD_QUAD_REPS = 1024;              // most distinct rows numbered by a quad, by a CTA (as above)
 constexpr int DD_CTA_REPS = 4096;
 constexpr int DD_AHEAD_XW = 5;                  // widest rows whose next round is loaded ahead
-constexpr int DD_K = 2;                         // rows per thread per round (feature rows of 1-2 words)
+constexpr int DD_K = 1;                         // rows per thread per round
 constexpr int DD_XW = NARROW_WD;                // widest feature row (words) of dedup_kernel<false>
 constexpr int DD_XW_WIDE = 16;                  // widest of dedup_kernel<true> (one row in flight)
 constexpr int DEDUP_PROBES = 8;                 // linear-probe limit
@@ -348,7 +348,7 @@ __device__ bool dd_finish(const DedupArgs& a, int c, int nrep, int t)
 // One group of G warps finds the representatives of context c and writes
 // them, in stream order, to rep_list[row_off[c] + k] with their duplicate
 // counts in rep_dup; rep_count[c] = number of representatives.  Each thread
-// takes DD_K rows a round (one for feature rows of 3 or more words).  Table slot: (fingerprint, smallest row index
+// takes DD_K rows a round.  Table slot: (fingerprint, smallest row index
 // of that content) plus a duplicate counter; a full row comparison decides
 // every match, so a row is a duplicate only if it equals an earlier row.
 //
@@ -398,7 +398,7 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
     // once instead: 77,926 contexts 2,607 against 2,505 us, 4,096 contexts 284
     // against 275).
     constexpr bool AHEAD = XW <= DD_AHEAD_XW;
-    constexpr int K = (XW <= 2 && !AHEAD) ? DD_K : 1;
+    constexpr int K = DD_K;
     uint4 yn[K];
     uint32_t xn[K][XW];
     auto load_round = [&](int base) {
