@@ -15,7 +15,10 @@
 // shared memory binds; here 0.66 ms with one thread a row (ten instructions to
 // spread four bits and pack a parity, two warps a scheduler), 0.62 with two,
 // 0.54 with one mask a word and parities taken from sign bits.  The products
-// take 64 cycles each, 0.22 ms in all (tensor pipe 46% active).
+// take 64 cycles each, 0.22 ms in all (tensor pipe 46% active).  Rows read by
+// their own threads, four words at a time 4 * xw bytes apart, cost two batches
+// of 32,768 rows a context 1,864 us; read a tile ahead, coalesced, and staged in
+// shared memory, 1,830.
 #include "elim.cuh"
 #include "full.cuh"
 
@@ -46,6 +49,9 @@ constexpr int TC_A_BYTES = MAX_N * TC_N;
 constexpr uint32_t TC_IDESC = (1u << 4) |                          // fp32 sums
                               ((uint32_t)(TC_N >> 3) << 17) |      // N; A and B e4m3, both K-major
                               ((uint32_t)(TC_TILE >> 4) << 24);    // M
+constexpr int TC_STAGE_WORDS = TC_TILE * (MAX_N / 32 + 4);  // a group's rows
+constexpr int TC_ST = TC_TILE * (MAX_N / 32) / 256;         // words of them that a thread loads
+constexpr int TC_SMEM_BYTES = TC_A_BYTES + 2 * 4 * TC_STAGE_WORDS;
 constexpr int TC_COLS = 512;       // tensor memory columns: two groups of 128 sums and 2 x 64 of rows
 constexpr int TC_GROUP_COLS = 256;
 
@@ -208,40 +214,72 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
         const int64_t i1 = (i0 + FULL_CHUNK < T) ? i0 + FULL_CHUNK : T;
         const uint32_t* const xc = a.x + a.x_off[c];
         const int xw = cd.xw;
-        const uint32_t lm = (cd.n & 31) ? (1u << (cd.n & 31)) - 1u : 0xFFFFFFFFu;
         const bool vec = ((uintptr_t)xc & 15) == 0 && (xw & 3) == 0;
         const uint4 b = s.raw ? make_uint4(0, 0, 0, 0) : __ldg(s.bz + cd.slot_off);
         unsigned long long cnt = 0ull, first = ~0ull;
-        // the words of a chunk, and y, are loaded a chunk ahead
-        uint32_t xn[TC_KW];
-        auto fetch = [&](int64_t tile, int ch) {
-            const int64_t i = tile + 32 * wg + lane;
-            const uint32_t* const xr = xc + (i < i1 ? i : tile) * xw;
-            const int w0 = (2 * ch + half) * TC_KW;
+        // A tile's rows are contiguous: the group loads the next one into
+        // registers, coalesced, while it works on this one from shared memory.
+        // (Bits past the last feature meet zeros in the map.)
+        const int tg = t & 255;
+        const int rw = 4 * ((xw + 3) / 4) + 4;  // words of a staged row: 16-byte pieces, rows apart in the banks
+        uint32_t* const stage = reinterpret_cast<uint32_t*>(tc_smem + TC_A_BYTES) + g * TC_STAGE_WORDS;
+        uint32_t st[TC_ST];
+        auto fetch = [&](int64_t tile) {
+            const int rows = (int)(i1 - tile < TC_TILE ? i1 - tile : TC_TILE);
+            const uint32_t* const src = xc + tile * xw;
             if (vec) {
-                const uint4 u = w0 < xw ? __ldg(reinterpret_cast<const uint4*>(xr + w0)) : make_uint4(0, 0, 0, 0);
-                xn[0] = u.x;
-                xn[1] = u.y;
-                xn[2] = u.z;
-                xn[3] = u.w;
+#pragma unroll
+                for (int u = 0; u < TC_ST / 4; ++u) {
+                    const int k = tg + 256 * u;
+                    if (4 * k < rows * xw) {
+                        const uint4 v = __ldg(reinterpret_cast<const uint4*>(src) + k);
+                        st[4 * u] = v.x;
+                        st[4 * u + 1] = v.y;
+                        st[4 * u + 2] = v.z;
+                        st[4 * u + 3] = v.w;
+                    }
+                }
             } else {
 #pragma unroll
-                for (int v = 0; v < TC_KW; ++v) xn[v] = w0 + v < xw ? __ldg(xr + w0 + v) : 0u;
+                for (int u = 0; u < TC_ST; ++u) {
+                    const int k = tg + 256 * u;
+                    if (k < rows * xw) st[u] = __ldg(src + k);
+                }
+            }
+        };
+        auto put = [&]() {
+            if (vec) {
+                const int per = xw / 4;
+#pragma unroll
+                for (int u = 0; u < TC_ST / 4; ++u) {
+                    const int k = tg + 256 * u, r = k / per;
+                    if (r < TC_TILE)
+                        *reinterpret_cast<uint4*>(stage + r * rw + 4 * (k - r * per)) =
+                            make_uint4(st[4 * u], st[4 * u + 1], st[4 * u + 2], st[4 * u + 3]);
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < TC_ST; ++u) {
+                    const int k = tg + 256 * u, r = k / xw;
+                    if (r < TC_TILE) stage[r * rw + k - r * xw] = st[u];
+                }
             }
         };
         int64_t tile = i0 + (int64_t)g * TC_TILE;
-        if (tile < i1) fetch(tile, 0);
+        if (tile < i1) fetch(tile);
         for (; tile < i1; tile += 2 * TC_TILE) {
             const int64_t i = tile + 32 * wg + lane;
             const bool valid = i < i1;
+            // (the group is done with the last tile's rows: its sums were compared)
+            put();
+            asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory");
+            if (tile + 2 * TC_TILE < i1) fetch(tile + 2 * TC_TILE);
             const uint4 y = __ldg(a.y + r0 + (valid ? i : tile));
+            const uint32_t* const xr = stage + (32 * wg + lane) * rw;
             for (int ch = 0; ch < nch; ++ch, ++uses) {
                 const int w0 = (2 * ch + half) * TC_KW;
-                uint32_t x[TC_KW];
-#pragma unroll
-                for (int v = 0; v < TC_KW; ++v) x[v] = w0 + v == xw - 1 ? xn[v] & lm : xn[v];
-                if (ch + 1 < nch) fetch(tile, ch + 1);
-                else if (tile + 2 * TC_TILE < i1) fetch(tile + 2 * TC_TILE, 0);
+                const uint4 xv = w0 < xw ? *reinterpret_cast<const uint4*>(xr + w0) : make_uint4(0, 0, 0, 0);
+                const uint32_t x[TC_KW] = {xv.x, xv.y, xv.z, xv.w};
                 const int buf = (int)(uses & 1u);
                 const uint32_t use = uses >> 1;
                 if (use > 0 && !sm.failed && !mbar_wait_bounded(&sm.bar[g][buf], (use - 1) & 1u)) sm.failed = 1;
@@ -325,9 +363,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
 cudaError_t verify_launch_tc(const StoreDev& sd, const FullArgs& fa, int num_sms, cudaStream_t cs)
 {
     const cudaError_t e =
-        cudaFuncSetAttribute(verify_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_A_BYTES);
+        cudaFuncSetAttribute(verify_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BYTES);
     if (e != cudaSuccess) return e;
-    verify_tc_kernel<<<num_sms, TC_THREADS, TC_A_BYTES, cs>>>(sd, fa);
+    verify_tc_kernel<<<num_sms, TC_THREADS, TC_SMEM_BYTES, cs>>>(sd, fa);
     return cudaGetLastError();
 }
 
