@@ -1307,7 +1307,7 @@ cudaError_t launch_queues(K kernel, const StoreDev& sd, LearnArgs la, int max_wo
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     la.cta_region_words = (int)(smem / 4);
-    kernel<<<num_sms * resident_ctas(smem, per_sm), warps * 32, smem, cs>>>(sd, la);
+    f2_launch(kernel, num_sms * resident_ctas(smem, per_sm), warps * 32, smem, cs, sd.num_ctx <= EARLY_MAX_CTX, sd, la);
     return cudaGetLastError();
 }
 

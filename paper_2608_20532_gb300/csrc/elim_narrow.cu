@@ -12,6 +12,7 @@ namespace {
 // enough for a CTA per context has the SMs to spare and takes eight.
 __global__ void __launch_bounds__(LEARN_WARPS * 32, 2) elim_narrow_kernel(StoreDev s, LearnArgs a)
 {
+    pdl_wait();
     extern __shared__ __align__(16) uint32_t smem[];
     elim_queues<CLS_CTA, CLS_WARP, CLS_RESUME>(s, a, smem, a.warp_region_words, [&](int c, auto cta, uint32_t* region, int words) {
         switch (s.desc[c].wd) {

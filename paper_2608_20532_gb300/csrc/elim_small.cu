@@ -12,6 +12,7 @@ static_assert(DEFAULT_SMALL_REGION_BYTES / 4 >= 32 * SMALL_WD * row_stride(SMALL
 // slower on the 78k-context, 81M-row learn).
 __global__ void __launch_bounds__(LEARN_WARPS * 32, 3) elim_small_kernel(StoreDev s, LearnArgs a)
 {
+    pdl_wait();
     extern __shared__ __align__(16) uint32_t smem[];
     elim_queues<CLS_CTA_S, CLS_WARP_S, CLS_RESUME_S>(s, a, smem, a.small_region_words, [&](int c, auto cta, uint32_t* region, int words) {
         switch (s.desc[c].wd) {

@@ -7,6 +7,7 @@ namespace {
 template <int WDT, int CLS, int RESUME>
 __global__ void __launch_bounds__(WIDE_WARPS * 32, WDT <= WIDE_M_WD ? 2 : 1) elim_wide_kernel(StoreDev s, LearnArgs a)
 {
+    pdl_wait();
     extern __shared__ __align__(16) uint32_t smem[];
     elim_cta_queue<CLS, RESUME>(s, a, [&](int c) { elim_cta<WDT>(s, a, c, smem, a.cta_region_words); });
 }
@@ -90,6 +91,7 @@ __device__ __forceinline__ int open_top(const uint4* row, int lane)
 
 __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, LearnArgs a)
 {
+    pdl_wait();
     __shared__ OpenSmem sm;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int n_items = a.counters[CNT_COUNT + CLS_WIDE];
@@ -248,7 +250,8 @@ cudaError_t launch(K kernel, const StoreDev& sd, LearnArgs la, int max_d, int wd
     const size_t smem = 4 * (size_t)la.cta_region_words;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kernel<<<num_sms * resident_ctas(smem, per_sm), WIDE_WARPS * 32, smem, cs>>>(sd, la);
+    f2_launch(kernel, num_sms * resident_ctas(smem, per_sm), WIDE_WARPS * 32, smem, cs, sd.num_ctx <= EARLY_MAX_CTX, sd,
+              la);
     return cudaGetLastError();
 }
 
@@ -258,7 +261,7 @@ cudaError_t elim_launch_wide(const StoreDev& sd, LearnArgs la, int max_d, bool m
 {
     if (medium)
         return launch(elim_wide_kernel<WIDE_M_WD, CLS_WIDE_M, CLS_RESUME_W>, sd, la, max_d, WIDE_M_WD, 2, num_sms, cs);
-    elim_open_kernel<<<num_sms, OPEN_THREADS, 0, cs>>>(sd, la);
+    f2_launch(elim_open_kernel, num_sms, OPEN_THREADS, 0, cs, sd.num_ctx <= EARLY_MAX_CTX, sd, la);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch(elim_wide_kernel<WIDE_WD, CLS_WIDE, CLS_RESUME_W>, sd, la, max_d, WIDE_WD, 1, num_sms, cs);

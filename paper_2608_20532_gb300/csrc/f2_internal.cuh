@@ -24,6 +24,53 @@ struct NvtxRange {
 #define F2_NVTX_RANGE(name) ::f2::NvtxRange f2_nvtx_range_(name)
 
 constexpr unsigned FULL = 0xffffffffu;
+
+// Kernels launched "early" have programmatic stream serialisation: such a
+// kernel may be set up on the SMs while the kernel before it in the stream
+// still runs.  Every kernel that f2_launch starts begins with pdl_wait(), which
+// lets the kernel after it do the same and waits until everything the kernels
+// before it wrote is visible.  What a call of short kernels spends between them
+// shrinks: with the fill that small stores no longer launch, eight batches for
+// 4,096 contexts 418..444 -> 319 us, 4,096 contexts 275 -> 263, 64 contexts of
+// 1,024 bits 1,830 -> 1,781.  Calls of long kernels gain nothing (77,926 contexts
+// 2,516 us with it, 2,501 without; 10M queries 916 and 831), so stores of more than
+// EARLY_MAX_CTX contexts and the encoder do without.  The pointers that a kernel
+// loads from through the read-only path are passed through the wait, so that no
+// such load can be moved above it.
+template <typename P>
+__device__ __forceinline__ void through_wait(P& p)
+{
+    asm volatile("" : "+l"(p)::"memory");
+}
+template <typename... P>
+__device__ __forceinline__ void pdl_wait(P&... p)
+{
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    (through_wait(p), ...);
+}
+
+constexpr int EARLY_MAX_CTX = 8192;
+constexpr size_t EARLY_MAX_BYTES = size_t(16) << 20;  // of a fill or a copy
+
+// (The launch's error, if any, stays the last error.)
+template <typename... P, typename... A>
+inline void f2_launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t cs, bool early,
+                      A... args)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = cs;
+    cfg.attrs = &at;
+    cfg.numAttrs = early ? 1 : 0;
+    (void)cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 constexpr int MAX_N = 1024;          // feature bits per context
 constexpr int MAX_D = MAX_N + 1;     // row width with the affine constant
 constexpr int NARROW_WD = 9;         // widest row (32-bit words) handled by the narrow kernels

@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(256) rebase_kernel(const int64_t* __restrict__
                                                      int32_t c0, int32_t c1, int32_t C, int64_t xa,
                                                      int64_t* __restrict__ row_off, int64_t* __restrict__ x_off)
 {
+    pdl_wait(ro, xo);
     // contexts outside [c0, c1) get no rows; offsets of the chunk's contexts
     // count from the chunk's first row and first feature word
     const int64_t r0 = ro[0];
@@ -266,7 +267,8 @@ extern "C" int f2_learn_host(f2_store* st, const int64_t* row_off, const uint32_
         if (e != cudaSuccess) return f2_cuda_status(e);
         int blocks = (C + 256) / 256;
         if (blocks > st->num_sms * 4) blocks = st->num_sms * 4;
-        rebase_kernel<<<blocks, 256, 0, cs>>>(h->ro[b], h->xo[b], k.c0, k.c1, C, k.xa, h->row_off, h->x_off);
+        f2_launch(rebase_kernel, blocks, 256, 0, cs, C <= EARLY_MAX_CTX, h->ro[b], h->xo[b], k.c0, k.c1, C, k.xa,
+                  h->row_off, h->x_off);
         e = cudaGetLastError();
         if (e != cudaSuccess) return f2_cuda_status(e);
         rc = f2_learn_batched(st, h->row_off, h->x[b], h->x_off, reinterpret_cast<const uint32_t*>(h->y[b]),

@@ -831,6 +831,7 @@ __device__ bool dedup_wide_ctx(const StoreDev& s, const DedupArgs& a, int c, int
 template <bool WX>
 __global__ void __launch_bounds__(DD_THREADS, DD_CTAS_PER_SM) dedup_kernel(StoreDev s, DedupArgs a)
 {
+    pdl_wait();
     // WX: the contexts whose feature rows have DD_XW + 1 .. DD_XW_WIDE words
     constexpr int C_CTA = WX ? CLS_DDW_CTA : CLS_DD_CTA;
     constexpr int C_QUAD = WX ? CLS_DDW_QUAD : CLS_DD_QUAD;
@@ -970,6 +971,7 @@ constexpr int CHECK_SMEM_BYTES = 4 * CHECK_BASIS_WORDS + CHECK_CHUNK + 4 * CHECK
 
 __global__ void __launch_bounds__(256) check_snap_kernel(StoreDev s, CheckArgs a)
 {
+    pdl_wait();
     extern __shared__ __align__(16) uint32_t smem[];
     uint32_t* const S = smem;
     uint8_t* const flags = reinterpret_cast<uint8_t*>(smem + CHECK_BASIS_WORDS);
@@ -1123,7 +1125,19 @@ constexpr int PLAN_SUB = PLAN_BUCKETS * NARROW_WD;  // (bucket, width) keys per 
 constexpr int PLAN_KEYS = NUM_CLASSES * PLAN_SUB;
 static_assert(PLAN_KEYS <= PLAN_HIST_WORDS, "the plan histogram holds every key");
 
+// Scratch that a learn call counts in, cleared by the first plan of the call
+// where one block plans (plan_small_kernel), else by a fill before it.
+struct PlanZero {
+    int* work;                    // CNT_WORK .. CNT_WORDS of the counters; NULL: cleared already
+    int32_t* shard_done;          // [C]
+    int* full_ctr;                // [2C], and the late count at [4C]
+    unsigned long long* full_cnt; // [C]
+    unsigned long long* full_first;  // [C], all ones
+    int* hand;                    // two counts, and [2C] from 2 + 4C; NULL: not used in this call
+};
+
 struct PlanArgs {
+    PlanZero zero;
     const int64_t* row_off;
     const int64_t* x_off;
     int64_t total_rows;
@@ -1248,6 +1262,7 @@ __device__ __forceinline__ bool plan_done(const PlanArgs& p) { return p.after &&
 
 __global__ void __launch_bounds__(256) plan_key_kernel(StoreDev s, PlanArgs p)
 {
+    pdl_wait();
     if (plan_done(p)) return;
     __shared__ int hist[PLAN_KEYS];
     for (int i = threadIdx.x; i < PLAN_KEYS; i += blockDim.x) hist[i] = 0;
@@ -1324,6 +1339,7 @@ __device__ void plan_scan_block(int* hist, int* counters, int mode)
 
 __global__ void __launch_bounds__(1024) plan_scan_kernel(PlanArgs p)
 {
+    pdl_wait();
     if (plan_done(p)) return;
     plan_scan_block(p.hist, p.counters, p.mode);
 }
@@ -1343,6 +1359,7 @@ __device__ __forceinline__ void plan_place(const PlanArgs& p, int* cursor, int c
 
 __global__ void __launch_bounds__(256) plan_scatter_kernel(StoreDev s, PlanArgs p)
 {
+    pdl_wait();
     if (plan_done(p)) return;
     // the lanes of a warp with the same key take their slots with one atomic
     const int lane = threadIdx.x & 31;
@@ -1370,9 +1387,24 @@ __global__ void __launch_bounds__(256) plan_scatter_kernel(StoreDev s, PlanArgs 
 constexpr int PLAN_SMALL_MAX = 8192;
 __global__ void __launch_bounds__(1024) plan_small_kernel(StoreDev s, PlanArgs p)
 {
+    pdl_wait();
     __shared__ int hist[PLAN_KEYS];
     if (plan_done(p)) return;
     for (int i = threadIdx.x; i < PLAN_KEYS; i += blockDim.x) hist[i] = 0;
+    if (p.zero.work) {
+        const PlanZero& z = p.zero;
+        const int C = s.num_ctx;
+        if (threadIdx.x < CNT_WORDS - CNT_WORK) z.work[threadIdx.x] = 0;
+        if (threadIdx.x == 0) z.full_ctr[4 * C] = 0;
+        if (threadIdx.x < 2 && z.hand) z.hand[threadIdx.x] = 0;
+        for (int c = threadIdx.x; c < C; c += blockDim.x) {
+            z.shard_done[c] = 0;
+            z.full_ctr[c] = z.full_ctr[C + c] = 0;
+            z.full_cnt[c] = 0ull;
+            z.full_first[c] = ~0ull;
+            if (z.hand) z.hand[2 + 4 * C + c] = z.hand[2 + 5 * C + c] = 0;
+        }
+    }
     __syncthreads();
     const PlanLimits L = plan_limits(p);
     constexpr int PER = PLAN_SMALL_MAX / 1024;
@@ -1396,7 +1428,7 @@ __global__ void __launch_bounds__(1024) plan_small_kernel(StoreDev s, PlanArgs p
 int launch_plan(const StoreDev& sd, const PlanArgs& pa, int num_sms, cudaStream_t cs)
 {
     if (sd.num_ctx <= PLAN_SMALL_MAX) {
-        plan_small_kernel<<<1, 1024, 0, cs>>>(sd, pa);
+        f2_launch(plan_small_kernel, 1, 1024, 0, cs, sd.num_ctx <= EARLY_MAX_CTX, sd, pa);
         return f2_cuda_status(cudaGetLastError());
     }
     if (!pa.hist_zeroed) {
@@ -1406,9 +1438,9 @@ int launch_plan(const StoreDev& sd, const PlanArgs& pa, int num_sms, cudaStream_
     int blocks = (sd.num_ctx + 255) / 256;
     if (blocks > num_sms * 2) blocks = num_sms * 2;
     if (blocks < 1) blocks = 1;
-    plan_key_kernel<<<blocks, 256, 0, cs>>>(sd, pa);
-    plan_scan_kernel<<<1, 1024, 0, cs>>>(pa);
-    plan_scatter_kernel<<<blocks, 256, 0, cs>>>(sd, pa);
+    f2_launch(plan_key_kernel, blocks, 256, 0, cs, sd.num_ctx <= EARLY_MAX_CTX, sd, pa);
+    f2_launch(plan_scan_kernel, 1, 1024, 0, cs, sd.num_ctx <= EARLY_MAX_CTX, pa);
+    f2_launch(plan_scatter_kernel, blocks, 256, 0, cs, sd.num_ctx <= EARLY_MAX_CTX, sd, pa);
     return f2_cuda_status(cudaGetLastError());
 }
 
@@ -1440,6 +1472,7 @@ constexpr int FULL_TABLE_WORDS = 2 * FULL_ZH_BYTES / 4 + 256;  // both planes + 
 
 __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, FullArgs a)
 {
+    pdl_wait();
     extern __shared__ uint4 full_smem[];
     // the table at the first 1024-byte boundary of the dynamic shared memory
     const uint32_t pad = ((1024u - (smem_addr(full_smem) & 1023u)) & 1023u) / 4u;
@@ -1651,7 +1684,8 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
                        int64_t warp_work, int32_t* queue, int32_t* keybuf, int* hist, int num_sms,
                        const Widths& wv, int* full_ctr, unsigned long long* full_cnt,
                        unsigned long long* full_first, cudaStream_t cs, Fork* fk = nullptr, int scale = 0,
-                       bool prezeroed = false, int64_t long_rows = LONG_CALL_ROWS, const CheckArgs* check = nullptr)
+                       bool prezeroed = false, int64_t long_rows = LONG_CALL_ROWS, const CheckArgs* check = nullptr,
+                       const PlanZero& zero = PlanZero{})
 {
     // prezeroed: the caller has cleared full_ctr's first 2C words and late
     // count, full_cnt, full_first (to -1) and hist
@@ -1671,6 +1705,7 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
         if (e0 != cudaSuccess) return f2_cuda_status(e0);
     }
     PlanArgs pa;
+    pa.zero = zero;
     pa.row_off = row_off;
     pa.x_off = x_off;
     pa.total_rows = total_rows;
@@ -1724,7 +1759,7 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
         const size_t csmem = CHECK_SMEM_BYTES;
         e = cudaFuncSetAttribute(check_snap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem);
         if (e != cudaSuccess) return f2_cuda_status(e);
-        check_snap_kernel<<<num_sms * 2, 256, csmem, cs>>>(sd, *check);
+        f2_launch(check_snap_kernel, num_sms * 2, 256, csmem, cs, sd.num_ctx <= EARLY_MAX_CTX, sd, *check);
         e = cudaGetLastError();
         if (e != cudaSuccess) return f2_cuda_status(e);
         LearnArgs lr = lx;
@@ -1763,7 +1798,7 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, verify_full_kernel, FULL_THREADS, smem);
         if (e != cudaSuccess) return f2_cuda_status(e);
         if (per_sm < 1) per_sm = 1;
-        verify_full_kernel<<<num_sms * per_sm, FULL_THREADS, smem, cs>>>(sd, fa);
+        f2_launch(verify_full_kernel, num_sms * per_sm, FULL_THREADS, smem, cs, sd.num_ctx <= EARLY_MAX_CTX, sd, fa);
         e = cudaGetLastError();
         if (e != cudaSuccess) return f2_cuda_status(e);
     }
@@ -1855,20 +1890,25 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
         if (!st->timing && f2_dev_alloc(st, (void**)&st->timing, bytes, cs, true) != cudaSuccess) return F2_ERR_OOM;
         zl.add(st->timing, bytes);
     }
-    if (hand_min > 0) {  // hand-off: the two list counts and the chunk counters
-        zl.add(st->hand, sizeof(int) * 2);
-        zl.add(st->hand + 2 + 4 * C, sizeof(int) * 2 * C);
+    PlanZero zero{};
+    if (st->num_ctx <= PLAN_SMALL_MAX) {  // by the call's first plan
+        zero = {st->counters + CNT_WORK, st->shard_done, st->full_ctr, st->full_cnt, st->full_first,
+                hand_min > 0 ? st->hand : nullptr};
+    } else {
+        if (hand_min > 0) {  // hand-off: the two list counts and the chunk counters
+            zl.add(st->hand, sizeof(int) * 2);
+            zl.add(st->hand + 2 + 4 * C, sizeof(int) * 2 * C);
+        }
+        if (dedup) {  // the work totals and the shard items of the duplicate pass
+            zl.add(st->counters + CNT_WORK, (CNT_WORDS - CNT_WORK) * sizeof(int));
+            zl.add(st->shard_done, sizeof(int32_t) * C);
+        }
+        zl.add(st->full_ctr, sizeof(int) * 2 * C);        // full-rank chunks claimed and done
+        zl.add(st->full_ctr + 4 * C, sizeof(int));        // late count
+        zl.add(st->full_cnt, sizeof(unsigned long long) * C);
+        zl.add(st->full_first, sizeof(unsigned long long) * C, 0xff);
+        zl.add(st->plan_hist, sizeof(int) * 2 * PLAN_HIST_WORDS);  // the histograms of the two plans
     }
-    if (dedup) {  // the work totals and the shard items of the duplicate pass
-        zl.add(st->counters + CNT_WORK, (CNT_WORDS - CNT_WORK) * sizeof(int));
-        zl.add(st->shard_done, sizeof(int32_t) * C);
-    }
-    zl.add(st->full_ctr, sizeof(int) * 2 * C);        // full-rank chunks claimed and done
-    zl.add(st->full_ctr + 4 * C, sizeof(int));        // late count
-    zl.add(st->full_cnt, sizeof(unsigned long long) * C);
-    zl.add(st->full_first, sizeof(unsigned long long) * C, 0xff);
-    if (st->num_ctx > PLAN_SMALL_MAX)  // the histograms of the two plans (one block keeps its own)
-        zl.add(st->plan_hist, sizeof(int) * 2 * PLAN_HIST_WORDS);
     e = f2_fill(zl, cs);
     if (e != cudaSuccess) return f2_cuda_status(e);
     const StoreDev sd = st->dev();
@@ -1895,6 +1935,8 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
     }
     if (dedup) {
         PlanArgs pa;
+        pa.zero = zero;
+        zero = PlanZero{};  // (the second plan finds it cleared)
         pa.row_off = row_off;
         pa.x_off = x_off;
         pa.total_rows = total_rows;
@@ -1940,13 +1982,15 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
         if (e != cudaSuccess) return f2_cuda_status(e);
         cudaStream_t ks = fk.next(wide_rows ? 2 : 1);
         if (fk.e != cudaSuccess) return f2_cuda_status(fk.e);
-        dedup_kernel<false><<<DD_CTAS_PER_SM * st->num_sms, DD_THREADS, DD_SMEM, ks>>>(sd, da);
+        f2_launch(dedup_kernel<false>, DD_CTAS_PER_SM * st->num_sms, DD_THREADS, DD_SMEM, ks,
+                  sd.num_ctx <= EARLY_MAX_CTX, sd, da);
         e = cudaGetLastError();
         if (e != cudaSuccess) return f2_cuda_status(e);
         if (wide_rows) {
             e = cudaFuncSetAttribute(dedup_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DD_SMEM);
             if (e != cudaSuccess) return f2_cuda_status(e);
-            dedup_kernel<true><<<DD_CTAS_PER_SM * st->num_sms, DD_THREADS, DD_SMEM, fk.next(1)>>>(sd, da);
+            f2_launch(dedup_kernel<true>, DD_CTAS_PER_SM * st->num_sms, DD_THREADS, DD_SMEM, fk.next(1),
+                      sd.num_ctx <= EARLY_MAX_CTX, sd, da);
             e = cudaGetLastError();
             if (e != cudaSuccess) return f2_cuda_status(e);
         }
@@ -1997,7 +2041,7 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
     return launch_elimination(sd, la, row_off, x_off, total_rows, total_x_words, dedup ? st->rep_count : nullptr,
                               heavy, st->warp_work, st->queue, st->keybuf, st->plan_hist + PLAN_HIST_WORDS,
                               st->num_sms, wv, st->full_ctr, st->full_cnt, st->full_first, cs, &fk, scale, true,
-                              all_cta ? INT64_MAX : st->long_call_rows, &ca);
+                              all_cta ? INT64_MAX : st->long_call_rows, &ca, zero);
 }
 
 extern "C" int f2_learn_timing(const f2_store* st, uint64_t* out_host, f2_stream_t stream)
@@ -2053,6 +2097,7 @@ std::mutex g_noalloc_mu;
 __global__ void __launch_bounds__(1024) noalloc_desc_kernel(const int32_t* __restrict__ n_bits, int C, uint32_t raw,
                                                             CtxDesc* __restrict__ desc)
 {
+    pdl_wait(n_bits);
     constexpr int PER = (F2_NOALLOC_MAX_CTX + 1023) / 1024;
     __shared__ long long wsum[3][32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -2215,7 +2260,8 @@ extern "C" int f2_learn_batched_noalloc(int32_t num_ctx, const int32_t* n_bits_h
                             cs);
     }
     if (e != cudaSuccess) return f2_cuda_status(e);
-    noalloc_desc_kernel<<<1, 1024, 0, cs>>>(sc->n_bits, num_ctx, raw ? 1u : 0u, sc->desc);
+    f2_launch(noalloc_desc_kernel, 1, 1024, 0, cs, num_ctx <= EARLY_MAX_CTX, sc->n_bits, num_ctx, raw ? 1u : 0u,
+              sc->desc);
 
     StoreDev sd;
     sd.desc = sc->desc;

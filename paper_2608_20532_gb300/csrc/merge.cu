@@ -22,6 +22,7 @@ __global__ void __launch_bounds__(256) merge_gather_kernel(StoreDev s, const int
                                                            const int64_t* __restrict__ member_word,
                                                            uint32_t* __restrict__ x, uint4* __restrict__ y)
 {
+    pdl_wait(member_row, member_word);
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
     for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < s.num_ctx; c += warps) {
@@ -121,7 +122,8 @@ extern "C" int f2_merge_bases(const f2_store* src, int32_t num_groups, const int
     if (e == cudaSuccess && C > 0) {
         int blocks = (C + 7) / 8;
         if (blocks > src->num_sms * 16) blocks = src->num_sms * 16;
-        merge_gather_kernel<<<blocks, 256, 0, cs>>>(src->dev(), d_member_row, d_member_word, d_x, d_y);
+        f2_launch(merge_gather_kernel, blocks, 256, 0, cs, true, src->dev(), d_member_row, d_member_word, d_x,
+                  d_y);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && num_groups > 0) {

@@ -36,6 +36,7 @@ namespace {
 // segment's aligned head and tail, single bytes at both ends.
 __global__ void __launch_bounds__(256) fill_kernel(F2FillList L)
 {
+    pdl_wait();
     const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t nth = (size_t)gridDim.x * blockDim.x;
     for (int k = 0; k < L.n; ++k) {
@@ -65,7 +66,7 @@ cudaError_t f2_fill(const F2FillList& L, cudaStream_t cs)
     unsigned long long blocks = (total + 16383) / 16384;
     if (blocks > 1024) blocks = 1024;
     if (blocks < 1) blocks = 1;
-    fill_kernel<<<(unsigned)blocks, 256, 0, cs>>>(L);
+    f2_launch(fill_kernel, (unsigned)blocks, 256, 0, cs, total <= EARLY_MAX_BYTES, L);
     return cudaGetLastError();
 }
 
@@ -311,6 +312,7 @@ struct CopyList {
 
 __global__ void __launch_bounds__(256) copy_kernel(CopyList L)
 {
+    pdl_wait();
     const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t nth = (size_t)gridDim.x * blockDim.x;
     for (int k = 0; k < L.n; ++k) {
@@ -364,7 +366,7 @@ extern "C" int f2_get_basis(const f2_store* s, int32_t* rank, uint32_t* pivot_ma
     if (L.n == 0) return F2_OK;
     size_t blocks = (total + 8191) / 8192;  // 32 bytes a thread, at most eight blocks per SM
     if (blocks > (size_t)s->num_sms * 8) blocks = (size_t)s->num_sms * 8;
-    copy_kernel<<<(unsigned)blocks, 256, 0, st>>>(L);
+    f2_launch(copy_kernel, (unsigned)blocks, 256, 0, st, total <= EARLY_MAX_BYTES, L);
     return f2_cuda_status(cudaGetLastError());
 }
 
@@ -375,6 +377,7 @@ extern "C" int f2_get_basis(const f2_store* s, int32_t* rank, uint32_t* pivot_ma
 // over slots: coalesced 16-byte stores.
 __global__ void __launch_bounds__(256) solve_kernel(StoreDev s, uint4* __restrict__ W)
 {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
     for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < s.num_ctx; c += warps) {
@@ -397,7 +400,8 @@ extern "C" int f2_solve_affine(const f2_store* s, uint32_t* W, f2_stream_t strea
     int blocks = (int)((s->num_ctx + 7) / 8);
     const int cap = s->num_sms * 8;
     if (blocks > cap) blocks = cap;
-    solve_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(s->dev(), reinterpret_cast<uint4*>(W));
+    f2_launch(solve_kernel, blocks, threads, 0, (cudaStream_t)stream, s->num_ctx <= EARLY_MAX_CTX, s->dev(),
+              reinterpret_cast<uint4*>(W));
     return f2_cuda_status(cudaGetLastError());
 }
 

@@ -145,6 +145,7 @@ __device__ void tc_build(const StoreDev& s, const CtxDesc& cd, uint8_t* A, int k
 
 __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, FullArgs a)
 {
+    pdl_wait();
     extern __shared__ __align__(128) uint8_t tc_smem[];
     __shared__ TcSmem sm;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -365,7 +366,7 @@ cudaError_t verify_launch_tc(const StoreDev& sd, const FullArgs& fa, int num_sms
     const cudaError_t e =
         cudaFuncSetAttribute(verify_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BYTES);
     if (e != cudaSuccess) return e;
-    verify_tc_kernel<<<num_sms, TC_THREADS, TC_SMEM_BYTES, cs>>>(sd, fa);
+    f2_launch(verify_tc_kernel, num_sms, TC_THREADS, TC_SMEM_BYTES, cs, sd.num_ctx <= EARLY_MAX_CTX, sd, fa);
     return cudaGetLastError();
 }
 
