@@ -57,7 +57,13 @@ namespace {
 // records the first such one, and only representatives before the
 // context's first are counted.  The last chunk of a context commits its
 // counts; if some representative was outside the span, the context is
-// listed for resume_kernel from that one on.
+// listed for a second launch of the elimination from that one on.
+//
+// 10,000 contexts of 128..512 bits of parsed values, 13.4M rows: 443 us while
+// every CTA claimed its way through the whole list of contexts, an atomic each,
+// a row's words were loaded one by one and every basis row was XOR-ed whole;
+// now 190 (45% of the issue slots; warps wait at the barriers of a chunk and
+// for its rows).
 // ---------------------------------------------------------------------------
 struct CheckArgs {
     const int64_t* row_off;
@@ -935,85 +941,202 @@ __device__ __forceinline__ int64_t check_slot(const CheckArgs& a, int c)
     return a.row_off[c] / CHECK_CHUNK + c;  // the context's first chunk record (chunks never overlap)
 }
 
+// Feature words of a row of up to WD words (bits >= n cleared), by the widest
+// loads that every row of the context allows (`al` as in load_words).
+template <int WD>
+__device__ __forceinline__ void load_row_words(const uint32_t* __restrict__ p, int al, bool valid, int n, int xw,
+                                               uint32_t (&x)[WD])
+{
+#pragma unroll
+    for (int v = 0; v < WD; ++v) x[v] = 0;
+    if (valid) {
+        if (WD >= 4 && al >= 2) {
+#pragma unroll
+            for (int v = 0; v + 3 < WD; v += 4)
+                if (v < xw) {
+                    const uint4 t = __ldg(reinterpret_cast<const uint4*>(p + v));
+                    x[v] = t.x;
+                    x[v + 1] = t.y;
+                    x[v + 2] = t.z;
+                    x[v + 3] = t.w;
+                }
+        } else if (WD >= 2 && al >= 1) {
+#pragma unroll
+            for (int v = 0; v + 1 < WD; v += 2)
+                if (v < xw) {
+                    const uint2 t = __ldg(reinterpret_cast<const uint2*>(p + v));
+                    x[v] = t.x;
+                    x[v + 1] = t.y;
+                }
+        } else {
+#pragma unroll
+            for (int v = 0; v < WD; ++v)
+                if (v < xw) x[v] = __ldg(p + v);
+        }
+    }
+    const uint32_t last = (n & 31) ? (1u << (n & 31)) - 1u : FULL;
+#pragma unroll
+    for (int v = 0; v < WD; ++v) x[v] &= (v == xw - 1) ? last : FULL;
+}
+
+// Reduces q and y by the basis rows of pivot words W and up.  A basis row has no
+// bit above its pivot.
+template <int WD, int W>
+__device__ __forceinline__ void check_words(uint32_t (&q)[WD], uint4& y, const uint32_t* S, const uint32_t* Ps,
+                                            const uint32_t* Ds)
+{
+    constexpr int RS = row_stride(WD);
+    const uint32_t sel = q[W];
+    uint32_t uw = __reduce_or_sync(FULL, sel & Ps[W]);
+    uint32_t dw = uw & Ds[W];
+    uw &= ~dw;
+    while (uw) {  // two a step, their loads issued together
+        const int b0 = __ffs(uw) - 1;
+        uw &= uw - 1;
+        const bool two = uw != 0u;
+        const int b1 = two ? __ffs(uw) - 1 : b0;
+        uw &= uw - 1;
+        const uint4 z0 = *reinterpret_cast<const uint4*>(S + (32 * W + b0) * RS);
+        const uint4 z1 = *reinterpret_cast<const uint4*>(S + (32 * W + b1) * RS);
+        const uint32_t m0 = 0u - ((sel >> b0) & 1u);
+        const uint32_t m1 = two ? 0u - ((sel >> b1) & 1u) : 0u;
+        y.x ^= (z0.x & m0) ^ (z1.x & m1);
+        y.y ^= (z0.y & m0) ^ (z1.y & m1);
+        y.z ^= (z0.z & m0) ^ (z1.z & m1);
+        y.w ^= (z0.w & m0) ^ (z1.w & m1);
+    }
+    while (dw) {
+        const int b = __ffs(dw) - 1;
+        dw &= dw - 1;
+        const uint32_t* row = S + (32 * W + b) * RS;
+        const uint4 z = *reinterpret_cast<const uint4*>(row);
+        const uint32_t m = 0u - ((sel >> b) & 1u);
+        y.x ^= z.x & m;
+        y.y ^= z.y & m;
+        y.z ^= z.z & m;
+        y.w ^= z.w & m;
+#pragma unroll
+        for (int v4 = 0; v4 <= W / 4; ++v4) {
+            const uint4 e = *reinterpret_cast<const uint4*>(row + 4 + 4 * v4);
+            const uint32_t ev[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (4 * v4 + j <= W && 4 * v4 + j < WD) q[4 * v4 + j] ^= ev[j] & m;
+        }
+    }
+    if constexpr (W + 1 < WD) check_words<WD, W + 1>(q, y, S, Ps, Ds);
+}
+
+// Classes of the representatives kb .. ke-1 of a context under its basis S of
+// pivots Ps: 2 outside the span, 1 a contradiction, 0 redundant.  The basis is
+// reduced, so a row's pivot bits select its basis rows whatever their order;
+// and where a basis row is its pivot alone (not in Ds: with values that differ
+// in single bits, nearly every row) only its 128-bit word counts.
 template <int WD>
 __device__ void check_chunk(const StoreDev& s, const CheckArgs& a, int c, int kb, int ke, const uint32_t* S,
-                            const uint32_t (&P)[WD], uint8_t* flags)
+                            const uint32_t* Ps, const uint32_t* Ds, uint8_t* flags)
 {
     const CtxDesc cd = s.desc[c];
     const int64_t r0 = a.row_off[c];
     const int32_t* reps = a.rep_list ? a.rep_list + r0 : nullptr;
     const uint32_t* xc = a.x + a.x_off[c];
     const uint4* yc = a.y + r0;
-    const uint64_t mixed = mixed_words<WD>(P, cd.d, cd.wd);
+    const uintptr_t bits = (uintptr_t)xc | (uintptr_t)(4 * cd.xw);
+    const int al = (bits & 15) == 0 ? 2 : ((bits & 7) == 0 ? 1 : 0);
     // every lane of a warp in each round: the pivot walk is warp-uniform
     for (int base = kb; base < ke; base += blockDim.x) {
         const int k = base + (int)threadIdx.x;
         const bool valid = k < ke;
         const int i = valid ? (reps ? __ldg(reps + k) : k) : 0;
-        uint32_t xin[WD], q[1][WD];
-        uint4 yr[1];
-        load_raw<WD>(xc + (int64_t)i * cd.xw, yc + i, valid, cd.n, cd.xw, xin, yr[0]);
-        make_q<WD>(xin, valid, s.raw, q[0]);
-        reduce_rows<WD, 1>(q, yr, S, P, mixed);
+        uint32_t xin[WD], q[WD];
+        uint4 y = valid ? __ldg(yc + i) : make_uint4(0, 0, 0, 0);
+        load_row_words<WD>(xc + (int64_t)i * cd.xw, al, valid, cd.n, cd.xw, xin);
+        make_q<WD>(xin, valid, s.raw, q);
+        check_words<WD, 0>(q, y, S, Ps, Ds);
         uint32_t resid = 0;
 #pragma unroll
-        for (int w = 0; w < WD; ++w) resid |= q[0][w] & ~P[w];
-        // 2: outside the span, 1: a contradiction, 0: redundant
-        if (valid) flags[k - kb] = resid ? 2 : (nonzero4(yr[0]) ? 1 : 0);
+        for (int w = 0; w < WD; ++w) resid |= q[w] & ~Ps[w];
+        if (valid) flags[k - kb] = resid ? 2 : (nonzero4(y) ? 1 : 0);
     }
 }
 
 // Shared memory of the check: the basis (a slot of row_stride words per
 // column), the chunk's classes (CHECK_CHUNK bytes), then CHECK_CTL_WORDS of
-// control (the pivot words, the claimed chunk, the chunk's sums).
-constexpr int CHECK_CTL_WORDS = 64;
+// control (the pivot words, those whose rows have other columns too, the
+// claimed chunk, the chunk's sums).
+constexpr int CHECK_CTL_WORDS = 80;
 constexpr int CHECK_SMEM_BYTES = 4 * CHECK_BASIS_WORDS + CHECK_CHUNK + 4 * CHECK_CTL_WORDS;
 
-__global__ void __launch_bounds__(256) check_snap_kernel(StoreDev s, CheckArgs a)
+__global__ void __launch_bounds__(256, 3) check_snap_kernel(StoreDev s, CheckArgs a)
 {
     pdl_wait();
     extern __shared__ __align__(16) uint32_t smem[];
     uint32_t* const S = smem;
     uint8_t* const flags = reinterpret_cast<uint8_t*>(smem + CHECK_BASIS_WORDS);
     uint32_t* const ctl = smem + CHECK_BASIS_WORDS + CHECK_CHUNK / 4;
-    uint32_t* const Ps = ctl;  // 48 pivot words
+    uint32_t* const Ps = ctl;       // 24 pivot words (WIDE_M_WD at most)
+    uint32_t* const Ds = ctl + 24;  // 24 words
     int* const s_c = reinterpret_cast<int*>(ctl + 48);
     int* const s_k = s_c + 1;
     int* const s_first_out = s_c + 2;
     unsigned long long* const s_cnt = reinterpret_cast<unsigned long long*>(ctl + 52);
     long long* const s_first = reinterpret_cast<long long*>(ctl + 54);
     const int t = threadIdx.x;
-    int q = 0, built = -1;
+    // CTAs start at different contexts and go round; a CTA stays with a context
+    // while it has chunks left.  A warp looks at 32 contexts at a time.
+    const int nq = *a.snap_count;
+    const int q0 = nq > 0 ? (int)((int64_t)blockIdx.x * nq / gridDim.x) : 0;
+    int tried = 0, built = -1;
+    auto reps_of = [&](int c) {
+        return a.rep_list ? a.rep_count[c] : (int)(a.row_off[c + 1] - a.row_off[c]);
+    };
     for (;;) {
-        if (t == 0) {  // the next chunk, contexts in list order
+        if (t < 32) {
             int c = -1, k = 0;
-            const int nq = *a.snap_count;
-            for (; q < nq; ++q) {
-                const int cq = a.snap_list[q];
-                const int R = a.rep_list ? a.rep_count[cq] : (int)(a.row_off[cq + 1] - a.row_off[cq]);
-                k = atomicAdd(a.ctr + cq, 1);
-                if (a.snap_start[cq] + k * CHECK_CHUNK < R) {
-                    c = cq;
-                    break;
-                }
+            if (built >= 0) {
+                if (t == 0) k = atomicAdd(a.ctr + built, 1);
+                k = __shfl_sync(FULL, k, 0);
+                if (a.snap_start[built] + k * CHECK_CHUNK < reps_of(built)) c = built;
             }
-            *s_c = c;
-            *s_k = k;
-            *s_first_out = INT_MAX;
-            *s_cnt = 0ull;
-            *s_first = LLONG_MAX;
+            while (c < 0 && tried < nq) {
+                int cq = -1;
+                if (tried + t < nq) {
+                    const int at = q0 + tried + t;
+                    cq = a.snap_list[at < nq ? at : at - nq];
+                    if (a.snap_start[cq] + (int64_t)__ldcg(a.ctr + cq) * CHECK_CHUNK >= reps_of(cq)) cq = -1;
+                }
+                const uint32_t left = __ballot_sync(FULL, cq >= 0);
+                if (!left) {
+                    tried += 32;
+                    continue;
+                }
+                cq = __shfl_sync(FULL, cq, __ffs(left) - 1);
+                if (t == 0) k = atomicAdd(a.ctr + cq, 1);
+                k = __shfl_sync(FULL, k, 0);
+                if (a.snap_start[cq] + k * CHECK_CHUNK < reps_of(cq)) c = cq;
+            }
+            if (t == 0) {
+                *s_c = c;
+                *s_k = k;
+                *s_first_out = INT_MAX;
+                *s_cnt = 0ull;
+                *s_first = LLONG_MAX;
+            }
         }
         __syncthreads();
         const int c = *s_c;
         const int ck = *s_k;
         if (c < 0) break;
         const CtxDesc cd = s.desc[c];
-        const int R = a.rep_list ? a.rep_count[c] : (int)(a.row_off[c + 1] - a.row_off[c]);
+        const int R = reps_of(c);
         const int st0 = a.snap_start[c];
         const int kb = st0 + ck * CHECK_CHUNK;
         const int ke = (kb + CHECK_CHUNK < R) ? kb + CHECK_CHUNK : R;
         if (built != c) {  // the basis into shared memory (pivot rows only)
-            if (t < 48) Ps[t] = (t < cd.wd) ? s.pivot[cd.pw_off + t] : 0u;
+            if (t < 24) {
+                Ps[t] = (t < cd.wd) ? s.pivot[cd.pw_off + t] : 0u;
+                Ds[t] = 0u;
+            }
             __syncthreads();
             // the stride of the instance that checks it (rows of 10..17 words: the 17-word one)
             const int rs = row_stride(cd.wd <= NARROW_WD ? cd.wd : WIDE_M_WD);
@@ -1022,17 +1145,18 @@ __global__ void __launch_bounds__(256) check_snap_kernel(StoreDev s, CheckArgs a
                 uint32_t* row = S + kk * rs;
                 *reinterpret_cast<uint4*>(row) = s.bz[cd.slot_off + kk];
                 const uint32_t* src = s.bx + cd.xw_off + (int64_t)kk * cd.wd;
-                for (int v = 0; v < rs - 4; ++v) row[4 + v] = (v < cd.wd) ? src[v] : 0u;
+                uint32_t other = 0;
+                for (int v = 0; v < rs - 4; ++v) {
+                    const uint32_t e = (v < cd.wd) ? src[v] : 0u;
+                    row[4 + v] = e;
+                    if (v < cd.wd) other |= e & ~Ps[v];
+                }
+                if (other) atomicOr(Ds + (kk >> 5), 1u << (kk & 31));
             }
             built = c;
             __syncthreads();
         }
-#define F2_CHECK(W)                                                   \
-    {                                                                 \
-        uint32_t P[W];                                                \
-        for (int v = 0; v < W; ++v) P[v] = Ps[v];                     \
-        check_chunk<W>(s, a, c, kb, ke, S, P, flags);                 \
-    }
+#define F2_CHECK(W) check_chunk<W>(s, a, c, kb, ke, S, Ps, Ds, flags)
         switch (cd.wd) {
         case 1: F2_CHECK(1); break;
         case 2: F2_CHECK(2); break;
@@ -1759,7 +1883,7 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
         const size_t csmem = CHECK_SMEM_BYTES;
         e = cudaFuncSetAttribute(check_snap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem);
         if (e != cudaSuccess) return f2_cuda_status(e);
-        f2_launch(check_snap_kernel, num_sms * 2, 256, csmem, cs, sd.num_ctx <= EARLY_MAX_CTX, sd, *check);
+        f2_launch(check_snap_kernel, num_sms * 3, 256, csmem, cs, sd.num_ctx <= EARLY_MAX_CTX, sd, *check);
         e = cudaGetLastError();
         if (e != cudaSuccess) return f2_cuda_status(e);
         LearnArgs lr = lx;
