@@ -331,8 +331,7 @@ enum f2_option {
                                     sends the rest back to elimination from there); only in calls of at
                                     least 16x this many rows; 0 = never. Unless this is set, calls of at
                                     least 2^20 rows on a store with contexts of 10..17 words hand off
-                                    the contexts that hold an eighth of an SM's share of the call's
-                                    work or more (at least 2048 representatives) */
+                                    the contexts with at least 2048 representatives left */
 };
 int f2_set_option(f2_store* store, int option, int64_t value);
 

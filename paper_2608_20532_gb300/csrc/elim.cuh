@@ -36,8 +36,6 @@ struct LearnArgs {
     // with at least handoff_min representatives left, stops and is listed
     // here: check_snap_kernel checks the rest against its basis in parallel
     int handoff_min;             // 0 = never
-    int handoff_share;           // with it: and at least this share (in 1/16) of the call's work per SM, 0 = no such rule
-    int num_sms;
     int* snap_count;
     int32_t* snap_list;
     int32_t* snap_start;         // its first representative left
@@ -626,21 +624,18 @@ __device__ __forceinline__ void decompress_residual(const uint32_t (&cr)[RW], co
 // instances of the wide kernel (the 10..17-word one takes part).
 constexpr int HANDOFF_QUIET = 2;
 constexpr int CHECK_BASIS_WORDS = 14336;  // 56 KB
-constexpr int CHECK_CHUNK = 512;
+constexpr int CHECK_CHUNK = 1024;
 constexpr int HANDOFF_CALL_FACTOR = 16;  // calls of fewer rows than this many hand-off minimums hand off none
 constexpr int WIDE_WD = 33;    // widest row (d <= 1056)
 constexpr int WIDE_M_WD = 17;  // rows of 10..17 words (d <= 544): half the registers, two CTAs per SM
 
-// The fewest representatives left for a context of width d to hand off.  The
+// The fewest representatives left for a context to hand off.  The
 // check needs the representatives' list, which a context that skipped the
 // duplicate pass of this call has not.
-__device__ __forceinline__ int handoff_least(const LearnArgs& a, int d, bool deduped)
+__device__ __forceinline__ int handoff_least(const LearnArgs& a, bool deduped)
 {
     if (a.handoff_min <= 0 || a.resume_from || deduped != (a.rep_count != nullptr)) return INT_MAX;
-    if (a.handoff_share <= 0) return a.handoff_min;
-    const unsigned long long work = *reinterpret_cast<const unsigned long long*>(a.counters + CNT_WORK);
-    const unsigned long long least = work * (unsigned long long)a.handoff_share / (16ull * (unsigned)a.num_sms * (unsigned)d);
-    return least > (unsigned long long)a.handoff_min ? (least < INT_MAX ? (int)least : INT_MAX) : a.handoff_min;
+    return a.handoff_min;
 }
 
 // What a group knows of its context while it streams the rows.
@@ -1080,7 +1075,7 @@ __device__ void elim_cta(const StoreDev& s, const LearnArgs& a, int c, uint32_t*
     st.base = a.resume_from ? a.resume_from[c] : 0;  // the first representative of this launch
     if constexpr (WD > WIDE_M_WD) st.base = a.open_from[c];
     st.quiet = st.parity = 0;
-    st.hand_min = handoff_least(a, cd.d, deduped);
+    st.hand_min = handoff_least(a, deduped);
     st.first = LLONG_MAX;
     st.cnt = 0;
     if (t == 0) {

@@ -62,8 +62,9 @@ namespace {
 // 10,000 contexts of 128..512 bits of parsed values, 13.4M rows: 443 us while
 // every CTA claimed its way through the whole list of contexts, an atomic each,
 // a row's words were loaded one by one and every basis row was XOR-ed whole;
-// now 190 (45% of the issue slots; warps wait at the barriers of a chunk and
-// for its rows).
+// 190 without that (45% of the issue slots; warps wait at the barriers of a
+// chunk and for its rows).  Two rows a lane made no difference, nor fewer
+// barriers a chunk.
 // ---------------------------------------------------------------------------
 struct CheckArgs {
     const int64_t* row_off;
@@ -1043,11 +1044,14 @@ __device__ void check_chunk(const StoreDev& s, const CheckArgs& a, int c, int kb
     const uint4* yc = a.y + r0;
     const uintptr_t bits = (uintptr_t)xc | (uintptr_t)(4 * cd.xw);
     const int al = (bits & 15) == 0 ? 2 : ((bits & 7) == 0 ? 1 : 0);
+    int next = kb + (int)threadIdx.x < ke ? (reps ? __ldg(reps + kb + threadIdx.x) : kb + (int)threadIdx.x) : 0;
     // every lane of a warp in each round: the pivot walk is warp-uniform
     for (int base = kb; base < ke; base += blockDim.x) {
         const int k = base + (int)threadIdx.x;
         const bool valid = k < ke;
-        const int i = valid ? (reps ? __ldg(reps + k) : k) : 0;
+        const int i = next;
+        const int kn = k + (int)blockDim.x;
+        next = kn < ke ? (reps ? __ldg(reps + kn) : kn) : 0;
         uint32_t xin[WD], q[WD];
         uint4 y = valid ? __ldg(yc + i) : make_uint4(0, 0, 0, 0);
         load_row_words<WD>(xc + (int64_t)i * cd.xw, al, valid, cd.n, cd.xw, xin);
@@ -1063,8 +1067,8 @@ __device__ void check_chunk(const StoreDev& s, const CheckArgs& a, int c, int kb
 // Shared memory of the check: the basis (a slot of row_stride words per
 // column), the chunk's classes (CHECK_CHUNK bytes), then CHECK_CTL_WORDS of
 // control (the pivot words, those whose rows have other columns too, the
-// claimed chunk, the chunk's sums).
-constexpr int CHECK_CTL_WORDS = 80;
+// claimed chunk, the chunk's sums, the pivots).
+constexpr int CHECK_CTL_WORDS = 64 + 16 * WIDE_M_WD;
 constexpr int CHECK_SMEM_BYTES = 4 * CHECK_BASIS_WORDS + CHECK_CHUNK + 4 * CHECK_CTL_WORDS;
 
 __global__ void __launch_bounds__(256, 3) check_snap_kernel(StoreDev s, CheckArgs a)
@@ -1076,6 +1080,7 @@ __global__ void __launch_bounds__(256, 3) check_snap_kernel(StoreDev s, CheckArg
     uint32_t* const ctl = smem + CHECK_BASIS_WORDS + CHECK_CHUNK / 4;
     uint32_t* const Ps = ctl;       // 24 pivot words (WIDE_M_WD at most)
     uint32_t* const Ds = ctl + 24;  // 24 words
+    uint16_t* const list = reinterpret_cast<uint16_t*>(ctl + 64);  // 32 * WIDE_M_WD columns at most
     int* const s_c = reinterpret_cast<int*>(ctl + 48);
     int* const s_k = s_c + 1;
     int* const s_first_out = s_c + 2;
@@ -1140,18 +1145,23 @@ __global__ void __launch_bounds__(256, 3) check_snap_kernel(StoreDev s, CheckArg
             __syncthreads();
             // the stride of the instance that checks it (rows of 10..17 words: the 17-word one)
             const int rs = row_stride(cd.wd <= NARROW_WD ? cd.wd : WIDE_M_WD);
-            for (int kk = t; kk < cd.d; kk += blockDim.x) {
-                if (!((Ps[kk >> 5] >> (kk & 31)) & 1u)) continue;
-                uint32_t* row = S + kk * rs;
-                *reinterpret_cast<uint4*>(row) = s.bz[cd.slot_off + kk];
-                const uint32_t* src = s.bx + cd.xw_off + (int64_t)kk * cd.wd;
-                uint32_t other = 0;
-                for (int v = 0; v < rs - 4; ++v) {
-                    const uint32_t e = (v < cd.wd) ? src[v] : 0u;
-                    row[4 + v] = e;
-                    if (v < cd.wd) other |= e & ~Ps[v];
-                }
-                if (other) atomicOr(Ds + (kk >> 5), 1u << (kk & 31));
+            int np = 0;  // the pivots in a list, then a thread a word of their rows
+            for (int v = 0; v < cd.wd; ++v) {
+                const uint32_t P = Ps[v];
+                const int b = t - (32 * v & 255);
+                if (b >= 0 && b < 32 && ((P >> b) & 1u)) list[np + __popc(P & ((1u << b) - 1u))] = (uint16_t)(32 * v + b);
+                np += __popc(P);
+            }
+            __syncthreads();
+            for (int r = t; r < np; r += blockDim.x)
+                *reinterpret_cast<uint4*>(S + list[r] * rs) = s.bz[cd.slot_off + list[r]];
+            const int per = rs - 4, all = np * per;
+#pragma unroll 4
+            for (int j = t; j < all; j += 256) {
+                const int r = j / per, v = j - r * per, kk = list[r];
+                const uint32_t e = v < cd.wd ? s.bx[cd.xw_off + (int64_t)kk * cd.wd + v] : 0u;
+                S[kk * rs + 4 + v] = e;
+                if (v < cd.wd && (e & ~Ps[v])) atomicOr(Ds + (kk >> 5), 1u << (kk & 31));
             }
             built = c;
             __syncthreads();
@@ -1759,15 +1769,14 @@ __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, F
 }
 
 // The default hand-off (see f2_learn_batched): calls of at least this many
-// rows, contexts with at least this many representatives left that are at
-// least HANDOFF_SHARE / 16 of an SM's share of the call's representatives x d.
-// On 10,000 contexts of parsed values (13.6M rows) the learn call took 1,515 us
-// without, 1,415 / 1,286 / 1,347 / 1,400 / 1,398 / 1,583 at 1 / 2 / 3 / 4 / 6 / 8.
-// Calls without rows of 10..17 words gain nothing: 4,096 contexts took 268 us
-// without and 293 or more with it, 77,926 contexts 2,379 and 2,467 or more.
+// rows on stores with rows of 10..17 words, contexts with at least this many
+// representatives left.  On 10,000 contexts of parsed values (13.4M rows) the
+// learn call takes 1,054 us; 1,060 from 1,024 representatives on, 1,066 where a
+// context must also hold a sixteenth of an SM's share of the call's work (1,102
+// with chunks of 512, where an eighth took 1,162).  Other stores gain nothing:
+// 4,096 contexts 262 us without, 278 with it, 77,926 contexts 2,510 and 2,579.
 constexpr int64_t HANDOFF_AUTO_ROWS = int64_t(1) << 20;
 constexpr int HANDOFF_AUTO_REPS = 2048;
-constexpr int HANDOFF_SHARE = 2;
 
 // Which elimination kernels a store needs, and their widest bases.
 
@@ -1987,9 +1996,7 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
     }
     const Widths& wv = st->widths;
     // Hand-off of saturated contexts, in calls long enough to have some.  By
-    // default only in calls with contexts of 10..17 words, whose rows cost
-    // most, and there for the few contexts that hold HANDOFF_SHARE / 16 of an
-    // SM's share of the call's work or more.
+    // default only in calls with contexts of 10..17 words, whose rows cost most.
     const bool auto_hand = st->handoff_min < 0 && dedup && wv.has_wide_m && total_rows >= HANDOFF_AUTO_ROWS;
     const int hand_min = auto_hand ? HANDOFF_AUTO_REPS
                          : (st->handoff_min > 0 && total_rows >= HANDOFF_CALL_FACTOR * st->handoff_min)
@@ -2137,8 +2144,6 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
     la.small_region_words = (int)(st->small_basis_bytes / 4);
     la.cta_region_words = 0;  // set per launch
     la.handoff_min = hand_min;
-    la.handoff_share = auto_hand ? HANDOFF_SHARE : 0;
-    la.num_sms = st->num_sms;
     la.snap_count = st->hand;
     la.snap_list = st->hand + 2;
     la.snap_start = st->hand + 2 + C;
@@ -2415,8 +2420,6 @@ extern "C" int f2_learn_batched_noalloc(int32_t num_ctx, const int32_t* n_bits_h
     la.small_region_words = DEFAULT_SMALL_REGION_BYTES / 4;
     la.cta_region_words = 0;
     la.handoff_min = 0;
-    la.handoff_share = 0;
-    la.num_sms = nd->num_sms;
     la.snap_count = nullptr;
     la.snap_list = nullptr;
     la.snap_start = nullptr;
