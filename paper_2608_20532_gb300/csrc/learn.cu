@@ -13,28 +13,36 @@
 //
 //  Pass 2 (elimination) streams the representatives of each context, in
 //  order, through a reduced basis B[k] = (r_k, z_k) held in shared memory:
-//   1. reduce: each lane reduces its row against the basis as it stood at
+//   1. open: an empty basis is filled from the first rows, a few a lane, each
+//      pivot applied to the group's rows at once, so that they stay reduced
+//      among themselves and no stored row is read (rows of more than 17 words:
+//      1,024 rows, a thread each, elim_open_kernel);
+//   2. reduce: each lane reduces its row against the basis as it stood at
 //      the start of the round (the snapshot).  The basis is reduced (RREF,
 //      the paper's step (5)), so the rows to XOR are exactly the pivots set
-//      in the row itself; the warp walks the union of those pivots and every
-//      lane XORs the broadcast row under its own bit;
-//   2. classify: a zero feature residual means the row lies in the span of
+//      in the row itself: the warp walks the union of those pivots and every
+//      lane XORs the broadcast row under its own bit, or, where it fits and
+//      pays, looks four columns at a time up in a table of the basis that is
+//      kept while the rows inserted since are few;
+//   3. classify: a zero feature residual means the row lies in the span of
 //      the snapshot, and the map T fixed by the snapshot never changes
 //      afterwards (contradicting rows are not inserted, insertions only
 //      extend it), so the classification equals the one-row-at-a-time one:
 //      zero word residual -> redundant, else contradiction (steps (2)-(3)).
 //      A contradicting representative counts once for itself and once per
 //      duplicate; its index is the first of them;
-//   3. insert: the remaining rows (candidates) are eliminated among
+//   4. insert: the remaining rows (candidates) are eliminated among
 //      themselves in stream order inside the warp (step (4)), then merged:
 //      new rows go to their pivot slots and every older row is cleared at
 //      the new pivot columns (step (5)).  The basis, including every z_k, is
 //      the sequential algorithm's.
 //
 // Both passes give one warp to small contexts (many per CTA) and a whole CTA
-// to large ones; contexts wider than 288 bits (d up to 1025) are eliminated
-// by a separate wide kernel.  Single-block plan kernels validate the CSR
-// batch and order the work longest-first.
+// to large ones.  Contexts of few rows go to the elimination without the first
+// pass.  The elimination is in elim.cuh, instantiated by width in
+// elim_small.cu (d <= 96), elim_narrow.cu (d <= 288) and elim_wide.cu (up to
+// d = 1025); the full-rank check on the tensor cores in verify_tc.cu.  Plan
+// kernels validate the CSR batch and order the work longest-first.
 #include <string.h>
 
 #include <mutex>
@@ -2046,7 +2054,7 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
     // Hand-off of saturated contexts, in calls long enough to have some.  By
     // default only in calls with contexts of 10..17 words, whose rows cost most.
     const bool auto_hand = st->handoff_min < 0 && dedup && wv.has_wide_m && total_rows >= HANDOFF_AUTO_ROWS;
-    const int hand_min = auto_hand ? HANDOFF_AUTO_REPS
+    int hand_min = auto_hand ? HANDOFF_AUTO_REPS
                          : (st->handoff_min > 0 && total_rows >= HANDOFF_CALL_FACTOR * st->handoff_min)
                              ? (int)st->handoff_min
                              : 0;
@@ -2058,9 +2066,14 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
             if (st->check_rec) cudaFreeAsync(st->check_rec, cs);
             st->check_rec = nullptr;
             st->check_rec_cap = 0;
-            if (f2_dev_alloc(st, (void**)&st->check_rec, 2 * sizeof(uint4) * (size_t)slots, cs, true) != cudaSuccess)
-                return F2_ERR_OOM;
-            st->check_rec_cap = slots;
+            if (f2_dev_alloc(st, (void**)&st->check_rec, 2 * sizeof(uint4) * (size_t)slots, cs, true) == cudaSuccess) {
+                st->check_rec_cap = slots;
+            } else {
+                st->check_rec = nullptr;
+                if (!auto_hand) return F2_ERR_OOM;
+                hand_min = 0;  // not asked for: the call goes without
+                (void)cudaGetLastError();
+            }
         }
     }
     F2FillList zl;

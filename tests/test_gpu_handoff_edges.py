@@ -9,7 +9,8 @@ import pytest
 import torch
 
 import oracle
-from gpu_util import assert_basis_equal, cuda_device, dev_arrays, lib
+from paper_2608_20532_gb300 import workloads
+from gpu_util import KEYS, as_bytes, assert_basis_equal, cuda_device, dev_arrays, gpu_learn_workload, lib
 
 pytestmark = pytest.mark.gpu
 
@@ -68,3 +69,26 @@ def test_check(shift, raw):
         assert st.device_status() == binding.F2_OK
         assert_basis_equal(binding, st.basis(), O.export())
         st.close()
+
+
+def test_default_without_memory():
+    """A call that would hand off by default goes without where the check's
+    records cannot be allocated: nothing that the caller did not ask for may
+    fail the call."""
+    dev = cuda_device()
+    binding = lib()
+    cfg = dict(num_ctx=16, layout=workloads.LAYOUT_UNIFORM_BITS, n_fixed=300, rows_fixed=66000, dup_frac=0.5,
+               density=0.05, n_contra=3)
+    wl = workloads.generate(cfg, 31)
+    assert wl.total_rows >= 1 << 20
+    got = []
+    for fail_at in (-1, 2):  # after the two lists of the duplicate pass
+        st = binding.Store(wl.n_bits, device=dev)
+        st.set_option(binding.F2_OPT_FAIL_ALLOC, fail_at)
+        gpu_learn_workload(binding, st, wl, dev)
+        torch.cuda.synchronize()
+        assert st.device_status() == binding.F2_OK
+        got.append({k: as_bytes(binding.to_numpy(v)).copy() for k, v in st.basis().items()})
+        st.close()
+    for k in KEYS:
+        assert np.array_equal(got[0][k], got[1][k]), k
