@@ -37,7 +37,6 @@ METRIC = "GF(2) rows eliminated/sec and words encoded/sec at 1 GB300; % HBM/INT 
 HBM_FALLBACK_GBS = 6800.0
 SMS = 152
 INT_LANES_PER_SM = 64      # 32-bit logic lanes per SM per clock (4 SMSPs x 16)
-SMEM_BYTES_PER_CLK = 128   # shared-memory bandwidth per SM per clock (32 banks x 4 bytes)
 SM_MAX_MHZ_FALLBACK = 2070.0
 
 
@@ -481,8 +480,8 @@ def run_ours(args):
 
     # ---- full-rank verification (config 5 after saturation): one more
     # incremental call on the saturated store, timed alone -- every row is a
-    # check y = T(phi(x)) by verify_full_kernel (ceil(d/4) 16-byte lookups a
-    # row from a table in shared memory; the plan kernels are the rest)
+    # check y = T(phi(x)) by verify_tc_kernel (the plan kernels and the empty
+    # launches of the others are the rest)
     verify = None
     if cfg_id == 5:
         ro1, xo1 = batches[1]
@@ -497,12 +496,8 @@ def run_ours(args):
         torch.cuda.synchronize()
         v_ms = v0.elapsed_time(v1) / K
         rows1 = int(wl.batches[1][0][-1] - wl.batches[1][0][0])
-        d = int(wl.n_bits.max()) + 1
-        lookups = rows1 * ((d + 3) // 4)
-        smem_bytes = lookups * 16
         verify = {"ms_per_call": v_ms, "rows_per_call": rows1, "rows_per_s": rows1 / (v_ms / 1e3),
-                  "lookups_per_row": (d + 3) // 4, "smem_bytes_per_call": smem_bytes,
-                  "kernel": "verify_full_kernel (+ plan kernels), one incremental call on full-rank contexts"}
+                  "kernel": "verify_tc_kernel (+ plan kernels), one incremental call on full-rank contexts"}
 
     # ---- encode epilogue (Appendix C/D): scheduler control merged at bit 105,
     # opaque-mask bits restored from recorded state; timed on its own, after
@@ -660,8 +655,8 @@ def run_ours(args):
     # learn roofline is HBM.  ops_learn is kept as the naive-method reference.
     learn_bound = "hbm"
     rl_learn = {
-        "kernel": "f2_learn_batched (fill, plan kernels, dedup_kernel, elim_narrow_kernel<true/false>, "
-                  "elim_wide_kernel, verify_full_kernel)",
+        "kernel": "f2_learn_batched (fill, plan kernels, dedup_kernel, elim_small_kernel, elim_narrow_kernel, "
+                  "elim_open_kernel, elim_wide_kernel, check_snap_kernel, verify_tc_kernel, verify_full_kernel)",
         "hbm": {"achieved": bytes_learn / learn_mean / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": (bytes_learn / learn_mean) / hbm_peak, "bytes_per_launch": bytes_learn},
         # The naive method's word-XOR count (every row reduced against the
@@ -717,14 +712,10 @@ def run_ours(args):
             "traffic": profile_traffic("f2_encode_batched"),
         }
     if verify is not None:
-        # the shared-memory pipe: 128 bytes a clock per SM (32 banks x 4 bytes)
-        smem_peak = SMS * SMEM_BYTES_PER_CLK * peaks["sm_max_mhz"] * 1e6
-        ach = verify["smem_bytes_per_call"] / (verify["ms_per_call"] / 1e3)
+        ach = verify["rows_per_call"] * (16 + 4 * int(wl.n_bits.max() // 32)) / (verify["ms_per_call"] / 1e3)
         result["roofline_verify"] = {
-            "bound": "smem", "achieved": ach / 1e9, "peak": smem_peak / 1e9, "unit": "GB/s (shared memory)",
-            "frac": ach / smem_peak, "peak_source": "derived: 152 SMs x 128 B/clock x max SM clock",
-            "hbm_frac": (verify["rows_per_call"] * (16 + 4 * int(wl.n_bits.max() // 32)) /
-                         (verify["ms_per_call"] / 1e3)) / (peaks["hbm_gbs"] * 1e9), **verify}
+            "bound": "hbm", "achieved": ach / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
+            "frac": ach / (peaks["hbm_gbs"] * 1e9), "peak_source": peaks["source"], **verify}
     if epilogue is not None:
         epilogue["frac_of_measured_hbm"] = epilogue["achieved_gbs"] / peaks["hbm_gbs"]
         result["encode_epilogue"] = epilogue
@@ -741,23 +732,32 @@ def run_ours(args):
 
 def launches_per_step(wl, has_q: bool) -> int:
     """Kernels one step enqueues (the host logic of the library): the reset's
-    fill; per learn call the fill of its counters, a plan (one kernel for at
-    most 8,192 contexts, else three) and dedup_kernel (a second instance when
-    some feature row has more than 9 words) for the duplicate pass, a plan,
-    the elimination kernel of each width class present (d <= 96, 96 < d <=
-    288, 288 < d <= 544, wider) and the full-rank check; solve_kernel; per
-    2^25 queries the encode's fill and its seven kernels (count, table,
-    build, scan, scatter, runs, short), or one kernel for a pass of at most
-    65,536 queries."""
+    fill; per learn call the fill of its counters (more than 8,192 contexts;
+    else its first plan clears them), a plan (one kernel for at most 8,192
+    contexts, else three) and dedup_kernel (a second instance when some feature
+    row has more than 9 words) for the duplicate pass, a plan, the elimination
+    kernel of each width class present (d <= 96, 96 < d <= 288, 288 < d <= 544,
+    wider: that one after elim_open_kernel), with rows of 10..17 words in a call
+    of at least 2^20 rows the hand-off check and the classes it can send back,
+    and the full-rank check (two kernels with 192 features or more and 2,048
+    rows); solve_kernel; per 2^25 queries the encode's fill and its seven kernels
+    (count, table, build, scan, scatter, runs, short), or one kernel for a pass
+    of at most 65,536 queries."""
     wd = (wl.n_bits.astype(np.int64) + 1 + 31) // 32
     xw = (wl.n_bits.astype(np.int64) + 31) // 32
-    plan = 1 if wl.num_ctx <= 8192 else 3
-    elim = (int((wd <= 3).any()) + int(((wd > 3) & (wd <= 9)).any()) + int(((wd > 9) & (wd <= 17)).any())
-            + int((wd > 17).any()))
-    learn = 1 + plan + 1 + int((xw > 9).any()) + plan + elim + 1
+    small = wl.num_ctx <= 8192
+    plan = 1 if small else 3
+    taken_up = int((wd <= 3).any()) + int(((wd > 3) & (wd <= 9)).any()) + int(((wd > 9) & (wd <= 17)).any())
+    learn = 0
+    for row_off, _ in wl.batches:
+        rows = int(row_off[-1]) - int(row_off[0])
+        learn += int(not small) + plan + 1 + int((xw > 9).any()) + plan + taken_up + 2 * int((wd > 17).any())
+        if rows >= 1 << 20 and ((wd > 9) & (wd <= 17)).any():
+            learn += 1 + taken_up
+        learn += 1 + int(wl.n_bits.max() >= 192 and rows >= 2048)
     nq = len(wl.queries.ctx_id) if has_q else 0
     enc = (1 if nq <= 65536 else 8 * ((nq + (1 << 25) - 1) >> 25)) if has_q else 0
-    return 1 + len(wl.batches) * learn + 1 + enc
+    return 1 + learn + 1 + enc
 
 
 def basis_bytes_touched(wl, store) -> int:
@@ -769,7 +769,8 @@ def basis_bytes_touched(wl, store) -> int:
 
 
 # the translation units of each library call's kernels
-KERNEL_SOURCES = {"f2_learn_batched": ("learn.cu", "f2_internal.cuh"),
+KERNEL_SOURCES = {"f2_learn_batched": ("learn.cu", "elim.cuh", "elim_small.cu", "elim_narrow.cu", "elim_wide.cu",
+                                       "full.cuh", "verify_tc.cu", "f2_internal.cuh"),
                   "f2_encode_batched": ("encode.cu", "f2_internal.cuh")}
 
 

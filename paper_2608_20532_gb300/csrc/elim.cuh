@@ -1209,7 +1209,7 @@ __device__ void elim_cta(const StoreDev& s, const LearnArgs& a, int c, uint32_t*
     if (t == 0) {
         s.rank[c] = st.rank;
         commit_stats(s, c, *first_s, *cnt_s);
-        if (snap_at >= 0) {  // rows_seen is advanced by check_snap_kernel (or resume_kernel)
+        if (snap_at >= 0) {  // rows_seen is advanced by check_snap_kernel (or the launch that resumes it)
             a.snap_start[c] = snap_at;
             a.snap_list[atomicAdd(a.snap_count, 1)] = c;
         } else if (stop_at < 0) {

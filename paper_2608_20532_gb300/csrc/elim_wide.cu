@@ -21,12 +21,14 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, WDT <= WIDE_M_WD ? 2 : 1) eli
 // (broadcast loads, only the words up to the pivot's).  The rows stay reduced
 // among themselves, so what remains is the reduced basis.  (One row a barrier
 // took 1,475 cycles a pivot, four take 1,310, of which the XORs alone 610: 38
-// integer instructions a warp at half rate.)  Streaming 256 rows at a time against a basis in shared
-// memory, the 1,025 pivots of a dense 1,024-bit context took 3,000 cycles
-// each, most of it in reading older rows a lane each.  Two batches of 65,536
-// rows for 64 such contexts went from 3,012 to 2,256 us.  Dense rows are a few pivots short of full
-// rank after d rows: up to OPEN_EXTRA further rows are reduced one at a time
-// by all threads (a XOR reduction of the rows their bits select).
+// integer instructions a warp at half rate; groups of 8, 16 and 32 rows were
+// no faster.)  Streaming 256 rows at a time against a basis in shared memory,
+// the 1,025 pivots of a dense 1,024-bit context took 3,000 cycles each, most of
+// it in reading older rows a lane each.  Two batches of 65,536 rows for 64 such
+// contexts went from 3,012 to 2,256 us, and to 2,180 with four rows a barrier.
+// Dense rows are a few pivots short of full rank after d rows: up to OPEN_EXTRA
+// further rows are reduced one at a time by all threads (a XOR reduction of the
+// rows their bits select).
 // ---------------------------------------------------------------------------
 constexpr int OPEN_THREADS = 1024;
 constexpr int OPEN_GROUP = 4;

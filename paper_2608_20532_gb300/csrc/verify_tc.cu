@@ -17,7 +17,7 @@
 // 0.54 with one mask a word and parities taken from sign bits.  The products
 // take 64 cycles each, 0.22 ms in all (tensor pipe 46% active).  Rows read by
 // their own threads, four words at a time 4 * xw bytes apart, cost two batches
-// of 32,768 rows a context 1,864 us; read a tile ahead, coalesced, and staged in
+// of 65,536 rows a context 1,864 us; read a tile ahead, coalesced, and staged in
 // shared memory, 1,830.
 #include "elim.cuh"
 #include "full.cuh"
