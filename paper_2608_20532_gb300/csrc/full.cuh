@@ -25,7 +25,7 @@ struct FullArgs {
 
 // A context with n features and T rows to check goes to the tensor cores: the
 // table check costs d/4 lookups of 16 bytes a row, 0.71 ms for 4.2M rows of
-// 1,024 features, the tensor cores 0.54 ms; spreading the map over a CTA's
+// 1,024 features, the tensor cores 0.49 ms; spreading the map over a CTA's
 // shared memory (128 bytes a feature) wants a few thousand rows to pay.
 constexpr int TC_MIN_N = 192;
 constexpr int TC_MIN_ROWS = 2048;
@@ -33,6 +33,66 @@ __host__ __device__ __forceinline__ bool full_by_tensor(int n, int64_t T) { retu
 
 cudaError_t verify_launch_tc(const StoreDev& sd, const FullArgs& fa, int num_sms, cudaStream_t cs);
 cudaError_t verify_load_tc();
+
+// The contexts to check: full at the start of the call, then full mid-call.
+struct FullList {
+    int nfull, begin, n;
+    __device__ __forceinline__ FullList(const FullArgs& a)
+        : nfull(a.counters[CNT_COUNT + CLS_FULL]), begin(a.counters[CNT_BEGIN + CLS_FULL]), n(nfull + *a.late_count)
+    {
+    }
+    __device__ __forceinline__ int ctx(const FullArgs& a, int q) const
+    {
+        return q < nfull ? a.queue[begin + q] : a.late_list[q - nfull];
+    }
+    __device__ __forceinline__ int64_t start(const FullArgs& a, int q, int c) const
+    {
+        return q < nfull ? 0 : (int64_t)a.late_start[c];
+    }
+};
+
+// A warp claims the next chunk k of a listed context: of the one at `stay` while
+// it has any, else of the first with chunks left, 32 looked at together, from
+// q0 round the list (`tried` of it are used up).  Returns its place in the list,
+// or -1.  (One thread that went from context to context, an atomic on each, took
+// most of the 29.6 us of the table kernel on 64 contexts that are all the other
+// kernel's, now 5.1, and 28 of the 513 us of that one on 4.2M rows.)
+__device__ __forceinline__ int full_claim(const StoreDev& s, const FullArgs& a, const FullList& l, bool tensor, int q0,
+                                          int stay, int& tried, int lane, int& k)
+{
+    auto rows_left = [&](int q, int& c) {
+        c = l.ctx(a, q);
+        return a.row_off[c + 1] - a.row_off[c] - l.start(a, q, c);
+    };
+    auto take = [&](int q) {
+        int c;
+        const int64_t T = rows_left(q, c);
+        if (lane == 0) k = atomicAdd(a.ctr + c, 1);
+        k = __shfl_sync(FULL, k, 0);
+        return (int64_t)k * FULL_CHUNK < T;
+    };
+    k = 0;
+    if (stay >= 0 && take(stay)) return stay;
+    while (tried < l.n) {
+        int at = -1;
+        if (tried + lane < l.n) {
+            at = q0 + tried + lane;
+            if (at >= l.n) at -= l.n;
+            int c;
+            const int64_t T = rows_left(at, c);
+            if ((a.tensor && full_by_tensor(s.desc[c].n, T)) != tensor || (int64_t)__ldcg(a.ctr + c) * FULL_CHUNK >= T)
+                at = -1;
+        }
+        const uint32_t left = __ballot_sync(FULL, at >= 0);
+        if (!left) {
+            tried += 32;
+            continue;
+        }
+        at = __shfl_sync(FULL, at, __ffs(left) - 1);
+        if (take(at)) return at;
+    }
+    return -1;
+}
 
 // A chunk of context c's rows is checked (one thread): cnt contradictions, the
 // first at `first`; the last chunk of the context commits its counts and

@@ -1671,35 +1671,26 @@ __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, F
     __shared__ int s_q, s_k;
     __shared__ unsigned long long s_cnt, s_first;
     const int t = threadIdx.x, lane = t & 31;
-    const int nfull = a.counters[CNT_COUNT + CLS_FULL];
-    const int qb = a.counters[CNT_BEGIN + CLS_FULL];
-    const int nq = nfull + *a.late_count;  // full at the start of the call, then full mid-call
-    auto ctx_of = [&](int qq) { return qq < nfull ? a.queue[qb + qq] : a.late_list[qq - nfull]; };
-    auto start_of = [&](int qq, int c) { return qq < nfull ? (int64_t)0 : (int64_t)a.late_start[c]; };
-    int q = 0, built = -1;
+    const FullList list(a);
+    const int q0 = (int)((long long)blockIdx.x * list.n / gridDim.x);
+    int q = -1, tried = 0, built = -1;
     for (;;) {
-        if (t == 0) {
-            int k = 0;
-            while (q < nq) {
-                const int c = ctx_of(q);
-                const int64_t T = a.row_off[c + 1] - a.row_off[c] - start_of(q, c);
-                if (!(a.tensor && full_by_tensor(s.desc[c].n, T))) {
-                    k = atomicAdd(a.ctr + c, 1);
-                    if ((int64_t)k * FULL_CHUNK < T) break;
-                }
-                ++q;
+        if (t < 32) {
+            int k;
+            const int qn = full_claim(s, a, list, false, q0, q, tried, lane, k);
+            if (t == 0) {
+                s_q = qn;
+                s_k = k;
+                s_cnt = 0ull;
+                s_first = ~0ull;
             }
-            s_q = q;
-            s_k = k;
-            s_cnt = 0ull;
-            s_first = ~0ull;
         }
         __syncthreads();
         q = s_q;
-        if (q >= nq) break;
+        if (q < 0) break;
         const int k = s_k;
-        const int c = ctx_of(q);
-        const int64_t i_first = start_of(q, c);
+        const int c = list.ctx(a, q);
+        const int64_t i_first = list.start(a, q, c);
         const CtxDesc cd = s.desc[c];
         const int np = (cd.d + 3) >> 2;
         const int nw = (np + 7) >> 3;  // words of q, eight groups each

@@ -18,7 +18,7 @@
 // take 64 cycles each, 0.22 ms in all (tensor pipe 46% active).  Rows read by
 // their own threads, four words at a time 4 * xw bytes apart, cost two batches
 // of 65,536 rows a context 1,864 us; read a tile ahead, coalesced, and staged in
-// shared memory, 1,830.
+// shared memory, 1,830.  The kernel now takes 0.49 ms.
 #include "elim.cuh"
 #include "full.cuh"
 
@@ -152,12 +152,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
     // group, the half of each row's features and sums that is this thread's, and
     // the quarter of the rows (a warp reaches 32 lanes of tensor memory)
     const int g = warp >> 3, half = (warp >> 2) & 1, wg = warp & 3;
-    const int nfull = a.counters[CNT_COUNT + CLS_FULL];
-    const int qb = a.counters[CNT_BEGIN + CLS_FULL];
-    const int nq = nfull + *a.late_count;
-    if (nq == 0) return;
-    auto ctx_of = [&](int qq) { return qq < nfull ? a.queue[qb + qq] : a.late_list[qq - nfull]; };
-    auto start_of = [&](int qq, int c) { return qq < nfull ? (int64_t)0 : (int64_t)a.late_start[c]; };
+    const FullList list(a);
+    if (list.n == 0) return;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&sm.tmem)),
                      "r"(TC_COLS)
@@ -176,31 +172,25 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
     const uint32_t lanes = (uint32_t)(32 * wg) << 16;
     const uint32_t a_addr = smem_addr(tc_smem);
     // CTAs start at different contexts and go round, so that each builds few maps
-    int q = (int)((long long)blockIdx.x * nq / gridDim.x), tried = 0, built = -1;
+    const int q0 = (int)((long long)blockIdx.x * list.n / gridDim.x);
+    int q = -1, tried = 0, built = -1;
     uint32_t uses = 0;  // chunks this group has issued
     for (;;) {
-        if (t == 0) {
-            int k = 0;
-            while (tried < nq) {
-                const int c = ctx_of(q);
-                const int64_t T = a.row_off[c + 1] - a.row_off[c] - start_of(q, c);
-                if (full_by_tensor(s.desc[c].n, T)) {
-                    k = atomicAdd(a.ctr + c, 1);
-                    if ((int64_t)k * FULL_CHUNK < T) break;
-                }
-                q = q + 1 < nq ? q + 1 : 0;
-                ++tried;
+        if (t < 32) {
+            int k;
+            const int qn = full_claim(s, a, list, true, q0, q, tried, lane, k);
+            if (t == 0) {
+                sm.q = qn;
+                sm.k = k;
+                sm.cnt = 0ull;
+                sm.first = ~0ull;
             }
-            sm.q = tried < nq ? q : -1;
-            sm.k = k;
-            sm.cnt = 0ull;
-            sm.first = ~0ull;
         }
         __syncthreads();
         q = sm.q;
         if (q < 0) break;
-        const int c = ctx_of(q);
-        const int64_t i_first = start_of(q, c);
+        const int c = list.ctx(a, q);
+        const int64_t i_first = list.start(a, q, c);
         const CtxDesc cd = s.desc[c];
         const int nch = (cd.n + TC_KC - 1) / TC_KC;
         if (built != c) {  // (every product of the last context is done: its sums were read)
