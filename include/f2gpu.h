@@ -322,7 +322,7 @@ enum f2_option {
                                     tables (one kernel launch); default 65536, 0 = never */
     F2_OPT_LONG_CALL_ROWS = 15,  /* f2_learn_batched calls of at least this many rows eliminate the contexts
                                     of 4..9 words in CTAs of four warps instead of eight (more contexts
-                                    side by side; the longest contexts take longer); default 0. A store
+                                    side by side; the longest contexts take longer); default 2^25. A store
                                     small enough for a CTA per context keeps eight */
     F2_OPT_HANDOFF_REPS = 16,    /* a context owned by a whole CTA whose rank has stopped growing hands
                                     the rest of its call off to a parallel check when at least this many

@@ -5,11 +5,13 @@ namespace f2 {
 namespace {
 
 // CTA-owned contexts first (longest first), then warp-owned ones, 16 warps per
-// SM at 128 registers, in CTAs of four warps: a CTA-owned context's insertions
-// run one warp at a time, so smaller groups waste less (eight against four:
-// 2,434 against 2,388 us on the 77,926-context learn, 269 against 261 on 4,096
-// contexts, 1,560 against 1,515 on 10,000 of parsed values).  A store small
-// enough for a CTA per context has the SMs to spare and takes eight.
+// SM at 128 registers.  A CTA-owned context's insertions run one warp at a time,
+// so CTAs of four warps waste less (2,388 against 2,434 us on the 77,926-context
+// learn), but a long context takes longer in them: calls of fewer than
+// DEFAULT_LONG_CALL_ROWS rows, which one such context can hold up, take eight.
+// 4,096 contexts with a few of 10,000 and more rows: 398 us with four, 307 with
+// eight; where no context stands out 265 and 268, 10,000 contexts of parsed
+// values 1,051 and 1,061.
 __global__ void __launch_bounds__(LEARN_WARPS * 32, 2) elim_narrow_kernel(StoreDev s, LearnArgs a)
 {
     pdl_wait();

@@ -80,7 +80,7 @@ constexpr int PLAN_BUCKETS = 48;     // log2(work) buckets for longest-first ord
 constexpr int DEFAULT_WARP_REGION_BYTES = 13824;  // shared memory of one warp-owned context
 constexpr int DEFAULT_SMALL_REGION_BYTES = 9472;  // the same in the small-width kernel (d <= 96)
 constexpr int64_t DEFAULT_ENCODE_DIRECT_MAX = 65536;  // encode passes this small skip the grouping
-constexpr int64_t DEFAULT_LONG_CALL_ROWS = 0;  // learn calls this long: 4-warp CTAs (4..9 words)
+constexpr int64_t DEFAULT_LONG_CALL_ROWS = int64_t(1) << 25;  // learn calls this long: 4-warp CTAs (4..9 words)
 constexpr int64_t DEFAULT_HANDOFF_REPS = -1;  // representatives left for a saturated context to hand off (0: never, -1: by the call's work)
 constexpr int DEFAULT_HEAVY_ROWS = 4096;          // rows from which a context gets a whole CTA (at most)
 constexpr int HEAVY_ROWS_MIN = 1024;              // ... and at least, when it scales with the batch:
