@@ -86,6 +86,17 @@ __device__ __forceinline__ void tc_commit(unsigned long long* bar)
                  : "memory");
 }
 
+// Waits, with a limit, for the products that complete the phase of `bar`;
+// false if they did not.  The lanes leave the wait at different times and the
+// tensor-memory instructions after it take a whole warp, so they vote first;
+// the fence orders those instructions after the products.
+__device__ __forceinline__ bool tc_wait(unsigned long long* bar, uint32_t parity)
+{
+    const bool ok = __all_sync(FULL, mbar_wait_bounded(bar, parity)) != 0;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    return ok;
+}
+
 __device__ __forceinline__ void tc_store32(uint32_t addr, const uint32_t (&v)[32])
 {
     asm volatile(
@@ -175,6 +186,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
     const int q0 = (int)((long long)blockIdx.x * list.n / gridDim.x);
     int q = -1, tried = 0, built = -1;
     uint32_t uses = 0;  // chunks this group has issued
+    bool in_time = true;  // no wait of this warp has given up
     for (;;) {
         if (t < 32) {
             int k;
@@ -273,7 +285,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
                 const uint32_t x[TC_KW] = {xv.x, xv.y, xv.z, xv.w};
                 const int buf = (int)(uses & 1u);
                 const uint32_t use = uses >> 1;
-                if (use > 0 && !sm.failed && !mbar_wait_bounded(&sm.bar[g][buf], (use - 1) & 1u)) sm.failed = 1;
+                if (use > 0 && in_time && !tc_wait(&sm.bar[g][buf], (use - 1) & 1u)) in_time = false;
                 const uint32_t at = base + TC_N + (uint32_t)(buf * (TC_KC / 4));
                 uint32_t e[32];
 #pragma unroll
@@ -299,8 +311,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
             }
             // the tile's sums
             const uint32_t last = uses - 1;
-            if (!sm.failed && !mbar_wait_bounded(&sm.bar[g][last & 1u], (last >> 1) & 1u)) sm.failed = 1;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (in_time && !tc_wait(&sm.bar[g][last & 1u], (last >> 1) & 1u)) in_time = false;
+            if (!in_time) sm.failed = 1;
             uint32_t bad = 0;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -342,7 +354,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
     }
     // (done already, unless a wait gave up)
     for (uint32_t u = uses < 2 ? 0 : uses - 2; u < uses; ++u)
-        (void)mbar_wait_bounded(&sm.bar[g][u & 1u], (u >> 1) & 1u);
+        (void)tc_wait(&sm.bar[g][u & 1u], (u >> 1) & 1u);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
