@@ -62,7 +62,9 @@ enum f2_status {
     F2_ERR_ALIGN = 4,       /* a pointer misses its required alignment */
     F2_ERR_OOM = 5,         /* device or host allocation failed */
     F2_ERR_CUDA = 6,        /* a CUDA runtime call failed */
-    F2_ERR_TIMEOUT = 7,     /* (device) a bounded device-side wait gave up */
+    F2_ERR_TIMEOUT = 7,     /* (device) a bounded device-side wait gave up: the queries it was for are
+                               not written; a full-rank context whose rows it was for keeps its
+                               contradiction records and its row count as they were */
     F2_ERR_ROWS = 8,        /* (device) CSR offsets of a context are decreasing or out of bounds;
                                that context's rows were skipped */
     F2_ERR_STRIDE = 9       /* (device) a query's context needs more words than x_stride_words */
@@ -331,6 +333,9 @@ enum f2_option {
                                     least 16x this many rows; 0 = never. Unless this is set, calls of at
                                     least 2^20 rows on a store with contexts of 10..17 words hand off
                                     the contexts with at least 2048 representatives left */
+    F2_OPT_FAIL_WAIT = 17,       /* test hook: 1: the waits of f2_learn_batched's tensor-core full-rank check
+                                    (192 features and more) act as if they had given up
+                                    (F2_ERR_TIMEOUT); 0 (default): off */
 };
 int f2_set_option(f2_store* store, int option, int64_t value);
 

@@ -44,6 +44,7 @@ F2_OPT_DEDUP_SHARDS = 13
 F2_OPT_ENCODE_DIRECT_MAX = 14
 F2_OPT_LONG_CALL_ROWS = 15
 F2_OPT_HANDOFF_REPS = 16
+F2_OPT_FAIL_WAIT = 17
 
 # every entry point of include/f2gpu.h
 EXPORTS = (

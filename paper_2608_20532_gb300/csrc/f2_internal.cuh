@@ -470,6 +470,7 @@ struct f2_store {
     // test hook (F2_OPT_FAIL_ALLOC): device allocations left before one is
     // made to fail; -1 = off
     mutable int64_t fail_alloc_in;
+    int fail_wait;          // test hook (F2_OPT_FAIL_WAIT)
     // diagnostics (F2_OPT_TIMING): per-context timestamps of the last learn call
     int timing_on;
     unsigned long long* timing;

@@ -21,6 +21,7 @@ struct FullArgs {
     unsigned long long* first;        // [C] first contradicting row of the call (all ones: none)
     int table_words;                  // FULL_TABLE_WORDS
     int tensor;                       // contexts of full_by_tensor are left to verify_tc_kernel
+    int fail_wait;                    // test hook: verify_tc_kernel's waits for sums give up
 };
 
 // A context with n features and T rows to check goes to the tensor cores: the
@@ -96,11 +97,17 @@ __device__ __forceinline__ int full_claim(const StoreDev& s, const FullArgs& a, 
 
 // A chunk of context c's rows is checked (one thread): cnt contradictions, the
 // first at `first`; the last chunk of the context commits its counts and
-// advances rows_seen.
+// advances rows_seen.  Where a chunk's check failed (a wait gave up) its counts
+// are unknown, so nothing of the context is committed: the mark is a bit that
+// no count reaches.
+constexpr unsigned long long FULL_FAILED = 1ull << 63;
+
 __device__ __forceinline__ void full_commit(const StoreDev& s, const FullArgs& a, int c, int64_t i_first, int64_t T,
-                                            unsigned long long cnt, unsigned long long first)
+                                            unsigned long long cnt, unsigned long long first, bool failed)
 {
-    if (cnt) {
+    if (failed) {
+        atomicOr(a.cnt + c, FULL_FAILED);
+    } else if (cnt) {
         atomicAdd(a.cnt + c, cnt);
         atomicMin(a.first + c, first);
     }
@@ -109,6 +116,7 @@ __device__ __forceinline__ void full_commit(const StoreDev& s, const FullArgs& a
     if (atomicAdd(a.ctr + s.num_ctx + c, 1) != nch - 1) return;
     __threadfence();
     const unsigned long long tot = atomicAdd(a.cnt + c, 0ull);
+    if (tot & FULL_FAILED) return;
     const unsigned long long fi = atomicMin(a.first + c, ~0ull);
     const long long seen = s.rows_seen[c];
     if (tot) {

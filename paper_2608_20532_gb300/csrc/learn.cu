@@ -1810,7 +1810,7 @@ __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, F
             atomicMin(&s_first, first);
         }
         __syncthreads();
-        if (t == 0) full_commit(s, a, c, i_first, T, s_cnt, s_first);
+        if (t == 0) full_commit(s, a, c, i_first, T, s_cnt, s_first, false);
         __syncthreads();
     }
 }
@@ -1865,7 +1865,7 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
                        const Widths& wv, int* full_ctr, unsigned long long* full_cnt,
                        unsigned long long* full_first, cudaStream_t cs, Fork* fk = nullptr, int scale = 0,
                        bool prezeroed = false, int64_t long_rows = LONG_CALL_ROWS, const CheckArgs* check = nullptr,
-                       const PlanZero& zero = PlanZero{})
+                       const PlanZero& zero = PlanZero{}, int fail_wait = 0)
 {
     // prezeroed: the caller has cleared full_ctr's first 2C words and late
     // count, full_cnt, full_first (to -1) and hist
@@ -1966,6 +1966,7 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
         fa.cnt = full_cnt;
         fa.first = full_first;
         fa.table_words = FULL_TABLE_WORDS;
+        fa.fail_wait = fail_wait;
         fa.tensor = wv.max_n >= TC_MIN_N && total_rows >= TC_MIN_ROWS;
         if (fa.tensor) {
             e = verify_launch_tc(sd, fa, num_sms, cs);
@@ -2222,7 +2223,7 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
     return launch_elimination(sd, la, row_off, x_off, total_rows, total_x_words, dedup ? st->rep_count : nullptr,
                               heavy, st->warp_work, st->queue, st->keybuf, st->plan_hist + PLAN_HIST_WORDS,
                               st->num_sms, wv, st->full_ctr, st->full_cnt, st->full_first, cs, &fk, scale, true,
-                              all_cta ? INT64_MAX : st->long_call_rows, &ca, zero);
+                              all_cta ? INT64_MAX : st->long_call_rows, &ca, zero, st->fail_wait);
 }
 
 extern "C" int f2_learn_timing(const f2_store* st, uint64_t* out_host, f2_stream_t stream)

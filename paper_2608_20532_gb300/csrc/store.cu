@@ -559,6 +559,10 @@ extern "C" int f2_set_option(f2_store* s, int option, int64_t value)
         if (value < -1) return F2_ERR_INVALID_ARG;
         s->fail_alloc_in = value;
         return F2_OK;
+    case F2_OPT_FAIL_WAIT:
+        if (value != 0 && value != 1) return F2_ERR_INVALID_ARG;
+        s->fail_wait = (int)value;
+        return F2_OK;
     case F2_OPT_ELIM_TABLES:
         if (value != 0 && value != 1) return F2_ERR_INVALID_ARG;
         s->elim_tables = (int)value;

@@ -58,7 +58,6 @@ constexpr int TC_GROUP_COLS = 256;
 struct TcSmem {
     unsigned long long bar[2][2];  // [group][buffer]: the products of a buffer are done
     uint32_t tmem;
-    int failed;
     int q, k;
     uint32_t bad[2][4];            // [group][quarter]: rows that the second threads found contradicting
     unsigned long long cnt, first;
@@ -123,6 +122,21 @@ __device__ __forceinline__ void tc_load32(uint32_t addr, uint32_t (&v)[32])
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// Barrier of a group (named barrier 1 + g): whether any of its threads says so.
+__device__ __forceinline__ bool tc_any(int g, bool p)
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "barrier.cta.red.or.pred q, %2, 256, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"((uint32_t)p), "r"(1 + g)
+        : "memory");
+    return r != 0u;
+}
+
 // A (column j of the map = the word of feature j) as bytes; features from n to
 // kp are zero.
 __device__ void tc_build(const StoreDev& s, const CtxDesc& cd, uint8_t* A, int kp, int t)
@@ -174,7 +188,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
     if (t == 0) {
         for (int i = 0; i < 4; ++i) mbar_init(&sm.bar[i >> 1][i & 1], 1);
         mbar_init_fence();
-        sm.failed = 0;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -186,7 +199,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
     const int q0 = (int)((long long)blockIdx.x * list.n / gridDim.x);
     int q = -1, tried = 0, built = -1;
     uint32_t uses = 0;  // chunks this group has issued
-    bool in_time = true;  // no wait of this warp has given up
     for (;;) {
         if (t < 32) {
             int k;
@@ -270,7 +282,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
         };
         int64_t tile = i0 + (int64_t)g * TC_TILE;
         if (tile < i1) fetch(tile);
-        for (; tile < i1; tile += 2 * TC_TILE) {
+        // A wait that gives up ends the group's work (the group agrees on it at
+        // its next barrier): the sums are unknown and the buffers in use.
+        bool gone = false;
+        for (; tile < i1 && !gone; tile += 2 * TC_TILE) {
             const int64_t i = tile + 32 * wg + lane;
             const bool valid = i < i1;
             // (the group is done with the last tile's rows: its sums were compared)
@@ -279,13 +294,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
             if (tile + 2 * TC_TILE < i1) fetch(tile + 2 * TC_TILE);
             const uint4 y = __ldg(a.y + r0 + (valid ? i : tile));
             const uint32_t* const xr = stage + (32 * wg + lane) * rw;
-            for (int ch = 0; ch < nch; ++ch, ++uses) {
+            for (int ch = 0; ch < nch && !gone; ++ch) {
                 const int w0 = (2 * ch + half) * TC_KW;
                 const uint4 xv = w0 < xw ? *reinterpret_cast<const uint4*>(xr + w0) : make_uint4(0, 0, 0, 0);
                 const uint32_t x[TC_KW] = {xv.x, xv.y, xv.z, xv.w};
                 const int buf = (int)(uses & 1u);
                 const uint32_t use = uses >> 1;
-                if (use > 0 && in_time && !tc_wait(&sm.bar[g][buf], (use - 1) & 1u)) in_time = false;
+                const bool ok = use == 0 || tc_wait(&sm.bar[g][buf], (use - 1) & 1u);
                 const uint32_t at = base + TC_N + (uint32_t)(buf * (TC_KC / 4));
                 uint32_t e[32];
 #pragma unroll
@@ -295,10 +310,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
                     for (int w = 0; w < 8; ++w)
                         e[8 * v + w] = (w < 3 ? up : (w < 7 ? x[v] : down)) & (0x01010101u << tc_bit(w));
                 }
-                tc_store32(at + lanes + (uint32_t)(32 * half), e);
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                if (ok) {
+                    tc_store32(at + lanes + (uint32_t)(32 * half), e);
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                }
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory");
+                gone = tc_any(g, !ok);
+                if (gone) break;
                 if ((warp & 7) == 0 && lane == 0) {
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
@@ -308,14 +326,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
                     tc_commit(&sm.bar[g][buf]);
                 }
                 __syncwarp();
+                ++uses;
             }
+            if (gone) break;
             // the tile's sums
             const uint32_t last = uses - 1;
-            if (in_time && !tc_wait(&sm.bar[g][last & 1u], (last >> 1) & 1u)) in_time = false;
-            if (!in_time) sm.failed = 1;
+            const bool ok = !a.fail_wait && tc_wait(&sm.bar[g][last & 1u], (last >> 1) & 1u);
             uint32_t bad = 0;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            for (int h = 0; h < 2 && ok; ++h) {
                 uint32_t v[32];
                 tc_load32(base + lanes + (uint32_t)(64 * half + 32 * h), v);
                 uint32_t word = 0;
@@ -328,8 +347,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
                 const uint32_t m = __ballot_sync(FULL, bad != 0u);
                 if (lane == 0) sm.bad[g][wg] = m;
             }
-            asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory");
-            if (!half && valid && (bad || ((sm.bad[g][wg] >> lane) & 1u))) {
+            gone = tc_any(g, !ok);
+            if (!half && !gone && valid && (bad || ((sm.bad[g][wg] >> lane) & 1u))) {
                 ++cnt;
                 if ((unsigned long long)i < first) first = (unsigned long long)i;
             }
@@ -345,14 +364,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
             atomicAdd(&sm.cnt, cnt);
             atomicMin(&sm.first, first);
         }
-        __syncthreads();
+        const bool failed = __syncthreads_or(gone) != 0;
         if (t == 0) {
-            if (sm.failed) record_status(s.status, F2_ERR_TIMEOUT);
-            full_commit(s, a, c, i_first, T, sm.cnt, sm.first);
+            if (failed) record_status(s.status, F2_ERR_TIMEOUT);
+            full_commit(s, a, c, i_first, T, sm.cnt, sm.first, failed);
         }
         __syncthreads();
+        if (failed) break;  // other CTAs take what is left
     }
-    // (done already, unless a wait gave up)
+    // the products still in flight (none, unless a wait gave up)
     for (uint32_t u = uses < 2 ? 0 : uses - 2; u < uses; ++u)
         (void)tc_wait(&sm.bar[g][u & 1u], (u >> 1) & 1u);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

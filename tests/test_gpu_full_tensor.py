@@ -63,3 +63,50 @@ def test_full_rank_by_tensor(raw, shift):
         assert_basis_equal(binding, st.basis(), O.export())
     assert int((st.basis()["rank"].cpu().numpy() == np.array(n_bits) + (0 if raw else 1)).sum()) >= len(n_bits) - 2
     st.close()
+
+
+@pytest.mark.parametrize("raw", [False, True])
+def test_a_wait_that_gives_up_commits_nothing(raw):
+    """A call whose check gives up reports it and leaves the contradiction
+    records and row counts of the contexts it was checking as they were (the
+    narrow context, checked by the table kernel, is counted); the next call
+    goes on from there."""
+    dev = cuda_device()
+    binding = lib()
+    rng = np.random.default_rng(15)
+    n_bits = [192, 257, 1024, 40]
+    wide = np.array(n_bits) >= 192
+    maps = [(rng.integers(0, 2, (n, 128)).astype(np.float32), 0 if raw else rng.integers(0, 2, 128)) for n in n_bits]
+    st = binding.Store(np.array(n_bits, np.int32), raw=raw, device=dev)
+    O = oracle.Oracle(np.array(n_bits, np.int32), raw=raw)
+
+    def learn(counts, flips, learner):
+        ro, xo, x, y = _batch(rng, n_bits, counts, maps, flips, 0)
+        ro_t, x_t, xo_t, y_t = dev_arrays(binding, dev, ro, x, xo, y)
+        st.learn(ro_t, x_t, xo_t, y_t)
+        torch.cuda.synchronize()
+        if learner is not None:
+            learner.learn(ro, xo, x, y)
+
+    def state():
+        return {k: binding.to_numpy(v).copy() for k, v in st.basis().items()}
+
+    learn([n + 80 for n in n_bits], [(), (330,), (), ()], O)  # one recorded already
+    before = state()
+    assert (before["rank"] == np.array(n_bits) + (0 if raw else 1)).all()
+    st.set_option(binding.F2_OPT_FAIL_WAIT, 1)
+    learn([4300, 2048, 9000, 3000], [(0, 2100)] * 4, None)
+    assert st.device_status() == binding.F2_ERR_TIMEOUT
+    after = state()
+    for k in ("contra", "first_contra", "n_contra", "rows_seen"):
+        assert np.array_equal(after[k][wide], before[k][wide]), k
+        assert (after[k][~wide] != before[k][~wide]).all(), k
+    for k in ("rank", "pivot_mask", "basis_x", "basis_z"):
+        assert np.array_equal(after[k], before[k]), k
+    st.set_option(binding.F2_OPT_FAIL_WAIT, 0)
+    learn([4300, 2048, 9000, 0], [(7, 4000)] * 4, O)
+    assert st.device_status() == binding.F2_OK
+    ref, got = O.export(), state()
+    for k in ("rank", "contra", "first_contra", "n_contra", "rows_seen"):
+        assert np.array_equal(got[k][wide].astype(np.int64), ref[k][wide].astype(np.int64)), k
+    st.close()
