@@ -120,17 +120,17 @@ __device__ __forceinline__ uint64_t mixed_words(const uint32_t (&P)[WD], int d, 
 
 // Feature words exactly as supplied (bits >= n cleared), and the word.
 template <int WD>
-__device__ __forceinline__ void load_raw(const uint32_t* __restrict__ xrow, const uint4* __restrict__ yrow,
+__device__ __forceinline__ void load_raw(const uint32_t* xrow, const uint4* yrow,
                                          bool valid, int n, int xw, uint32_t (&xin)[WD], uint4& y)
 {
 #pragma unroll
     for (int v = 0; v < WD; ++v) {
         uint32_t t = 0;
-        if (valid && v < xw) t = __ldg(xrow + v);
+        if (valid && v < xw) t = ld(xrow + v);
         if (v == xw - 1 && (n & 31)) t &= (1u << (n & 31)) - 1u;
         xin[v] = t;
     }
-    y = valid ? __ldg(yrow) : make_uint4(0, 0, 0, 0);
+    y = valid ? ld(yrow) : make_uint4(0, 0, 0, 0);
 }
 
 // q = [1 || x] (index 0 = constant) or x itself for raw feature rows.
@@ -184,8 +184,8 @@ template <int WD>
 __device__ __forceinline__ void fetch_row(const RowStream& rs, int k, Row<WD>& r)
 {
     r.valid = k < rs.R;
-    r.i = r.valid ? (rs.reps ? __ldg(rs.reps + k) : k) : 0;
-    r.weight = 1u + ((r.valid && rs.dups) ? (uint32_t)__ldg(rs.dups + k) : 0u);
+    r.i = r.valid ? (rs.reps ? ld(rs.reps + k) : k) : 0;
+    r.weight = 1u + ((r.valid && rs.dups) ? (uint32_t)ld(rs.dups + k) : 0u);
     load_raw<WD>(rs.xc + (int64_t)r.i * rs.xw, rs.yc + r.i, r.valid, rs.n, rs.xw, r.x, r.y);
 }
 
@@ -905,8 +905,8 @@ __device__ __forceinline__ void open_basis(const RowStream& rs, ElimState<WD>& s
         }
         const int kr = 32 * t + lane;
         if (kr < rs.R && pk[0] < 0 && nonzero4(yr[0])) {  // in the span of the rows before it
-            st.cnt += 1u + (rs.dups ? (uint32_t)__ldg(rs.dups + kr) : 0u);
-            st.first = min(st.first, rs.seen + (rs.reps ? __ldg(rs.reps + kr) : kr));
+            st.cnt += 1u + (rs.dups ? (uint32_t)ld(rs.dups + kr) : 0u);
+            st.first = min(st.first, rs.seen + (rs.reps ? ld(rs.reps + kr) : kr));
         }
         // slot 1 becomes slot 0, slot 0 the last
         uint32_t x0[WD];

@@ -166,13 +166,13 @@ __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, 
             __syncthreads();
             uint4* const arow = sm.row[0][0];
             uint32_t* const acc = reinterpret_cast<uint32_t*>(arow);
-            const int i = rs.reps ? __ldg(rs.reps + base) : base;
+            const int i = rs.reps ? ld(rs.reps + base) : base;
             if (warp == 0) {
                 const uint32_t* xr = rs.xc + (int64_t)i * rs.xw;
                 for (int w = lane; w < WIDE_WD + 3; w += 32) {
                     auto word = [&](int v) {
                         if (v < 0 || v >= rs.xw) return 0u;
-                        uint32_t u = __ldg(xr + v);
+                        uint32_t u = ld(xr + v);
                         if (v == rs.xw - 1 && (rs.n & 31)) u &= (1u << (rs.n & 31)) - 1u;
                         return u;
                     };
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, 
                     sm.q[w] = q;
                 }
                 if (lane == 0) {
-                    arow[OPEN_Z] = __ldg(rs.yc + i);
+                    arow[OPEN_Z] = ld(rs.yc + i);
                     sm.holder = OPEN_THREADS;
                 }
             }
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, 
             const uint4 z = arow[OPEN_Z];
             if (k < 0) {
                 if (t == 0 && nonzero4(z)) {
-                    sm.cnt += 1u + (rs.dups ? (uint32_t)__ldg(rs.dups + base) : 0u);
+                    sm.cnt += 1u + (rs.dups ? (uint32_t)ld(rs.dups + base) : 0u);
                     if (rs.seen + (long long)i < sm.first) sm.first = rs.seen + (long long)i;
                 }
                 continue;

@@ -34,20 +34,22 @@ constexpr unsigned FULL = 0xffffffffu;
 // 4,096 contexts 418..444 -> 319 us, 4,096 contexts 275 -> 263, 64 contexts of
 // 1,024 bits 1,830 -> 1,781.  Calls of long kernels gain nothing (77,926 contexts
 // 2,516 us with it, 2,501 without; 10M queries 916 and 831), so stores of more than
-// EARLY_MAX_CTX contexts and the encoder do without.  The pointers that a kernel
-// loads from through the read-only path are passed through the wait, so that no
-// such load can be moved above it.
-template <typename P>
-__device__ __forceinline__ void through_wait(P& p)
-{
-    asm volatile("" : "+l"(p)::"memory");
-}
-template <typename... P>
-__device__ __forceinline__ void pdl_wait(P&... p)
+// EARLY_MAX_CTX contexts and the encoder do without.
+__device__ __forceinline__ void pdl_wait()
 {
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    (through_wait(p), ...);
+}
+
+// A kernel's load from global memory.  A chain of early kernels can all be set
+// up while the first of them, or a kernel of the caller's before it, still
+// writes what the last one reads, and the read-only path (__ldg, or const
+// __restrict__ parameters of a kernel) promises that nothing writes the data
+// while the kernel is there: kernels that begin with pdl_wait() load with this.
+template <typename T>
+__device__ __forceinline__ T ld(const T* p)
+{
+    return *p;
 }
 
 constexpr int EARLY_MAX_CTX = 8192;

@@ -55,11 +55,11 @@ struct HostIO {
 
 namespace {
 
-__global__ void __launch_bounds__(256) rebase_kernel(const int64_t* __restrict__ ro, const int64_t* __restrict__ xo,
+__global__ void __launch_bounds__(256) rebase_kernel(const int64_t* ro, const int64_t* xo,
                                                      int32_t c0, int32_t c1, int32_t C, int64_t xa,
-                                                     int64_t* __restrict__ row_off, int64_t* __restrict__ x_off)
+                                                     int64_t* row_off, int64_t* x_off)
 {
-    pdl_wait(ro, xo);
+    pdl_wait();
     // contexts outside [c0, c1) get no rows; offsets of the chunk's contexts
     // count from the chunk's first row and first feature word
     const int64_t r0 = ro[0];

@@ -198,15 +198,15 @@ static_assert(DD_WARPS * DD_WARP_REGION * 4 <= DD_SMEM, "warp regions exceed the
 __device__ __forceinline__ uint32_t last_mask(int n) { return (n & 31) ? ((1u << (n & 31)) - 1u) : 0xffffffffu; }
 
 // Full comparison of rows i and j of a context (feature bits < n and word).
-__device__ __forceinline__ bool rows_equal(const uint32_t* __restrict__ xc, const uint4* __restrict__ yc, int xw, int n,
+__device__ __forceinline__ bool rows_equal(const uint32_t* xc, const uint4* yc, int xw, int n,
                                            int64_t i, const uint4& yi, int64_t j)
 {
-    const uint4 yj = __ldg(yc + j);
+    const uint4 yj = ld(yc + j);
     if (yj.x != yi.x || yj.y != yi.y || yj.z != yi.z || yj.w != yi.w) return false;
     const uint32_t lm = last_mask(n);
     for (int v = 0; v < xw; ++v) {
         const uint32_t m = (v == xw - 1) ? lm : 0xffffffffu;
-        if (((__ldg(xc + i * xw + v) ^ __ldg(xc + j * xw + v)) & m) != 0u) return false;
+        if (((ld(xc + i * xw + v) ^ ld(xc + j * xw + v)) & m) != 0u) return false;
     }
     return true;
 }
@@ -216,7 +216,7 @@ __device__ __forceinline__ bool rows_equal(const uint32_t* __restrict__ xc, cons
 // index of that content), or -1 when the probe budget runs out (the row then
 // counts as its own representative, which is always exact).
 __device__ __noinline__ int dd_find_insert(uint2* tab, int E, uint32_t h, int64_t i, const uint4& yi,
-                                           const uint32_t* __restrict__ xc, const uint4* __restrict__ yc, int xw,
+                                           const uint32_t* xc, const uint4* yc, int xw,
                                            int n, uint32_t slot, int budget)
 {
     const uint32_t fp = h | 1u;
@@ -240,12 +240,12 @@ __device__ __noinline__ int dd_find_insert(uint2* tab, int E, uint32_t h, int64_
 // Feature words of a row: the widest loads that every row of the context
 // allows (`al`: log2 of the words its rows are aligned to).
 template <int XW>
-__device__ __forceinline__ void load_words(const uint32_t* __restrict__ p, int al, uint32_t (&x)[XW])
+__device__ __forceinline__ void load_words(const uint32_t* p, int al, uint32_t (&x)[XW])
 {
     if (XW % 4 == 0 && al >= 2) {
 #pragma unroll
         for (int v = 0; v + 3 < XW; v += 4) {
-            const uint4 t = __ldg(reinterpret_cast<const uint4*>(p + v));
+            const uint4 t = ld(reinterpret_cast<const uint4*>(p + v));
             x[v] = t.x;
             x[v + 1] = t.y;
             x[v + 2] = t.z;
@@ -254,13 +254,13 @@ __device__ __forceinline__ void load_words(const uint32_t* __restrict__ p, int a
     } else if (XW % 2 == 0 && al >= 1) {
 #pragma unroll
         for (int v = 0; v + 1 < XW; v += 2) {
-            const uint2 t = __ldg(reinterpret_cast<const uint2*>(p + v));
+            const uint2 t = ld(reinterpret_cast<const uint2*>(p + v));
             x[v] = t.x;
             x[v + 1] = t.y;
         }
     } else {
 #pragma unroll
-        for (int v = 0; v < XW; ++v) x[v] = __ldg(p + v);
+        for (int v = 0; v < XW; ++v) x[v] = ld(p + v);
     }
 }
 
@@ -421,7 +421,7 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
         for (int j = 0; j < K; ++j) {
             const int i = base + j * NT + t;
             const int ic = i < T ? i : T - 1;  // (a row read twice, not counted)
-            yn[j] = __ldg(yc + ic);
+            yn[j] = ld(yc + ic);
             load_words<XW>(xc + (int64_t)ic * XW, al, xn[j]);
         }
     };
@@ -491,7 +491,7 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
 #pragma unroll
             for (int v = 0; v < XW; ++v) xo[j][v] = 0u;
             if (need[j]) {
-                yo[j] = __ldg(yc + o);
+                yo[j] = ld(yc + o);
                 load_words<XW>(xc + o * XW, al, xo[j]);
             }
         }
@@ -639,7 +639,7 @@ __device__ __forceinline__ DdSmem dd_layout(int region, int region_words, int T,
 // Row (x, y) equals the row numbered r, whose smallest index so far is i0.
 template <int XW>
 __device__ __forceinline__ bool dd_same(const DdSmem& m, int r, const uint32_t (&x)[XW], const uint4& y,
-                                        const uint32_t* __restrict__ xc, const uint4* __restrict__ yc, uint32_t lm)
+                                        const uint32_t* xc, const uint4* yc, uint32_t lm)
 {
     uint4 o;
     uint32_t diff = 0;
@@ -649,10 +649,10 @@ __device__ __forceinline__ bool dd_same(const DdSmem& m, int r, const uint32_t (
         for (int v = 0; v < XW; ++v) diff |= dd_smem()[m.xs + r * XW + v] ^ x[v];
     } else {
         const int64_t j = (int64_t)*reinterpret_cast<const volatile uint32_t*>(dd_smem() + m.idx + r);
-        o = __ldg(yc + j);
+        o = ld(yc + j);
 #pragma unroll
         for (int v = 0; v < XW; ++v) {
-            const uint32_t w = __ldg(xc + j * XW + v);
+            const uint32_t w = ld(xc + j * XW + v);
             diff |= (v == XW - 1 ? w & lm : w) ^ x[v];
         }
     }
@@ -665,7 +665,7 @@ __device__ __forceinline__ bool dd_same(const DdSmem& m, int r, const uint32_t (
 // another, so the warps hide each other's latencies; the first rows are put in
 // order at the end, through a bitmap.
 template <int G, int XW>
-__device__ int dedup_rows(const uint32_t* __restrict__ xc, const uint4* __restrict__ yc, int T, int off, uint32_t lm,
+__device__ int dedup_rows(const uint32_t* xc, const uint4* yc, int T, int off, uint32_t lm,
                           int al, const DdSmem& m, int32_t* __restrict__ rep, int32_t* __restrict__ dups, int* wcnt)
 {
     constexpr int NT = 32 * G;
@@ -679,7 +679,7 @@ __device__ int dedup_rows(const uint32_t* __restrict__ xc, const uint4* __restri
     for (int base = 0; base < T; base += NT) {
         const int i = base + t;
         const int ic = i < T ? i : T - 1;  // (a row read twice, not counted)
-        const uint4 y = __ldg(yc + ic);
+        const uint4 y = ld(yc + ic);
         uint32_t x[XW];
         load_words<XW>(xc + (int64_t)ic * XW, al, x);
         x[XW - 1] &= lm;
@@ -953,7 +953,7 @@ __device__ __forceinline__ int64_t check_slot(const CheckArgs& a, int c)
 // Feature words of a row of up to WD words (bits >= n cleared), by the widest
 // loads that every row of the context allows (`al` as in load_words).
 template <int WD>
-__device__ __forceinline__ void load_row_words(const uint32_t* __restrict__ p, int al, bool valid, int n, int xw,
+__device__ __forceinline__ void load_row_words(const uint32_t* p, int al, bool valid, int n, int xw,
                                                uint32_t (&x)[WD])
 {
 #pragma unroll
@@ -963,7 +963,7 @@ __device__ __forceinline__ void load_row_words(const uint32_t* __restrict__ p, i
 #pragma unroll
             for (int v = 0; v + 3 < WD; v += 4)
                 if (v < xw) {
-                    const uint4 t = __ldg(reinterpret_cast<const uint4*>(p + v));
+                    const uint4 t = ld(reinterpret_cast<const uint4*>(p + v));
                     x[v] = t.x;
                     x[v + 1] = t.y;
                     x[v + 2] = t.z;
@@ -973,14 +973,14 @@ __device__ __forceinline__ void load_row_words(const uint32_t* __restrict__ p, i
 #pragma unroll
             for (int v = 0; v + 1 < WD; v += 2)
                 if (v < xw) {
-                    const uint2 t = __ldg(reinterpret_cast<const uint2*>(p + v));
+                    const uint2 t = ld(reinterpret_cast<const uint2*>(p + v));
                     x[v] = t.x;
                     x[v + 1] = t.y;
                 }
         } else {
 #pragma unroll
             for (int v = 0; v < WD; ++v)
-                if (v < xw) x[v] = __ldg(p + v);
+                if (v < xw) x[v] = ld(p + v);
         }
     }
     const uint32_t last = (n & 31) ? (1u << (n & 31)) - 1u : FULL;
@@ -1052,16 +1052,16 @@ __device__ void check_chunk(const StoreDev& s, const CheckArgs& a, int c, int kb
     const uint4* yc = a.y + r0;
     const uintptr_t bits = (uintptr_t)xc | (uintptr_t)(4 * cd.xw);
     const int al = (bits & 15) == 0 ? 2 : ((bits & 7) == 0 ? 1 : 0);
-    int next = kb + (int)threadIdx.x < ke ? (reps ? __ldg(reps + kb + threadIdx.x) : kb + (int)threadIdx.x) : 0;
+    int next = kb + (int)threadIdx.x < ke ? (reps ? ld(reps + kb + threadIdx.x) : kb + (int)threadIdx.x) : 0;
     // every lane of a warp in each round: the pivot walk is warp-uniform
     for (int base = kb; base < ke; base += blockDim.x) {
         const int k = base + (int)threadIdx.x;
         const bool valid = k < ke;
         const int i = next;
         const int kn = k + (int)blockDim.x;
-        next = kn < ke ? (reps ? __ldg(reps + kn) : kn) : 0;
+        next = kn < ke ? (reps ? ld(reps + kn) : kn) : 0;
         uint32_t xin[WD], q[WD];
-        uint4 y = valid ? __ldg(yc + i) : make_uint4(0, 0, 0, 0);
+        uint4 y = valid ? ld(yc + i) : make_uint4(0, 0, 0, 0);
         load_row_words<WD>(xc + (int64_t)i * cd.xw, al, valid, cd.n, cd.xw, xin);
         make_q<WD>(xin, valid, s.raw, q);
         check_words<WD, 0>(q, y, S, Ps, Ds);
@@ -1200,8 +1200,8 @@ __global__ void __launch_bounds__(256, 3) check_snap_kernel(StoreDev s, CheckArg
         for (int j = t; j < ke - kb && kb + j < fo; j += blockDim.x) {
             if (flags[j] != 1) continue;
             const int k = kb + j;
-            const int i = a.rep_list ? __ldg(a.rep_list + a.row_off[c] + k) : k;
-            cnt += 1u + (a.rep_dup ? (uint32_t)__ldg(a.rep_dup + a.row_off[c] + k) : 0u);
+            const int i = a.rep_list ? ld(a.rep_list + a.row_off[c] + k) : k;
+            cnt += 1u + (a.rep_dup ? (uint32_t)ld(a.rep_dup + a.row_off[c] + k) : 0u);
             first = min(first, (long long)i);
         }
         if (cnt) {
@@ -1698,7 +1698,7 @@ __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, F
         uint2* Zh = Zl + FULL_ZH_BYTES / 8;
         if (built != c) {
             for (int j = t; j < 4 * np; j += FULL_THREADS) {
-                const uint4 z = (j < cd.d) ? __ldg(s.bz + cd.slot_off + j) : make_uint4(0, 0, 0, 0);
+                const uint4 z = (j < cd.d) ? ld(s.bz + cd.slot_off + j) : make_uint4(0, 0, 0, 0);
                 const int e = (j >> 2) * 16 + (1 << (j & 3));
                 Zl[e] = make_uint2(z.x, z.y);
                 Zh[e] = make_uint2(z.z, z.w);
@@ -1751,7 +1751,7 @@ __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, F
                 int r = t / xw, v = t - (t / xw) * xw;
                 const int dr = FULL_THREADS / xw, dv = FULL_THREADS - dr * xw;
                 for (int w = t; w < nb * xw; w += FULL_THREADS) {
-                    stage[r * sst + v] = __ldg(src + w);
+                    stage[r * sst + v] = ld(src + w);
                     r += dr;
                     v += dv;
                     if (v >= xw) {
@@ -1763,7 +1763,7 @@ __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, F
             __syncthreads();
             if (t < nb) {
                 const int64_t i = b0 + t;
-                const uint4 yi = __ldg(a.y + r0 + i);
+                const uint4 yi = ld(a.y + r0 + i);
                 const uint32_t* xr = stage + t * sst;
                 uint32_t a0 = 0, a1 = 0, a2 = 0, a3 = 0, prev = 0;
                 const char* const zt = reinterpret_cast<const char*>(tabw);
@@ -2276,10 +2276,10 @@ std::mutex g_noalloc_mu;
 
 // Context descriptors and canonical offsets (exclusive prefix sums of d,
 // d*wd and wd) for up to F2_NOALLOC_MAX_CTX contexts, one block.
-__global__ void __launch_bounds__(1024) noalloc_desc_kernel(const int32_t* __restrict__ n_bits, int C, uint32_t raw,
-                                                            CtxDesc* __restrict__ desc)
+__global__ void __launch_bounds__(1024) noalloc_desc_kernel(const int32_t* n_bits, int C, uint32_t raw,
+                                                            CtxDesc* desc)
 {
-    pdl_wait(n_bits);
+    pdl_wait();
     constexpr int PER = (F2_NOALLOC_MAX_CTX + 1023) / 1024;
     __shared__ long long wsum[3][32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;

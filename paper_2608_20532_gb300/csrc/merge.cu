@@ -18,11 +18,11 @@ namespace {
 
 // One warp per source context: lane over slots; the i-th pivot row of
 // context c becomes row member_row[c] + i of the merge batch.
-__global__ void __launch_bounds__(256) merge_gather_kernel(StoreDev s, const int64_t* __restrict__ member_row,
-                                                           const int64_t* __restrict__ member_word,
-                                                           uint32_t* __restrict__ x, uint4* __restrict__ y)
+__global__ void __launch_bounds__(256) merge_gather_kernel(StoreDev s, const int64_t* member_row,
+                                                           const int64_t* member_word,
+                                                           uint32_t* x, uint4* y)
 {
-    pdl_wait(member_row, member_word);
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
     for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < s.num_ctx; c += warps) {
@@ -32,14 +32,14 @@ __global__ void __launch_bounds__(256) merge_gather_kernel(StoreDev s, const int
         const uint32_t* P = s.pivot + cd.pw_off;
         int below = 0;  // pivots in the words before the current one
         for (int w = 0; w < cd.wd; ++w) {
-            const uint32_t pw = __ldg(P + w);
+            const uint32_t pw = ld(P + w);
             const int k = 32 * w + lane;
             if ((pw >> lane) & 1u) {
                 const int i = below + __popc(pw & ((1u << lane) - 1u));
-                y[r0 + i] = __ldg(s.bz + cd.slot_off + k);
+                y[r0 + i] = ld(s.bz + cd.slot_off + k);
                 const uint32_t* src = s.bx + cd.xw_off + (int64_t)k * cd.wd;
                 uint32_t* dst = x + member_word[c] + (int64_t)i * cd.wd;
-                for (int v = 0; v < cd.wd; ++v) dst[v] = __ldg(src + v);
+                for (int v = 0; v < cd.wd; ++v) dst[v] = ld(src + v);
             }
             below += __popc(pw);
         }

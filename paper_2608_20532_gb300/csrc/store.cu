@@ -375,7 +375,7 @@ extern "C" int f2_get_basis(const f2_store* s, int32_t* rank, uint32_t* pivot_ma
 // W[c][j] = z_j for a pivot j, 0 otherwise (the learned map T of Sec. 2.3
 // extended by zero on the free coordinates).  One warp per context, lanes
 // over slots: coalesced 16-byte stores.
-__global__ void __launch_bounds__(256) solve_kernel(StoreDev s, uint4* __restrict__ W)
+__global__ void __launch_bounds__(256) solve_kernel(StoreDev s, uint4* W)
 {
     pdl_wait();
     const int lane = threadIdx.x & 31;
@@ -384,8 +384,8 @@ __global__ void __launch_bounds__(256) solve_kernel(StoreDev s, uint4* __restric
         const CtxDesc cd = s.desc[c];
         const uint32_t* P = s.pivot + cd.pw_off;
         for (int j = lane; j < cd.d; j += 32) {
-            const bool piv = (__ldg(P + (j >> 5)) >> (j & 31)) & 1u;
-            W[cd.slot_off + j] = piv ? __ldg(s.bz + cd.slot_off + j) : make_uint4(0, 0, 0, 0);
+            const bool piv = (ld(P + (j >> 5)) >> (j & 31)) & 1u;
+            W[cd.slot_off + j] = piv ? ld(s.bz + cd.slot_off + j) : make_uint4(0, 0, 0, 0);
         }
     }
 }

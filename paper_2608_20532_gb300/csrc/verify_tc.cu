@@ -149,7 +149,7 @@ __device__ void tc_build(const StoreDev& s, const CtxDesc& cd, uint8_t* A, int k
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int f = (k & ~31) + 8 * j + w8;
-            z[j] = f < cd.n ? __ldg(s.bz + cd.slot_off + first + f) : make_uint4(0, 0, 0, 0);
+            z[j] = f < cd.n ? ld(s.bz + cd.slot_off + first + f) : make_uint4(0, 0, 0, 0);
         }
         uint8_t* const col = A + (k >> 4) * TC_LBO + (k & 15);
 #pragma unroll
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
         const uint32_t* const xc = a.x + a.x_off[c];
         const int xw = cd.xw;
         const bool vec = ((uintptr_t)xc & 15) == 0 && (xw & 3) == 0;
-        const uint4 b = s.raw ? make_uint4(0, 0, 0, 0) : __ldg(s.bz + cd.slot_off);
+        const uint4 b = s.raw ? make_uint4(0, 0, 0, 0) : ld(s.bz + cd.slot_off);
         unsigned long long cnt = 0ull, first = ~0ull;
         // A tile's rows are contiguous: the group loads the next one into
         // registers, coalesced, while it works on this one from shared memory.
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
                 for (int u = 0; u < TC_ST / 4; ++u) {
                     const int k = tg + 256 * u;
                     if (4 * k < rows * xw) {
-                        const uint4 v = __ldg(reinterpret_cast<const uint4*>(src) + k);
+                        const uint4 v = ld(reinterpret_cast<const uint4*>(src) + k);
                         st[4 * u] = v.x;
                         st[4 * u + 1] = v.y;
                         st[4 * u + 2] = v.z;
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
 #pragma unroll
                 for (int u = 0; u < TC_ST; ++u) {
                     const int k = tg + 256 * u;
-                    if (k < rows * xw) st[u] = __ldg(src + k);
+                    if (k < rows * xw) st[u] = ld(src + k);
                 }
             }
         };
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) verify_tc_kernel(StoreDev s, Fu
             put();
             asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory");
             if (tile + 2 * TC_TILE < i1) fetch(tile + 2 * TC_TILE);
-            const uint4 y = __ldg(a.y + r0 + (valid ? i : tile));
+            const uint4 y = ld(a.y + r0 + (valid ? i : tile));
             const uint32_t* const xr = stage + (32 * wg + lane) * rw;
             for (int ch = 0; ch < nch && !gone; ++ch) {
                 const int w0 = (2 * ch + half) * TC_KW;

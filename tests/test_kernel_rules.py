@@ -36,3 +36,17 @@ def test_tensor_memory_follows_a_warp_wide_wait():
     kernel = _function(text, "verify_tc_kernel")
     for use in ("tc_store32(", "tc_load32("):
         assert 0 <= kernel.find("tc_wait(") < kernel.find(use)
+
+
+def test_early_kernels_load_coherently():
+    """A kernel that begins with pdl_wait() may be set up while kernels before
+    it still write what it reads, so neither it nor the device code it shares
+    uses the read-only path."""
+    files = [f for f in sorted(os.listdir(CSRC)) if f.endswith((".cu", ".cuh"))]
+    early = [f for f in files if re.search(r"\bpdl_wait\(", _source(f)) or f in ("elim.cuh", "full.cuh")]
+    assert {"learn.cu", "store.cu", "merge.cu", "host_io.cu", "verify_tc.cu", "elim_wide.cu"} <= set(early)
+    for f in early:
+        text = _source(f)
+        assert not re.search(r"__ldg\(|ld\.global\.nc", text), f
+        for kernel in re.finditer(r"__global__[^{;]*?\w+\(([^{;]*)\)\s*\{", text):
+            assert "__restrict__" not in kernel.group(1), (f, kernel.group(1))
