@@ -181,9 +181,10 @@ struct Row {
 };
 
 template <int WD>
-__device__ __forceinline__ void fetch_row(const RowStream& rs, int k, Row<WD>& r)
+__device__ __forceinline__ void fetch_row(const RowStream& rs, int base, int j, Row<WD>& r)
 {
-    r.valid = k < rs.R;
+    const int k = (int)((uint32_t)base + (uint32_t)j);
+    r.valid = item_in(base, j, rs.R);
     r.i = r.valid ? (rs.reps ? ld(rs.reps + k) : k) : 0;
     r.weight = 1u + ((r.valid && rs.dups) ? (uint32_t)ld(rs.dups + k) : 0u);
     load_raw<WD>(rs.xc + (int64_t)r.i * rs.xw, rs.yc + r.i, r.valid, rs.n, rs.xw, r.x, r.y);
@@ -693,7 +694,7 @@ __device__ int table_rounds(const LearnArgs& a, const RowStream& rs, ElimState<W
     for (int u = 0; u < RW; ++u) NP[u] = 0u;
     int n_new = 0, spent = 0, snap_at = -1;
     Row<WD> nx;
-    fetch_row<WD>(rs, st.base + 32 * warp + lane, nx);
+    fetch_row<WD>(rs, st.base, 32 * warp + lane, nx);
     while (st.base < rs.R) {
         const bool valid = nx.valid;
         uint32_t q[WD], cr[RW];
@@ -701,7 +702,7 @@ __device__ int table_rounds(const LearnArgs& a, const RowStream& rs, ElimState<W
         const long long idx = rs.seen + nx.i;
         const uint32_t weight = nx.weight;
         make_q<WD>(nx.x, valid, rs.raw, q);
-        fetch_row<WD>(rs, st.base + nt + 32 * warp + lane, nx);  // the next round's row, in flight
+        fetch_row<WD>(rs, st.base, nt + 32 * warp + lane, nx);  // the next round's row, in flight
         table_reduce<RW, WD>(TB, np, q, acc, cr);
         xor4(yr[0], acc);
         if (n_new) {
@@ -795,7 +796,7 @@ __device__ int table_rounds(const LearnArgs& a, const RowStream& rs, ElimState<W
                 for (int u = 0; u < RW; ++u) NP[u] |= N1[u];
             }
         }
-        st.base += nt;
+        st.base = step_to(st.base, nt, rs.R);
         if constexpr (CTA) {
             st.quiet = inserted ? 0 : st.quiet + 1;
             if (st.quiet >= HANDOFF_QUIET && rs.R - st.base >= st.hand_min && st.rank + n_new < d && d * RS <= CHECK_BASIS_WORDS) {
@@ -877,13 +878,12 @@ __device__ __forceinline__ void open_basis(const RowStream& rs, ElimState<WD>& s
     uint32_t xr[K][WD];
     uint4 yr[K];
     int pk[K];
-    const int rounds = (rs.R + 31) >> 5;
-    const int n_live = rounds < K ? rounds : K;
+    const int n_live = rs.R > 32 * (K - 1) ? K : (rs.R + 31) >> 5;
     uint32_t live = (1u << n_live) - 1u;
 #pragma unroll
     for (int t = 0; t < K; ++t) {
         Row<WD> r;
-        fetch_row<WD>(rs, 32 * t + lane, r);
+        fetch_row<WD>(rs, 0, 32 * t + lane, r);
         make_q<WD>(r.x, r.valid, rs.raw, xr[t]);
         yr[t] = r.y;
         pk[t] = -1;
@@ -931,7 +931,7 @@ __device__ __forceinline__ void open_basis(const RowStream& rs, ElimState<WD>& s
     for (int t = 0; t < K; ++t)
         if (pk[t] >= 0) store_row<WD>(S + pk[t] * RS, xr[t], yr[t]);
     __syncwarp();
-    st.base = 32 * n_live;
+    st.base = step_to(0, 32 * n_live, rs.R);
 }
 
 // A round of 32 rows by one warp against the basis itself: walk, insert the
@@ -942,7 +942,7 @@ __device__ __forceinline__ void walk_round(const RowStream& rs, ElimState<WD>& s
     constexpr int RS = row_stride(WD);
     uint32_t xr[1][WD];
     Row<WD> r;
-    fetch_row<WD>(rs, st.base + lane, r);
+    fetch_row<WD>(rs, st.base, lane, r);
     uint4 yr[1] = {r.y};
     const long long idx = rs.seen + r.i;
     make_q<WD>(r.x, r.valid, rs.raw, xr[0]);
@@ -966,7 +966,7 @@ __device__ __forceinline__ void walk_round(const RowStream& rs, ElimState<WD>& s
 #pragma unroll
         for (int v = 0; v < WD; ++v) st.P[v] |= NP[v];
     }
-    st.base += 32;
+    st.base = step_to(st.base, 32, rs.R);
 }
 
 __device__ __forceinline__ RowStream row_stream(const StoreDev& s, const LearnArgs& a, const CtxDesc& cd, int c,
@@ -975,9 +975,9 @@ __device__ __forceinline__ RowStream row_stream(const StoreDev& s, const LearnAr
     RowStream rs;
     const int64_t r0 = a.row_off[c];
     const int T = (int)(a.row_off[c + 1] - r0);
-    const int rc = a.rep_count ? a.rep_count[c] : -(T + 2);
+    const int rc = a.rep_count ? a.rep_count[c] : all_rows(T);
     deduped = rc >= 0;
-    rs.R = deduped ? rc : -(rc + 2);
+    rs.R = deduped ? rc : rows_of(rc);
     rs.reps = deduped ? a.rep_list + r0 : nullptr;
     rs.dups = deduped ? a.rep_dup + r0 : nullptr;
     rs.xc = a.x + a.x_off[c];
@@ -1026,7 +1026,7 @@ __device__ void elim_warp(const StoreDev& s, const LearnArgs& a, int c, uint32_t
         // from the rounds left where the saving covers the build.
         const int rw = table_planes(cd.d - st.rank);
         if (a.tables && rw <= WARP_TABLE_RW && table_room(cd.d, rw) <= tab_cap &&
-            ((left + 31) >> 5) * (14 * st.rank - 8 * np) > 40 * np) {
+            (((int64_t)left + 31) >> 5) * (14 * st.rank - 8 * np) > 40 * np) {
             (void)table_phase<WD, 1, false>(a, rs, st, S, TB, FL, cd.d, cd.wd, nullptr, nullptr);
         } else {
             walk_round<WD>(rs, st, S, cd.d, cd.wd, lane);
@@ -1094,7 +1094,7 @@ __device__ void elim_cta(const StoreDev& s, const LearnArgs& a, int c, uint32_t*
     const int tab_cap = region_words - FL_WORDS - CTL_WORDS - cd.d * RS;
     const int np = (cd.d + 3) >> 2;
     Row<WD> nx;
-    fetch_row<WD>(rs, st.base + t, nx);
+    fetch_row<WD>(rs, st.base, t, nx);
     int snap_at = -1;  // handed off from this representative on
     while (st.base < rs.R && stop_at < 0) {
         if constexpr (WD <= TABLE_MAX_WD) {
@@ -1107,7 +1107,7 @@ __device__ void elim_cta(const StoreDev& s, const LearnArgs& a, int c, uint32_t*
                 else snap_at = table_phase<WD, 4, true>(a, rs, st, S, TB, FL, cd.d, cd.wd, wc, NPR);
                 if (snap_at >= 0) break;
                 mixed = mixed_words<WD>(st.P, cd.d, cd.wd);
-                fetch_row<WD>(rs, st.base + t, nx);
+                fetch_row<WD>(rs, st.base, t, nx);
                 continue;
             }
         }
@@ -1117,7 +1117,7 @@ __device__ void elim_cta(const StoreDev& s, const LearnArgs& a, int c, uint32_t*
         const long long idx = rs.seen + nx.i;
         const uint32_t weight = nx.weight;
         make_q<WD>(nx.x, valid, rs.raw, xr[0]);
-        fetch_row<WD>(rs, st.base + nt + t, nx);
+        fetch_row<WD>(rs, st.base, nt + t, nx);
         if (st.rank) reduce_rows<WD, 1>(xr, yr, S, st.P, mixed);
         uint32_t nz = 0;
 #pragma unroll
@@ -1131,7 +1131,7 @@ __device__ void elim_cta(const StoreDev& s, const LearnArgs& a, int c, uint32_t*
         }
         uint32_t cand = __ballot_sync(FULL, valid && nz != 0u);
         uint32_t wmask = publish_candidates(cand, wc, st.parity, warp, lane, G);
-        st.base += nt;
+        st.base = step_to(st.base, nt, rs.R);
         st.quiet = wmask ? 0 : st.quiet + 1;
         // the first warp with candidates inserts them; then every warp clears
         // its share of the older rows (step (5)) and reduces its own

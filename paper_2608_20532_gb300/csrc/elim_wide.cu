@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, 
         const RowStream rs = row_stream(s, a, cd, c, deduped);
         const int n = rs.R < OPEN_THREADS ? rs.R : OPEN_THREADS;
         Row<WIDE_WD> r;
-        fetch_row<WIDE_WD>(rs, t, r);
+        fetch_row<WIDE_WD>(rs, 0, t, r);
         uint32_t x[WIDE_WD];
         make_q<WIDE_WD>(r.x, r.valid, rs.raw, x);
         uint4 y = r.y;

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "f2gpu.h"
+#include "ranges.cuh"
 
 namespace f2 {
 

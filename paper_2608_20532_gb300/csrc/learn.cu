@@ -397,6 +397,7 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
     const int lo = (int)(((long long)Tc * shard) / nsh);
     const int64_t r0 = a.row_off[c] + lo;  // this shard's rows, and its part of rep_list / rep_dup
     const int T = (int)(((long long)Tc * (shard + 1)) / nsh) - lo;
+    const uint32_t Tu = (uint32_t)T;  // (rows past the last are counted unsigned: T may be 2^31 - 1)
     const uint32_t* xc = a.x + a.x_off[c] + (int64_t)lo * XW;
     const uint4* yc = a.y + r0;
     const uint32_t lm = last_mask(n);
@@ -416,17 +417,17 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
     constexpr int K = DD_K;
     uint4 yn[K];
     uint32_t xn[K][XW];
-    auto load_round = [&](int base) {
+    auto load_round = [&](uint32_t base) {
 #pragma unroll
         for (int j = 0; j < K; ++j) {
-            const int i = base + j * NT + t;
-            const int ic = i < T ? i : T - 1;  // (a row read twice, not counted)
+            const uint32_t i = base + (uint32_t)(j * NT + t);
+            const int ic = i < Tu ? (int)i : T - 1;  // (a row read twice, not counted)
             yn[j] = ld(yc + ic);
             load_words<XW>(xc + (int64_t)ic * XW, al, xn[j]);
         }
     };
     if (AHEAD) load_round(0);
-    for (int base = 0; base < T; base += NT * K) {
+    for (uint32_t base = 0; base < Tu; base += NT * K) {
         int mine[K];
         uint32_t h[K];
         uint4 yv[K];
@@ -449,18 +450,18 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
         uint32_t cs[K];
 #pragma unroll
         for (int j = 0; j < K; ++j) {
-            const int i = base + j * NT + t;
-            mine[j] = (i < T) ? -2 : -1;  // -2 = unresolved
+            const uint32_t i = base + (uint32_t)(j * NT + t);
+            mine[j] = (i < Tu) ? -2 : -1;  // -2 = unresolved
             ent[j] = make_uint2(0u, 0u);
             cs[j] = 0u;
-            if (i < T) {
+            if (i < Tu) {
                 const uint32_t fp = h[j] | 1u;
                 uint32_t slot = (h[j] >> 7) & emask;
                 int p = 0;
                 for (; p < DEDUP_PROBES; ++p, slot = (slot + 1) & emask) {
                     uint2 e = tab[slot];
                     if (e.x == 0u) {
-                        const unsigned long long want = ((unsigned long long)(uint32_t)i << 32) | fp;
+                        const unsigned long long want = ((unsigned long long)i << 32) | fp;
                         const unsigned long long old =
                             atomicCAS(reinterpret_cast<unsigned long long*>(tab + slot), 0ull, want);
                         if (old == 0ull) {
@@ -504,9 +505,9 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
                 const uint32_t w = (v == XW - 1) ? (xo[j][v] & lm) : xo[j][v];
                 e = e && (w == xv[j][v]);
             }
-            const int i = base + j * NT + t;
+            const uint32_t i = base + (uint32_t)(j * NT + t);
             if (e) {
-                if ((uint32_t)i < ent[j].y) atomicMin(&tab[cs[j]].y, (uint32_t)i);
+                if (i < ent[j].y) atomicMin(&tab[cs[j]].y, (uint32_t)i);
                 mine[j] = (int)cs[j];
             } else {  // a different row with the same fingerprint: keep probing
                 mine[j] = dd_find_insert(tab, E, h[j], i, yv[j], xc, yc, XW, n, (cs[j] + 1) & emask,
@@ -517,9 +518,9 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
         uint32_t bal[K];
 #pragma unroll
         for (int j = 0; j < K; ++j) {
-            const int i = base + j * NT + t;
-            const bool valid = i < T;
-            const int rep = (valid && mine[j] >= 0) ? (int)tab[mine[j]].y : i;
+            const uint32_t i = base + (uint32_t)(j * NT + t);
+            const bool valid = i < Tu;
+            const uint32_t rep = (valid && mine[j] >= 0) ? tab[mine[j]].y : i;
             const bool isrep = valid && rep == i;
             if (valid && !isrep) atomicAdd(D + mine[j], 1);
             bal[j] = __ballot_sync(FULL, isrep);
@@ -536,7 +537,7 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
             }
             if ((bal[j] >> lane) & 1u) {
                 const int pos = nrep + before + __popc(bal[j] & ((1u << lane) - 1u));
-                a.rep_list[r0 + pos] = base + j * NT + t;  // within the shard (see below)
+                a.rep_list[r0 + pos] = (int32_t)(base + (uint32_t)(j * NT + t));  // within the shard (see below)
                 a.rep_dup[r0 + pos] = mine[j];
             }
             nrep += total;
@@ -544,7 +545,7 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
         // (the next round's first barrier comes before it writes wcnt again)
     }
     dd_sync<G>();
-    for (int k = t; k < nrep; k += NT) {
+    for (uint32_t k = t; k < (uint32_t)nrep; k += NT) {
         const int slot = a.rep_dup[r0 + k];
         a.rep_dup[r0 + k] = (slot >= 0) ? D[slot] : 0;
     }
@@ -826,8 +827,9 @@ __device__ bool dedup_wide_ctx(const StoreDev& s, const DedupArgs& a, int c, int
     const uint32_t lm = last_mask(s.desc[c].n);
     const int al = ((uintptr_t)xc & 15) == 0 ? 2 : (((uintptr_t)xc & 7) == 0 ? 1 : 0);
     int nrep = 0;
-    for (int s0 = 0; s0 < T; s0 += SEG) {
-        const int n = T - s0 < SEG ? T - s0 : SEG;
+    for (int s0 = 0, s1; s0 < T; s0 = s1) {
+        s1 = step_to(s0, SEG, T);
+        const int n = s1 - s0;
         const DdSmem m = dd_layout<XW>(region, G * DD_WARP_REGION, n, MOST);
         // (a piece starts at a multiple of SEG rows, so its rows keep the alignment)
         nrep += dedup_rows<G, XW>(xc + (int64_t)s0 * XW, a.y + r0 + s0, n, s0, lm, al, m, a.rep_list + r0 + nrep,
@@ -873,8 +875,7 @@ __global__ void __launch_bounds__(DD_THREADS, DD_CTAS_PER_SM) dedup_kernel(Store
             const int c = (int)(qi & (SHARD_CTX_LIMIT - 1));
             const int nsh = (int)(qi >> 28) + 1;
             const int T = (int)(a.row_off[c + 1] - a.row_off[c]);
-            int E = pow2_at_least(2 * ((T + nsh - 1) / nsh));
-            if (E > DD_CTA_E) E = DD_CTA_E;
+            const int E = table_entries((int)(((int64_t)T + nsh - 1) / nsh), DD_CTA_E);
             // a split context's pass: from its first shard's start to the end of the last one
             if (threadIdx.x == 0 && ((qi >> 24) & 7u) == 0) time_mark(a.timing, c, 0);
             bool done = true;
@@ -903,8 +904,7 @@ __global__ void __launch_bounds__(DD_THREADS, DD_CTAS_PER_SM) dedup_kernel(Store
             if (item >= n) break;
             const int c = a.queue[b + item];
             const int T = (int)(a.row_off[c + 1] - a.row_off[c]);
-            int E = pow2_at_least(2 * T);
-            if (E > DD_QUAD_E) E = DD_QUAD_E;
+            const int E = table_entries(T, DD_QUAD_E);
             if ((warp & 3) == 0 && lane == 0) time_mark(a.timing, c, 0);
 #define F2_DD_QUAD(W) dedup_ctx<4, W>(s, a, c, region, E, wcnt + q * 4 * DD_K)
 #define F2_DDW_QUAD(W) dedup_wide_ctx<4, W>(s, a, c, q * 4 * DD_WARP_REGION, wcnt + q * 4 * DD_K)
@@ -929,7 +929,7 @@ __global__ void __launch_bounds__(DD_THREADS, DD_CTAS_PER_SM) dedup_kernel(Store
             if (item >= n) break;
             const int c = a.queue[b + item];
             const int T = (int)(a.row_off[c + 1] - a.row_off[c]);
-            const int E = pow2_at_least(2 * T);
+            const int E = table_entries(T, DD_WARP_E);
             if (lane == 0) time_mark(a.timing, c, 0);
 #define F2_DD_WARP(W) dedup_ctx<1, W>(s, a, c, region, E, nullptr)
 #define F2_DDW_WARP(W) dedup_wide_ctx<1, W>(s, a, c, warp * DD_WARP_REGION, nullptr)
@@ -1052,14 +1052,15 @@ __device__ void check_chunk(const StoreDev& s, const CheckArgs& a, int c, int kb
     const uint4* yc = a.y + r0;
     const uintptr_t bits = (uintptr_t)xc | (uintptr_t)(4 * cd.xw);
     const int al = (bits & 15) == 0 ? 2 : ((bits & 7) == 0 ? 1 : 0);
-    int next = kb + (int)threadIdx.x < ke ? (reps ? ld(reps + kb + threadIdx.x) : kb + (int)threadIdx.x) : 0;
+    const int n = ke - kb;
+    auto row_of = [&](int j) { return j < n ? (reps ? ld(reps + kb + j) : kb + j) : 0; };
+    int next = row_of(threadIdx.x);
     // every lane of a warp in each round: the pivot walk is warp-uniform
-    for (int base = kb; base < ke; base += blockDim.x) {
-        const int k = base + (int)threadIdx.x;
-        const bool valid = k < ke;
+    for (int base = 0; base < n; base += blockDim.x) {
+        const int j = base + (int)threadIdx.x;
+        const bool valid = j < n;
         const int i = next;
-        const int kn = k + (int)blockDim.x;
-        next = kn < ke ? (reps ? ld(reps + kn) : kn) : 0;
+        next = row_of(j + (int)blockDim.x);
         uint32_t xin[WD], q[WD];
         uint4 y = valid ? ld(yc + i) : make_uint4(0, 0, 0, 0);
         load_row_words<WD>(xc + (int64_t)i * cd.xw, al, valid, cd.n, cd.xw, xin);
@@ -1068,7 +1069,7 @@ __device__ void check_chunk(const StoreDev& s, const CheckArgs& a, int c, int kb
         uint32_t resid = 0;
 #pragma unroll
         for (int w = 0; w < WD; ++w) resid |= q[w] & ~Ps[w];
-        if (valid) flags[k - kb] = resid ? 2 : (nonzero4(y) ? 1 : 0);
+        if (valid) flags[j] = resid ? 2 : (nonzero4(y) ? 1 : 0);
     }
 }
 
@@ -1109,14 +1110,14 @@ __global__ void __launch_bounds__(256, 3) check_snap_kernel(StoreDev s, CheckArg
             if (built >= 0) {
                 if (t == 0) k = atomicAdd(a.ctr + built, 1);
                 k = __shfl_sync(FULL, k, 0);
-                if (a.snap_start[built] + k * CHECK_CHUNK < reps_of(built)) c = built;
+                if (chunk_exists(a.snap_start[built], k, CHECK_CHUNK, reps_of(built))) c = built;
             }
             while (c < 0 && tried < nq) {
                 int cq = -1;
                 if (tried + t < nq) {
                     const int at = q0 + tried + t;
                     cq = a.snap_list[at < nq ? at : at - nq];
-                    if (a.snap_start[cq] + (int64_t)__ldcg(a.ctr + cq) * CHECK_CHUNK >= reps_of(cq)) cq = -1;
+                    if (!chunk_exists(a.snap_start[cq], __ldcg(a.ctr + cq), CHECK_CHUNK, reps_of(cq))) cq = -1;
                 }
                 const uint32_t left = __ballot_sync(FULL, cq >= 0);
                 if (!left) {
@@ -1126,7 +1127,7 @@ __global__ void __launch_bounds__(256, 3) check_snap_kernel(StoreDev s, CheckArg
                 cq = __shfl_sync(FULL, cq, __ffs(left) - 1);
                 if (t == 0) k = atomicAdd(a.ctr + cq, 1);
                 k = __shfl_sync(FULL, k, 0);
-                if (a.snap_start[cq] + k * CHECK_CHUNK < reps_of(cq)) c = cq;
+                if (chunk_exists(a.snap_start[cq], k, CHECK_CHUNK, reps_of(cq))) c = cq;
             }
             if (t == 0) {
                 *s_c = c;
@@ -1144,7 +1145,7 @@ __global__ void __launch_bounds__(256, 3) check_snap_kernel(StoreDev s, CheckArg
         const int R = reps_of(c);
         const int st0 = a.snap_start[c];
         const int kb = st0 + ck * CHECK_CHUNK;
-        const int ke = (kb + CHECK_CHUNK < R) ? kb + CHECK_CHUNK : R;
+        const int ke = step_to(kb, CHECK_CHUNK, R);
         if (built != c) {  // the basis into shared memory (pivot rows only)
             if (t < 24) {
                 Ps[t] = (t < cd.wd) ? s.pivot[cd.pw_off + t] : 0u;
@@ -1216,7 +1217,7 @@ __global__ void __launch_bounds__(256, 3) check_snap_kernel(StoreDev s, CheckArg
             a.rec[2 * slot] = make_uint4((uint32_t)fo, (uint32_t)sc, (uint32_t)(sc >> 32), 0u);
             a.rec[2 * slot + 1] = make_uint4((uint32_t)sf, (uint32_t)((unsigned long long)sf >> 32), 0u, 0u);
             __threadfence();
-            const int nch = (R - st0 + CHECK_CHUNK - 1) / CHECK_CHUNK;
+            const int nch = chunk_count(st0, CHECK_CHUNK, R);
             if (atomicAdd(a.ctr + s.num_ctx + c, 1) == nch - 1) {  // the context's last chunk
                 __threadfence();
                 const int64_t s0 = check_slot(a, c);
@@ -1259,7 +1260,7 @@ __global__ void __launch_bounds__(256, 3) check_snap_kernel(StoreDev s, CheckArg
 //     rows and at most DD_XW_WIDE feature words goes to the warp, quad or CTA
 //     dedup queue by its row count, the others straight to an elimination
 //     queue; rep_count[c] becomes 0 (filled by the dedup pass), -1 (invalid,
-//     skipped) or -(T+2) (every row is its own representative);
+//     skipped) or all_rows(T) (every row is its own representative);
 //   mode 1 (elimination plan): contexts with rows to eliminate go to the
 //     warp, CTA or wide elimination queue.  After a mode-0 plan that sent no
 //     context to the duplicate pass it has nothing to do and returns.
@@ -1356,7 +1357,7 @@ __device__ __forceinline__ int plan_key_of(const StoreDev& s, const PlanArgs& p,
     bool direct = p.mode == 1;  // to an elimination queue
     if (p.mode == 1 && p.rep_count) {
         R = r.reps;
-        if (R <= -2) R = -(R + 2);
+        if (R <= -2) R = rows_of((int32_t)R);
     } else {
         const int64_t a0 = r.a0, a1 = r.a1;
         const int64_t rows = a1 - a0;
@@ -1369,7 +1370,7 @@ __device__ __forceinline__ int plan_key_of(const StoreDev& s, const PlanArgs& p,
             // wide rows and short contexts are not deduplicated; rows of a
             // full-rank context are checked one by one (verify_full_kernel)
             if (R > 0 && (cd.xw > DD_XW_WIDE || R <= p.dedup_min || r.rank == cd.d)) {
-                p.rep_count[c] = (int32_t)(-(R + 2));
+                p.rep_count[c] = all_rows(R);
                 direct = true;
             } else {
                 p.rep_count[c] = (R > 0) ? 0 : (int32_t)R;
