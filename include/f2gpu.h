@@ -31,7 +31,10 @@
  *   - Every call is asynchronous on the caller's stream and ordered with the
  *     caller's other work on that stream; results are valid once the stream
  *     has been synchronized.  Calls on one store must not overlap on
- *     different streams.
+ *     different streams.  The device that the store was created on is the
+ *     current one, and `stream` a stream of it, in every call on the store
+ *     (f2_get_basis, f2_device_status, f2_learn_timing, f2_store_export and
+ *     f2_store_import copy only and take any current device).
  *   - Return value: F2_OK or an F2_ERR_* code for errors detected on the host
  *     before anything is enqueued (nothing is enqueued on error).  Errors that
  *     only the device can detect (bad CSR offsets, out-of-range context ids)

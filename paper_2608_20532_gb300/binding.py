@@ -122,6 +122,12 @@ def _check(code: int, what: str):
         raise F2Error(code, what)
 
 
+def _current_stream(index: int) -> int:
+    """The current stream of a device, as torch's own launchers take it (a Stream object costs a
+    microsecond a call)."""
+    return torch._C._cuda_getCurrentRawStream(index)
+
+
 def _stream(stream=None) -> int:
     s = stream if stream is not None else torch.cuda.current_stream()
     return int(s.cuda_stream)
@@ -163,9 +169,10 @@ class Store:
         self.n_bits = nb
         self.raw = bool(raw)
         self.device = torch.device(device) if device is not None else torch.device("cuda", torch.cuda.current_device())
+        self._index = self.device.index if self.device.index is not None else torch.cuda.current_device()
         if _handle is None:
             h = ctypes.c_void_p()
-            with torch.cuda.device(self.device):
+            with torch.cuda.device(self._index):
                 _check(self._lib.f2_create(ctypes.byref(h), int(nb.shape[0]), nb.ctypes.data,
                                            F2_FLAG_RAW_FEATURES if raw else 0, _stream(stream)), "f2_create")
         else:  # a store the library created (f2_merge_bases)
@@ -178,9 +185,22 @@ class Store:
         _check(self._lib.f2_layout(self._h, self.slot_off.ctypes.data, self.xw_off.ctypes.data,
                                    self.pw_off.ctypes.data), "f2_layout")
 
+    def _call(self, name, stream, *args):
+        """Call the library on the store's handle with the store's device current (kernels launch on
+        the current device) and `stream`, or that device's current stream."""
+        fn = getattr(self._lib, name)
+        raw = int(stream.cuda_stream) if stream is not None else _current_stream(self._index)
+        if torch.cuda.current_device() == self._index:
+            code = fn(self._h, *args, raw)
+        else:
+            with torch.cuda.device(self._index):
+                code = fn(self._h, *args, raw)
+        _check(code, name)
+
     def close(self):
         if getattr(self, "_h", None) and self._h.value:
-            self._lib.f2_destroy(self._h)  # frees device memory: the device has synchronized
+            with torch.cuda.device(self._index):
+                self._lib.f2_destroy(self._h)  # frees device memory: the device has synchronized
             self._h = ctypes.c_void_p()
         self._held = []
 
@@ -198,16 +218,15 @@ class Store:
         _check(self._lib.f2_set_option(self._h, option, int(value)), "f2_set_option")
 
     def reset(self, stream=None):
-        _check(self._lib.f2_reset(self._h, _stream(stream)), "f2_reset")
+        self._call("f2_reset", stream)
 
     def learn(self, row_off: torch.Tensor, x: torch.Tensor, x_off: torch.Tensor, y: torch.Tensor, stream=None):
         """One batch: row_off int64[C+1], x int32/uint32 words, x_off int64[C], y int32[R, 4]."""
         if row_off.dtype != torch.int64 or x_off.dtype != torch.int64:
             raise TypeError("row_off and x_off must be int64")
         total_rows = y.numel() // 4
-        _check(self._lib.f2_learn_batched(self._h, _dptr(row_off), _dptr(x), _dptr(x_off), _dptr(y),
-                                          int(total_rows), int(x.numel()), _stream(stream)),
-               "f2_learn_batched")
+        self._call("f2_learn_batched", stream, _dptr(row_off), _dptr(x), _dptr(x_off), _dptr(y), int(total_rows),
+                   int(x.numel()))
 
     def _hold(self, arrays, stream):
         """Keep host arrays alive until `stream` has passed the call that reads or writes them."""
@@ -216,32 +235,28 @@ class Store:
             held = self._held = []
         held[:] = [(ev, refs) for ev, refs in held if not ev.query()]
         ev = torch.cuda.Event()
-        ev.record(stream if stream is not None else torch.cuda.current_stream(self.device))
+        ev.record(stream if stream is not None else torch.cuda.current_stream(self._index))
         held.append((ev, tuple(arrays)))
 
     def learn_host(self, row_off, x, x_off, y, stream=None):
         """One batch from host memory (f2_learn_host): row_off int64[C+1], x 32-bit words,
         x_off int64[C], y 32-bit words [R, 4]; pinned CPU tensors let copies overlap."""
-        with torch.cuda.device(self.device):
-            _check(self._lib.f2_learn_host(self._h, _hptr(row_off), _hptr(x), _hptr(x_off), _hptr(y),
-                                           int(_hsize(y) // 4), int(_hsize(x)), _stream(stream)),
-                   "f2_learn_host")
-            self._hold((row_off, x, x_off, y), stream)
+        self._call("f2_learn_host", stream, _hptr(row_off), _hptr(x), _hptr(x_off), _hptr(y), int(_hsize(y) // 4),
+                   int(_hsize(x)))
+        self._hold((row_off, x, x_off, y), stream)
 
     def encode_host(self, ctx_id, x, y_out, in_span, stream=None):
         """Queries in host memory (f2_encode_host): ctx_id int32[Q], x 32-bit words [Q, stride];
         y_out 32-bit words [Q, 4] and in_span uint8[Q] are written once `stream` passes the call."""
         Q = int(_hsize(ctx_id))
         stride = int(x.shape[1]) if len(x.shape) == 2 else 1
-        with torch.cuda.device(self.device):
-            _check(self._lib.f2_encode_host(self._h, Q, _hptr(ctx_id), _hptr(x), stride, _hptr(y_out),
-                                            _hptr(in_span), _stream(stream)), "f2_encode_host")
-            self._hold((ctx_id, x, y_out, in_span), stream)
+        self._call("f2_encode_host", stream, Q, _hptr(ctx_id), _hptr(x), stride, _hptr(y_out), _hptr(in_span))
+        self._hold((ctx_id, x, y_out, in_span), stream)
         return y_out, in_span
 
     def basis(self, stream=None) -> dict:
         C = self.num_ctx
-        dev = self.device
+        dev = self._index
         out = {
             "rank": torch.empty(C, dtype=torch.int32, device=dev),
             "pivot_mask": torch.empty(int(self.pw_off[-1]), dtype=torch.int32, device=dev),
@@ -253,13 +268,13 @@ class Store:
             "rows_seen": torch.empty(C, dtype=torch.int64, device=dev),
         }
         keys = ("rank", "pivot_mask", "basis_x", "basis_z", "contra", "first_contra", "n_contra", "rows_seen")
-        _check(self._lib.f2_get_basis(self._h, *(_dptr(out[k]) for k in keys), _stream(stream)), "f2_get_basis")
+        self._call("f2_get_basis", stream, *(_dptr(out[k]) for k in keys))
         return out
 
     def solve(self, out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
         if out is None:
-            out = torch.empty((int(self.slot_off[-1]), 4), dtype=torch.int32, device=self.device)
-        _check(self._lib.f2_solve_affine(self._h, _dptr(out), _stream(stream)), "f2_solve_affine")
+            out = torch.empty((int(self.slot_off[-1]), 4), dtype=torch.int32, device=self._index)
+        self._call("f2_solve_affine", stream, _dptr(out))
         return out
 
     def encode(self, ctx_id: torch.Tensor, x: torch.Tensor, y_out: Optional[torch.Tensor] = None,
@@ -268,11 +283,10 @@ class Store:
         Q = int(ctx_id.numel())
         stride = int(x.shape[1]) if x.dim() == 2 else 1
         if y_out is None:
-            y_out = torch.empty((Q, 4), dtype=torch.int32, device=self.device)
+            y_out = torch.empty((Q, 4), dtype=torch.int32, device=self._index)
         if in_span is None:
-            in_span = torch.empty(Q, dtype=torch.uint8, device=self.device)
-        _check(self._lib.f2_encode_batched(self._h, Q, _dptr(ctx_id), _dptr(x), stride, _dptr(y_out),
-                                           _dptr(in_span), _stream(stream)), "f2_encode_batched")
+            in_span = torch.empty(Q, dtype=torch.uint8, device=self._index)
+        self._call("f2_encode_batched", stream, Q, _dptr(ctx_id), _dptr(x), stride, _dptr(y_out), _dptr(in_span))
         return y_out, in_span
 
     def encode_epilogue(self, ctx_id: torch.Tensor, in_span: torch.Tensor, y: torch.Tensor, sched=None,
@@ -281,11 +295,9 @@ class Store:
         of opaque_mask[ctx] taken from state; rejected queries untouched.
         sched int32[Q], state int32[Q, 4], opaque_mask int32[num_ctx, 4]."""
         Q = int(ctx_id.numel())
-        _check(self._lib.f2_encode_epilogue(self._h, Q, _dptr(ctx_id), _dptr(in_span),
-                                            _dptr(sched) if sched is not None else None,
-                                            _dptr(state) if state is not None else None,
-                                            _dptr(opaque_mask) if opaque_mask is not None else None,
-                                            _dptr(y), _stream(stream)), "f2_encode_epilogue")
+        self._call("f2_encode_epilogue", stream, Q, _dptr(ctx_id), _dptr(in_span),
+                   _dptr(sched) if sched is not None else None, _dptr(state) if state is not None else None,
+                   _dptr(opaque_mask) if opaque_mask is not None else None, _dptr(y))
         return y
 
     def merge(self, group_of, num_groups: int, out_mask=None, stream=None):
@@ -296,37 +308,35 @@ class Store:
         m = None if out_mask is None else np.ascontiguousarray(np.asarray(out_mask, dtype=np.uint32))
         ok = np.zeros(max(int(num_groups), 1), np.uint8)
         h = ctypes.c_void_p()
-        with torch.cuda.device(self.device):
-            _check(self._lib.f2_merge_bases(self._h, int(num_groups), g.ctypes.data,
-                                            m.ctypes.data if m is not None else None, ctypes.byref(h),
-                                            ok.ctypes.data, _stream(stream)), "f2_merge_bases")
+        self._call("f2_merge_bases", stream, int(num_groups), g.ctypes.data,
+                   m.ctypes.data if m is not None else None, ctypes.byref(h), ok.ctypes.data)
         d = np.zeros(int(num_groups), np.int32)
         member = g >= 0
         d[g[member]] = self.n_bits[member] + (0 if self.raw else 1)
-        return Store(d, raw=True, device=self.device, _handle=h), ok[:int(num_groups)]
+        return Store(d, raw=True, device=torch.device("cuda", self._index), _handle=h), ok[:int(num_groups)]
 
     def learn_timing(self, stream=None) -> np.ndarray:
         """Per-context timestamps of the last learn call (F2_OPT_TIMING on):
         uint64[num_ctx, 6] = dedup start/end, elimination start/end (ns), their SM ids."""
         out = np.zeros((self.num_ctx, 6), np.uint64)
-        _check(self._lib.f2_learn_timing(self._h, out.ctypes.data, _stream(stream)), "f2_learn_timing")
+        self._call("f2_learn_timing", stream, out.ctypes.data)
         return out
 
     def device_status(self, stream=None) -> int:
         v = ctypes.c_int(0)
-        _check(self._lib.f2_device_status(self._h, ctypes.byref(v), _stream(stream)), "f2_device_status")
+        self._call("f2_device_status", stream, ctypes.byref(v))
         return int(v.value)
 
     def export_state(self, stream=None) -> bytes:
         n = ctypes.c_size_t(0)
-        _check(self._lib.f2_store_export(self._h, None, ctypes.byref(n), _stream(stream)), "f2_store_export")
+        self._call("f2_store_export", stream, None, ctypes.byref(n))
         buf = ctypes.create_string_buffer(n.value)
-        _check(self._lib.f2_store_export(self._h, buf, ctypes.byref(n), _stream(stream)), "f2_store_export")
+        self._call("f2_store_export", stream, buf, ctypes.byref(n))
         return buf.raw[:n.value]
 
     def import_state(self, data: bytes, stream=None):
         buf = ctypes.create_string_buffer(data, len(data))
-        _check(self._lib.f2_store_import(self._h, buf, len(data), _stream(stream)), "f2_store_import")
+        self._call("f2_store_import", stream, buf, len(data))
 
 
 def peak_lop3(blocks: int, iters: int, out: torch.Tensor, stream=None) -> int:

@@ -364,10 +364,22 @@ extern "C" int f2_get_basis(const f2_store* s, int32_t* rank, uint32_t* pivot_ma
     cp(n_contra, s->n_contra, sizeof(uint64_t) * C);
     cp(rows_seen, s->rows_seen, sizeof(int64_t) * C);
     if (L.n == 0) return F2_OK;
-    size_t blocks = (total + 8191) / 8192;  // 32 bytes a thread, at most eight blocks per SM
-    if (blocks > (size_t)s->num_sms * 8) blocks = (size_t)s->num_sms * 8;
-    f2_launch(copy_kernel, (unsigned)blocks, 256, 0, st, total <= EARLY_MAX_BYTES, L);
-    return f2_cuda_status(cudaGetLastError());
+    // A kernel runs on the store's device and a stream of it; copies, where the
+    // caller's device or stream is another one, on any.
+    int cur = -1;
+    cudaError_t e = cudaGetDevice(&cur);
+    if (e != cudaSuccess) return f2_cuda_status(e);
+    if (cur == s->device) {
+        size_t blocks = (total + 8191) / 8192;  // 32 bytes a thread, at most eight blocks per SM
+        if (blocks > (size_t)s->num_sms * 8) blocks = (size_t)s->num_sms * 8;
+        f2_launch(copy_kernel, (unsigned)blocks, 256, 0, st, total <= EARLY_MAX_BYTES, L);
+        e = cudaGetLastError();
+        if (e != cudaErrorInvalidResourceHandle) return f2_cuda_status(e);
+        e = cudaSuccess;
+    }
+    for (int k = 0; k < L.n && e == cudaSuccess; ++k)
+        e = cudaMemcpyAsync(L.dst[k], L.src[k], L.bytes[k], cudaMemcpyDeviceToDevice, st);
+    return f2_cuda_status(e);
 }
 
 // ------------------------------------------------------------ affine solve
