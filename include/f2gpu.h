@@ -310,7 +310,9 @@ enum f2_option {
                                     laid out chunk by chunk (the others keep one run); default 512 */
     F2_OPT_FAIL_ALLOC = 9,       /* test hook: the device allocation made after `value` more successful
                                     ones by calls on this store fails as if out of memory (the call
-                                    returns F2_ERR_OOM; the store stays usable); -1 (default) = off */
+                                    returns F2_ERR_OOM and the store stays usable; where it was for a
+                                    hand-off that the call makes by default, the call goes without);
+                                    -1 (default) = off */
     F2_OPT_TIMING = 10,          /* 1: f2_learn_batched records per-context timestamps (f2_learn_timing);
                                     0 (default): off */
     F2_OPT_ELIM_TABLES = 11,     /* 1 (default): step (1) against the basis uses a 4-bit lookup table of it
@@ -333,9 +335,10 @@ enum f2_option {
                                     the rest of its call off to a parallel check when at least this many
                                     of its representatives are left (a representative outside the basis
                                     sends the rest back to elimination from there); only in calls of at
-                                    least 16x this many rows; 0 = never. Unless this is set, calls of at
+                                    least 16x this many rows; 0 = never. -1 (default): calls of at
                                     least 2^20 rows on a store with contexts of 10..17 words hand off
-                                    the contexts with at least 2048 representatives left */
+                                    the contexts with at least 2048 representatives left that do not
+                                    run against a lookup table */
     F2_OPT_FAIL_WAIT = 17,       /* test hook: 1: the waits of f2_learn_batched's tensor-core full-rank check
                                     (192 features and more) act as if they had given up
                                     (F2_ERR_TIMEOUT); 0 (default): off */

@@ -36,6 +36,7 @@ struct LearnArgs {
     // with at least handoff_min representatives left, stops and is listed
     // here: check_snap_kernel checks the rest against its basis in parallel
     int handoff_min;             // 0 = never
+    int handoff_tables;          // also contexts that run against a lookup table
     int* snap_count;
     int32_t* snap_list;
     int32_t* snap_start;         // its first representative left
@@ -799,7 +800,8 @@ __device__ int table_rounds(const LearnArgs& a, const RowStream& rs, ElimState<W
         st.base = step_to(st.base, nt, rs.R);
         if constexpr (CTA) {
             st.quiet = inserted ? 0 : st.quiet + 1;
-            if (st.quiet >= HANDOFF_QUIET && rs.R - st.base >= st.hand_min && st.rank + n_new < d && d * RS <= CHECK_BASIS_WORDS) {
+            if (a.handoff_tables && st.quiet >= HANDOFF_QUIET && rs.R - st.base >= st.hand_min && st.rank + n_new < d &&
+                d * RS <= CHECK_BASIS_WORDS) {
                 snap_at = st.base;
                 break;
             }
@@ -1182,7 +1184,8 @@ __device__ void elim_cta(const StoreDev& s, const LearnArgs& a, int c, uint32_t*
         if constexpr (WD <= NARROW_WD || WD == WIDE_M_WD) {
             // a saturated context with many representatives left hands the
             // rest off to the parallel check (block-uniform)
-            if (st.quiet >= HANDOFF_QUIET && rs.R - st.base >= st.hand_min && st.rank < cd.d && cd.d * RS <= CHECK_BASIS_WORDS) {
+            if (st.quiet >= HANDOFF_QUIET && rs.R - st.base >= st.hand_min && st.rank < cd.d &&
+                cd.d * RS <= CHECK_BASIS_WORDS) {
                 snap_at = st.base;
                 break;
             }

@@ -1818,11 +1818,19 @@ __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, F
 
 // The default hand-off (see f2_learn_batched): calls of at least this many
 // rows on stores with rows of 10..17 words, contexts with at least this many
-// representatives left.  On 10,000 contexts of parsed values (13.4M rows) the
-// learn call takes 1,054 us; 1,060 from 1,024 representatives on, 1,066 where a
-// context must also hold a sixteenth of an SM's share of the call's work (1,102
-// with chunks of 512, where an eighth took 1,162).  Other stores gain nothing:
-// 4,096 contexts 262 us without, 278 with it, 77,926 contexts 2,510 and 2,579.
+// representatives left that walk their pivots.  On 10,000 contexts of parsed
+// values (13.4M rows) the learn call takes 1,054 us; 1,060 from 1,024
+// representatives on, 1,066 where a context must also hold a sixteenth of an
+// SM's share of the call's work (1,102 with chunks of 512, where an eighth took
+// 1,162).  Contexts that run against a lookup table stay: the check walks the
+// pivots, which costs a context of high rank more than its table, and one context
+// of 10..17 words would turn that on for a whole store.  With one such context,
+// without the hand-off / with it / with it for contexts with a table too:
+// 10,000 contexts of 100..256 features (16.3M rows) 2,343 / 2,362 / 2,642 us,
+// 4,096 of 32..128 (2.5M) 308 / 321 / 350, 77,926 (80M) 2,459 / 2,482 / 2,534,
+// 5,000 of parsed values of 128..256 bits (6.7M) 800 / 466 / 466; where a few long
+// contexts with tables bound the call it would gain: 1,000 contexts (8.2M rows)
+// 1,507 / 1,528 / 1,363, 5,000 of one parsed value 491 / 513 / 290.
 constexpr int64_t HANDOFF_AUTO_ROWS = int64_t(1) << 20;
 constexpr int HANDOFF_AUTO_REPS = 2048;
 
@@ -2198,6 +2206,7 @@ extern "C" int f2_learn_batched(f2_store* st, const int64_t* row_off, const uint
     la.small_region_words = (int)(st->small_basis_bytes / 4);
     la.cta_region_words = 0;  // set per launch
     la.handoff_min = hand_min;
+    la.handoff_tables = !auto_hand;
     la.snap_count = st->hand;
     la.snap_list = st->hand + 2;
     la.snap_start = st->hand + 2 + C;
@@ -2474,6 +2483,7 @@ extern "C" int f2_learn_batched_noalloc(int32_t num_ctx, const int32_t* n_bits_h
     la.small_region_words = DEFAULT_SMALL_REGION_BYTES / 4;
     la.cta_region_words = 0;
     la.handoff_min = 0;
+    la.handoff_tables = 0;
     la.snap_count = nullptr;
     la.snap_list = nullptr;
     la.snap_start = nullptr;

@@ -584,7 +584,7 @@ extern "C" int f2_set_option(f2_store* s, int option, int64_t value)
         s->small_basis_bytes = (value / 16) * 16;
         return F2_OK;
     case F2_OPT_HANDOFF_REPS:
-        if (value < 0 || value > (int64_t(1) << 30)) return F2_ERR_INVALID_ARG;
+        if (value < -1 || value > (int64_t(1) << 30)) return F2_ERR_INVALID_ARG;  // -1: the default
         s->handoff_min = value;
         return F2_OK;
     case F2_OPT_LONG_CALL_ROWS:

@@ -92,3 +92,55 @@ def test_default_without_memory():
         st.close()
     for k in KEYS:
         assert np.array_equal(got[0][k], got[1][k]), k
+
+
+def test_default_of_a_mixed_store():
+    """The default hand-off of a store that mixes contexts of every width, long
+    contexts of low rank (which walk their pivots) and of high rank (which run
+    against a lookup table), some with a row outside the span late; and the
+    option set and set back to the default."""
+    dev = cuda_device()
+    binding = lib()
+    rng = np.random.default_rng(88)
+    n_bits, ranks = [], []
+    for n in (40, 64, 95, 128, 200, 287, 320, 500):
+        for r in (3, 9, n // 3, n - 2):
+            n_bits.append(n)
+            ranks.append(r)
+    T = 33000
+    nb = np.array(n_bits, np.int32)
+    W = (nb.astype(np.int64) + 31) // 32
+    row_off = np.arange(len(n_bits) + 1, dtype=np.int64) * T
+    assert int(row_off[-1]) >= 1 << 20
+    x_off = np.concatenate([[0], np.cumsum(T * W)[:-1]]).astype(np.int64)
+    x = np.zeros(int(T * W.sum()), np.uint32)
+    y = np.zeros((int(row_off[-1]), 4), np.uint32)
+    for c, (n, r) in enumerate(zip(n_bits, ranks)):
+        G = rng.integers(0, 2, (r, n)).astype(np.float32)
+        A = rng.integers(0, 2, (n, 128)).astype(np.float32)
+        xb = np.zeros((T, 32 * int(W[c])), np.uint8)
+        xb[:, :n] = (rng.integers(0, 2, (T, r)).astype(np.float32) @ G).astype(np.int64) & 1
+        if c % 3 == 0:
+            xb[T - 1 - 7 * c, int(rng.integers(n))] ^= 1
+        yb = ((xb[:, :n].astype(np.float32) @ A).astype(np.int64) & 1).astype(np.uint8)
+        yc = np.packbits(yb, axis=1, bitorder="little").view(np.uint32).copy()
+        for i in rng.integers(T // 2, T, c % 4):
+            yc[i, 2] ^= 16
+        x[x_off[c]:x_off[c] + T * W[c]] = np.packbits(xb, axis=1, bitorder="little").view(np.uint32).reshape(-1)
+        y[row_off[c]:row_off[c + 1]] = yc
+    O = oracle.Oracle(nb)
+    O.learn(row_off, x_off, x, y)
+    ref = O.export()
+    st = binding.Store(nb, device=dev)
+    ro_t, x_t, xo_t, y_t = dev_arrays(binding, dev, row_off, x, x_off, y)
+    for option in (None, 0, -1, 2048):
+        if option is not None:
+            st.set_option(binding.F2_OPT_HANDOFF_REPS, option)
+        st.reset()
+        st.learn(ro_t, x_t, xo_t, y_t)
+        torch.cuda.synchronize()
+        assert st.device_status() == binding.F2_OK
+        assert_basis_equal(binding, st.basis(), ref)
+    with pytest.raises(binding.F2Error):
+        st.set_option(binding.F2_OPT_HANDOFF_REPS, -2)
+    st.close()
