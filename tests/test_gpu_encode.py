@@ -170,6 +170,35 @@ def test_bad_ids_and_stride_in_long_runs(env):
         assert st.device_status() == 9
 
 
+@pytest.mark.parametrize("contexts", [1, 3, 64])
+def test_warps_of_one_context(env, contexts):
+    """The counting of a small store's queries, a warp at a time: warps whose 32 queries are of one
+    context, in which one lane differs, which name no context, and the pass's ragged end."""
+    binding, dev = env
+    rng = np.random.default_rng(31 + contexts)
+    wl = wlmod.generate(dict(num_ctx=contexts, layout=wlmod.LAYOUT_CYCLIC_FIELDS, n_min=20, n_max=90, rows_fixed=60,
+                             dup_frac=0.2, density=0.05, n_contra=0), 7)
+    st = binding.Store(wl.n_bits, device=dev)
+    gpu_learn_workload(binding, st, wl, dev)
+    O = oracle_for(wl)
+    kinds = rng.integers(0, 4, 160)
+    ctx = np.repeat(rng.integers(0, contexts, 160), 32).astype(np.int32).reshape(160, 32)
+    ctx[kinds == 1, 31] = (ctx[kinds == 1, 31] + 1) % (contexts + 1)  # contexts: names none
+    ctx[kinds == 2] = contexts + 5
+    ctx[kinds == 3, 0] = -1
+    for n in (ctx.size, ctx.size - 1, ctx.size - 40, 33):
+        c = ctx.reshape(-1)[:n].copy()
+        x = rng.integers(0, 2 ** 32, (n, 3), dtype=np.uint64).astype(np.uint32)
+        good = (c >= 0) & (c < contexts)
+        ry, rok = O.encode(np.where(good, c, 0).astype(np.int32), x)
+        for tm in (16, DIRECT):
+            y, ok = _encode_all(binding, st, c, x, tm)
+            assert np.array_equal(ok, np.where(good, rok, 0xFF).astype(np.uint8)), (n, tm)
+            assert np.array_equal(y[good], ry[good]), (n, tm)
+            assert st.device_status() == (binding.F2_OK if good.all() else binding.F2_ERR_CTX_RANGE)
+    st.close()
+
+
 def test_zipf_config3_scaled_table_mins(env):
     binding, dev = env
     wl = wlmod.generate(wlmod.scaled(3, 2000), 313, query_count=200000)
