@@ -739,22 +739,24 @@ def launches_per_step(wl, has_q: bool) -> int:
     kernel of each width class present (d <= 96, 96 < d <= 288, 288 < d <= 544,
     wider: that one after elim_open_kernel), with rows of 10..17 words in a call
     of at least 2^20 rows the hand-off check and the classes it can send back,
-    and the full-rank check (two kernels with 192 features or more and 2,048
-    rows); solve_kernel; per 2^25 queries the encode's fill and its seven kernels
-    (count, table, build, scan, scatter, runs, short), or one kernel for a pass
-    of at most 65,536 queries."""
+    and the full-rank check (two kernels where some context's features suit the
+    tensor cores, in a call of at least 2,048 rows); solve_kernel; per 2^25
+    queries the encode's fill and its seven kernels (count, table, build, scan,
+    scatter, runs, short), or one kernel for a pass of at most 65,536 queries."""
     wd = (wl.n_bits.astype(np.int64) + 1 + 31) // 32
     xw = (wl.n_bits.astype(np.int64) + 31) // 32
     small = wl.num_ctx <= 8192
     plan = 1 if small else 3
     taken_up = int((wd <= 3).any()) + int(((wd > 3) & (wd <= 9)).any()) + int(((wd > 9) & (wd <= 17)).any())
+    nb = wl.n_bits.astype(np.int64)
+    tensor = bool((2 * nb > 400 + 255 * ((nb + 255) // 256) + 195 * (xw % 4 != 0)).any())
     learn = 0
     for row_off, _ in wl.batches:
         rows = int(row_off[-1]) - int(row_off[0])
         learn += int(not small) + plan + 1 + int((xw > 9).any()) + plan + taken_up + 2 * int((wd > 17).any())
         if rows >= 1 << 20 and ((wd > 9) & (wd <= 17)).any():
             learn += 1 + taken_up
-        learn += 1 + int(wl.n_bits.max() >= 192 and rows >= 2048)
+        learn += 1 + int(tensor and rows >= 2048)
     nq = len(wl.queries.ctx_id) if has_q else 0
     enc = (1 if nq <= 65536 else 8 * ((nq + (1 << 25) - 1) >> 25)) if has_q else 0
     return 1 + learn + 1 + enc

@@ -340,7 +340,7 @@ enum f2_option {
                                     the contexts with at least 2048 representatives left that do not
                                     run against a lookup table */
     F2_OPT_FAIL_WAIT = 17,       /* test hook: 1: the waits of f2_learn_batched's tensor-core full-rank check
-                                    (192 features and more) act as if they had given up
+                                    (contexts of many features) act as if they had given up
                                     (F2_ERR_TIMEOUT); 0 (default): off */
 };
 int f2_set_option(f2_store* store, int option, int64_t value);

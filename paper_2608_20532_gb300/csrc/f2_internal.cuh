@@ -136,7 +136,8 @@ constexpr int PLAN_HIST_WORDS = 8192;  // key histogram of the plan kernels (>= 
 // rows of each width class of a store.
 struct Widths {
     int max_small_words = 0, max_narrow_words = 0, max_wide_m_d = 0, max_wide_d = 0;
-    int max_d = 0, max_n = 0, max_xw = 0;  // over every context (any may reach full rank)
+    int max_d = 0, max_xw = 0;  // over every context (any may reach full rank)
+    bool has_tensor = false;    // some context's features suit the tensor-core check
     bool has_small = false, has_narrow = false, has_wide_m = false, has_wide = false;
 };
 

@@ -24,13 +24,29 @@ struct FullArgs {
     int fail_wait;                    // test hook: verify_tc_kernel's waits for sums give up
 };
 
-// A context with n features and T rows to check goes to the tensor cores: the
-// table check costs d/4 lookups of 16 bytes a row, 0.71 ms for 4.2M rows of
-// 1,024 features, the tensor cores 0.49 ms; spreading the map over a CTA's
-// shared memory (128 bytes a feature) wants a few thousand rows to pay.
-constexpr int TC_MIN_N = 192;
+// Which check a context with n features and T rows takes.  By rows of 300
+// contexts with 16,384 each, the table check (n/4 lookups of 16 bytes a row)
+// takes 125 + 0.67 n us and the tensor check 255 + 85 for each chunk of 256
+// features, begun or whole, and 65 more where a feature row is not a multiple of
+// 16 bytes (one word a load instead of four).  Table / tensor: 256 features
+// 288 / 339 us, 384 379 / 423, 512 466 / 437, 544 492 / 581, 640 549 / 514,
+// 736 629 / 583, 768 632 / 516, 800 666 / 636, 1,000 793 / 598.  Its map (128 bytes a
+// feature, spread over a CTA's shared memory) wants rows, too: 600 contexts with
+// 4,096 rows of 512 features 269 / 270, of 1,024 443 / 360, with 2,048 rows 159 / 172
+// and 250 / 224; but where it runs at all, its CTAs' look through a list of 600
+// contexts that are not its own costs 20 us, so the line is not drawn above 2,048.
+constexpr int TC_CHUNK = 256;  // features of a chunk
 constexpr int TC_MIN_ROWS = 2048;
-__host__ __device__ __forceinline__ bool full_by_tensor(int n, int64_t T) { return n >= TC_MIN_N && T >= TC_MIN_ROWS; }
+__host__ __device__ __forceinline__ bool tensor_features(int n)
+{
+    const int chunks = (n + TC_CHUNK - 1) / TC_CHUNK;
+    const int odd = (((n + 31) / 32) & 3) ? 195 : 0;
+    return 2 * n > 400 + 255 * chunks + odd;
+}
+__host__ __device__ __forceinline__ bool full_by_tensor(int n, int64_t T)
+{
+    return T >= TC_MIN_ROWS && tensor_features(n);
+}
 
 cudaError_t verify_launch_tc(const StoreDev& sd, const FullArgs& fa, int num_sms, cudaStream_t cs);
 cudaError_t verify_load_tc();

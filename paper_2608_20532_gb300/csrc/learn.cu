@@ -1976,7 +1976,7 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
         fa.first = full_first;
         fa.table_words = FULL_TABLE_WORDS;
         fa.fail_wait = fail_wait;
-        fa.tensor = wv.max_n >= TC_MIN_N && total_rows >= TC_MIN_ROWS;
+        fa.tensor = wv.has_tensor && total_rows >= TC_MIN_ROWS;
         if (fa.tensor) {
             e = verify_launch_tc(sd, fa, num_sms, cs);
             if (e != cudaSuccess) return f2_cuda_status(e);
@@ -2003,7 +2003,7 @@ Widths width_summary(const int32_t* n_bits, int32_t num_ctx, bool raw)
         const int wd = (d + 31) / 32;
         const int words = elim_words(d, wd);
         if (d > w.max_d) w.max_d = d;
-        if (n_bits[c] > w.max_n) w.max_n = n_bits[c];
+        if (tensor_features(n_bits[c])) w.has_tensor = true;
         if ((n_bits[c] + 31) / 32 > w.max_xw) w.max_xw = (n_bits[c] + 31) / 32;
         if (wd <= SMALL_WD) {
             w.has_small = true;

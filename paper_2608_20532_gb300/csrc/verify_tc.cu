@@ -27,7 +27,7 @@ namespace {
 
 constexpr int TC_THREADS = 512;
 constexpr int TC_TILE = 128;       // rows of a tile: two threads of a group each
-constexpr int TC_KC = 256;         // features of a chunk (bytes of A, 64 columns of tensor memory)
+constexpr int TC_KC = TC_CHUNK;    // features of a chunk (bytes of A, 64 columns of tensor memory)
 constexpr int TC_KW = TC_KC / 64;  // its words for each of a row's two threads
 constexpr int TC_N = 128;          // bits of y
 // The order of the features along K is free, so the byte at 32 v + 4 w + j of a

@@ -65,6 +65,35 @@ def test_full_rank_by_tensor(raw, shift):
     st.close()
 
 
+@pytest.mark.parametrize("shift", [0, 1])
+def test_by_features_and_rows(shift):
+    """The smallest contexts that go to the tensor cores and the largest that
+    stay with the tables, by features (whole and begun chunks, feature rows of
+    whole 16-byte pieces and not) and by rows."""
+    dev = cuda_device()
+    binding = lib()
+    rng = np.random.default_rng(25 + shift)
+    n_bits, counts = [], []
+    for n in (455, 456, 480, 481, 512, 513, 609, 640, 641, 680, 681, 736, 768, 769, 807, 808, 864, 865, 1023, 1024):
+        for T in (2047, 2048, 5000):
+            n_bits.append(n)
+            counts.append(T)
+    maps = [(rng.integers(0, 2, (n, 128)).astype(np.float32), rng.integers(0, 2, 128)) for n in n_bits]
+    flips = [() if c % 5 == 0 else (0, 129, 2047, 2048, counts[c] - 1) for c in range(len(n_bits))]
+    nb = np.array(n_bits, np.int32)
+    st = binding.Store(nb, device=dev)
+    O = oracle.Oracle(nb)
+    for cnt, fl in (([n + 80 for n in n_bits], [()] * len(n_bits)), (counts, flips)):
+        ro, xo, x, y = _batch(rng, n_bits, cnt, maps, fl, shift)
+        ro_t, x_t, xo_t, y_t = dev_arrays(binding, dev, ro, x, xo, y)
+        st.learn(ro_t, x_t, xo_t, y_t)
+        O.learn(ro, xo, x, y)
+        torch.cuda.synchronize()
+        assert st.device_status() == binding.F2_OK
+        assert_basis_equal(binding, st.basis(), O.export())
+    st.close()
+
+
 @pytest.mark.parametrize("raw", [False, True])
 def test_a_wait_that_gives_up_commits_nothing(raw):
     """A call whose check gives up reports it and leaves the contradiction
@@ -74,8 +103,8 @@ def test_a_wait_that_gives_up_commits_nothing(raw):
     dev = cuda_device()
     binding = lib()
     rng = np.random.default_rng(15)
-    n_bits = [192, 257, 1024, 40]
-    wide = np.array(n_bits) >= 192
+    n_bits = [500, 768, 1024, 40]
+    wide = np.array(n_bits) >= 500
     maps = [(rng.integers(0, 2, (n, 128)).astype(np.float32), 0 if raw else rng.integers(0, 2, 128)) for n in n_bits]
     st = binding.Store(np.array(n_bits, np.int32), raw=raw, device=dev)
     O = oracle.Oracle(np.array(n_bits, np.int32), raw=raw)
@@ -91,11 +120,11 @@ def test_a_wait_that_gives_up_commits_nothing(raw):
     def state():
         return {k: binding.to_numpy(v).copy() for k, v in st.basis().items()}
 
-    learn([n + 80 for n in n_bits], [(), (330,), (), ()], O)  # one recorded already
+    learn([n + 80 for n in n_bits], [(), (840,), (), ()], O)  # one recorded already
     before = state()
     assert (before["rank"] == np.array(n_bits) + (0 if raw else 1)).all()
     st.set_option(binding.F2_OPT_FAIL_WAIT, 1)
-    learn([4300, 2048, 9000, 3000], [(0, 2100)] * 4, None)
+    learn([4300, 3000, 9000, 3000], [(0, 2100)] * 4, None)
     assert st.device_status() == binding.F2_ERR_TIMEOUT
     after = state()
     for k in ("contra", "first_contra", "n_contra", "rows_seen"):
@@ -104,7 +133,7 @@ def test_a_wait_that_gives_up_commits_nothing(raw):
     for k in ("rank", "pivot_mask", "basis_x", "basis_z"):
         assert np.array_equal(after[k], before[k]), k
     st.set_option(binding.F2_OPT_FAIL_WAIT, 0)
-    learn([4300, 2048, 9000, 0], [(7, 4000)] * 4, O)
+    learn([4300, 2731, 9000, 0], [(7, 4000)] * 4, O)
     assert st.device_status() == binding.F2_OK
     ref, got = O.export(), state()
     for k in ("rank", "contra", "first_contra", "n_contra", "rows_seen"):
