@@ -28,7 +28,8 @@ __global__ void __launch_bounds__(WIDE_WARPS * 32, WDT <= WIDE_M_WD ? 2 : 1) eli
 // contexts went from 3,012 to 2,256 us, and to 2,180 with four rows a barrier.
 // Dense rows are a few pivots short of full rank after d rows: up to OPEN_EXTRA
 // further rows are reduced one at a time by all threads (a XOR reduction of the
-// rows their bits select).
+// rows their bits select).  (Rows this wide are never deduplicated: each stands
+// for itself.)
 // ---------------------------------------------------------------------------
 constexpr int OPEN_THREADS = 1024;
 constexpr int OPEN_GROUP = 4;
@@ -158,17 +159,16 @@ __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, 
         }
         // rows without a pivot lie in the span of the rows before them
         if (t < n && pk < 0 && nonzero4(y)) {
-            atomicAdd(&sm.cnt, (unsigned long long)r.weight);
-            atomicMin(&sm.first, rs.seen + (long long)r.i);
+            atomicAdd(&sm.cnt, 1ull);
+            atomicMin(&sm.first, rs.seen + t);
         }
         int base = n;
         for (int extra = 0; rank < cd.d && base < rs.R && extra < OPEN_EXTRA; ++extra, ++base) {
             __syncthreads();
             uint4* const arow = sm.row[0][0];
             uint32_t* const acc = reinterpret_cast<uint32_t*>(arow);
-            const int i = rs.reps ? ld(rs.reps + base) : base;
             if (warp == 0) {
-                const uint32_t* xr = rs.xc + (int64_t)i * rs.xw;
+                const uint32_t* xr = rs.xc + (int64_t)base * rs.xw;
                 for (int w = lane; w < WIDE_WD + 3; w += 32) {
                     auto word = [&](int v) {
                         if (v < 0 || v >= rs.xw) return 0u;
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, 
                     sm.q[w] = q;
                 }
                 if (lane == 0) {
-                    arow[OPEN_Z] = ld(rs.yc + i);
+                    arow[OPEN_Z] = ld(rs.yc + base);
                     sm.holder = OPEN_THREADS;
                 }
             }
@@ -207,8 +207,8 @@ __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, 
             const uint4 z = arow[OPEN_Z];
             if (k < 0) {
                 if (t == 0 && nonzero4(z)) {
-                    sm.cnt += 1u + (rs.dups ? (uint32_t)ld(rs.dups + base) : 0u);
-                    if (rs.seen + (long long)i < sm.first) sm.first = rs.seen + (long long)i;
+                    ++sm.cnt;
+                    if (rs.seen + base < sm.first) sm.first = rs.seen + base;
                 }
                 continue;
             }
