@@ -1252,7 +1252,8 @@ __device__ __forceinline__ void elim_cta_queue(const StoreDev& s, const LearnArg
         if (item >= n) break;
         const int c = list[item];
         if (resume && width_class(s.desc[c].wd) != CLS) continue;
-        if (threadIdx.x == 0 && !resume) time_mark(a.timing, c, 2);
+        // (elim_open_kernel marks the start of the widest ones)
+        if (threadIdx.x == 0 && !resume && CLS != CLS_WIDE) time_mark(a.timing, c, 2);
         run(c);
         if (threadIdx.x == 0) time_mark(a.timing, c, 3);
     }

@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(OPEN_THREADS, 1) elim_open_kernel(StoreDev s, 
     const int32_t* const list = a.queue + a.counters[CNT_BEGIN + CLS_WIDE];
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         const int c = list[item];
+        if (t == 0) time_mark(a.timing, c, 2);
         if (s.rank[c] != 0) {
             if (t == 0) a.open_from[c] = 0;
             continue;

@@ -85,3 +85,23 @@ def test_opening(kind, raw):
         full = [c for c, (n, T) in enumerate(zip(n_bits, counts)) if n == 1024 and T > 1024]
         assert (ref["rank"][full] == 1025).all()
     st.close()
+
+
+def test_timing_includes_the_opening():
+    """The elimination's time of a wide context runs from its opening: 1,000
+    dense rows, which all go into it, take hundreds of microseconds there and a
+    few in the kernel after it."""
+    dev = cuda_device()
+    binding = lib()
+    rng = np.random.default_rng(4)
+    n_bits, counts = [1024, 40], [1000, 1000]
+    maps = [(rng.integers(0, 2, (n, 128)).astype(np.float32), rng.integers(0, 2, 128)) for n in n_bits]
+    st = binding.Store(np.array(n_bits, np.int32), device=dev)
+    st.set_option(binding.F2_OPT_TIMING, 1)
+    ro, xo, x, y = _batch(rng, n_bits, counts, ["dense"] * 2, maps)
+    ro_t, x_t, xo_t, y_t = dev_arrays(binding, dev, ro, x, xo, y)
+    st.learn(ro_t, x_t, xo_t, y_t)
+    times = st.learn_timing()
+    start, end = int(times[0, 2]), int(times[0, 3])
+    assert start and end - start > 200_000  # ns; 1,000 pivots of about 0.7 us
+    st.close()
