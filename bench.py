@@ -19,7 +19,6 @@ Other workloads: ``--config 1|2|5`` (learn + solve, plus encode for 1).
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import os
 import statistics
@@ -668,10 +667,9 @@ def run_ours(args):
                                 "alu_peak_ops_per_s": alu_peak,
                                 "peak_probe_lop3_ops_per_s": probe if probe else None},
     }
-    traffic = profile_traffic("f2_learn_batched")
     dom = rl_learn[learn_bound]
     roofline = {"bound": learn_bound, "achieved": dom["achieved"], "peak": dom["peak"], "unit": dom["unit"],
-                "frac": dom["frac"], "traffic": traffic,
+                "frac": dom["frac"], "traffic": None,  # no DRAM counters of a whole call are taken
                 "peak_source": peaks["source"] if learn_bound == "hbm" else
                 "derived: 152 SMs x 64 INT32 lanes x max SM clock"}
     result = {
@@ -709,7 +707,7 @@ def run_ours(args):
             # a reference rate; long runs are encoded with 4-bit tables instead
             "naive_alu_reference": {"ops_per_launch": ops_enc, "naive_ops_per_s": ops_enc / enc_mean,
                                     "alu_peak_ops_per_s": alu_peak},
-            "traffic": profile_traffic("f2_encode_batched"),
+            "traffic": None,
         }
     if verify is not None:
         ach = verify["rows_per_call"] * (16 + 4 * int(wl.n_bits.max() // 32)) / (verify["ms_per_call"] / 1e3)
@@ -768,35 +766,6 @@ def basis_bytes_touched(wl, store) -> int:
     d = wl.n_bits.astype(np.int64)[used] + 1
     wd = (d + 31) // 32
     return int((d * (16 + 4 * wd) + 4 * wd).sum())
-
-
-# the translation units of each library call's kernels
-KERNEL_SOURCES = {"f2_learn_batched": ("learn.cu", "elim.cuh", "elim_small.cu", "elim_narrow.cu", "elim_wide.cu",
-                                       "full.cuh", "verify_tc.cu", "f2_internal.cuh"),
-                  "f2_encode_batched": ("encode.cu", "f2_internal.cuh")}
-
-
-def kernel_source_hash(call: str) -> str:
-    h = hashlib.sha256()
-    csrc = os.path.join(ROOT, "paper_2608_20532_gb300", "csrc")
-    for f in KERNEL_SOURCES[call]:
-        with open(os.path.join(csrc, f), "rb") as fh:
-            h.update(fh.read())
-    return h.hexdigest()[:16]
-
-
-def profile_traffic(call: str):
-    """DRAM bytes per call from a committed ncu summary, if it was taken on
-    the current sources of that call's kernels (null otherwise)."""
-    p = os.path.join(ROOT, "profiles", "traffic.json")
-    if not os.path.exists(p):
-        return None
-    with open(p) as f:
-        d = json.load(f)
-    e = d.get(call)
-    if not e or e.get("source_hash") != kernel_source_hash(call):
-        return None
-    return e.get("dram_bytes_per_launch")
 
 
 # ------------------------------------------------------------ CPU oracle

@@ -48,3 +48,22 @@ def test_single_process_is_identity():
 
     assert bench.reduce_across_ranks(3.5, "max") == 3.5
     assert bench.reduce_across_ranks(7, "sum") == 7.0
+
+
+def test_profiles_hold_no_whole_step_counters():
+    """Counters other than durations come from one kernel of a small case: no
+    command of profiles/ captures them over every kernel of a step, and the
+    bench quotes no such figure."""
+    import re
+
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    for f in sorted(os.listdir(os.path.join(root, "profiles"))):
+        with open(os.path.join(root, "profiles", f)) as fh:
+            text = fh.read().replace("\\\n", " ")
+        for cmd in re.findall(r"ncu -[^\n]*", text):
+            assert "--clock-control none" in cmd, (f, cmd)
+            assert "--set full" not in cmd, (f, cmd)
+            if cmd.split("--metrics ")[-1].split()[0] != "gpu__time_duration.sum":
+                assert re.search(r"-k regex:\w+ -c [123] ", cmd) and "bench.py" not in cmd, (f, cmd)
+    with open(os.path.join(root, "bench.py")) as fh:
+        assert "profiles" not in fh.read()
