@@ -370,7 +370,7 @@ int f2_learn_timing(const f2_store* store, uint64_t* out_host, f2_stream_t strea
  * cudaFree or allocating library routine.  The caller owns every buffer;
  * the scheduling scratch (context descriptors, work queues, counters) lives
  * in one fixed, file-scope device array of the library, sized for
- * F2_NOALLOC_MAX_CTX contexts (about 0.9 MB), that every GPU which loads the
+ * F2_NOALLOC_MAX_CTX contexts (about 1.6 MB), that every GPU which loads the
  * library holds until the process exits.
  *
  *   num_ctx        in [0, F2_NOALLOC_MAX_CTX]; larger values are rejected

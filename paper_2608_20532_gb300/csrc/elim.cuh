@@ -159,7 +159,7 @@ __device__ __forceinline__ void group_sync()
 //
 // One group (a warp, or a whole CTA) streams the representatives of a context
 // through a basis in shared memory: slot k holds [z_k (4 words) | r_k], padded
-// to row_stride(WD) words.  Rows live in registers, one or two a lane.
+// to row_stride(WD) words.  Rows live in registers, one a lane (the opening: four).
 
 // The rows that a group streams, and one of them as loaded.
 struct RowStream {
@@ -191,27 +191,21 @@ __device__ __forceinline__ void fetch_row(const RowStream& rs, int base, int j, 
     load_raw<WD>(rs.xc + (int64_t)r.i * rs.xw, rs.yc + r.i, r.valid, rs.n, rs.xw, r.x, r.y);
 }
 
-// Step (1): XOR into each lane's K rows the stored rows of the pivots M that
-// the row has set.  A stored row never changes another pivot bit of M, so the
-// bit that selects row b is the row's own bit b however the rows are ordered:
-// the warp walks the union of its rows' pivots, two per step with their loads
-// issued together, every lane under its own bits.  A broadcast load and its
-// address serve the K rows of a lane.  Words that only pivots fill (not in
+// Step (1): XOR into each lane's row the stored rows of the pivots M that the
+// row has set.  A stored row never changes another pivot bit of M, so the bit
+// that selects row b is the row's own bit b however the rows are ordered: the
+// warp walks the union of its rows' pivots, two per step with their loads issued
+// together, every lane under its own bits.  Words that only pivots fill (not in
 // `mixed`) are never XOR-ed: the caller clears the pivot columns.
-template <int WD, int K>
-__device__ __forceinline__ void reduce_rows(uint32_t (&xr)[K][WD], uint4 (&yr)[K], const uint32_t* __restrict__ S,
+template <int WD>
+__device__ __forceinline__ void reduce_rows(uint32_t (&xr)[WD], uint4& yr, const uint32_t* __restrict__ S,
                                             const uint32_t (&M)[WD], uint64_t mixed)
 {
     constexpr int RS = row_stride(WD);
 #pragma unroll
     for (int w = 0; w < WD; ++w) {
-        uint32_t any = xr[0][w], sel[K];
-#pragma unroll
-        for (int t = 0; t < K; ++t) {
-            sel[t] = xr[t][w];
-            any |= sel[t];
-        }
-        uint32_t uw = __reduce_or_sync(FULL, any & M[w]);
+        const uint32_t sel = xr[w];
+        uint32_t uw = __reduce_or_sync(FULL, sel & M[w]);
         const bool xwork = (mixed & ((2ull << w) - 1ull)) != 0;
         while (uw) {
             const int b0 = __ffs(uw) - 1;
@@ -223,16 +217,12 @@ __device__ __forceinline__ void reduce_rows(uint32_t (&xr)[K][WD], uint4 (&yr)[K
             const uint32_t* row1 = S + (32 * w + b1) * RS;
             const uint4 z0 = *reinterpret_cast<const uint4*>(row0);
             const uint4 z1 = *reinterpret_cast<const uint4*>(row1);
-            uint32_t m0[K], m1[K];
-#pragma unroll
-            for (int t = 0; t < K; ++t) {
-                m0[t] = 0u - ((sel[t] >> b0) & 1u);
-                m1[t] = two ? 0u - ((sel[t] >> b1) & 1u) : 0u;
-                yr[t].x ^= (z0.x & m0[t]) ^ (z1.x & m1[t]);
-                yr[t].y ^= (z0.y & m0[t]) ^ (z1.y & m1[t]);
-                yr[t].z ^= (z0.z & m0[t]) ^ (z1.z & m1[t]);
-                yr[t].w ^= (z0.w & m0[t]) ^ (z1.w & m1[t]);
-            }
+            const uint32_t m0 = 0u - ((sel >> b0) & 1u);
+            const uint32_t m1 = two ? 0u - ((sel >> b1) & 1u) : 0u;
+            yr.x ^= (z0.x & m0) ^ (z1.x & m1);
+            yr.y ^= (z0.y & m0) ^ (z1.y & m1);
+            yr.z ^= (z0.z & m0) ^ (z1.z & m1);
+            yr.w ^= (z0.w & m0) ^ (z1.w & m1);
             if (xwork) {
 #pragma unroll
                 for (int v4 = 0; v4 <= w / 4; ++v4) {
@@ -244,10 +234,7 @@ __device__ __forceinline__ void reduce_rows(uint32_t (&xr)[K][WD], uint4 (&yr)[K
                     for (int j = 0; j < 4; ++j) {
                         const int v = 4 * v4 + j;
                         if (v <= w && v < WD)
-                            if ((mixed >> v) & 1ull) {
-#pragma unroll
-                                for (int t = 0; t < K; ++t) xr[t][v] ^= (ea[j] & m0[t]) ^ (eb[j] & m1[t]);
-                            }
+                            if ((mixed >> v) & 1ull) xr[v] ^= (ea[j] & m0) ^ (eb[j] & m1);
                     }
                 }
             }
@@ -731,71 +718,69 @@ __device__ int table_rounds(const LearnArgs& a, const RowStream& rs, ElimState<W
             st.first = min(st.first, idx);
         }
         bool inserted = false;
-        if constexpr (RW > 0) {
-            uint32_t c1 = __ballot_sync(FULL, valid && nz != 0u);
-            uint32_t xr[1][RW], N1[RW];
+        uint32_t c1 = __ballot_sync(FULL, valid && nz != 0u);
+        uint32_t xr[1][RW], N1[RW];
 #pragma unroll
-            for (int u = 0; u < RW; ++u) xr[0][u] = cr[u];
-            if constexpr (CTA) {
-                uint32_t wmask = publish_candidates(c1, wc, st.parity, warp, lane, G);
-                inserted = wmask != 0u;
-                while (wmask) {
-                    const int fw = __ffs(wmask) - 1;
-                    if (warp == fw) {
-                        (void)insert_rows<RW, RS>(xr, yr, c1, S, FL, lane, idx, weight, st.first, st.cnt, N1);
-                        if (lane < RW) {
-                            uint32_t t = 0;
+        for (int u = 0; u < RW; ++u) xr[0][u] = cr[u];
+        if constexpr (CTA) {
+            uint32_t wmask = publish_candidates(c1, wc, st.parity, warp, lane, G);
+            inserted = wmask != 0u;
+            while (wmask) {
+                const int fw = __ffs(wmask) - 1;
+                if (warp == fw) {
+                    (void)insert_rows<RW, RS>(xr, yr, c1, S, FL, lane, idx, weight, st.first, st.cnt, N1);
+                    if (lane < RW) {
+                        uint32_t t = 0;
 #pragma unroll
-                            for (int u = 0; u < RW; ++u)
-                                if (u == lane) t = N1[u];
-                            NPR[lane] = t;
-                        }
-                        c1 = 0u;
+                        for (int u = 0; u < RW; ++u)
+                            if (u == lane) t = N1[u];
+                        NPR[lane] = t;
                     }
-                    __syncthreads();
+                    c1 = 0u;
+                }
+                __syncthreads();
+#pragma unroll
+                for (int u = 0; u < RW; ++u) {
+                    N1[u] = NPR[u];
+                    n_new += __popc(N1[u]);
+                }
+                back_clear<RW, RS>(S, FL, NP, N1, lane, warp, G);
+                if (warp > fw && c1) {
 #pragma unroll
                     for (int u = 0; u < RW; ++u) {
-                        N1[u] = NPR[u];
-                        n_new += __popc(N1[u]);
-                    }
-                    back_clear<RW, RS>(S, FL, NP, N1, lane, warp, G);
-                    if (warp > fw && c1) {
+                        const uint32_t sel = xr[0][u];
+                        uint32_t uw = __reduce_or_sync(FULL, sel & N1[u]);
+                        while (uw) {
+                            const int b = __ffs(uw) - 1;
+                            uw &= uw - 1;
+                            const uint32_t* row = S + (int)FL[32 * u + b] * RS;
+                            if ((sel >> b) & 1u) {
+                                xor4(yr[0], *reinterpret_cast<const uint4*>(row));
 #pragma unroll
-                        for (int u = 0; u < RW; ++u) {
-                            const uint32_t sel = xr[0][u];
-                            uint32_t uw = __reduce_or_sync(FULL, sel & N1[u]);
-                            while (uw) {
-                                const int b = __ffs(uw) - 1;
-                                uw &= uw - 1;
-                                const uint32_t* row = S + (int)FL[32 * u + b] * RS;
-                                if ((sel >> b) & 1u) {
-                                    xor4(yr[0], *reinterpret_cast<const uint4*>(row));
-#pragma unroll
-                                    for (int v = 0; v <= u; ++v) xr[0][v] ^= row[4 + v];
-                                }
+                                for (int v = 0; v <= u; ++v) xr[0][v] ^= row[4 + v];
                             }
                         }
-                        uint32_t left = 0;
-#pragma unroll
-                        for (int u = 0; u < RW; ++u) left |= xr[0][u];
-                        if (((c1 >> lane) & 1u) && !left && nonzero4(yr[0])) {
-                            st.cnt += weight;
-                            st.first = min(st.first, idx);
-                        }
-                        c1 = __ballot_sync(FULL, left != 0u);
                     }
+                    uint32_t left = 0;
 #pragma unroll
-                    for (int u = 0; u < RW; ++u) NP[u] |= N1[u];
-                    wmask = publish_candidates(c1, wc, st.parity, warp, lane, G);
+                    for (int u = 0; u < RW; ++u) left |= xr[0][u];
+                    if (((c1 >> lane) & 1u) && !left && nonzero4(yr[0])) {
+                        st.cnt += weight;
+                        st.first = min(st.first, idx);
+                    }
+                    c1 = __ballot_sync(FULL, left != 0u);
                 }
-            } else if (c1) {
-                inserted = true;
-                n_new += insert_rows<RW, RS>(xr, yr, c1, S, FL, lane, idx, weight, st.first, st.cnt, N1);
-                back_clear<RW, RS>(S, FL, NP, N1, lane, 0, 1);
-                __syncwarp();
 #pragma unroll
                 for (int u = 0; u < RW; ++u) NP[u] |= N1[u];
+                wmask = publish_candidates(c1, wc, st.parity, warp, lane, G);
             }
+        } else if (c1) {
+            inserted = true;
+            n_new += insert_rows<RW, RS>(xr, yr, c1, S, FL, lane, idx, weight, st.first, st.cnt, N1);
+            back_clear<RW, RS>(S, FL, NP, N1, lane, 0, 1);
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < RW; ++u) NP[u] |= N1[u];
         }
         st.base = step_to(st.base, nt, rs.R);
         if constexpr (CTA) {
@@ -809,36 +794,34 @@ __device__ int table_rounds(const LearnArgs& a, const RowStream& rs, ElimState<W
         spent += n_new;
         if (n_new && spent > (CTA ? 64 : 4 * np)) break;  // a new table pays
     }
-    if constexpr (RW > 0) {
-        if (n_new) {
-            // N into the basis: full residuals, then step (5) on the older rows
-            uint32_t NF[WD];
+    if (n_new) {
+        // N into the basis: full residuals, then step (5) on the older rows
+        uint32_t NF[WD];
 #pragma unroll
-            for (int v = 0; v < WD; ++v) NF[v] = 0u;
+        for (int v = 0; v < WD; ++v) NF[v] = 0u;
 #pragma unroll
-            for (int u = 0; u < RW; ++u) {
-                const bool mine = (NP[u] >> lane) & 1u;
-                const int coord = mine ? (int)FL[32 * u + lane] : 0;
-                if (mine && (!CTA || u % G == warp)) {
-                    uint32_t* row = S + coord * RS;
-                    uint32_t c[RW], xf[WD];
+        for (int u = 0; u < RW; ++u) {
+            const bool mine = (NP[u] >> lane) & 1u;
+            const int coord = mine ? (int)FL[32 * u + lane] : 0;
+            if (mine && (!CTA || u % G == warp)) {
+                uint32_t* row = S + coord * RS;
+                uint32_t c[RW], xf[WD];
 #pragma unroll
-                    for (int v = 0; v < RW; ++v) c[v] = row[4 + v];
-                    decompress_residual<WD, RW>(c, FL, xf);
+                for (int v = 0; v < RW; ++v) c[v] = row[4 + v];
+                decompress_residual<WD, RW>(c, FL, xf);
 #pragma unroll
-                    for (int v = 0; v < WD; ++v) row[4 + v] = xf[v];
-                }
-#pragma unroll
-                for (int v = 0; v < WD; ++v)
-                    NF[v] |= __reduce_or_sync(FULL, (mine && (coord >> 5) == v) ? 1u << (coord & 31) : 0u);
+                for (int v = 0; v < WD; ++v) row[4 + v] = xf[v];
             }
-            group_sync<CTA>();
-            back_clear<WD, RS>(S, nullptr, st.P, NF, lane, warp, G);
-            group_sync<CTA>();
 #pragma unroll
-            for (int v = 0; v < WD; ++v) st.P[v] |= NF[v];
-            st.rank += n_new;
+            for (int v = 0; v < WD; ++v)
+                NF[v] |= __reduce_or_sync(FULL, (mine && (coord >> 5) == v) ? 1u << (coord & 31) : 0u);
         }
+        group_sync<CTA>();
+        back_clear<WD, RS>(S, nullptr, st.P, NF, lane, warp, G);
+        group_sync<CTA>();
+#pragma unroll
+        for (int v = 0; v < WD; ++v) st.P[v] |= NF[v];
+        st.rank += n_new;
     }
     return snap_at;
 }
@@ -948,7 +931,7 @@ __device__ __forceinline__ void walk_round(const RowStream& rs, ElimState<WD>& s
     uint4 yr[1] = {r.y};
     const long long idx = rs.seen + r.i;
     make_q<WD>(r.x, r.valid, rs.raw, xr[0]);
-    if (st.rank) reduce_rows<WD, 1>(xr, yr, S, st.P, mixed_words<WD>(st.P, d, wd));
+    if (st.rank) reduce_rows<WD>(xr[0], yr[0], S, st.P, mixed_words<WD>(st.P, d, wd));
     uint32_t nz = 0;
 #pragma unroll
     for (int v = 0; v < WD; ++v) {
@@ -1120,7 +1103,7 @@ __device__ void elim_cta(const StoreDev& s, const LearnArgs& a, int c, uint32_t*
         const uint32_t weight = nx.weight;
         make_q<WD>(nx.x, valid, rs.raw, xr[0]);
         fetch_row<WD>(rs, st.base, nt + t, nx);
-        if (st.rank) reduce_rows<WD, 1>(xr, yr, S, st.P, mixed);
+        if (st.rank) reduce_rows<WD>(xr[0], yr[0], S, st.P, mixed);
         uint32_t nz = 0;
 #pragma unroll
         for (int v = 0; v < WD; ++v) {
@@ -1158,7 +1141,7 @@ __device__ void elim_cta(const StoreDev& s, const LearnArgs& a, int c, uint32_t*
             }
             back_clear<WD, RS>(S, nullptr, st.P, NP, lane, warp, G);
             if (warp > fw && cand) {
-                reduce_rows<WD, 1>(xr, yr, S, NP, ~0ull);
+                reduce_rows<WD>(xr[0], yr[0], S, NP, ~0ull);
                 uint32_t left = 0;
 #pragma unroll
                 for (int v = 0; v < WD; ++v) left |= xr[0][v];

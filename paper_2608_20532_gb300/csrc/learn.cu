@@ -129,7 +129,6 @@ constexpr int DD_SEG_ROWS = 16384;              // rows a CTA takes at a time (1
 constexpr int DD_QUAD_REPS = 1024;              // most distinct rows numbered by a quad, by a CTA (as above)
 constexpr int DD_CTA_REPS = 4096;
 constexpr int DD_AHEAD_XW = 5;                  // widest rows whose next round is loaded ahead
-constexpr int DD_K = 1;                         // rows per thread per round
 constexpr int DD_XW = NARROW_WD;                // widest feature row (words) of dedup_kernel<false>
 constexpr int DD_XW_WIDE = 16;                  // widest of dedup_kernel<true> (one row in flight)
 constexpr int DEDUP_PROBES = 8;                 // linear-probe limit
@@ -363,7 +362,7 @@ __device__ bool dd_finish(const DedupArgs& a, int c, int nrep, int t)
 // One group of G warps finds the representatives of context c and writes
 // them, in stream order, to rep_list[row_off[c] + k] with their duplicate
 // counts in rep_dup; rep_count[c] = number of representatives.  Each thread
-// takes DD_K rows a round.  Table slot: (fingerprint, smallest row index
+// takes a row a round.  Table slot: (fingerprint, smallest row index
 // of that content) plus a duplicate counter; a full row comparison decides
 // every match, so a row is a duplicate only if it equals an earlier row.
 //
@@ -414,134 +413,98 @@ __device__ bool dedup_ctx(const StoreDev& s, const DedupArgs& a, int c, uint32_t
     // once instead: 77,926 contexts 2,607 against 2,505 us, 4,096 contexts 284
     // against 275).
     constexpr bool AHEAD = XW <= DD_AHEAD_XW;
-    constexpr int K = DD_K;
-    uint4 yn[K];
-    uint32_t xn[K][XW];
+    uint4 yn;
+    uint32_t xn[XW];
     auto load_round = [&](uint32_t base) {
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-            const uint32_t i = base + (uint32_t)(j * NT + t);
-            const int ic = i < Tu ? (int)i : T - 1;  // (a row read twice, not counted)
-            yn[j] = ld(yc + ic);
-            load_words<XW>(xc + (int64_t)ic * XW, al, xn[j]);
-        }
+        const uint32_t i = base + (uint32_t)t;
+        const int ic = i < Tu ? (int)i : T - 1;  // (a row read twice, not counted)
+        yn = ld(yc + ic);
+        load_words<XW>(xc + (int64_t)ic * XW, al, xn);
     };
     if (AHEAD) load_round(0);
-    for (uint32_t base = 0; base < Tu; base += NT * K) {
-        int mine[K];
-        uint32_t h[K];
-        uint4 yv[K];
-        uint32_t xv[K][XW];
+    for (uint32_t base = 0; base < Tu; base += NT) {
         if (!AHEAD) load_round(base);
+        const uint32_t i = base + (uint32_t)t;
+        const bool valid = i < Tu;
+        const uint4 yv = yn;
+        uint32_t xv[XW];
 #pragma unroll
-        for (int j = 0; j < K; ++j) {
-            yv[j] = yn[j];
-#pragma unroll
-            for (int v = 0; v < XW; ++v) xv[j][v] = (v == XW - 1) ? xn[j][v] & lm : xn[j][v];
-        }
-        if (AHEAD) load_round(base + NT * K);
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-            h[j] = dd_hash<XW>(xv[j], yv[j]);
-        }
+        for (int v = 0; v < XW; ++v) xv[v] = (v == XW - 1) ? xn[v] & lm : xn[v];
+        if (AHEAD) load_round(base + NT);
+        const uint32_t h = dd_hash<XW>(xv, yv);
         // probe by fingerprint only (shared memory): the first slot holding
         // this fingerprint, or an empty slot that the row then claims
-        uint2 ent[K];
-        uint32_t cs[K];
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-            const uint32_t i = base + (uint32_t)(j * NT + t);
-            mine[j] = (i < Tu) ? -2 : -1;  // -2 = unresolved
-            ent[j] = make_uint2(0u, 0u);
-            cs[j] = 0u;
-            if (i < Tu) {
-                const uint32_t fp = h[j] | 1u;
-                uint32_t slot = (h[j] >> 7) & emask;
-                int p = 0;
-                for (; p < DEDUP_PROBES; ++p, slot = (slot + 1) & emask) {
-                    uint2 e = tab[slot];
-                    if (e.x == 0u) {
-                        const unsigned long long want = ((unsigned long long)i << 32) | fp;
-                        const unsigned long long old =
-                            atomicCAS(reinterpret_cast<unsigned long long*>(tab + slot), 0ull, want);
-                        if (old == 0ull) {
-                            mine[j] = (int)slot;
-                            break;
-                        }
-                        e.x = (uint32_t)old;
-                        e.y = (uint32_t)(old >> 32);
-                    }
-                    if (e.x == fp) {
-                        ent[j] = e;
-                        cs[j] = slot;
+        int mine = valid ? -2 : -1;  // -2 = unresolved
+        uint2 ent = make_uint2(0u, 0u);
+        uint32_t cs = 0u;
+        if (valid) {
+            const uint32_t fp = h | 1u;
+            uint32_t slot = (h >> 7) & emask;
+            int p = 0;
+            for (; p < DEDUP_PROBES; ++p, slot = (slot + 1) & emask) {
+                uint2 e = tab[slot];
+                if (e.x == 0u) {
+                    const unsigned long long want = ((unsigned long long)i << 32) | fp;
+                    const unsigned long long old =
+                        atomicCAS(reinterpret_cast<unsigned long long*>(tab + slot), 0ull, want);
+                    if (old == 0ull) {
+                        mine = (int)slot;
                         break;
                     }
+                    e.x = (uint32_t)old;
+                    e.y = (uint32_t)(old >> 32);
                 }
-                if (p == DEDUP_PROBES) mine[j] = -1;  // table region full: own representative
+                if (e.x == fp) {
+                    ent = e;
+                    cs = slot;
+                    break;
+                }
             }
+            if (p == DEDUP_PROBES) mine = -1;  // table region full: own representative
         }
-        // full comparison with the fingerprint matches: every load first
-        bool need[K];
-        uint4 yo[K];
-        uint32_t xo[K][XW];
+        // full comparison with the row of that fingerprint
+        const bool need = mine == -2;
+        uint4 yo = make_uint4(0, 0, 0, 0);
+        uint32_t xo[XW];
 #pragma unroll
-        for (int j = 0; j < K; ++j) {
-            need[j] = mine[j] == -2;
-            const int64_t o = need[j] ? (int64_t)ent[j].y : 0;
-            yo[j] = make_uint4(0, 0, 0, 0);
-#pragma unroll
-            for (int v = 0; v < XW; ++v) xo[j][v] = 0u;
-            if (need[j]) {
-                yo[j] = ld(yc + o);
-                load_words<XW>(xc + o * XW, al, xo[j]);
-            }
+        for (int v = 0; v < XW; ++v) xo[v] = 0u;
+        if (need) {
+            yo = ld(yc + ent.y);
+            load_words<XW>(xc + (int64_t)ent.y * XW, al, xo);
         }
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-            if (!need[j]) continue;
-            bool e = yo[j].x == yv[j].x && yo[j].y == yv[j].y && yo[j].z == yv[j].z && yo[j].w == yv[j].w;
+        if (need) {
+            bool e = yo.x == yv.x && yo.y == yv.y && yo.z == yv.z && yo.w == yv.w;
 #pragma unroll
             for (int v = 0; v < XW; ++v) {
-                const uint32_t w = (v == XW - 1) ? (xo[j][v] & lm) : xo[j][v];
-                e = e && (w == xv[j][v]);
+                const uint32_t w = (v == XW - 1) ? (xo[v] & lm) : xo[v];
+                e = e && (w == xv[v]);
             }
-            const uint32_t i = base + (uint32_t)(j * NT + t);
             if (e) {
-                if (i < ent[j].y) atomicMin(&tab[cs[j]].y, (uint32_t)i);
-                mine[j] = (int)cs[j];
+                if (i < ent.y) atomicMin(&tab[cs].y, i);
+                mine = (int)cs;
             } else {  // a different row with the same fingerprint: keep probing
-                mine[j] = dd_find_insert(tab, E, h[j], i, yv[j], xc, yc, XW, n, (cs[j] + 1) & emask,
-                                         DEDUP_PROBES - 1);
+                mine = dd_find_insert(tab, E, h, i, yv, xc, yc, XW, n, (cs + 1) & emask, DEDUP_PROBES - 1);
             }
         }
         dd_sync<G>();
-        uint32_t bal[K];
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-            const uint32_t i = base + (uint32_t)(j * NT + t);
-            const bool valid = i < Tu;
-            const uint32_t rep = (valid && mine[j] >= 0) ? tab[mine[j]].y : i;
-            const bool isrep = valid && rep == i;
-            if (valid && !isrep) atomicAdd(D + mine[j], 1);
-            bal[j] = __ballot_sync(FULL, isrep);
-            if (G > 1 && lane == 0) wcnt[gw * K + j] = __popc(bal[j]);
+        const uint32_t rep = (valid && mine >= 0) ? tab[mine].y : i;
+        const bool isrep = valid && rep == i;
+        if (valid && !isrep) atomicAdd(D + mine, 1);
+        const uint32_t bal = __ballot_sync(FULL, isrep);
+        int before = 0, total = __popc(bal);
+        if (G > 1) {
+            if (lane == 0) wcnt[gw] = total;
+            dd_sync<G>();
+            const int v = lane < G ? wcnt[lane] : 0;
+            total = __reduce_add_sync(FULL, v);
+            before = __reduce_add_sync(FULL, lane < gw ? v : 0);
         }
-        if (G > 1) dd_sync<G>();
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-            int before = 0, total = __popc(bal[j]);
-            if (G > 1) {
-                const int v = lane < G ? wcnt[lane * K + j] : 0;
-                total = __reduce_add_sync(FULL, v);
-                before = __reduce_add_sync(FULL, lane < gw ? v : 0);
-            }
-            if ((bal[j] >> lane) & 1u) {
-                const int pos = nrep + before + __popc(bal[j] & ((1u << lane) - 1u));
-                a.rep_list[r0 + pos] = (int32_t)(base + (uint32_t)(j * NT + t));  // within the shard (see below)
-                a.rep_dup[r0 + pos] = mine[j];
-            }
-            nrep += total;
+        if (isrep) {
+            const int pos = nrep + before + __popc(bal & ((1u << lane) - 1u));
+            a.rep_list[r0 + pos] = (int32_t)i;  // within the shard
+            a.rep_dup[r0 + pos] = mine;
         }
+        nrep += total;
         // (the next round's first barrier comes before it writes wcnt again)
     }
     dd_sync<G>();
@@ -662,7 +625,7 @@ __device__ __forceinline__ bool dd_same(const DdSmem& m, int r, const uint32_t (
 
 // The distinct rows among T <= DD_SEG_ROWS rows, by a group of G warps: their
 // indices (plus `off`), in stream order, and repeats go to rep / dups; returns
-// their number.  Each thread takes K rows a round and no round waits for
+// their number.  Each thread takes a row a round and no round waits for
 // another, so the warps hide each other's latencies; the first rows are put in
 // order at the end, through a bitmap.
 template <int G, int XW>
@@ -855,7 +818,7 @@ __global__ void __launch_bounds__(DD_THREADS, DD_CTAS_PER_SM) dedup_kernel(Store
     constexpr int C_WARP = WX ? CLS_DDW_WARP : CLS_DD_WARP;
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ int s_item[DD_WARPS];
-    __shared__ int wcnt[DD_WARPS * DD_K];
+    __shared__ int wcnt[DD_WARPS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (a.counters[CNT_DEDUPED] == 0) return;
     {
@@ -906,8 +869,8 @@ __global__ void __launch_bounds__(DD_THREADS, DD_CTAS_PER_SM) dedup_kernel(Store
             const int T = (int)(a.row_off[c + 1] - a.row_off[c]);
             const int E = table_entries(T, DD_QUAD_E);
             if ((warp & 3) == 0 && lane == 0) time_mark(a.timing, c, 0);
-#define F2_DD_QUAD(W) dedup_ctx<4, W>(s, a, c, region, E, wcnt + q * 4 * DD_K)
-#define F2_DDW_QUAD(W) dedup_wide_ctx<4, W>(s, a, c, q * 4 * DD_WARP_REGION, wcnt + q * 4 * DD_K)
+#define F2_DD_QUAD(W) dedup_ctx<4, W>(s, a, c, region, E, wcnt + q * 4)
+#define F2_DDW_QUAD(W) dedup_wide_ctx<4, W>(s, a, c, q * 4 * DD_WARP_REGION, wcnt + q * 4)
             if constexpr (WX) {
                 F2_XWIDE_SWITCH(s.desc[c].xw, F2_DDW_QUAD)
             } else {
@@ -1834,12 +1797,6 @@ __global__ void __launch_bounds__(FULL_THREADS) verify_full_kernel(StoreDev s, F
 constexpr int64_t HANDOFF_AUTO_ROWS = int64_t(1) << 20;
 constexpr int HANDOFF_AUTO_REPS = 2048;
 
-// Which elimination kernels a store needs, and their widest bases.
-
-// Calls of at least this many rows run the 4..9-word elimination in CTAs of
-// four warps (see elim_narrow_kernel; F2_OPT_LONG_CALL_ROWS).
-constexpr int64_t LONG_CALL_ROWS = DEFAULT_LONG_CALL_ROWS;
-
 // A second stream for kernels that work on disjoint contexts: the first
 // such kernel goes to `aux` (forked from the caller's stream), the others to
 // the caller's stream, and join() makes the caller's stream wait for `aux`.
@@ -1873,7 +1830,7 @@ int launch_elimination(const StoreDev& sd, const LearnArgs& la, const int64_t* r
                        int64_t warp_work, int32_t* queue, int32_t* keybuf, int* hist, int num_sms,
                        const Widths& wv, int* full_ctr, unsigned long long* full_cnt,
                        unsigned long long* full_first, cudaStream_t cs, Fork* fk = nullptr, int scale = 0,
-                       bool prezeroed = false, int64_t long_rows = LONG_CALL_ROWS, const CheckArgs* check = nullptr,
+                       bool prezeroed = false, int64_t long_rows = DEFAULT_LONG_CALL_ROWS, const CheckArgs* check = nullptr,
                        const PlanZero& zero = PlanZero{}, int fail_wait = 0)
 {
     // prezeroed: the caller has cleared full_ctr's first 2C words and late
