@@ -84,7 +84,8 @@ constexpr int DEFAULT_WARP_REGION_BYTES = 13824;  // shared memory of one warp-o
 constexpr int DEFAULT_SMALL_REGION_BYTES = 9472;  // the same in the small-width kernel (d <= 96)
 constexpr int64_t DEFAULT_ENCODE_DIRECT_MAX = 65536;  // encode passes this small skip the grouping
 constexpr int64_t DEFAULT_LONG_CALL_ROWS = int64_t(1) << 25;  // learn calls this long: 4-warp CTAs (4..9 words)
-constexpr int64_t DEFAULT_HANDOFF_REPS = -1;  // representatives left for a saturated context to hand off (0: never, -1: by the call's work)
+// representatives left for a saturated context to hand off (0: never, -1: by the call and the store)
+constexpr int64_t DEFAULT_HANDOFF_REPS = -1;
 constexpr int DEFAULT_HEAVY_ROWS = 4096;          // rows from which a context gets a whole CTA (at most)
 constexpr int HEAVY_ROWS_MIN = 1024;              // ... and at least, when it scales with the batch:
 constexpr int HEAVY_ROWS_BATCH_DIV = 20000;       // batch rows / this (no duplicate pass), or
@@ -129,8 +130,8 @@ enum Class {
     NUM_CLASSES = 16
 };
 static_assert(NUM_CLASSES <= CNT_BEGIN - CNT_HEAD, "counter blocks hold one entry per class");
-constexpr int SMALL_WD = 3;
-constexpr int PLAN_HIST_WORDS = 8192;  // key histogram of the plan kernels (>= number of keys)  // contexts of d <= 96 bits: fewer registers, twice the warps per SM
+constexpr int SMALL_WD = 3;  // contexts of d <= 96 bits: fewer registers, more warps per SM
+constexpr int PLAN_HIST_WORDS = 8192;  // key histogram of the plan kernels (>= number of keys)
 
 // Shared-memory and kernel selection of the elimination launches: the widest
 // rows of each width class of a store.
@@ -412,8 +413,8 @@ struct f2_store {
     int dd_shards;              // most CTAs one context's duplicate pass is split over
     int64_t enc_direct_max;     // encode passes of at most this many queries skip the grouping
     int64_t long_call_rows;     // learn calls of at least this many rows: 4-warp CTAs for 4..9-word contexts
-    int64_t handoff_min;        // representatives left for a saturated context to hand off (0: never, -1: by the call's work)
-    int* hand;                  // hand-off lists: counts [2], snap list/start [2C], resume list/from [2C], chunk counters [2C]
+    int64_t handoff_min;        // representatives left for a saturated context to hand off (as DEFAULT_HANDOFF_REPS)
+    int* hand;                  // hand-off: counts [2], snap list/start [2C], resume list/from [2C], chunk counters [2C]
     uint4* check_rec;           // the check's chunk records (2 x uint4 each), grown per call
     int64_t check_rec_cap;
     f2::Widths widths;      // width classes of the contexts (computed on first use)

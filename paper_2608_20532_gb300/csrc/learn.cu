@@ -70,9 +70,9 @@ namespace {
 // 10,000 contexts of 128..512 bits of parsed values, 13.4M rows: 443 us while
 // every CTA claimed its way through the whole list of contexts, an atomic each,
 // a row's words were loaded one by one and every basis row was XOR-ed whole;
-// 190 without that (45% of the issue slots; warps wait at the barriers of a
-// chunk and for its rows).  Two rows a lane made no difference, nor fewer
-// barriers a chunk.
+// 190 without that, 228 now that it is handed every long context that walks its
+// pivots (41..48% of the issue slots; warps wait at the barriers of a chunk and
+// for its rows).  Two rows a lane made no difference, nor fewer barriers a chunk.
 // ---------------------------------------------------------------------------
 struct CheckArgs {
     const int64_t* row_off;

@@ -300,8 +300,8 @@ namespace {
 // Copies of several device arrays in one launch.  A small store's arrays are
 // a few KB each, so eight copies cost eight launches' latency and little
 // else: a 256-context reset + learn + solve + basis went from 102 to 85 us, a
-// 77,926-context one (126 MB of basis) from 2,771 to 2,726.  Whole 16-byte words where both ends are 16-byte aligned, bytes
-// otherwise and at the tail.
+// 77,926-context one (126 MB of basis) from 2,771 to 2,726.  Whole 16-byte words
+// where both ends are 16-byte aligned, bytes otherwise and at the tail.
 struct CopyList {
     static constexpr int MAX = 8;
     void* dst[MAX];

@@ -15,7 +15,7 @@
 // shared memory binds; here 0.66 ms with one thread a row (ten instructions to
 // spread four bits and pack a parity, two warps a scheduler), 0.62 with two,
 // 0.54 with one mask a word and parities taken from sign bits.  The products
-// take 64 cycles each, 0.22 ms in all (tensor pipe 46% active).  Rows read by
+// take 64 cycles each, 0.22 ms in all (tensor pipe 45% active).  Rows read by
 // their own threads, four words at a time 4 * xw bytes apart, cost two batches
 // of 65,536 rows a context 1,864 us; read a tile ahead, coalesced, and staged in
 // shared memory, 1,830.  The kernel now takes 0.49 ms.
